@@ -901,7 +901,7 @@ cudaError_t launch(const TcParams& p, cudaStream_t stream, int sms, bool f16) {
 namespace ppc {
 
 pp_status tc_prepare() {
-  if (prepare() != cudaSuccess || device_sms() <= 0) return PP_ERR_CUDA;
+  if (prepare() != cudaSuccess || device_sms() <= 0 || tcr_prepare() != PP_OK) return PP_ERR_CUDA;
   // the entry point is process-wide; looked up at the first set-up of each device
   const cudaError_t e = g_encode_once.run([](int) {
     void* fn = nullptr;
@@ -1047,7 +1047,7 @@ pp_status tc_build16(TcLayout* T, const pp_packed* pk, float input_bound, cudaSt
   return PP_OK;
 }
 
-// Geometry the launch will use: orientation and tile width for a map width.
+// Geometry the row-tiled kernel would use: orientation and tile width for a map width.
 void tc_geometry(const TcLayout& T, int W, bool pool, int* ori, int* tw) {
   const bool f16 = T.f16;
   // a pixel-major tile with 128 filters holds one output row (its accumulator
@@ -1094,6 +1094,10 @@ pp_status tc_launch(const TcLayout& T, const LayerMeta& M, const float* x, float
   p.flags = flags;
   int ori, tw;
   tc_geometry(T, W, (flags & PP_POOL2) != 0, &ori, &tw);
+  if (ori != ORI_FP && tcr_applicable(T, M.Ci, N, H, ori == ORI_PFR)) {
+    const pp_status st = tcr_launch(T, M, x, y, skip, N, H, W, flags, stream);
+    if (st != PP_ERR_UNSUPPORTED) return st;
+  }
   const int sms = device_sms();
   cudaError_t e;
   if (ori == ORI_PF)

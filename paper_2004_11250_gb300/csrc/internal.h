@@ -115,6 +115,13 @@ pp_status tc_status(const TcLayout& T, int* device_error);
 // Build the f16 tiles and scales (precision PP_PRECISION_F16X3) for inputs bounded by input_bound.
 pp_status tc_build16(TcLayout* T, const pp_packed* pk, float input_bound, cudaStream_t stream);
 void tc_free(TcLayout* T);
+// Layers with at most 64 filters and 64 input channels: weights resident in shared memory, CTA pairs (conv_tcr.cu);
+// returns PP_ERR_UNSUPPORTED for others and where pairs cannot be launched.  narrow: the row-tiled kernel would
+// flatten the map's rows.
+bool tcr_applicable(const TcLayout& T, int Ci, int N, int H, bool narrow);
+pp_status tcr_prepare();
+pp_status tcr_launch(const TcLayout& T, const LayerMeta& M, const float* x, float* y, const float* skip, int N, int H,
+                     int W, int flags, cudaStream_t stream);
 // Flat variant (maps up to 128 pixels wide, 128-filter blocks); returns
 // PP_ERR_UNSUPPORTED for shapes it does not handle.
 pp_status tcf_launch(const TcLayout& T, const LayerMeta& M, const float* x, float* y, const float* skip, int N,

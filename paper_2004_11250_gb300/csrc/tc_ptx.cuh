@@ -82,6 +82,8 @@ __device__ __forceinline__ void tm_ld8(uint32_t ta, float (&v)[8]) {
                : "=f"(v[0]), "=f"(v[1]), "=f"(v[2]), "=f"(v[3]), "=f"(v[4]), "=f"(v[5]), "=f"(v[6]), "=f"(v[7])
                : "r"(ta));
 }
+__device__ __forceinline__ void tm_ld(uint32_t ta, float (&v)[16]) { tm_ld16(ta, v); }
+__device__ __forceinline__ void tm_ld(uint32_t ta, float (&v)[8]) { tm_ld8(ta, v); }
 __device__ __forceinline__ void mma_tf32(uint32_t d, uint64_t a, uint64_t b, uint32_t id, uint32_t acc) {
   asm volatile(
       "{ .reg .pred p; setp.ne.b32 p, %4, 0; tcgen05.mma.cta_group::1.kind::tf32 [%0], %1, %2, %3, p; }" ::"r"(d),
@@ -134,6 +136,37 @@ __device__ __forceinline__ void mbar_arrive_remote(uint32_t cluster_addr) {
   asm volatile("mbarrier.arrive.release.cluster.shared::cluster.b64 _, [%0];" ::"r"(cluster_addr) : "memory");
 }
 
+// the same with the default scope: hands over operands that the async proxy reads (after fence.proxy.async) or
+// tensor memory; it does not wait for the thread's global stores, as the cluster-scope release does
+__device__ __forceinline__ void mbar_arrive_pair(uint32_t cluster_addr) {
+  asm volatile("mbarrier.arrive.shared::cluster.b64 _, [%0];" ::"r"(cluster_addr) : "memory");
+}
+
+// Two fp32 operations per instruction (each element rounded as the scalar one).
+__device__ __forceinline__ uint64_t pack2(float a, float b) {
+  uint64_t r;
+  asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(a), "f"(b));
+  return r;
+}
+__device__ __forceinline__ void unpack2(uint64_t v, float& a, float& b) {
+  asm("mov.b64 {%0, %1}, %2;" : "=f"(a), "=f"(b) : "l"(v));
+}
+__device__ __forceinline__ uint64_t add2(uint64_t a, uint64_t b) {
+  uint64_t r;
+  asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+  return r;
+}
+__device__ __forceinline__ uint64_t mul2(uint64_t a, uint64_t b) {
+  uint64_t r;
+  asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+  return r;
+}
+__device__ __forceinline__ uint64_t fma2(uint64_t a, uint64_t b, uint64_t c) {
+  uint64_t r;
+  asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
+  return r;
+}
+
 // tf32 split of an fp32 value: hi keeps the sign, exponent and 10 explicit
 // mantissa bits (exact in tf32); lo = v - hi is exact in fp32.
 __device__ __forceinline__ float tf32_hi(float v) { return __uint_as_float(__float_as_uint(v) & 0xFFFFE000u); }
@@ -161,6 +194,33 @@ __device__ __forceinline__ uint32_t split_f16x8(const float* v, float sc, uint4&
   h = make_uint4(hw[0], hw[1], hw[2], hw[3]);
   l = make_uint4(lw[0], lw[1], lw[2], lw[3]);
   return bad;
+}
+
+// The same split with packed fp32 operations and the range test as a running maximum of |hi| (NaN propagates): the
+// caller tests the result with f16_max_bad once at the end.
+__device__ __forceinline__ void split_f16x8_max(const float* v, float sc, uint4& h, uint4& l, __half2& mx) {
+  uint32_t hw[4], lw[4];
+  const uint64_t s2 = pack2(sc, sc), m1 = pack2(-1.f, -1.f), e2 = pack2(2048.f, 2048.f);
+#pragma unroll
+  for (int k = 0; k < 4; ++k) {
+    const uint64_t vs = mul2(pack2(v[2 * k], v[2 * k + 1]), s2);
+    float a, b;
+    unpack2(vs, a, b);
+    const __half2 hh = __floats2half2_rn(a, b);
+    const float2 hf = __half22float2(hh);
+    unpack2(mul2(fma2(pack2(hf.x, hf.y), m1, vs), e2), a, b);
+    const __half2 ll = __floats2half2_rn(a, b);
+    hw[k] = *reinterpret_cast<const uint32_t*>(&hh);
+    lw[k] = *reinterpret_cast<const uint32_t*>(&ll);
+    mx = __hmax2_nan(mx, __habs2(hh));
+  }
+  h = make_uint4(hw[0], hw[1], hw[2], hw[3]);
+  l = make_uint4(lw[0], lw[1], lw[2], lw[3]);
+}
+// nonzero when some |hi| in the running maximum was infinite or NaN
+__device__ __forceinline__ bool f16_max_bad(__half2 mx) {
+  const uint32_t w = *reinterpret_cast<const uint32_t*>(&mx);
+  return (((w & 0x7FFF7FFFu) + 0x04000400u) & 0x80008000u) != 0;
 }
 
 }  // namespace ppc_ptx

@@ -1069,3 +1069,67 @@ def test_f16_input_range(pp, runner, oracle_mod, kernel):
         assert pp.pp_layer_precision(dl.handle) == (0, 1.0)
     finally:
         dl.close()
+
+
+# The resident-weight kernel (at most 64 filters and 64 input channels, maps wider than 62): ragged channel chunks and
+# filter counts, columns at the edges of its 128-pixel tiles and strips, one and a few rows, odd numbers of strips (cut
+# at half height), more tiles (tf32) and rows (f16) than CTAs, rows that are not 16-byte aligned.
+RESIDENT_CASES = [
+    # N, Ci, Co, H, W
+    (1, 1, 1, 1, 63),
+    (1, 8, 5, 2, 127),
+    (1, 9, 33, 3, 128),
+    (2, 16, 32, 5, 129),
+    (1, 17, 64, 7, 130),
+    (3, 63, 40, 4, 131),
+    (1, 64, 64, 9, 257),
+    (1, 64, 64, 46, 200),
+    (5, 3, 7, 33, 65),
+    (1, 8, 8, 330, 384),
+    (7, 2, 3, 64, 640),
+]
+
+
+@pytest.mark.parametrize("case", RESIDENT_CASES)
+@pytest.mark.parametrize("flags", ["none", "skip_relu", "skip_pool_relu"])
+@pytest.mark.parametrize("precision", [0, 1])
+def test_resident_weight_kernel(pp, runner, oracle_mod, case, flags, precision):
+    N, Ci, Co, H, W = case
+    pool = "pool" in flags
+    if pool:
+        H, W = H + H % 2, W + W % 2
+    rng = np.random.default_rng(sum(case) + len(flags) + precision)
+    L = synth.small_random_layer(rng, Co, Ci, P=8, keep=0.5 if Ci > 3 else 1.0)
+    x = rng.uniform(-1, 1, (N, Ci, H, W)).astype(np.float32)
+    skip = rng.uniform(-1, 1, (N, Co, H, W)).astype(np.float32) if "skip" in flags else None
+    g = run_layer(pp, runner, L, x, skip, "relu" in flags, pool, kernel=pp.PP_KERNEL_TC, precision=precision)
+    y, s = oracle_layer_full(oracle_mod, L, x, skip, "relu" in flags, pool)
+    check_within(g, y, s, f"resident-weight kernel {case} {flags} precision {precision}")
+    # a second launch gives the same bits (a fixed order of sums)
+    g2 = run_layer(pp, runner, L, x, skip, "relu" in flags, pool, kernel=pp.PP_KERNEL_TC, precision=precision)
+    assert np.array_equal(g, g2)
+
+
+@pytest.mark.parametrize("precision", [0, 1])
+def test_resident_weight_kernel_unaligned_input(pp, runner, oracle_mod, precision):
+    """x only 4-byte aligned, and the layer's filters stored in another channel order."""
+    rng = np.random.default_rng(41)
+    N, Ci, Co, H, W = 1, 24, 40, 11, 140
+    L = synth.small_random_layer(rng, Co, Ci, P=8, keep=0.5)
+    x = rng.uniform(-1, 1, (N, Ci, H, W)).astype(np.float32)
+    order = rng.permutation(Co).astype(np.int32)
+    d = runner.DeviceLayer(L, precision=precision)
+    try:
+        pp.pp_layer_set_kernel(d.handle, pp.PP_KERNEL_TC)
+        pp.pp_layer_set_output_order(d.handle, order, torch.cuda.current_stream())
+        buf = torch.empty(x.size + 1, device="cuda")
+        buf[1:] = torch.from_numpy(x.ravel()).cuda()
+        y = torch.full((N, Co, H, W), float("nan"), device="cuda")
+        d.forward(buf[1:], y, None, N, H, W, 0, torch.cuda.current_stream())
+        torch.cuda.synchronize()
+        assert pp.pp_layer_device_status(d.handle) == 0
+        g = y.cpu().numpy()[:, order]
+    finally:
+        d.close()
+    yo, s = oracle_layer_full(oracle_mod, L, x)
+    check_within(g, yo, s, "unaligned input")
