@@ -936,8 +936,8 @@ extern "C" pp_status pp_layer_info(const pp_layer* L, int* Co, int* Ci, int64_t*
   if (Co) *Co = L->Co;
   if (Ci) *Ci = L->Ci;
   if (device_bytes)
-    *device_bytes = (int64_t)(L->dbytes + L->tm.dbytes + L->tc.dbytes + L->tc.dbytes16 +
-                              (L->direct.w ? ((size_t)L->Co * L->Ci * 9 + (L->direct.bias ? L->Co : 0)) * 4 : 0));
+    *device_bytes =
+        (int64_t)(L->dbytes + L->tm.dbytes + L->tc.dbytes + L->tc.dbytes16 + L->direct.dbytes);
   return PP_OK;
 }
 
@@ -980,34 +980,10 @@ extern "C" pp_status pp_dense_create(const float* w, const float* bias, int Co, 
   if (prepare_kernels() != cudaSuccess) return PP_ERR_CUDA;
   pp_dense* D = new (std::nothrow) pp_dense;
   if (!D) return PP_ERR_OOM;
-  D->base.mode = MODE_GENERIC;
-  // A dense kernel is three entries of the generic path: taps 0-3, 4-7 and 8.
-  std::vector<std::vector<Entry>> per_filter(Co);
-  std::vector<int32_t> perm(Co);
-  for (int o = 0; o < Co; ++o) {
-    perm[o] = o;
-    for (int i = 0; i < Ci; ++i) {
-      const float* k = w + ((size_t)o * Ci + i) * 9;
-      for (int part = 0; part < 3; ++part) {
-        Entry en;
-        en.ch = i;
-        en.slot = 0;
-        const int t0 = part * 4;
-        const int nt = part < 2 ? 4 : 1;
-        en.payload = 0;
-        for (int s = 0; s < nt; ++s) en.payload |= uint32_t(t0 + s) << (4 * s);
-        en.payload |= uint32_t(nt - 1) << 28;
-        for (int s = 0; s < 4; ++s) en.w[s] = s < nt ? k[t0 + s] : 0.f;
-        per_filter[o].push_back(en);
-      }
-    }
-  }
-  // three entries per kernel: 5 channels per stage keep a warp's stage at <= EMAX entries
-  pp_status st = build_layer(&D->base, Co, Ci, 5, per_filter, perm, bias, (cudaStream_t)stream);
-  if (st == PP_OK && ppc::direct_applicable(Co, Ci)) {
-    st = ppc::direct_build(&D->base.direct, w, bias, Co, Ci, (cudaStream_t)stream);
-    if (st == PP_OK) D->base.kernel = D->base.auto_kernel = PP_KERNEL_DIRECT;
-  }
+  D->base.Co = Co;
+  D->base.Ci = Ci;
+  const pp_status st = ppc::direct_build(&D->base.direct, w, bias, Co, Ci, (cudaStream_t)stream);
+  D->base.kernel = D->base.auto_kernel = PP_KERNEL_DIRECT;
   if (st != PP_OK) {
     pp_dense_destroy(D);
     return st;

@@ -1,42 +1,68 @@
 // Direct 3x3 convolution on the FP32 FMA pipes for layers with few input or
 // few output channels (the first and last layers of the networks: VGG-16's
 // 3 -> 64, the VDSR-shaped stack's 1 -> 64 and 64 -> 1 dense convolutions, the
-// 16 -> 16 single layer).  For these the tensor-core kernels cannot fill an
-// MMA (K = 8 channels per chunk, M = 64 or 128 filters) and their per-tile
-// start-up dominates, while the FMA kernels built for pattern dispatch carry
-// machinery these shapes do not need.
+// 16 -> 16 single layer) and for dense layers of any width.  For the former the
+// tensor-core kernels cannot fill an MMA (K = 8 channels per chunk, M = 64 or
+// 128 filters) and their per-tile start-up dominates; the latter have no
+// pattern structure, and the register kernel's dispatch per entry ran them at
+// 2 % of the FP32 rate.
 //
-// The weights are expanded to dense [Co][Ci][9] (pruned taps and kernels are
-// exact zeros, so the sum is the one of Section 2 with zero terms added).
-// CTA: a 32 x 32 output tile and FBD filters; 256 threads, each owning a 2 x 2
-// pixel block and accumulating FBD x 4 outputs in registers.  Input channels
-// are staged CC at a time (tile plus one-pixel zero halo) together with their
-// weights, double-buffered with cp.async; per channel a thread reads its 4 x 4
-// input window once and runs FBD x 36 FMAs on it, the weights coming from
-// shared memory as warp-wide broadcasts.  Epilogue: + bias, + skip, ReLU,
-// optional 2 x 2 max pool, stored in the original channel order.
+// The weights are expanded to the dense 9 taps (pruned taps and kernels are
+// exact zeros, so the sum is the one of Section 2 with zero terms added).  Input
+// channels are staged a few at a time (tile plus one-pixel zero halo) together
+// with their weights, in a ring of stages filled by cp.async.  Epilogue: + bias, + skip,
+// ReLU, optional 2 x 2 max pool, stored in the original channel order.
+//
+// ppconv_direct_kernel: a CTA of 256 threads owns FBD filters of a tile; a
+// thread owns a 2 x 2 pixel block and FBD x 4 accumulators.  What bounds it is
+// instruction issue and, on large maps, the FMA pipe (64 -> 64 at 224 x 224,
+// batch 4: 45 of 73 TFLOP/s), so two filters share each packed FMA
+// (fma.rn.f32x2): the weights lie as pairs of filters, 9 pairs per channel padded
+// to 80 bytes, read as broadcasts; the thread's 4 x 4 window is duplicated once
+// per channel.  Maps with few tiles split the staged channels over KS groups of
+// threads on tiles of 1024 / KS pixels, whose sums meet in shared memory in group
+// order: 64 -> 64 at 56 x 56 would otherwise have 4 tiles (register kernel 268
+// us, here 13.5).  Each chunk of channels is summed by itself and then added,
+// which halves the rounding error of one long sum (1.1e-7 against 2.2e-7 of the
+// result at 64 channels).
+//
+// ppconv_direct_wide_kernel: at most 4 filters on wide maps (a network's last
+// layer).  These read far more than they compute (64 -> 1 at 720 x 1280: 236 MB
+// of input), and with 2 x 2 blocks the shared-memory reads of the windows (16
+// for 36 FMAs) took longer than the copies.  A thread owns 4 x 4 pixels, a warp 4
+// rows of 128, so a window row is one 16-byte read and two shuffles for 12 FMAs a
+// row and filter, and three stages of two channels keep 40 KB per CTA in flight.
+// 64 -> 1 at 720 x 1280 with the residual: 97 -> 61 us (4.0 TB/s of the input).
+//
+// ppconv_direct_first_kernel: at most 4 input channels (a network's first
+// layer) on maps wider than a tile's half.  These write far more than they read:
+// a CTA stages its tile's input once for up to 64 filters, 8 at a time, and a
+// thread's 2 x 4 pixels leave in 16-byte stores.
 #include <cuda_runtime.h>
 
+#include <algorithm>
 #include <cstring>
 #include <vector>
 
 #include "internal.h"
+#include "tc_ptx.cuh"
 
 namespace {
 
-constexpr int DT = 32;        // output tile edge
-constexpr int DTW = DT + 2;   // staged rows (one-pixel halo)
-constexpr int DCOLS = DT + 8; // staged columns: c0 - 4 .. c0 + 35 (16-byte aligned groups of 4)
-constexpr int DPITCH = DCOLS; // shared-memory row pitch in floats
+using namespace ppc_ptx;
+
 constexpr int DTHREADS = 256;
+constexpr int FBMAX = 8;      // filters per CTA at most
+constexpr int WPAIR = 20;     // floats of one channel of a filter pair: 9 taps x 2 filters, padded to 80 bytes
 
 struct DirectParams {
   const float* x;
   float* y;
   const float* skip;
-  const float* w;     // [Co][Ci][9], original filter order
+  const float* w;     // [Ci][npair][WPAIR]: tap t of filters 2 q, 2 q + 1 at 2 t, 2 t + 1; original filter order
   const float* bias;  // [Co] or null
   int N, Ci, Co, H, W, flags;
+  int npair;
   int tiles_x, tiles_y;
   int vec;  // x 16-byte aligned and W a multiple of 4: rows staged in 16-byte copies
 };
@@ -50,89 +76,148 @@ __device__ __forceinline__ void cp_async16(float* dst, const float* src, bool va
   asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(d), "l"(src), "r"(valid ? 16 : 0) : "memory");
 }
 
-template <int CC, int FBD>
-__global__ void __launch_bounds__(DTHREADS, FBD >= 16 ? 2 : 3) ppconv_direct_kernel(const DirectParams p) {
-  // two stages of [CC][DTW][DPITCH] input and [CC][FBD][12] weights (9 taps padded to 12)
+// Stages rows r0 - 1 .. r0 + ROWS - 2 and columns c0 - 4 .. c0 + COLS - 5 of some channels of an image, zero outside it
+// and beyond Ci, as [channel][ROWS][COLS].  With W a multiple of 4 every 16-byte group is wholly inside or outside;
+// otherwise only the columns c0 - 1 .. c0 + COLS - 8 that are read are copied, one by one.  A thread copies the same
+// places of every channel: their offsets are worked out once (vec), so a copy costs an add and the copy itself.
+template <int ROWS, int COLS, int NT>
+struct XStage {
+  static constexpr int GROUPS = ROWS * (COLS / 4), NE = (GROUPS + NT - 1) / NT;
+  int src[NE];  // offset within a channel of x, or -1 outside the image
+  __device__ __forceinline__ void init(const DirectParams& p, int r0, int c0, int tid) {
+#pragma unroll
+    for (int i = 0; i < NE; ++i) {
+      const int e = tid + i * NT, rr = e / (COLS / 4), g = e - rr * (COLS / 4);
+      const int r = r0 - 1 + rr, col = c0 - 4 + 4 * g;
+      src[i] = e < GROUPS && (unsigned)r < (unsigned)p.H && (unsigned)col < (unsigned)p.W ? r * p.W + col : -1;
+    }
+  }
+  template <int CC>
+  __device__ __forceinline__ void copy(float* dst, const DirectParams& p, const float* xb, int ch0, int r0, int c0,
+                                       int tid) const {
+    const size_t plane = (size_t)p.H * p.W;
+    const float* xc = xb + (size_t)ch0 * plane;
+    if (p.vec) {
+#pragma unroll
+      for (int k = 0; k < CC; ++k, xc += plane) {
+        const bool have = ch0 + k < p.Ci;
+#pragma unroll
+        for (int i = 0; i < NE; ++i)
+          if ((i + 1) * NT <= GROUPS || tid + i * NT < GROUPS) {
+            const bool in = have && src[i] >= 0;
+            cp_async16(dst + k * ROWS * COLS + 4 * (tid + i * NT), in ? xc + src[i] : p.x, in);
+          }
+      }
+    } else {
+      constexpr int USED = COLS - 6;
+      for (int e = tid; e < ROWS * USED; e += NT) {
+        const int rr = e / USED, cc = e - rr * USED;
+        const int r = r0 - 1 + rr, col = c0 - 1 + cc;
+        const bool inside = (unsigned)r < (unsigned)p.H && (unsigned)col < (unsigned)p.W;
+        const float* sp = xc + (size_t)r * p.W + col;
+#pragma unroll
+        for (int k = 0; k < CC; ++k, sp += plane) {
+          const bool in = inside && ch0 + k < p.Ci;
+          cp_async4(dst + (k * ROWS + rr) * COLS + cc + 3, in ? sp : p.x, in);
+        }
+      }
+    }
+  }
+};
+
+template <int CC, int FBD, int KS>
+struct DirectGeo {
+  static constexpr int TH = KS == 1 ? 32 : 16, TW = KS == 4 ? 16 : 32;  // tile of 1024 / KS pixels
+  static constexpr int ROWS = TH + 2, COLS = TW + 8;                    // staged; columns from c0 - 4
+  static constexpr int XS = CC * ROWS * COLS, WS = CC * (FBD / 2) * WPAIR;
+  static constexpr int RED = KS > 1 ? (KS - 1) * (DTHREADS / KS) * FBD * 4 : 0;  // sums of groups 1 ..
+  // stages: one chunk's arithmetic does not cover the copies' latency (small tiles have less of it)
+  static constexpr int NS = KS == 1 ? 3 : 4;
+  static constexpr int FLOATS = NS * (XS + WS) > RED ? NS * (XS + WS) : RED;
+  static_assert(CC % KS == 0 && FBD % 2 == 0, "channels over the groups, filters in pairs");
+};
+
+template <int CC, int FBD, int KS>
+__global__ void __launch_bounds__(DTHREADS, 2) ppconv_direct_kernel(const DirectParams p) {
+  using G = DirectGeo<CC, FBD, KS>;
+  constexpr int NP = FBD / 2, GT = DTHREADS / KS, TX = G::TW / 2;
+  // NS stages of [CC][ROWS][COLS] input and [CC][NP][WPAIR] weights; at the end the groups' sums
   extern __shared__ __align__(16) float dsm[];
-  auto xs = reinterpret_cast<float(*)[CC][DTW][DPITCH]>(dsm);
-  auto ws = reinterpret_cast<float(*)[CC][FBD][12]>(dsm + 2 * CC * DTW * DPITCH);
-  const int tid = threadIdx.x, tx = tid & 15, ty = tid >> 4;
+  const int tid = threadIdx.x, grp = tid / GT, gt = tid % GT, tx = gt % TX, ty = gt / TX;
   int t = (int)blockIdx.x;
   const int bx = t % p.tiles_x;
   t /= p.tiles_x;
   const int by = t % p.tiles_y;
   const int n = t / p.tiles_y;
-  const int o0 = (int)blockIdx.y * FBD;
-  const int r0 = by * DT, c0 = bx * DT;
+  const int q0 = (int)(blockIdx.z * gridDim.y + blockIdx.y) * NP;  // first filter pair
+  if (q0 >= p.npair) return;
+  const int r0 = by * G::TH, c0 = bx * G::TW;
   const float* xb = p.x + (size_t)n * p.Ci * p.H * p.W;
   const int nchunks = (p.Ci + CC - 1) / CC;
 
-  // channels ch * CC .. of the input tile (zero outside the image and beyond
-  // Ci) and their weights for this CTA's filters (zero beyond Co) into buffer b
-  // staged column j holds image column c0 - 4 + j
-  auto stage = [&](int ch, int b) {
-    if (p.vec) {
-      // rows of 16-byte groups: with W a multiple of 4 each group is wholly inside or outside the image
-      for (int e = tid; e < CC * DTW * (DCOLS / 4); e += DTHREADS) {
-        const int k = e / (DTW * (DCOLS / 4)), rem = e - k * (DTW * (DCOLS / 4));
-        const int rr = rem / (DCOLS / 4), g = rem - rr * (DCOLS / 4);
-        const int c = ch * CC + k, r = r0 - 1 + rr, col = c0 - 4 + 4 * g;
-        const bool in = c < p.Ci && (unsigned)r < (unsigned)p.H && (unsigned)col < (unsigned)p.W;
-        cp_async16(&xs[b][k][rr][4 * g], in ? xb + ((size_t)c * p.H + r) * p.W + col : p.x, in);
-      }
-    } else {
-      for (int e = tid; e < CC * DTW * DTW; e += DTHREADS) {
-        const int k = e / (DTW * DTW), rem = e - k * (DTW * DTW);
-        const int rr = rem / DTW, cc = rem - rr * DTW;
-        const int c = ch * CC + k, r = r0 - 1 + rr, col = c0 - 1 + cc;
-        const bool in = c < p.Ci && (unsigned)r < (unsigned)p.H && (unsigned)col < (unsigned)p.W;
-        cp_async4(&xs[b][k][rr][cc + 3], in ? xb + ((size_t)c * p.H + r) * p.W + col : p.x, in);
+  XStage<G::ROWS, G::COLS, DTHREADS> xst;
+  xst.init(p, r0, c0, tid);
+  auto stage = [&](int ch) {
+    float* xs = dsm + (ch % G::NS) * (G::XS + G::WS);
+    if (ch < nchunks) {
+      xst.template copy<CC>(xs, p, xb, ch * CC, r0, c0, tid);
+      for (int e = tid; e < CC * NP * (WPAIR / 4); e += DTHREADS) {  // the layout is padded to FBMAX filters
+        const int k = e / (NP * (WPAIR / 4)), rem = e - k * (NP * (WPAIR / 4));
+        const bool in = ch * CC + k < p.Ci;
+        cp_async16(xs + G::XS + 4 * e, in ? p.w + ((size_t)(ch * CC + k) * p.npair + q0) * WPAIR + 4 * rem : p.w, in);
       }
     }
-    for (int e = tid; e < CC * FBD * 9; e += DTHREADS) {
-      const int k = e / (FBD * 9), rem = e - k * (FBD * 9);
-      const int o = rem / 9, tap = rem - o * 9;
-      const int c = ch * CC + k, oo = o0 + o;
-      const bool in = c < p.Ci && oo < p.Co;
-      cp_async4(&ws[b][k][o][tap], in ? p.w + ((size_t)oo * p.Ci + c) * 9 + tap : p.w, in);
-    }
-    asm volatile("cp.async.commit_group;" ::: "memory");
+    asm volatile("cp.async.commit_group;" ::: "memory");  // one group per step, empty past the last chunk
   };
 
-  float acc[FBD][4];
+  uint64_t acc[NP][4];
 #pragma unroll
-  for (int o = 0; o < FBD; ++o)
+  for (int o = 0; o < NP; ++o)
 #pragma unroll
-    for (int q = 0; q < 4; ++q) acc[o][q] = 0.f;
+    for (int q = 0; q < 4; ++q) acc[o][q] = 0;
 
   // programmatic dependent launch: nothing of the previous kernel in the
   // stream is read or overwritten before this wait
   asm volatile("griddepcontrol.wait;" ::: "memory");
-  stage(0, 0);
+#pragma unroll
+  for (int st = 0; st < G::NS - 1; ++st) stage(st);
   for (int ch = 0; ch < nchunks; ++ch) {
-    const int b = ch & 1;
-    if (ch + 1 < nchunks) {
-      stage(ch + 1, b ^ 1);
-      asm volatile("cp.async.wait_group 1;" ::: "memory");
-    } else {
-      asm volatile("cp.async.wait_group 0;" ::: "memory");
-    }
-    __syncthreads();
+    asm volatile("cp.async.wait_group %0;" ::"n"(G::NS - 2) : "memory");
+    __syncthreads();  // chunk ch has landed; every thread is done with the stage that is filled next
+    stage(ch + G::NS - 1);
+    const float* xs = dsm + (ch % G::NS) * (G::XS + G::WS);
+    const float* ws = xs + G::XS;
+    uint64_t part[NP][4];  // the chunk's sum: added to acc as one term, which keeps the rounding error of long sums low
 #pragma unroll
-    for (int k = 0; k < CC; ++k) {
-      // the thread's 4 x 4 input window: staged rows 2 ty .. 2 ty + 3, image
-      // columns c0 + 2 tx - 1 .. c0 + 2 tx + 2 (staged 2 tx + 3 .. 2 tx + 6)
-      float xv[4][4];
+    for (int o = 0; o < NP; ++o)
 #pragma unroll
-      for (int a = 0; a < 4; ++a)
+      for (int q = 0; q < 4; ++q) part[o][q] = 0;
+#pragma unroll 1
+    for (int kk = 0; kk < CC / KS; ++kk) {
+      const int k = kk * KS + grp;
+      if (ch * CC + k >= p.Ci) break;
+      // the thread's 4 x 4 input window (staged rows 2 ty .., columns 2 tx + 3 .. 2 tx + 6), each value twice
+      uint64_t xv[4][4];
 #pragma unroll
-        for (int q = 0; q < 4; ++q) xv[a][q] = xs[b][k][2 * ty + a][2 * tx + 3 + q];
+      for (int a = 0; a < 4; ++a) {
+        const float2* row = reinterpret_cast<const float2*>(xs + (k * G::ROWS + 2 * ty + a) * G::COLS + 2 * tx + 2);
+        const float2 u = row[0], v = row[1], w = row[2];
+        xv[a][0] = pack2(u.y, u.y);
+        xv[a][1] = pack2(v.x, v.x);
+        xv[a][2] = pack2(v.y, v.y);
+        xv[a][3] = pack2(w.x, w.x);
+      }
 #pragma unroll
-      for (int o = 0; o < FBD; ++o) {
-        const float4 w0 = *reinterpret_cast<const float4*>(&ws[b][k][o][0]);
-        const float4 w1 = *reinterpret_cast<const float4*>(&ws[b][k][o][4]);
-        const float w8 = ws[b][k][o][8];
-        const float wt[9] = {w0.x, w0.y, w0.z, w0.w, w1.x, w1.y, w1.z, w1.w, w8};
+      for (int o = 0; o < NP; ++o) {
+        const float* wp = ws + (k * NP + o) * WPAIR;
+        uint64_t wt[9];
+#pragma unroll
+        for (int e = 0; e < 4; ++e) {
+          const ulonglong2 v = *reinterpret_cast<const ulonglong2*>(wp + 4 * e);
+          wt[2 * e] = v.x;
+          wt[2 * e + 1] = v.y;
+        }
+        wt[8] = *reinterpret_cast<const uint64_t*>(wp + 16);
 #pragma unroll
         for (int dy = 0; dy < 3; ++dy)
 #pragma unroll
@@ -141,20 +226,42 @@ __global__ void __launch_bounds__(DTHREADS, FBD >= 16 ? 2 : 3) ppconv_direct_ker
             for (int py = 0; py < 2; ++py)
 #pragma unroll
               for (int px = 0; px < 2; ++px)
-                acc[o][py * 2 + px] = fmaf(wt[dy * 3 + dx], xv[py + dy][px + dx], acc[o][py * 2 + px]);
+                part[o][py * 2 + px] = fma2(wt[dy * 3 + dx], xv[py + dy][px + dx], part[o][py * 2 + px]);
       }
     }
-    __syncthreads();  // buffer b is restaged by the next iteration's copy
+#pragma unroll
+    for (int o = 0; o < NP; ++o)
+#pragma unroll
+      for (int q = 0; q < 4; ++q) acc[o][q] = add2(acc[o][q], part[o][q]);
   }
 
   // the next kernel may start its prologue (it waits for this grid to finish)
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+  if (KS > 1) {
+    // groups 1 .. hand their sums to group 0, which adds them in order
+    uint64_t* red = reinterpret_cast<uint64_t*>(dsm);
+    __syncthreads();  // every thread is done with the stages (no copy is in flight: the last groups are empty)
+    if (grp > 0) {
+#pragma unroll
+      for (int o = 0; o < NP; ++o)
+#pragma unroll
+        for (int q = 0; q < 4; ++q) red[((grp - 1) * NP * 4 + o * 4 + q) * GT + gt] = acc[o][q];
+    }
+    __syncthreads();
+    if (grp > 0) return;
+#pragma unroll
+    for (int g = 0; g < KS - 1; ++g)
+#pragma unroll
+      for (int o = 0; o < NP; ++o)
+#pragma unroll
+        for (int q = 0; q < 4; ++q) acc[o][q] = add2(acc[o][q], red[(g * NP * 4 + o * 4 + q) * GT + gt]);
+  }
   const bool relu = p.flags & PP_RELU, pool = p.flags & PP_POOL2;
   const float* skip = (p.flags & PP_ADD_SKIP) ? p.skip : nullptr;
   const int r = r0 + 2 * ty, c = c0 + 2 * tx;
 #pragma unroll
   for (int o = 0; o < FBD; ++o) {
-    const int oo = o0 + o;
+    const int oo = 2 * q0 + o;
     if (oo >= p.Co) break;
     const size_t plane = (size_t)n * p.Co + oo;
     const float bs = p.bias ? __ldg(p.bias + oo) : 0.f;
@@ -162,7 +269,9 @@ __global__ void __launch_bounds__(DTHREADS, FBD >= 16 ? 2 : 3) ppconv_direct_ker
 #pragma unroll
     for (int q = 0; q < 4; ++q) {
       const int rq = r + (q >> 1), cq = c + (q & 1);
-      v[q] = acc[o][q] + bs;
+      float lo, hi;
+      unpack2(acc[o / 2][q], lo, hi);
+      v[q] = (o & 1 ? hi : lo) + bs;
       if (skip && rq < p.H && cq < p.W) v[q] += __ldg(skip + (plane * p.H + rq) * p.W + cq);
       if (relu) v[q] = fmaxf(v[q], 0.f);
     }
@@ -187,13 +296,275 @@ __global__ void __launch_bounds__(DTHREADS, FBD >= 16 ? 2 : 3) ppconv_direct_ker
   }
 }
 
-template <int CC, int FBD>
-cudaError_t launch_one(const DirectParams& p, dim3 grid, cudaStream_t stream) {
-  constexpr int bytes = 2 * (CC * DTW * DPITCH + CC * FBD * 12) * 4;
-  static ppc::DeviceOnce attr_once;  // one per instantiation
-  const cudaError_t ea = attr_once.run([](int) {
-    return cudaFuncSetAttribute(ppconv_direct_kernel<CC, FBD>, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
-  });
+constexpr int VTHREADS = 128;                // 4 warps
+constexpr int VH = 16, VW = 128;             // tile: 4 rows of 128 pixels per warp
+constexpr int VROWS = VH + 2, VCOLS = VW + 8;
+constexpr int VCC = 2, VST = 3;              // channels per stage, stages
+constexpr int VX = VCC * VROWS * VCOLS;
+
+template <int CO>
+__global__ void __launch_bounds__(VTHREADS, 3) ppconv_direct_wide_kernel(const DirectParams p) {
+  // VST stages of [VCC][VROWS][VCOLS] input and [VCC][CO][9][2] weights (each twice, for packed FMAs)
+  constexpr int VWS = VCC * CO * 20;
+  extern __shared__ __align__(16) float dsm[];
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  int t = (int)blockIdx.x;
+  const int bx = t % p.tiles_x;
+  t /= p.tiles_x;
+  const int by = t % p.tiles_y;
+  const int n = t / p.tiles_y;
+  const int r0 = by * VH, c0 = bx * VW;
+  const float* xb = p.x + (size_t)n * p.Ci * p.H * p.W;
+  const int nchunks = (p.Ci + VCC - 1) / VCC;
+
+  XStage<VROWS, VCOLS, VTHREADS> xst;
+  xst.init(p, r0, c0, tid);
+  auto stage = [&](int ch) {
+    float* xs = dsm + (ch % VST) * (VX + VWS);
+    if (ch < nchunks) {
+      xst.template copy<VCC>(xs, p, xb, ch * VCC, r0, c0, tid);
+      for (int e = tid; e < VCC * CO * 18; e += VTHREADS) {
+        const int k = e / (CO * 18), rem = e - k * (CO * 18), o = rem / 18, tap = (rem - o * 18) >> 1;
+        const bool in = ch * VCC + k < p.Ci;
+        cp_async4(xs + VX + (k * CO + o) * 20 + (rem - o * 18),
+                  in ? p.w + ((size_t)(ch * VCC + k) * p.npair + (o >> 1)) * WPAIR + 2 * tap + (o & 1) : p.w, in);
+      }
+    }
+    asm volatile("cp.async.commit_group;" ::: "memory");  // one group per step, empty past the last chunk
+  };
+
+  uint64_t acc[CO][4][2];  // 4 rows x 4 columns as pairs of columns
+#pragma unroll
+  for (int o = 0; o < CO; ++o)
+#pragma unroll
+    for (int r = 0; r < 4; ++r) acc[o][r][0] = acc[o][r][1] = 0;
+
+  asm volatile("griddepcontrol.wait;" ::: "memory");
+#pragma unroll
+  for (int s = 0; s < VST - 1; ++s) stage(s);
+  for (int ch = 0; ch < nchunks; ++ch) {
+    asm volatile("cp.async.wait_group %0;" ::"n"(VST - 2) : "memory");
+    __syncthreads();  // chunk ch has landed; every thread is done with the stage that is filled next
+    stage(ch + VST - 1);
+    const float* xs = dsm + (ch % VST) * (VX + VWS);
+#pragma unroll
+    for (int k = 0; k < VCC; ++k) {
+      if (ch * VCC + k >= p.Ci) break;
+      // window rows 0 .. 5, columns -1 .. 4 of the thread's block: pairs starting at each of the columns -1 .. 3
+      uint64_t xp[6][5];
+#pragma unroll
+      for (int a = 0; a < 6; ++a) {
+        const float* row = xs + (k * VROWS + 4 * warp + a) * VCOLS;
+        const float4 v = *reinterpret_cast<const float4*>(row + 4 * lane + 4);
+        const float edge = row[lane == 0 ? 3 : VW + 4];
+        float l = __shfl_up_sync(0xffffffffu, v.w, 1), r = __shfl_down_sync(0xffffffffu, v.x, 1);
+        l = lane == 0 ? edge : l;
+        r = lane == 31 ? edge : r;
+        xp[a][0] = pack2(l, v.x);
+        xp[a][1] = pack2(v.x, v.y);
+        xp[a][2] = pack2(v.y, v.z);
+        xp[a][3] = pack2(v.z, v.w);
+        xp[a][4] = pack2(v.w, r);
+      }
+#pragma unroll
+      for (int o = 0; o < CO; ++o) {
+        const float* wp = xs + VX + (k * CO + o) * 20;
+        uint64_t wt[9];
+#pragma unroll
+        for (int e = 0; e < 4; ++e) {
+          const ulonglong2 v = *reinterpret_cast<const ulonglong2*>(wp + 4 * e);
+          wt[2 * e] = v.x;
+          wt[2 * e + 1] = v.y;
+        }
+        wt[8] = *reinterpret_cast<const uint64_t*>(wp + 16);
+#pragma unroll
+        for (int dy = 0; dy < 3; ++dy)
+#pragma unroll
+          for (int dx = 0; dx < 3; ++dx)
+#pragma unroll
+            for (int r = 0; r < 4; ++r)
+#pragma unroll
+              for (int h = 0; h < 2; ++h)
+                acc[o][r][h] = fma2(wt[dy * 3 + dx], xp[r + dy][2 * h + dx], acc[o][r][h]);
+      }
+    }
+  }
+
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+  asm volatile("cp.async.wait_group 0;" ::: "memory");
+  const bool relu = p.flags & PP_RELU, pool = p.flags & PP_POOL2;
+  const float* skip = (p.flags & PP_ADD_SKIP) ? p.skip : nullptr;
+  const int row0 = r0 + 4 * warp, c = c0 + 4 * lane;
+  const bool wide = (p.W & 3) == 0;
+#pragma unroll
+  for (int o = 0; o < CO; ++o) {
+    const size_t plane = (size_t)n * p.Co + o;
+    const float bs = p.bias ? __ldg(p.bias + o) : 0.f;
+    float v[4][4];
+#pragma unroll
+    for (int r = 0; r < 4; ++r) {
+      unpack2(acc[o][r][0], v[r][0], v[r][1]);
+      unpack2(acc[o][r][1], v[r][2], v[r][3]);
+#pragma unroll
+      for (int k = 0; k < 4; ++k) {
+        v[r][k] += bs;
+        if (skip && row0 + r < p.H && c + k < p.W) v[r][k] += __ldg(skip + (plane * p.H + row0 + r) * p.W + c + k);
+        if (relu) v[r][k] = fmaxf(v[r][k], 0.f);
+      }
+    }
+    if (pool) {  // H and W are even, so a 2 x 2 window inside the image is whole
+#pragma unroll
+      for (int r = 0; r < 4; r += 2)
+#pragma unroll
+        for (int k = 0; k < 4; k += 2)
+          if (row0 + r < p.H && c + k < p.W)
+            p.y[(plane * (p.H / 2) + (row0 + r) / 2) * (p.W / 2) + (c + k) / 2] =
+                fmaxf(fmaxf(v[r][k], v[r][k + 1]), fmaxf(v[r + 1][k], v[r + 1][k + 1]));
+    } else {
+#pragma unroll
+      for (int r = 0; r < 4; ++r) {
+        if (row0 + r >= p.H) break;
+        float* yr = p.y + (plane * p.H + row0 + r) * p.W;
+        if (wide) {
+          if (c < p.W) *reinterpret_cast<float4*>(yr + c) = make_float4(v[r][0], v[r][1], v[r][2], v[r][3]);
+        } else {
+#pragma unroll
+          for (int k = 0; k < 4; ++k)
+            if (c + k < p.W) yr[c + k] = v[r][k];
+        }
+      }
+    }
+  }
+}
+
+constexpr int UTHREADS = 128;                // 4 warps
+constexpr int UH = 8, UW = 128;              // tile: 2 rows of 128 pixels per warp
+constexpr int UROWS = UH + 2, UCOLS = UW + 8;
+constexpr int UFMAX = 64;                    // filters per CTA at most
+
+template <int CI>
+__global__ void __launch_bounds__(UTHREADS, 3) ppconv_direct_first_kernel(const DirectParams p, int fpc) {
+  constexpr int NP = FBMAX / 2;
+  __shared__ __align__(16) float xs[CI * UROWS * UCOLS];
+  __shared__ __align__(16) float ws[CI * (UFMAX / 2) * WPAIR];  // [CI][fpc / 2][WPAIR]
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  int t = (int)blockIdx.x;
+  const int bx = t % p.tiles_x;
+  t /= p.tiles_x;
+  const int by = t % p.tiles_y;
+  const int n = t / p.tiles_y;
+  const int r0 = by * UH, c0 = bx * UW;
+  const int q0 = (int)blockIdx.y * (fpc / 2), nq = min(fpc / 2, p.npair - q0);  // filter pairs of this CTA
+  // the weights do not depend on the previous kernel in the stream
+  for (int e = tid; e < CI * nq * (WPAIR / 4); e += UTHREADS) {
+    const int k = e / (nq * (WPAIR / 4)), rem = e - k * (nq * (WPAIR / 4));
+    cp_async16(ws + 4 * e, p.w + ((size_t)k * p.npair + q0) * WPAIR + 4 * rem, true);
+  }
+  asm volatile("griddepcontrol.wait;" ::: "memory");
+  XStage<UROWS, UCOLS, UTHREADS> xst;
+  xst.init(p, r0, c0, tid);
+  xst.template copy<CI>(xs, p, p.x + (size_t)n * p.Ci * p.H * p.W, 0, r0, c0, tid);
+  asm volatile("cp.async.commit_group;\n\tcp.async.wait_group 0;" ::: "memory");
+  __syncthreads();
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+
+  const bool relu = p.flags & PP_RELU, pool = p.flags & PP_POOL2;
+  const float* skip = (p.flags & PP_ADD_SKIP) ? p.skip : nullptr;
+  const int row0 = r0 + 2 * warp, c = c0 + 4 * lane;
+  const bool wide = (p.W & 3) == 0;
+  for (int q = 0; q < nq; q += NP) {
+    uint64_t acc[NP][2][4];  // filter pairs x 2 rows x 4 columns
+#pragma unroll
+    for (int o = 0; o < NP; ++o)
+#pragma unroll
+      for (int e = 0; e < 8; ++e) acc[o][e >> 2][e & 3] = 0;
+#pragma unroll
+    for (int k = 0; k < CI; ++k) {
+      uint64_t xv[4][6];  // window rows, columns -1 .. 4 of the thread's block, each value twice
+#pragma unroll
+      for (int a = 0; a < 4; ++a) {
+        const float* row = xs + (k * UROWS + 2 * warp + a) * UCOLS;
+        const float4 v = *reinterpret_cast<const float4*>(row + 4 * lane + 4);
+        const float edge = row[lane == 0 ? 3 : UW + 4];
+        float l = __shfl_up_sync(0xffffffffu, v.w, 1), r = __shfl_down_sync(0xffffffffu, v.x, 1);
+        l = lane == 0 ? edge : l;
+        r = lane == 31 ? edge : r;
+        xv[a][0] = pack2(l, l);
+        xv[a][1] = pack2(v.x, v.x);
+        xv[a][2] = pack2(v.y, v.y);
+        xv[a][3] = pack2(v.z, v.z);
+        xv[a][4] = pack2(v.w, v.w);
+        xv[a][5] = pack2(r, r);
+      }
+#pragma unroll
+      for (int o = 0; o < NP; ++o) {
+        const float* wp = ws + (k * nq + q + o) * WPAIR;  // the layout is padded to whole groups of FBMAX filters
+        uint64_t wt[9];
+#pragma unroll
+        for (int e = 0; e < 4; ++e) {
+          const ulonglong2 v = *reinterpret_cast<const ulonglong2*>(wp + 4 * e);
+          wt[2 * e] = v.x;
+          wt[2 * e + 1] = v.y;
+        }
+        wt[8] = *reinterpret_cast<const uint64_t*>(wp + 16);
+#pragma unroll
+        for (int dy = 0; dy < 3; ++dy)
+#pragma unroll
+          for (int dx = 0; dx < 3; ++dx)
+#pragma unroll
+            for (int py = 0; py < 2; ++py)
+#pragma unroll
+              for (int px = 0; px < 4; ++px)
+                acc[o][py][px] = fma2(wt[dy * 3 + dx], xv[py + dy][px + dx], acc[o][py][px]);
+      }
+    }
+#pragma unroll
+    for (int o = 0; o < FBMAX; ++o) {
+      const int oo = 2 * (q0 + q) + o;
+      if (oo >= p.Co) break;
+      const size_t plane = (size_t)n * p.Co + oo;
+      const float bs = p.bias ? __ldg(p.bias + oo) : 0.f;
+      float v[2][4];
+#pragma unroll
+      for (int r = 0; r < 2; ++r)
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+          float lo, hi;
+          unpack2(acc[o / 2][r][k], lo, hi);
+          v[r][k] = (o & 1 ? hi : lo) + bs;
+          if (skip && row0 + r < p.H && c + k < p.W) v[r][k] += __ldg(skip + (plane * p.H + row0 + r) * p.W + c + k);
+          if (relu) v[r][k] = fmaxf(v[r][k], 0.f);
+        }
+      if (pool) {  // H and W are even, so a 2 x 2 window inside the image is whole
+#pragma unroll
+        for (int k = 0; k < 4; k += 2)
+          if (row0 < p.H && c + k < p.W)
+            p.y[(plane * (p.H / 2) + row0 / 2) * (p.W / 2) + (c + k) / 2] =
+                fmaxf(fmaxf(v[0][k], v[0][k + 1]), fmaxf(v[1][k], v[1][k + 1]));
+      } else {
+#pragma unroll
+        for (int r = 0; r < 2; ++r) {
+          if (row0 + r >= p.H) break;
+          float* yr = p.y + (plane * p.H + row0 + r) * p.W;
+          if (wide) {
+            if (c < p.W) *reinterpret_cast<float4*>(yr + c) = make_float4(v[r][0], v[r][1], v[r][2], v[r][3]);
+          } else {
+#pragma unroll
+            for (int k = 0; k < 4; ++k)
+              if (c + k < p.W) yr[c + k] = v[r][k];
+          }
+        }
+      }
+    }
+  }
+}
+
+// One launch of kernel K (its dynamic shared memory allowed once per device).
+template <class K, class... A>
+cudaError_t launch_kernel(K kernel, ppc::DeviceOnce& once, dim3 grid, int threads, int bytes, cudaStream_t stream,
+                          const A&... args) {
+  const cudaError_t ea =
+      once.run([&](int) { return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes); });
   if (ea != cudaSuccess) return ea;
   cudaLaunchConfig_t cfg = {};
   cudaLaunchAttribute at[1];
@@ -202,52 +573,83 @@ cudaError_t launch_one(const DirectParams& p, dim3 grid, cudaStream_t stream) {
   cfg.attrs = at;
   cfg.numAttrs = 1;
   cfg.gridDim = grid;
-  cfg.blockDim = dim3(DTHREADS);
-  cfg.dynamicSmemBytes = bytes;
+  cfg.blockDim = dim3((unsigned)threads);
+  cfg.dynamicSmemBytes = (size_t)bytes;
   cfg.stream = stream;
-  return cudaLaunchKernelEx(&cfg, ppconv_direct_kernel<CC, FBD>, p);
+  return cudaLaunchKernelEx(&cfg, kernel, args...);
 }
 
-template <int CC>
-cudaError_t launch_cc(const DirectParams& p, int fbd, dim3 grid, cudaStream_t stream) {
+template <int CC, int FBD, int KS>
+cudaError_t launch_one(DirectParams p, cudaStream_t stream) {
+  using G = DirectGeo<CC, FBD, KS>;
+  static ppc::DeviceOnce once;  // one per instantiation
+  p.tiles_x = (p.W + G::TW - 1) / G::TW;
+  p.tiles_y = (p.H + G::TH - 1) / G::TH;
+  const int64_t nt = (int64_t)p.N * p.tiles_x * p.tiles_y, nfb = (p.Co + FBD - 1) / FBD;
+  if (nt > INT32_MAX) return cudaErrorInvalidConfiguration;
+  const unsigned gy = (unsigned)std::min<int64_t>(nfb, 65535);  // the grid's y extent; the rest in z
+  return launch_kernel(ppconv_direct_kernel<CC, FBD, KS>, once, dim3((unsigned)nt, gy, (unsigned)((nfb + gy - 1) / gy)),
+                       DTHREADS, G::FLOATS * 4, stream, p);
+}
+
+template <int CO>
+cudaError_t launch_wide(DirectParams p, cudaStream_t stream) {
+  static ppc::DeviceOnce once;
+  p.tiles_x = (p.W + VW - 1) / VW;
+  p.tiles_y = (p.H + VH - 1) / VH;
+  const int64_t nt = (int64_t)p.N * p.tiles_x * p.tiles_y;
+  if (nt > INT32_MAX) return cudaErrorInvalidConfiguration;
+  return launch_kernel(ppconv_direct_wide_kernel<CO>, once, dim3((unsigned)nt), VTHREADS,
+                       VST * (VX + VCC * CO * 20) * 4, stream, p);
+}
+
+template <int CI>
+cudaError_t launch_first(DirectParams p, int fpc, cudaStream_t stream) {
+  static ppc::DeviceOnce once;
+  p.tiles_x = (p.W + UW - 1) / UW;
+  p.tiles_y = (p.H + UH - 1) / UH;
+  const int64_t nt = (int64_t)p.N * p.tiles_x * p.tiles_y, nf = (2 * (int64_t)p.npair + fpc - 1) / fpc;
+  if (nt > INT32_MAX || nf > 65535) return cudaErrorInvalidConfiguration;
+  return launch_kernel(ppconv_direct_first_kernel<CI>, once, dim3((unsigned)nt, (unsigned)nf), UTHREADS, 0, stream, p,
+                       fpc);
+}
+
+template <int CC, int KS>
+cudaError_t launch_fbd(const DirectParams& p, int fbd, cudaStream_t stream) {
   switch (fbd) {
-    case 1: return launch_one<CC, 1>(p, grid, stream);
-    case 2: return launch_one<CC, 2>(p, grid, stream);
-    case 4: return launch_one<CC, 4>(p, grid, stream);
-    case 8: return launch_one<CC, 8>(p, grid, stream);
-    default: return launch_one<CC, 16>(p, grid, stream);
+    case 2: return launch_one<CC, 2, KS>(p, stream);
+    case 4: return launch_one<CC, 4, KS>(p, stream);
+    default: return launch_one<CC, FBMAX, KS>(p, stream);
   }
-}
-
-int sm_count() {
-  static int sms[64] = {};
-  int dev = 0;
-  if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return 148;
-  if (!sms[dev] && cudaDeviceGetAttribute(&sms[dev], cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) {
-    cudaGetLastError();
-    return 148;
-  }
-  return sms[dev];
 }
 
 }  // namespace
 
 namespace ppc {
 
+// Pruned layers get a direct layout when one side is small (dense ones always do).
 bool direct_applicable(int Co, int Ci) {
   return (Ci <= kDirectMaxSmall || Co <= kDirectMaxSmall) && (int64_t)Co * Ci <= (int64_t(1) << 20);
 }
 
 pp_status direct_build(DirectLayout* D, const float* w_dense, const float* bias, int Co, int Ci,
                        cudaStream_t stream) {
-  if (!direct_applicable(Co, Ci)) return PP_ERR_UNSUPPORTED;
-  const size_t nw = (size_t)Co * Ci * 9, nb = bias ? (size_t)Co : 0;
+  // pairs of filters, padded to whole CTAs of FBMAX filters (zero weights)
+  const int npair = (Co + FBMAX - 1) / FBMAX * (FBMAX / 2);
+  const size_t nw = (size_t)Ci * npair * WPAIR, nb = bias ? (size_t)Co : 0;
+  std::vector<float> host(nw, 0.f);
+  for (int o = 0; o < Co; ++o)
+    for (int i = 0; i < Ci; ++i) {
+      float* dst = &host[((size_t)i * npair + (o >> 1)) * WPAIR + (o & 1)];
+      const float* src = w_dense + ((size_t)o * Ci + i) * 9;
+      for (int t = 0; t < 9; ++t) dst[2 * t] = src[t];
+    }
   void* d = nullptr;
   if (cudaMalloc(&d, (nw + nb) * 4) != cudaSuccess) {
     cudaGetLastError();
     return PP_ERR_OOM;
   }
-  if (cudaMemcpyAsync(d, w_dense, nw * 4, cudaMemcpyHostToDevice, stream) != cudaSuccess ||
+  if (cudaMemcpyAsync(d, host.data(), nw * 4, cudaMemcpyHostToDevice, stream) != cudaSuccess ||
       (nb && cudaMemcpyAsync(static_cast<float*>(d) + nw, bias, nb * 4, cudaMemcpyHostToDevice, stream) !=
                  cudaSuccess) ||
       cudaStreamSynchronize(stream) != cudaSuccess) {
@@ -255,8 +657,10 @@ pp_status direct_build(DirectLayout* D, const float* w_dense, const float* bias,
     return PP_ERR_CUDA;
   }
   D->dmem = d;
+  D->dbytes = (nw + nb) * 4;
   D->w = static_cast<const float*>(d);
   D->bias = nb ? static_cast<const float*>(d) + nw : nullptr;
+  D->npair = npair;
   D->Co = Co;
   D->Ci = Ci;
   return PP_OK;
@@ -265,6 +669,8 @@ pp_status direct_build(DirectLayout* D, const float* w_dense, const float* bias,
 pp_status direct_launch(const DirectLayout& D, const float* x, float* y, const float* skip, int N, int H, int W,
                         int flags, cudaStream_t stream) {
   if (!D.w) return PP_ERR_UNSUPPORTED;
+  const int64_t sms = device_sms();
+  if (sms <= 0) return PP_ERR_CUDA;
   DirectParams p;
   p.x = x;
   p.y = y;
@@ -277,26 +683,64 @@ pp_status direct_launch(const DirectLayout& D, const float* x, float* y, const f
   p.H = H;
   p.W = W;
   p.flags = flags;
-  p.tiles_x = (W + DT - 1) / DT;
-  p.tiles_y = (H + DT - 1) / DT;
+  p.npair = D.npair;
+  p.tiles_x = p.tiles_y = 0;
   p.vec = (W & 3) == 0 && ((uintptr_t)x & 15) == 0;
-  // filters per CTA: up to 16, fewer when the layer has too few tiles to give
-  // every SM a few CTAs (the input tile is then staged once per filter block)
-  const int64_t nt = (int64_t)N * p.tiles_x * p.tiles_y;
-  int fbd = 16;
-  while (fbd > 1 && (fbd / 2 >= D.Co || nt * ((D.Co + fbd - 1) / fbd) < 2 * (int64_t)sm_count())) fbd /= 2;
-  const int64_t nfb = (D.Co + fbd - 1) / fbd;
-  if (nt > INT32_MAX || nfb > 65535) return PP_ERR_UNSUPPORTED;
-  const dim3 grid((unsigned)nt, (unsigned)nfb);
+  const auto ctas = [&](int th, int tw, int fbd) {
+    return (int64_t)N * ((H + th - 1) / th) * ((W + tw - 1) / tw) * ((D.Co + fbd - 1) / fbd);
+  };
   cudaError_t e;
-  switch (D.Ci) {
-    case 1: e = launch_cc<1>(p, fbd, grid, stream); break;
-    case 2: e = launch_cc<2>(p, fbd, grid, stream); break;
-    case 3: e = launch_cc<3>(p, fbd, grid, stream); break;
-    case 4: e = launch_cc<4>(p, fbd, grid, stream); break;
-    default: e = launch_cc<8>(p, fbd, grid, stream); break;  // fewer, larger copy steps
+  if (D.Co <= 4 && D.Ci >= 8 && ctas(VH, VW, 4) >= sms) {
+    // (64 -> 1 at 720 x 1280 61 us, 64 -> 3 109 us; 2 x 2 pixel blocks 97 and 147.  Fewer tiles than SMs: the split
+    // channels below, 64 -> 1 at 224 x 224 10.5 us)
+    switch (D.Co) {
+      case 1: e = launch_wide<1>(p, stream); break;
+      case 2: e = launch_wide<2>(p, stream); break;
+      case 3: e = launch_wide<3>(p, stream); break;
+      default: e = launch_wide<4>(p, stream); break;
+    }
+  } else if (D.Ci <= 4 && W > UW / 2 && D.Co > 4 && D.Co <= 65535 && ctas(UH, UW, FBMAX) >= sms / 2) {
+    // (1 -> 64 at 720 x 1280 48 us against 86 with the 32 x 32 tiles, 3 -> 64 at 224 x 224 7.2 against 9.1; below half
+    // a CTA per SM the smaller tiles win: 1 -> 64 at 64 x 96, 64 CTAs, 3.0 against 2.7)
+    int fpc = UFMAX;
+    while (fpc > FBMAX && ctas(UH, UW, fpc) < 2 * sms) fpc /= 2;
+    switch (D.Ci) {
+      case 1: e = launch_first<1>(p, fpc, stream); break;
+      case 2: e = launch_first<2>(p, fpc, stream); break;
+      case 3: e = launch_first<3>(p, fpc, stream); break;
+      default: e = launch_first<4>(p, fpc, stream); break;
+    }
+  } else {
+    // Filters per CTA: as many as there are, up to 8; channel groups while the grid would leave SMs without two CTAs,
+    // and fewer filters (the input tile is then staged more often) only when even four groups leave a quarter of the
+    // SMs idle (64 -> 64 at 56 x 56, 128 CTAs of 8 filters: 13.5 us, of 4 filters 19.7).
+    int fbd = D.Co > 4 ? 8 : D.Co > 2 ? 4 : 2, ks = 1;
+    const auto grid = [&]() { return ctas(ks == 1 ? 32 : 16, ks == 4 ? 16 : 32, fbd); };
+    if (D.Ci > 4) {
+      if (grid() < 2 * sms) ks = 2;
+      if (grid() < 2 * sms) ks = 4;
+    }
+    while (fbd > 2 && grid() < (ks == 4 ? sms * 3 / 4 : 2 * sms)) fbd /= 2;
+    if (D.Ci <= 4) {
+      switch (D.Ci) {
+        case 1: e = launch_fbd<1, 1>(p, fbd, stream); break;
+        case 2: e = launch_fbd<2, 1>(p, fbd, stream); break;
+        case 3: e = launch_fbd<3, 1>(p, fbd, stream); break;
+        default: e = launch_fbd<4, 1>(p, fbd, stream); break;
+      }
+    } else {
+      e = ks == 1 ? launch_fbd<4, 1>(p, fbd, stream)
+                  : ks == 2 ? launch_fbd<4, 2>(p, fbd, stream) : launch_fbd<4, 4>(p, fbd, stream);
+    }
   }
-  if (e != cudaSuccess) return PP_ERR_CUDA;
+  if (e == cudaErrorInvalidConfiguration) {
+    cudaGetLastError();
+    return PP_ERR_UNSUPPORTED;
+  }
+  if (e != cudaSuccess) {
+    cudaGetLastError();
+    return PP_ERR_CUDA;
+  }
   return PP_OK;
 }
 

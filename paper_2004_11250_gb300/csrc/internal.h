@@ -136,11 +136,14 @@ bool tcf_can_run(const TcLayout& T, int N, int H, int W, int flags, int R, int S
 // The geometry pinned for this shape, or R = S = 0.
 void tcf_pinned(const TcLayout& T, int N, int H, int W, int flags, int* R, int* S);
 
-// Direct FMA kernel for layers with few input or few output channels: dense
-// [Co][Ci][9] fp32 weights (zeros where pruned) and the bias, original order.
+// Direct FMA kernels for layers with few input or few output channels and for
+// dense layers: the 9 taps of every kernel in fp32 (zeros where pruned), filters
+// in pairs, and the bias, original order.
 constexpr int kDirectMaxSmall = 16;
 struct DirectLayout {
   void* dmem = nullptr;
+  size_t dbytes = 0;
+  int npair = 0;
   const float* w = nullptr;
   const float* bias = nullptr;
   int Co = 0, Ci = 0;

@@ -1133,3 +1133,30 @@ def test_resident_weight_kernel_unaligned_input(pp, runner, oracle_mod, precisio
         d.close()
     yo, s = oracle_layer_full(oracle_mod, L, x)
     check_within(g, yo, s, "unaligned input")
+
+
+# The direct kernels: dense layers between wide layers, channel groups (1, 2 or 4) on small and large grids, ragged
+# channel counts and filter pairs; the wide kernel of last layers (1 - 4 filters) and the first-layer kernel (1 - 4
+# channels) at tile edges, with and without rows of whole 16-byte groups, with more than one filter block per CTA.
+DIRECT_SHAPES = [
+    # N, Ci, Co, H, W
+    (1, 33, 47, 14, 14), (2, 20, 24, 40, 37), (1, 18, 17, 1, 1), (1, 64, 64, 33, 65), (5, 24, 40, 96, 96), (3, 17, 21, 130, 128),
+    (2, 8, 1, 720, 260), (1, 9, 2, 1250, 255), (3, 10, 3, 416, 256), (1, 16, 4, 2500, 130), (1, 8, 3, 16, 128),
+    (1, 1, 64, 18, 129), (2, 2, 70, 64, 130), (1, 3, 130, 41, 200), (1, 4, 9, 300, 257), (1, 3, 33, 6, 66), (2, 1, 5, 2000, 68),
+]
+
+
+@pytest.mark.parametrize("shape", DIRECT_SHAPES)
+@pytest.mark.parametrize("flags", ["none", "skip_relu", "skip_pool_relu"])
+def test_direct_kernels_dense(pp, runner, oracle_mod, shape, flags):
+    N, Ci, Co, H, W = shape
+    pool = "pool" in flags
+    if pool:
+        H, W = H + H % 2, W + W % 2
+    rng = np.random.default_rng(sum(shape) + len(flags))
+    D = synth.make_dense_layer(rng, Co, Ci, synth.he_std(Ci), 0.01)
+    x = rng.uniform(-1, 1, (N, Ci, H, W)).astype(np.float32)
+    skip = rng.uniform(-1, 1, (N, Co, H, W)).astype(np.float32) if "skip" in flags else None
+    g = run_layer(pp, runner, D, x, skip, "relu" in flags, pool)
+    y, s = oracle_layer_full(oracle_mod, D, x, skip, "relu" in flags, pool)
+    check_within(g, y, s, f"dense {shape} {flags}")
