@@ -260,12 +260,13 @@ pp_status pp_layer_precision(const pp_layer* layer, int* precision, float* input
  *                       consecutive of its 8 neighbours).
  *   PP_KERNEL_REGISTER  FP32 FMA over kept taps, accumulators in registers;
  *                       any pattern set.
- *   PP_KERNEL_DIRECT    FP32 FMA over all 9 taps of dense [Co][Ci][9] weights
- *                       (zeros where pruned), one 2 x 2 pixel block and up to
- *                       16 filters per thread; layers with at most 16 input
- *                       or at most 16 output channels (first and last layers).
+ *   PP_KERNEL_DIRECT    FP32 FMA over all 9 taps of dense weights (zeros where
+ *                       pruned), a block of pixels and up to 8 filters per
+ *                       thread; layers with at most 16 input or at most 16
+ *                       output channels (first and last layers).
  * PP_KERNEL_AUTO picks by an estimate of each kernel's time for the layer's
- * density (the direct kernel for Ci <= 4).  Setting a kernel the layer cannot
+ * density (the direct kernel for Ci <= 4, and in place of an FMA kernel that it
+ * beats, then also with more channels).  Setting a kernel the layer cannot
  * run returns PP_ERR_UNSUPPORTED. */
 #define PP_KERNEL_AUTO 0
 #define PP_KERNEL_TMEM 1
@@ -376,9 +377,8 @@ typedef struct pp_dense pp_dense;
 /* w [Co][Ci][9] and bias [Co] (or NULL) are host fp32; copied to the device. */
 pp_status pp_dense_create(const float* w, const float* bias, int Co, int Ci, void* stream, pp_dense** out);
 
-/* Same contract as pp_conv_forward, over all 9 taps of every kernel.  Layers
- * with at most 16 input or at most 16 output channels run the direct FMA
- * kernel (PP_KERNEL_DIRECT); others the register-accumulator kernel. */
+/* Same contract as pp_conv_forward, over all 9 taps of every kernel, by the
+ * direct FMA kernels (PP_KERNEL_DIRECT). */
 pp_status pp_dense_forward(const pp_dense* layer, const float* x, float* y, const float* skip, int N, int H, int W,
                            int flags, void* stream);
 

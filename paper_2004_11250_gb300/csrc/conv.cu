@@ -99,14 +99,12 @@ struct ConvParams {
   int nch, G;
   int tiles_x;
   int flags;
-  int cc;      // input channels per stage (<= CC; entries per warp and stage stay <= EMAX)
   int ksplit;  // CTAs of a cluster sharing one output tile (split over input chunks)
   int cpk;     // input chunks per split
 };
 
 // Entry code layout: bits 0..15 pattern payload (MODE_RING8: ring index;
-// MODE_GENERIC: 4 taps x 4 bits), 16..19 slot, 20..27 channel within the stage,
-// 28..29 number of taps - 1 (MODE_GENERIC).
+// MODE_GENERIC: 4 taps x 4 bits), 16..19 slot, 20..27 channel within the stage.
 __device__ __forceinline__ int code_slot(uint32_t c) { return (c >> 16) & 15; }
 __device__ __forceinline__ int code_ch(uint32_t c) { return (c >> 20) & 255; }
 
@@ -189,11 +187,10 @@ __device__ __forceinline__ void dispatch(float (&acc)[F][PX], const float (&win)
     }
   } else {
     const int slot9 = code_slot(code) * 9;
-    const int nt = ((code >> 28) & 3) + 1;
     uint32_t taps = code & 0xffff;
     float wv[4] = {w.x, w.y, w.z, w.w};
 #pragma unroll 1
-    for (int s = 0; s < nt; ++s) {
+    for (int s = 0; s < 4; ++s) {
       const float ws = s == 0 ? wv[0] : s == 1 ? wv[1] : s == 2 ? wv[2] : wv[3];
       switch (slot9 + (int)(taps & 15)) {
 #define PP_TAP_CASE(J, T) \
@@ -291,7 +288,7 @@ __global__ void __launch_bounds__(NTHREADS, 2) ppconv_kernel(const ConvParams p)
 
   auto issue = [&](int c) {
     unsigned char* st = smem + (c & 1) * STAGE_BYTES;
-    stage_input(reinterpret_cast<float*>(st + OFF_IN), p, n, c * p.cc, min(p.cc, p.Ci - c * p.cc), r0, c0);
+    stage_input(reinterpret_cast<float*>(st + OFF_IN), p, n, c * CC, min(CC, p.Ci - c * CC), r0, c0);
     if (active) stage_entries(st, p, warp, lane, __ldg(cofs + c), __ldg(cofs + c + 1));
     cp_async_commit();
   };
@@ -401,9 +398,9 @@ struct pp_layer {
   int auto_kernel = 2;
   ppc::TmLayout tm;
   ppc::TcLayout tc;
-  ppc::DirectLayout direct;  // built for layers with few input or output channels
+  ppc::DirectLayout direct;  // built for layers with few input or output channels and where the default choice is it
+  bool direct_ok = false;    // few input or output channels: pp_layer_set_kernel accepts PP_KERNEL_DIRECT
   int G = 0, nch = 0;
-  int cc = CC;  // input channels per stage
   int64_t nE = 0;
   bool has_bias = false;
   void* dmem = nullptr;  // one allocation holding every array below
@@ -453,13 +450,12 @@ bool ring_map(const uint8_t* taps, int P, std::vector<int>& map) {
 
 // Build the device layout from per-filter entry lists (filters already in
 // reordered order) and upload it.
-pp_status build_layer(pp_layer* L, int Co, int Ci, int cc, const std::vector<std::vector<Entry>>& per_filter,
+pp_status build_layer(pp_layer* L, int Co, int Ci, const std::vector<std::vector<Entry>>& per_filter,
                       const std::vector<int32_t>& perm, const float* bias_reordered, cudaStream_t stream) {
   L->Co = Co;
   L->Ci = Ci;
-  L->cc = cc;
   L->G = (Co + F - 1) / F;
-  L->nch = (Ci + cc - 1) / cc;
+  L->nch = (Ci + CC - 1) / CC;
   L->has_bias = bias_reordered != nullptr;
   std::vector<int> cofs((size_t)L->G * (L->nch + 1));
   std::vector<uint32_t> code;
@@ -476,14 +472,14 @@ pp_status build_layer(pp_layer* L, int Co, int Ci, int cc, const std::vector<std
     });
     size_t k = 0;
     for (int c = 0; c <= L->nch; ++c) {
-      while (k < es.size() && es[k].ch < c * cc) ++k;
+      while (k < es.size() && es[k].ch < c * CC) ++k;
       cofs[(size_t)q * (L->nch + 1) + c] = (int)(code.size() + k);
     }
     for (int c = 0; c < L->nch; ++c)  // the kernel stages at most EMAX entries per warp and chunk
       if (cofs[(size_t)q * (L->nch + 1) + c + 1] - cofs[(size_t)q * (L->nch + 1) + c] > EMAX)
         return PP_ERR_UNSUPPORTED;
     for (const Entry& e : es) {
-      code.push_back(e.payload | (uint32_t(e.slot) << 16) | (uint32_t(e.ch % cc) << 20));
+      code.push_back(e.payload | (uint32_t(e.slot) << 16) | (uint32_t(e.ch % CC) << 20));
       for (int s = 0; s < 4; ++s) wts.push_back(e.w[s]);
     }
   }
@@ -595,7 +591,6 @@ pp_status launch(const pp_layer* L, const float* x, float* y, const float* skip,
   p.H = H;
   p.W = W;
   p.nch = L->nch;
-  p.cc = L->cc;
   p.G = L->G;
   p.tiles_x = tiles_x;
   p.flags = flags;
@@ -673,13 +668,13 @@ extern "C" pp_status pp_layer_create(const pp_packed* pk, const float* bias, voi
         en.payload = (uint32_t)rmap[p];
       } else {
         const uint8_t* t = &pk->taps[4 * p];
-        en.payload = t[0] | (t[1] << 4) | (t[2] << 8) | (t[3] << 12) | (3u << 28);
+        en.payload = t[0] | (t[1] << 4) | (t[2] << 8) | (t[3] << 12);
       }
       for (int s = 0; s < 4; ++s) en.w[s] = pk->kw[(size_t)e * 4 + s];
       per_filter[j].push_back(en);
     }
   }
-  pp_status st = build_layer(L, pk->Co, pk->Ci, CC, per_filter, pk->perm, bias ? bias_r.data() : nullptr,
+  pp_status st = build_layer(L, pk->Co, pk->Ci, per_filter, pk->perm, bias ? bias_r.data() : nullptr,
                              (cudaStream_t)stream);
   if (st == PP_OK && L->mode == MODE_RING8) {
     st = ppc::tm_prepare();
@@ -694,7 +689,27 @@ extern "C" pp_status pp_layer_create(const pp_packed* pk, const float* bias, voi
     L->tc_ok = st == PP_OK;
     if (L->tc_ok) L->packed = *pk;
   }
-  if (st == PP_OK && ppc::direct_applicable(pk->Co, pk->Ci)) {
+  // Kernel choice by estimated SM cycles per pixel: the tensor cores run the
+  // dense 9-tap contraction (filters padded to 128, channels to 8) three times
+  // at ~1800 multiply-adds per cycle; the FMA kernels run only the kept taps
+  // at a quarter of the 128 FMA lanes (what they reach on these layers).
+  const double nk = (double)pk->kidx.size();
+  const double tc_cycles = 27.0 * (double)((pk->Co + 127) / 128 * 128) * (double)((pk->Ci + 7) / 8 * 8) / 1800.0;
+  const double fma_cycles = 4.0 * nk / 32.0;
+  L->auto_kernel = (L->tc_ok && tc_cycles < fma_cycles) ? (L->tc.FB == 128 ? PP_KERNEL_TC_FLAT : PP_KERNEL_TC)
+                                                         : (L->tm_ok ? PP_KERNEL_TMEM : PP_KERNEL_REGISTER);
+  // Where the estimate wants FP32, the direct kernel's 9 taps on packed FMAs beat the register kernel's dispatch at
+  // any density (64 -> 24 at 128 x 128, keep 0.2 / 0.5 / 0.9: 21 us against 54 / 110 / 181) and the TMEM kernel on
+  // layers that leave its 64-filter CTAs half empty (21 against 21 / 25 / 30; 64 -> 48 keep 0.2: 31 against 25).  Layers
+  // of a few dozen kernels are bound by the launch and keep their choice.
+  const bool fma = L->auto_kernel == PP_KERNEL_REGISTER || (L->auto_kernel == PP_KERNEL_TMEM && pk->Co <= 32);
+  const int64_t pairs = (int64_t)pk->Co * pk->Ci;
+  const bool direct_auto = fma && pairs >= 256 && pairs <= (int64_t(1) << 20);
+  // layers with a handful of input channels (a network's first layer) run the
+  // direct kernel: the others cannot fill their tiles
+  L->direct_ok = ppc::direct_applicable(pk->Co, pk->Ci);
+  if (direct_auto || (L->direct_ok && pk->Ci <= 4)) L->auto_kernel = PP_KERNEL_DIRECT;
+  if (st == PP_OK && (L->direct_ok || direct_auto)) {
     // dense [Co][Ci][9] in the original filter order, zeros where pruned
     std::vector<float> wd((size_t)pk->Co * pk->Ci * 9, 0.f);
     for (int j = 0; j < pk->Co; ++j)
@@ -712,18 +727,6 @@ extern "C" pp_status pp_layer_create(const pp_packed* pk, const float* bias, voi
     return st;
   }
   L->pk_perm = pk->perm;
-  // Kernel choice by estimated SM cycles per pixel: the tensor cores run the
-  // dense 9-tap contraction (filters padded to 128, channels to 8) three times
-  // at ~1800 multiply-adds per cycle; the FMA kernels run only the kept taps
-  // at a quarter of the 128 FMA lanes (what they reach on these layers).
-  const double nk = (double)pk->kidx.size();
-  const double tc_cycles = 27.0 * (double)((pk->Co + 127) / 128 * 128) * (double)((pk->Ci + 7) / 8 * 8) / 1800.0;
-  const double fma_cycles = 4.0 * nk / 32.0;
-  L->auto_kernel = (L->tc_ok && tc_cycles < fma_cycles) ? (L->tc.FB == 128 ? PP_KERNEL_TC_FLAT : PP_KERNEL_TC)
-                                                         : (L->tm_ok ? PP_KERNEL_TMEM : PP_KERNEL_REGISTER);
-  // layers with a handful of input channels (a network's first layer) run the
-  // direct kernel: the others cannot fill their tiles
-  if (L->direct.w && pk->Ci <= 4) L->auto_kernel = PP_KERNEL_DIRECT;
   L->kernel = L->auto_kernel;
   *out = L;
   return PP_OK;
@@ -809,7 +812,7 @@ extern "C" pp_status pp_layer_set_kernel(pp_layer* L, int kernel) {
       return PP_OK;
     case PP_KERNEL_REGISTER: L->kernel = kernel; return PP_OK;
     case PP_KERNEL_DIRECT:
-      if (!L->direct.w) return PP_ERR_UNSUPPORTED;
+      if (!L->direct_ok) return PP_ERR_UNSUPPORTED;
       L->kernel = kernel;
       return PP_OK;
     default: return PP_ERR_INVALID_ARG;
