@@ -266,6 +266,7 @@ __global__ void __launch_bounds__(flat_threads<SPLIT, F16>(), 1) ppconv_tcf_kern
   // compiler keeps every access below in the shared state space.
   unsigned char* smem = smem_raw + ((1024u - (su32(smem_raw) & 1023u)) & 1023u);
   __shared__ __align__(8) uint64_t full[2], raw_full[2], empty[2], acc_full[2], acc_empty[2], done_bar;
+  __shared__ __align__(8) uint64_t raw_empty[2];  // f16 with a box ring: every loader warp has read the chunk's box
   __shared__ __align__(8) uint64_t wempty[WSL_MAX];  // a weight-ring slot has been read by its MMAs
   __shared__ __align__(8) uint64_t pfull[2];  // PAIR, even CTA: the odd CTA's stage is full
   __shared__ uint32_t tmem_s;
@@ -288,12 +289,14 @@ __global__ void __launch_bounds__(flat_threads<SPLIT, F16>(), 1) ppconv_tcf_kern
 
   if (tid == 0) {
     for (int s = 0; s < 2; ++s) {
-      // a stage is full once every loader thread has stored its part of the
-      // input operands and the chunk's weight copies (one more arrival each,
+      // a stage is full once every loader thread (f16 with a box ring: one
+      // arrival per loader warp) has stored its part of the input operands and the
+      // chunk's weight copies (one more arrival each,
       // with its bytes: the three group copies, or without the ring the whole
       // chunk) have landed: the MMA thread waits on one barrier per chunk
-      mbar_init(su32(&full[s]), NLOAD + (WR ? NGRP : 1));
+      mbar_init(su32(&full[s]), (F16 && p.use_tma && p.sep ? MMA_WARP : NLOAD) + (WR ? NGRP : 1));
       mbar_init(su32(&raw_full[s]), 1);
+      mbar_init(su32(&raw_empty[s]), MMA_WARP);
       mbar_init(su32(&empty[s]), 1);
       mbar_init(su32(&acc_full[s]), 1);
       mbar_init(su32(&acc_empty[s]), NEPI);
@@ -429,8 +432,10 @@ __global__ void __launch_bounds__(flat_threads<SPLIT, F16>(), 1) ppconv_tcf_kern
     if (tid == 0 && p.use_tma && p.sep)
       for (; raw_issued < p.sep && raw_issued < nall; ++raw_issued)
         issue_raw(raw_issued, smem + p.raw_off + raw_issued * p.raw_slot);
-    bool stop = false;  // identical in every loader thread (decided by group_any)
-    uint32_t range_bad = 0;  // f16: nonzero once an input is non-finite or overflows fp16 after scaling
+    bool stop = false;  // identical in every loader thread (decided by group_any), f16 with a box ring in every lane of a warp
+    __half2 hmax = __floats2half2_rn(0.f, 0.f);  // f16: largest |x| after scaling: infinite or NaN out of fp16's range
+    const bool early = p.use_tma && p.sep;
+    const int nit = (2 * p.npix + NLOAD - 1) / NLOAD;  // items per thread
     for (int i = 0; i < nmine && !stop; ++i) {
       const Tile T = my_tile(tile_index(i));
       const float* xb = p.x + (size_t)T.n * p.Ci * p.H * p.W;
@@ -445,9 +450,12 @@ __global__ void __launch_bounds__(flat_threads<SPLIT, F16>(), 1) ppconv_tcf_kern
         // there (the tf32 split is cheap and follows the stage wait).
         // v holds an item's input values, or (f16, read early) its packed hi words then lo words
         float v[ITEMS_MAX][CPH];
-        const bool early = p.use_tma && p.sep;
         if (early) {
-          if (group_any<NLOAD>(!wait(&raw_full[s], (uint32_t)(use & 1)))) {
+          // f16: no barrier over the loader warps; each waits for the box itself, and thread 0 alone waits until all
+          // have read it before it issues the next copy into the slot (256 -> 256 at 56 x 56, batch 8: 70.8 -> 67.9 us
+          // with the cheaper split; the tf32 loaders, whose warps have little to do per chunk, ran 5 % slower so).
+          const bool landed = wait(&raw_full[s], (uint32_t)(use & 1));
+          if (F16 ? !__all_sync(0xffffffffu, landed) : group_any<NLOAD>(!landed)) {
             stop = true;
             break;
           }
@@ -455,12 +463,13 @@ __global__ void __launch_bounds__(flat_threads<SPLIT, F16>(), 1) ppconv_tcf_kern
 #pragma unroll
           for (int b = 0; b < ITEMS_MAX; ++b) {
             if constexpr (F16) {
+              if (b >= nit) break;
               // split as soon as read: only the packed halves stay live
               float u[CPH];
 #pragma unroll
               for (int k = 0; k < CPH; ++k) u[k] = roff[b] >= 0 ? raw[roff[b] + tsh + k * cstride] : 0.f;
-              uint4 h = make_uint4(0, 0, 0, 0), l = h;
-              if (doff[b] >= 0) range_bad |= split_f16x8(u, p.xscale, h, l);
+              uint4 h, l;
+              split_f16x8_max(u, p.xscale, h, l, hmax);
               v[b][0] = __uint_as_float(h.x);
               v[b][1] = __uint_as_float(h.y);
               v[b][2] = __uint_as_float(h.z);
@@ -475,12 +484,22 @@ __global__ void __launch_bounds__(flat_threads<SPLIT, F16>(), 1) ppconv_tcf_kern
             }
           }
           // the slot is rewritten next by a tensor-map copy (async proxy): each thread orders its reads of
-          // it before that copy with a proxy fence, then the loader barrier lets thread 0 issue it
+          // it before that copy with a proxy fence
           asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-          group_sync<NLOAD>();
-          if (tid == 0 && raw_issued < nall && raw_issued == g + p.sep) {
-            issue_raw(raw_issued, smem + p.raw_off + (size_t)(raw_issued & (p.sep - 1)) * p.raw_slot);
-            ++raw_issued;
+          if constexpr (F16) {
+            __syncwarp();
+            if (lane == 0) mbar_arrive(su32(&raw_empty[s]));
+            if (tid == 0 && raw_issued < nall && raw_issued == g + p.sep && wait(&raw_empty[s], (uint32_t)(use & 1))) {
+              issue_raw(raw_issued, smem + p.raw_off + (size_t)(raw_issued & (p.sep - 1)) * p.raw_slot);
+              ++raw_issued;
+            }
+            __syncwarp();
+          } else {
+            group_sync<NLOAD>();
+            if (tid == 0 && raw_issued < nall && raw_issued == g + p.sep) {
+              issue_raw(raw_issued, smem + p.raw_off + (size_t)(raw_issued & (p.sep - 1)) * p.raw_slot);
+              ++raw_issued;
+            }
           }
         }
         if (!p.use_tma) {
@@ -496,7 +515,8 @@ __global__ void __launch_bounds__(flat_threads<SPLIT, F16>(), 1) ppconv_tcf_kern
             }
           }
         }
-        if (group_any<NLOAD>(use > 0 && !wait(&empty[s], (uint32_t)((use - 1) & 1)))) {
+        const bool freed = use == 0 || wait(&empty[s], (uint32_t)((use - 1) & 1));
+        if (F16 && early ? !__all_sync(0xffffffffu, freed) : group_any<NLOAD>(!freed)) {
           stop = true;
           break;
         }
@@ -535,6 +555,7 @@ __global__ void __launch_bounds__(flat_threads<SPLIT, F16>(), 1) ppconv_tcf_kern
         }
 #pragma unroll
         for (int b = 0; b < ITEMS_MAX; ++b) {
+          if (F16 && b >= nit) break;
           if (doff[b] >= 0) {
             const int dst = doff[b];
             if constexpr (F16) {
@@ -545,7 +566,7 @@ __global__ void __launch_bounds__(flat_threads<SPLIT, F16>(), 1) ppconv_tcf_kern
                 l = make_uint4(__float_as_uint(v[b][4]), __float_as_uint(v[b][5]), __float_as_uint(v[b][6]),
                                __float_as_uint(v[b][7]));
               } else {
-                range_bad |= split_f16x8(&v[b][0], p.xscale, h, l);
+                split_f16x8_max(&v[b][0], p.xscale, h, l, hmax);
               }
               reinterpret_cast<uint4*>(hi)[dst] = h;
               reinterpret_cast<uint4*>(lo)[dst] = l;
@@ -561,10 +582,15 @@ __global__ void __launch_bounds__(flat_threads<SPLIT, F16>(), 1) ppconv_tcf_kern
           }
         }
         asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-        mbar_arrive(su32(&full[s]));
+        if (F16 && early) {
+          __syncwarp();
+          if (lane == 0) mbar_arrive(su32(&full[s]));
+        } else {
+          mbar_arrive(su32(&full[s]));
+        }
       }
     }
-    if (F16 && range_bad != 0) atomicOr(p.status, ppc::kStatusF16Range);
+    if (F16 && f16_max_bad(hmax)) atomicOr(p.status, ppc::kStatusF16Range);
     if (tid == 0) {
       // No copy may still be writing shared memory when the CTA exits: wait
       // (bounded) for the last copies issued into each stage.  (After a timeout
