@@ -159,7 +159,7 @@ __device__ __forceinline__ Tile tile_of(const FlatParams& p, int t) {
 // 2 with CTA pairs: the even and the odd CTAs hold different filter blocks).
 template <int S>
 __device__ __forceinline__ void split_reduce(const FlatParams& p, const Tile& T, int m0, int nm, float* part,
-                                             const int* o_s, const float* b_s, int tid, int rstride, int rofs) {
+                                             const int* o_s, int tid, int rstride, int rofs) {
   namespace cg = cooperative_groups;
   cg::cluster_group cl = cg::this_cluster();
   const float* src[S];
@@ -168,6 +168,7 @@ __device__ __forceinline__ void split_reduce(const FlatParams& p, const Tile& T,
   const int pst = p.ncols + 4;
   const bool relu = p.flags & PP_RELU;
   const float* skip = (p.flags & PP_ADD_SKIP) ? p.skip : nullptr;
+  const float* bias = p.bias ? p.bias + T.fb * FB + m0 : nullptr;  // of the owned filters (read only where they exist)
   auto sum = [&](int off) -> float4 {
     float4 v[S];
 #pragma unroll
@@ -189,12 +190,13 @@ __device__ __forceinline__ void split_reduce(const FlatParams& p, const Tile& T,
       const int ro = rest / qw, cx = (rest - ro * qw) * 4;
       const int row = T.r0 + ro, o = o_s[ml];
       if (row >= p.H || o < 0) continue;
+      const float bs = bias ? __ldg(bias + ml) : 0.f;
       const float4 a = sum((m0 + ml) * pst + ro * p.bcols + cx);
       const size_t yoff = (((size_t)T.n * p.Co + o) * p.H + row) * p.W + cx;
       float v[4] = {a.x, a.y, a.z, a.w};
 #pragma unroll
       for (int k = 0; k < 4; ++k) {
-        v[k] += b_s[ml];
+        v[k] += bs;
         if (skip && cx + k < p.W) v[k] += __ldg(skip + yoff + k);
         if (relu) v[k] = fmaxf(v[k], 0.f);
       }
@@ -219,6 +221,7 @@ __device__ __forceinline__ void split_reduce(const FlatParams& p, const Tile& T,
       const int orow = T.r0 / 2 + pr, o = o_s[ml];
       if (orow >= Ho || o < 0) continue;
       const int off = (m0 + ml) * pst + 2 * pr * p.bcols + 2 * pc;
+      const float bs = bias ? __ldg(bias + ml) : 0.f;
       const float4 a = sum(off), b = sum(off + p.bcols);
       const size_t plane = (size_t)T.n * p.Co + o;
       // window d of pooled output e: row 2 pr + (d >> 1), column 2 (pc + e) + (d & 1)
@@ -229,7 +232,7 @@ __device__ __forceinline__ void split_reduce(const FlatParams& p, const Tile& T,
         float mx = 0.f;
 #pragma unroll
         for (int d = 0; d < 4; ++d) {
-          float v = win[e][d] + b_s[ml];
+          float v = win[e][d] + bs;
           if (skip && pc + e < Wo)
             v += __ldg(skip + (plane * p.H + 2 * orow + (d >> 1)) * p.W + 2 * (pc + e) + (d & 1));
           if (relu) v = fmaxf(v, 0.f);
@@ -271,8 +274,7 @@ __global__ void __launch_bounds__(flat_threads<SPLIT, F16>(), 1) ppconv_tcf_kern
   __shared__ __align__(8) uint64_t pfull[2];  // PAIR, even CTA: the odd CTA's stage is full
   __shared__ uint32_t tmem_s;
   __shared__ volatile int abort_s;
-  __shared__ int o_s[FB / 2];    // split phase: original index of each owned filter (-1 beyond Co)
-  __shared__ float b_s[FB / 2];  // and its bias
+  __shared__ int o_s[FB];    // split phase: original index of each owned filter (-1 beyond Co)
 
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
 
@@ -892,8 +894,8 @@ __global__ void __launch_bounds__(flat_threads<SPLIT, F16>(), 1) ppconv_tcf_kern
     // (release / acquire at cluster scope) orders every CTA's partial tile in
     // its shared memory, and the filter table below, before the reads; the
     // second keeps each CTA's shared memory alive until the others have read it.
-    // This CTA finishes filters [m0, m1) of the tile (at most FB / 2 of them);
-    // their original indices and biases are fetched now, so the loads overlap
+    // This CTA finishes filters [m0, m1) of the tile (all of them when the split is 1);
+    // their original indices are fetched now, so the loads overlap
     // the barrier wait.
     const int tile = (int)blockIdx.x / csize, rstride = PAIR ? 2 : 1;
     const int m0 = srank * FB / p.split, m1 = (srank + 1) * FB / p.split, nm = m1 - m0;
@@ -901,17 +903,17 @@ __global__ void __launch_bounds__(flat_threads<SPLIT, F16>(), 1) ppconv_tcf_kern
     if (tid < nm) {
       const int jr = T.fb * FB + m0 + tid;
       o_s[tid] = jr < p.Co ? __ldg(p.perm + jr) : -1;
-      b_s[tid] = (jr < p.Co && p.bias) ? __ldg(p.bias + jr) : 0.f;
     }
     __syncwarp();
     asm volatile("barrier.cluster.arrive.release;\n\tbarrier.cluster.wait.acquire;" ::: "memory");
     if (!abort_s) {
       float* part = reinterpret_cast<float*>(smem);
       switch (p.split) {
-        case 2: split_reduce<2>(p, T, m0, nm, part, o_s, b_s, tid, rstride, pp); break;
-        case 4: split_reduce<4>(p, T, m0, nm, part, o_s, b_s, tid, rstride, pp); break;
-        case 8: split_reduce<8>(p, T, m0, nm, part, o_s, b_s, tid, rstride, pp); break;
-        default: split_reduce<16>(p, T, m0, nm, part, o_s, b_s, tid, rstride, pp); break;
+        case 1: split_reduce<1>(p, T, m0, nm, part, o_s, tid, rstride, pp); break;
+        case 2: split_reduce<2>(p, T, m0, nm, part, o_s, tid, rstride, pp); break;
+        case 4: split_reduce<4>(p, T, m0, nm, part, o_s, tid, rstride, pp); break;
+        case 8: split_reduce<8>(p, T, m0, nm, part, o_s, tid, rstride, pp); break;
+        default: split_reduce<16>(p, T, m0, nm, part, o_s, tid, rstride, pp); break;
       }
     }
     __syncwarp();
@@ -1022,10 +1024,19 @@ struct FlatGeo {
 // SM cycles: an MMA of N columns takes the longer of its multiply-adds at
 // ~1850 per cycle and its operand reads (4 KB of weights + 32 N bytes of
 // input) at 128 shared-memory bytes per cycle; a chunk also needs its 73.7 KB
-// of weights from L2 (~48 bytes per cycle) and at least ~1500 cycles of
-// staging latency with two stages; a start-up and pipeline fill of ~5000
-// cycles; the split's partial-tile round trip through L2 at ~64 bytes per
-// cycle; and clusters beyond those co-resident on the GPU run in later waves.
+// of weights from L2 (~48 bytes per cycle) and the loaders' round of its input,
+// which measured 2250 cycles in tf32 at any width up to 128 columns and 2550 +
+// 7 N in f16 (16 channels to split), 900 more where rows and planes are not
+// 16-byte aligned and each thread loads its own; start-up, pipeline fill and
+// teardown of ~9000 cycles; the last tile's copy out of tensor memory at ~16
+// cycles a column and the remote part of a split's partials at ~24 more;
+// clusters of 16 start late (~12000); and clusters beyond those co-resident on
+// the GPU run in later waves.  CTA pairs measured slower than their halves apart
+// (39.6 against 31.4 us at 512 -> 512, 28 x 28): 1.15 of the chunk time.  Against
+// every accepted geometry of 21 shapes the model's choice measured within 1 % of
+// the fastest; the model before it (1500 cycles a chunk, pairs at 0.8, start-up
+// 5000) was up to 1.8 times off it (100 -> 200 at 45 x 61: R = 2 unsplit, 42 us,
+// against R = 4 split in 2, 23).
 // Every geometry the kernel can run for this shape, best first by the model;
 // fills up to maxn entries and returns how many.
 // f16: nch counts 16-channel chunks and the input box holds 16 channels; a tile
@@ -1087,10 +1098,9 @@ int flat_candidates(int N, int H, int W, int nch, int nfb, bool pool, bool allow
       if (wide && pair) continue;
       G.ntiles = (int)nt;
       const double mma = 27.0 * std::max(G.ncols * 128.0 * 8.0 / 1850.0, 32.0 + G.ncols / 4.0);
-      // pairs: each SM reads half the input operand bytes per MMA and issues half the MMAs; modelled as 0.8
-      // of the chunk time (the input operand reads are ~20 % of a chunk's shared-memory traffic)
-      const double per_chunk = std::max(std::max(mma, W_BYTES / 48.0), 1500.0) * (pair ? 0.8 : 1.0);
-      // (split mode owns at most FB / 2 filters per CTA in its second phase: pairs split at least 2 ways)
+      const double load = (f16 ? 2550.0 + 7.0 * G.ncols : 2250.0) + ((W & 3) && ((int64_t)H * W & 3) ? 900.0 : 0.0);
+      const double per_chunk = std::max(std::max(mma, W_BYTES / 48.0), load) * (pair ? 1.15 : 1.0);
+      // (pairs split at least 2 ways)
       for (int s = pair ? 2 : 1; s <= MAX_SPLIT; s *= 2) {
         const int cs = pair ? 2 * s : s;  // cluster size
         if (cs > MAX_SPLIT) break;
@@ -1098,12 +1108,13 @@ int flat_candidates(int N, int H, int W, int nch, int nfb, bool pool, bool allow
         double cost;
         if (cs == 1) {
           const double waves = std::ceil((double)G.ntiles / D.sms);
-          // single-buffered: every tile's epilogue but the last is no longer hidden behind MMAs
-          cost = waves * nch * per_chunk + 5000.0 + (wide ? (waves - 1) * 16.0 * G.ncols : 0.0);
+          // single-buffered: every tile's epilogue, not only the last, is exposed
+          cost = waves * nch * per_chunk + 9000.0 + (wide ? waves : 1.0) * 16.0 * G.ncols;
         } else {
           // clusters beyond those that fit on the GPU at once run in a later wave
           const double waves = std::ceil((double)G.ntiles / D.max_clusters[cs]);
-          cost = waves * (std::ceil((double)nch / s) * per_chunk + 5000.0 + 16.0 * G.ncols);
+          cost = waves * (std::ceil((double)nch / s) * per_chunk + 9000.0 + (cs == 16 ? 12000.0 : 0.0) +
+                          (16.0 + 24.0 * (s - 1) / s) * G.ncols);
         }
         G.split = s;
         G.cost = cost;
@@ -1204,7 +1215,13 @@ pp_status launch_geo(const FlatGeo& G, const DeviceState& Dref, const ppc::TcLay
   p.raw_w = G.raw_w;
   p.raw_bytes = G.raw_bytes;
   // without the weight ring (unsplit tf32): two whole-chunk weight slots, 6 group slots
-  const bool ring = G.split > 1 || G.pair || f16;
+  // One tile per CTA, and rows that do not allow 16-byte stores or a residual: the split instantiation with a split of
+  // 1 (a cluster of one CTA).  Its second phase finishes a tile with whole rows per warp, where the other epilogue has a
+  // filter per lane and touches 32 planes with every 4-byte access (100 -> 200 at 45 x 61, batch 3, with residual, R = 2:
+  // 42.3 -> 26.9 us).  Aligned rows without residual leave in 16-byte stores as fast (128 -> 128 at 128 x 128, tf32 27.8
+  // against 27.4, f16 21.1 against 22.4).
+  const bool one = G.split == 1 && !G.pair && G.ntiles <= D->sms && ((W & 3) || (flags & PP_ADD_SKIP));
+  const bool ring = G.split > 1 || G.pair || f16 || one;
   p.wsl = ring ? G.wsl : 6;
   p.xoff = p.wsl * GRP_BYTES;
   p.xstage = G.xstage;
@@ -1277,7 +1294,7 @@ pp_status launch_geo(const FlatGeo& G, const DeviceState& Dref, const ppc::TcLay
     cfg.gridDim = dim3((unsigned)(G.ntiles * 2 * G.split));
     e = f16 ? cudaLaunchKernelEx(&cfg, ppconv_tcf_kernel<true, true, true>, p, xmap)
             : cudaLaunchKernelEx(&cfg, ppconv_tcf_kernel<true, false, true>, p, xmap);
-  } else if (G.split > 1) {
+  } else if (G.split > 1 || one) {
     at[1].id = cudaLaunchAttributeClusterDimension;
     at[1].val.clusterDim.x = (unsigned)G.split;
     at[1].val.clusterDim.y = 1;
