@@ -159,7 +159,7 @@ __device__ __forceinline__ Tile tile_of(const FlatParams& p, int t) {
 // 2 with CTA pairs: the even and the odd CTAs hold different filter blocks).
 template <int S>
 __device__ __forceinline__ void split_reduce(const FlatParams& p, const Tile& T, int m0, int nm, float* part,
-                                             const int* o_s, int tid, int rstride, int rofs) {
+                                             const int* o_s, const float* b_s, int tid, int rstride, int rofs) {
   namespace cg = cooperative_groups;
   cg::cluster_group cl = cg::this_cluster();
   const float* src[S];
@@ -168,7 +168,9 @@ __device__ __forceinline__ void split_reduce(const FlatParams& p, const Tile& T,
   const int pst = p.ncols + 4;
   const bool relu = p.flags & PP_RELU;
   const float* skip = (p.flags & PP_ADD_SKIP) ? p.skip : nullptr;
-  const float* bias = p.bias ? p.bias + T.fb * FB + m0 : nullptr;  // of the owned filters (read only where they exist)
+  const auto bias_of = [&](int ml) -> float {
+    return S > 1 ? b_s[ml] : (p.bias ? __ldg(p.bias + T.fb * FB + m0 + ml) : 0.f);  // only filters that exist
+  };
   auto sum = [&](int off) -> float4 {
     float4 v[S];
 #pragma unroll
@@ -190,7 +192,7 @@ __device__ __forceinline__ void split_reduce(const FlatParams& p, const Tile& T,
       const int ro = rest / qw, cx = (rest - ro * qw) * 4;
       const int row = T.r0 + ro, o = o_s[ml];
       if (row >= p.H || o < 0) continue;
-      const float bs = bias ? __ldg(bias + ml) : 0.f;
+      const float bs = bias_of(ml);
       const float4 a = sum((m0 + ml) * pst + ro * p.bcols + cx);
       const size_t yoff = (((size_t)T.n * p.Co + o) * p.H + row) * p.W + cx;
       float v[4] = {a.x, a.y, a.z, a.w};
@@ -221,7 +223,7 @@ __device__ __forceinline__ void split_reduce(const FlatParams& p, const Tile& T,
       const int orow = T.r0 / 2 + pr, o = o_s[ml];
       if (orow >= Ho || o < 0) continue;
       const int off = (m0 + ml) * pst + 2 * pr * p.bcols + 2 * pc;
-      const float bs = bias ? __ldg(bias + ml) : 0.f;
+      const float bs = bias_of(ml);
       const float4 a = sum(off), b = sum(off + p.bcols);
       const size_t plane = (size_t)T.n * p.Co + o;
       // window d of pooled output e: row 2 pr + (d >> 1), column 2 (pc + e) + (d & 1)
@@ -274,7 +276,8 @@ __global__ void __launch_bounds__(flat_threads<SPLIT, F16>(), 1) ppconv_tcf_kern
   __shared__ __align__(8) uint64_t pfull[2];  // PAIR, even CTA: the odd CTA's stage is full
   __shared__ uint32_t tmem_s;
   __shared__ volatile int abort_s;
-  __shared__ int o_s[FB];    // split phase: original index of each owned filter (-1 beyond Co)
+  __shared__ int o_s[FB];        // split phase: original index of each owned filter (-1 beyond Co)
+  __shared__ float b_s[FB / 2];  // and, with a split of 2 or more, its bias (shared memory has no room for 128)
 
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
 
@@ -895,7 +898,7 @@ __global__ void __launch_bounds__(flat_threads<SPLIT, F16>(), 1) ppconv_tcf_kern
     // its shared memory, and the filter table below, before the reads; the
     // second keeps each CTA's shared memory alive until the others have read it.
     // This CTA finishes filters [m0, m1) of the tile (all of them when the split is 1);
-    // their original indices are fetched now, so the loads overlap
+    // their original indices and biases are fetched now, so the loads overlap
     // the barrier wait.
     const int tile = (int)blockIdx.x / csize, rstride = PAIR ? 2 : 1;
     const int m0 = srank * FB / p.split, m1 = (srank + 1) * FB / p.split, nm = m1 - m0;
@@ -903,17 +906,18 @@ __global__ void __launch_bounds__(flat_threads<SPLIT, F16>(), 1) ppconv_tcf_kern
     if (tid < nm) {
       const int jr = T.fb * FB + m0 + tid;
       o_s[tid] = jr < p.Co ? __ldg(p.perm + jr) : -1;
+      if (nm <= FB / 2) b_s[tid] = (jr < p.Co && p.bias) ? __ldg(p.bias + jr) : 0.f;
     }
     __syncwarp();
     asm volatile("barrier.cluster.arrive.release;\n\tbarrier.cluster.wait.acquire;" ::: "memory");
     if (!abort_s) {
       float* part = reinterpret_cast<float*>(smem);
       switch (p.split) {
-        case 1: split_reduce<1>(p, T, m0, nm, part, o_s, tid, rstride, pp); break;
-        case 2: split_reduce<2>(p, T, m0, nm, part, o_s, tid, rstride, pp); break;
-        case 4: split_reduce<4>(p, T, m0, nm, part, o_s, tid, rstride, pp); break;
-        case 8: split_reduce<8>(p, T, m0, nm, part, o_s, tid, rstride, pp); break;
-        default: split_reduce<16>(p, T, m0, nm, part, o_s, tid, rstride, pp); break;
+        case 1: split_reduce<1>(p, T, m0, nm, part, o_s, b_s, tid, rstride, pp); break;
+        case 2: split_reduce<2>(p, T, m0, nm, part, o_s, b_s, tid, rstride, pp); break;
+        case 4: split_reduce<4>(p, T, m0, nm, part, o_s, b_s, tid, rstride, pp); break;
+        case 8: split_reduce<8>(p, T, m0, nm, part, o_s, b_s, tid, rstride, pp); break;
+        default: split_reduce<16>(p, T, m0, nm, part, o_s, b_s, tid, rstride, pp); break;
       }
     }
     __syncwarp();
