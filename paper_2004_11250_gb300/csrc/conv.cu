@@ -858,6 +858,10 @@ extern "C" pp_status pp_layer_autotune(pp_layer* L, int N, int H, int W, int fla
     cudaFree(y);
     return PP_ERR_OOM;
   }
+  // Wide maps of 128-filter tf32 blocks: the row-tiled kernel's place is taken by the one that streams weights to CTA
+  // pairs, which needs its own copy of the weight tiles (built once, kept: a captured graph may use it from now on;
+  // without memory for it the row-tiled kernel runs).
+  if (L->tc_ok && L->tc.FB == 128 && !L->tc.f16 && !(flags & PP_POOL2) && W >= 96) ppc::tcr_pair_layout(&L->tc, stream);
   pp_status st = PP_OK;
   if (cudaMemsetAsync(x, 0, in_elems * 4, stream) != cudaSuccess ||
       (sk && cudaMemsetAsync(sk, 0, out_elems * 4, stream) != cudaSuccess))
@@ -940,7 +944,7 @@ extern "C" pp_status pp_layer_info(const pp_layer* L, int* Co, int* Ci, int64_t*
   if (Ci) *Ci = L->Ci;
   if (device_bytes)
     *device_bytes =
-        (int64_t)(L->dbytes + L->tm.dbytes + L->tc.dbytes + L->tc.dbytes16 + L->direct.dbytes);
+        (int64_t)(L->dbytes + L->tm.dbytes + L->tc.dbytes + L->tc.dbytes16 + L->tc.dbytesp + L->direct.dbytes);
   return PP_OK;
 }
 

@@ -975,7 +975,8 @@ pp_status tc_build(TcLayout* T, const pp_packed* pk, cudaStream_t stream) {
   T->dbytes = total + 256;
   T->a = static_cast<const unsigned char*>(d);
   T->status = reinterpret_cast<int*>(static_cast<unsigned char*>(d) + total);
-  return PP_OK;
+  // 64-filter layers whose weights do not stay resident stream them in the pairs' order
+  return FB == 64 && tcr_streams(*T, Ci) ? tcr_pair_layout(T, stream) : PP_OK;
 }
 
 // The same layer for the fp16 split (PP_PRECISION_F16X3): per (filter block,
@@ -1121,6 +1122,7 @@ pp_status tc_launch(const TcLayout& T, const LayerMeta& M, const float* x, float
 }
 
 void tc_free(TcLayout* T) {
+  tcr_pair_free(T);
   if (T->dmem) cudaFree(T->dmem);
   T->dmem = nullptr;
   if (T->dmem16) cudaFree(T->dmem16);

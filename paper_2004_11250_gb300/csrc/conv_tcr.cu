@@ -1,8 +1,9 @@
-// Pattern-pruned 3x3 convolution on the tensor cores for layers with at most 64
-// filters and at most 64 input channels (the inner layers of super-resolution
-// stacks, the first blocks of VGG-like trunks): the
+// Pattern-pruned 3x3 convolution on CTA pairs of tensor cores, for layers with at
+// most 64 filters (the inner layers of super-resolution stacks, the first blocks
+// of VGG-like trunks) and 128-filter blocks on wide maps: the
 // same dense 9-tap contraction and the same hi / lo splits as conv_tc.cu, with
-// the layer's whole weight set resident in shared memory.
+// the whole weight set of a layer of at most 64 filters and 64 channels resident
+// in shared memory.
 //
 // Method: Niu et al., IJCAI-20 demo, Sections 2 (pattern and connectivity
 // pruning, here zeros of the dense 9-tap weights) and 3 (fused activation).
@@ -53,6 +54,14 @@
 // issuers on alternate rows, at once (170) or in turn (155 - 165), one issuer (197), releasing the accumulators before
 // the stores (154), polling with test_wait (174), tiles as in tf32 (181).
 //
+// Streamed weights (tf32).  Layers of at most 64 filters with more input channels, and 128-filter blocks (one output row
+// per CTA and tile, one issuer), take each chunk's weights with its input stage: one bulk copy per CTA and chunk, from a
+// second copy of the weight tiles in the pairs' row order.  The odd CTA's idle MMA warp reports its copies to the even
+// one.  Against the row-tiled kernel, whose 128-filter tile moves ~305 KB of a chunk through shared memory (2380 clocks)
+// for 1728 clocks of MMAs, the pair moves ~214 KB: 128 -> 128 at 128 x 128 26.7 -> 23.5 us, 2 x 200 x 200 119 -> 100,
+// 256 -> 256 at 120 x 160 150 -> 125; 64 filters: 100 -> 64 at 128 x 128 23.3 -> 19.0, 256 -> 48 at 100 x 130, batch 2
+// (rows not 16-byte aligned), 141 -> 70, 512 -> 64 at 28 x 28 94 -> 69.
+//
 // Every wait on an mbarrier is bounded; on timeout the kernel records an error
 // in the layer's device status word and skips the rest of its work.
 #include <cuda_runtime.h>
@@ -67,36 +76,40 @@ namespace {
 using namespace ppc_ptx;
 
 constexpr int NTAP = 9;
-constexpr int FB = 64;                  // filters
-constexpr int TW = 128, R = 2;          // output tile of one CTA
-constexpr int BROWS = R + 2, BCOLS = TW + 2, NPIX = BROWS * BCOLS;
-constexpr int IN_HALF = NPIX * 16;      // one K half of the hi or lo input operand
-constexpr int IN_BYTES = 2 * IN_HALF;
-constexpr int STAGE = 2 * IN_BYTES;     // hi, then lo
-constexpr int W_TAP = FB * 32;          // this CTA's 64 weight rows of a tap, 32 bytes (K) each
-constexpr int W_CHUNK = NTAP * W_TAP;
-constexpr int UNITS = 2 * BROWS + 1;    // loader units of a chunk: each staged row and K half, and the last 2 columns
+constexpr int TW = 128, BCOLS = TW + 2; // output columns of a tile, staged columns
 constexpr int NLOADW = 14;              // loader warps (24 warps in all: 80 registers per thread)
 constexpr int NEPIW = 8;                // warps 0-7: epilogue
 constexpr int MMA_WARP = NEPIW;         // warps 8 and 9: MMA issuers
-constexpr int LOAD_WARP0 = MMA_WARP + R;
+constexpr int LOAD_WARP0 = MMA_WARP + 2;
 constexpr int NTHREADS = 32 * (LOAD_WARP0 + NLOADW);
 constexpr long WAIT_LIMIT = PP_WAIT_POLLS;
-constexpr int MAX_CI = 64;
+constexpr int MAX_CI = 64;              // input channels whose weights stay resident (64 filters)
+constexpr int KCH32 = 8, KCH16 = 16;    // input channels per chunk
 
-// tf32: 8-channel chunks in a ring of two stages; f16: whole input rows (all channels) in a ring of four
-constexpr int KCH32 = 8, KCH16 = 16;         // input channels per chunk
-constexpr int MAXCH32 = MAX_CI / KCH32, MAXCH16 = MAX_CI / KCH16;
-constexpr int NST = 2;
-constexpr int X_OFF32 = MAXCH32 * W_CHUNK;
-constexpr int SMEM32 = X_OFF32 + NST * STAGE + 1024;
-constexpr int RING = 4;
-constexpr int ROW_HALF = BCOLS * 16;         // f16: one K half of a row's hi or lo operand in a chunk
-constexpr int ROW_CHUNK = 4 * ROW_HALF;      // hi (2 halves), lo
-constexpr int ROW_BYTES = MAXCH16 * ROW_CHUNK;
-constexpr int X_OFF16 = MAXCH16 * W_CHUNK;
-constexpr int SMEM16 = X_OFF16 + RING * ROW_BYTES + 1024;
-static_assert(SMEM32 <= 232448 - 2304 && SMEM16 <= 232448 - 2304, "shared memory plan");
+// One instantiation: FB filters (64, or 128 in tf32); STREAM (tf32): each chunk's weights come with its input stage
+// instead of staying resident.
+template <bool F16, int FB, bool STREAM>
+struct Geo {
+  static_assert(!F16 || (FB == 64 && !STREAM), "f16: resident weights of 64 filters");
+  static_assert(FB == 64 || STREAM, "128 filters' weights do not fit");
+  static constexpr int R = FB == 64 ? 2 : 1;           // output rows of a tile (tf32)
+  static constexpr int BROWS = R + 2, NPIX = BROWS * BCOLS;
+  static constexpr int IN_HALF = NPIX * 16;            // one K half of the hi or lo input operand of a chunk
+  static constexpr int IN_BYTES = 2 * IN_HALF;
+  static constexpr int W_TAP = FB * 32;                // this CTA's FB weight rows of a tap, 32 bytes (K) each
+  static constexpr int W_CHUNK = NTAP * W_TAP;
+  static constexpr int UNITS = 2 * BROWS + 1;          // loader units of a chunk: each row and K half, the last 2 columns
+  // tf32: chunks in a ring of stages (hi, lo; STREAM: weights first); f16: whole input rows in a ring of four
+  static constexpr int ROW_HALF = BCOLS * 16;          // f16: one K half of a row's hi or lo operand in a chunk
+  static constexpr int ROW_CHUNK = 4 * ROW_HALF;       // hi (2 halves), lo
+  static constexpr int NRING = F16 ? 4 : !STREAM ? 2 : FB == 64 ? 4 : 3;
+  static constexpr int ENTRY = F16 ? MAX_CI / KCH16 * ROW_CHUNK : 2 * IN_BYTES + (STREAM ? W_CHUNK : 0);
+  static constexpr int X_OFF = STREAM ? W_CHUNK : MAX_CI / (F16 ? KCH16 : KCH32) * W_CHUNK;  // input of entry s at + s ENTRY
+  static constexpr int SMEM = (STREAM ? 0 : X_OFF) + NRING * ENTRY + 1024;
+  // accumulator slots, one output row each: tf32 of 2 FB columns, f16 of 192 (256 apart)
+  static constexpr int NSLOT = F16 ? 2 : 512 / (2 * FB), SLOTC = F16 ? 256 : 2 * FB;
+  static_assert(SMEM <= 232448 - 2304, "shared memory plan");
+};
 
 struct TcrParams {
   const float* rscale;      // f16: per reordered filter, 1 / (weight scale x input scale)
@@ -104,13 +117,14 @@ struct TcrParams {
   const float* x;
   float* y;
   const float* skip;
-  const unsigned char* wt;  // [nch][9][K half][128 rows][16 bytes]: rows 0-63 hi, 64-127 lo
+  // resident: [nch][9][K half][128 rows][16 bytes], rows 0-63 hi, 64-127 lo; STREAM: [nfb][nch][rank][9][K half][FB rows]
+  const unsigned char* wt;
   const int* perm;
   const float* bias;
   int* status;
   int N, Ci, Co, H, W, nch, flags;
   int tiles_x, nstrips;     // 128-column strips of an image row; strips in all
-  int tiles_y, ntiles;      // tf32: tiles of R rows
+  int tiles_y, ntiles, nfb; // tf32: tiles of R rows; filter blocks
   int split, srows;         // f16: each strip is cut into `split` (1 or 2) pieces of srows rows
 };
 
@@ -146,22 +160,26 @@ struct Walk {
   }
 };
 
-template <bool F16, bool POOL>
+template <bool F16, bool POOL, int FB, bool STREAM>
 __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(NTHREADS, 1) ppconv_tcr_kernel(const TcrParams p) {
-  // accumulator slots, one output row each: tf32 4 of 128 columns, f16 2 of 192 (256 apart)
-  constexpr int NSLOT = F16 ? 2 : 4, SLOTC = F16 ? 256 : 128;
-  constexpr int NRING = F16 ? RING : NST;        // input ring: rows (f16) or chunk stages (tf32)
-  constexpr int X_OFF = F16 ? X_OFF16 : X_OFF32;
+  using G = Geo<F16, FB, STREAM>;
+  static_assert(!POOL || G::R == 2, "pooling reads row pairs of a tile");
+  constexpr int R = G::R, NSLOT = G::NSLOT, SLOTC = G::SLOTC, NRING = G::NRING, X_OFF = G::X_OFF, ENTRY = G::ENTRY;
+  constexpr int NPIX = G::NPIX, IN_HALF = G::IN_HALF, IN_BYTES = G::IN_BYTES, UNITS = G::UNITS;
+  constexpr int W_TAP = G::W_TAP, W_CHUNK = G::W_CHUNK, ROW_HALF = G::ROW_HALF, ROW_CHUNK = G::ROW_CHUNK;
+  constexpr int NISS = F16 ? 2 : R;  // MMA issuers
   extern __shared__ __align__(1024) unsigned char smem_raw[];
   unsigned char* smem = smem_raw + ((1024u - (su32(smem_raw) & 1023u)) & 1023u);
   // full (even CTA): both CTAs' loader warps have stored a ring entry; empty (tf32): the MMAs that read it are
   // complete; acc_full: a slot's row is accumulated (f16: and with it every earlier MMA is complete, which is what the
   // loaders wait for too); acc_empty (even CTA): both CTAs' epilogues have read it
   __shared__ __align__(8) uint64_t full[NRING], empty[NRING], acc_full[NSLOT], acc_empty[NSLOT], done_bar;
+  __shared__ __align__(8) uint64_t wfull[NRING];  // STREAM, odd CTA: its weights of a stage have landed
   __shared__ uint32_t tmem_s;
   // per filter: output channel x plane size of y and of skip (0 past the last filter), bias, inverse scale
-  __shared__ __align__(16) int yoff[FB], soff[FB];
-  __shared__ __align__(16) float bias_s[FB], scale_s[FB];
+  // (64 filters; 128-filter layers may have several blocks and read them from memory)
+  __shared__ __align__(16) int yoff[64], soff[64];
+  __shared__ __align__(16) float bias_s[64], scale_s[64];
   __shared__ volatile int abort_s;
 
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
@@ -182,14 +200,16 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(NTHREADS, 1) ppconv_
   const int units = F16 ? 2 * p.nch + 1 : UNITS;  // loader units of a ring entry
   if (tid == 0) {
     for (int s = 0; s < NRING; ++s) {
-      mbar_init(su32(&full[s]), 2 * units);
-      mbar_init(su32(&empty[s]), R);
+      // STREAM: and one more for each CTA's weights (the even CTA's with its bytes)
+      mbar_init(su32(&full[s]), 2 * units + (STREAM ? 2 : 0));
+      mbar_init(su32(&empty[s]), NISS);
+      mbar_init(su32(&wfull[s]), 1);
     }
     for (int s = 0; s < NSLOT; ++s) {
       mbar_init(su32(&acc_full[s]), F16 ? 2 : 1);
       mbar_init(su32(&acc_empty[s]), 2 * NEPIW);
     }
-    mbar_init(su32(&done_bar), R);
+    mbar_init(su32(&done_bar), NISS);
     abort_s = 0;
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
@@ -197,7 +217,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(NTHREADS, 1) ppconv_
     asm volatile("tcgen05.alloc.cta_group::2.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(su32(&tmem_s)), "n"(512));
     asm volatile("tcgen05.relinquish_alloc_permit.cta_group::2.sync.aligned;");
   }
-  if (tid < FB) {
+  if (FB == 64 && tid < FB) {
     const int o = tid < p.Co ? __ldg(p.perm + tid) : 0;
     yoff[tid] = o * (POOL ? (p.H / 2) * (p.W / 2) : p.H * p.W);
     soff[tid] = o * (p.H * p.W);
@@ -206,7 +226,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(NTHREADS, 1) ppconv_
   }
   // This CTA's half of the weights (they do not depend on the previous kernel in the stream):
   // even CTA rows hi 0-31, lo 32-63; odd CTA rows hi 32-63, lo 0-31 of every tap.
-  for (int i = tid; i < p.nch * NTAP * 128; i += NTHREADS) {
+  for (int i = tid; !STREAM && i < p.nch * NTAP * 128; i += NTHREADS) {
     const int r = i & 63, src = rank == 0 ? (r < 32 ? r : 64 + r) : 32 + r;
     reinterpret_cast<uint4*>(smem)[i] = __ldg(reinterpret_cast<const uint4*>(p.wt) + (i >> 6) * 128 + src);
   }
@@ -216,12 +236,15 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(NTHREADS, 1) ppconv_
   tm_fence_after();
   const uint32_t tmem = tmem_s;
 
-  // tf32: tile i of this CTA is tile blockIdx.x + i gridDim.x (the CTAs of a pair are neighbours); both run the
-  // even CTA's number of tiles, and a tile past the last is loaded as zeros and not stored.
-  const int first = (int)(blockIdx.x & ~1u);
-  const int nmine = p.ntiles > first ? (p.ntiles - 1 - first) / (int)gridDim.x + 1 : 0;
-  auto tile_of = [&](int i, int& n, int& r0, int& c0) -> bool {
-    int t = (int)blockIdx.x + i * (int)gridDim.x;
+  // tf32: work item i of a pair is item u = pair + i pairs, the filter block u % nfb of the neighbouring tiles 2 v and 2 v
+  // + 1, v = u / nfb; a tile past the last is loaded as zeros and not stored.
+  const int pair = (int)blockIdx.x >> 1, npairs = (int)gridDim.x >> 1;
+  const int items = (p.ntiles + 1) / 2 * p.nfb;
+  const int nmine = items > pair ? (items - 1 - pair) / npairs + 1 : 0;
+  auto tile_of = [&](int i, int& n, int& r0, int& c0, int& fb) -> bool {
+    const int u = pair + i * npairs;
+    fb = FB == 64 ? 0 : u % p.nfb;
+    int t = 2 * (FB == 64 ? u : u / p.nfb) + (int)rank;
     if (t >= p.ntiles) return false;
     c0 = (t % p.tiles_x) * TW;
     t /= p.tiles_x;
@@ -286,15 +309,15 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(NTHREADS, 1) ppconv_
       // pixels 32 j + lane; the last holds pixels 128 and 129 (lane l: chunk l >> 2, K half (l >> 1) & 1, pixel l & 1)
       int un = warp - LOAD_WARP0, k = 0, sq = 0;
       // Input row k of a run is last read for its output row min(k, len - 1).  last[0]: the output row (counted over
-      // all runs) after which the ring entry of row sq may be stored again, i.e. the last to read entry sq - RING.
-      int oc0 = 0, last[RING] = {0, 0, 0, 0};
+      // all runs) after which the ring entry of row sq may be stored again, i.e. the last to read entry sq - NRING.
+      int oc0 = 0, last[NRING] = {0, 0, 0, 0};
       auto settle = [&]() {
         while (more && un >= units) {
           un -= units;
           ++sq;
 #pragma unroll
-          for (int r = 0; r + 1 < RING; ++r) last[r] = last[r + 1];
-          last[RING - 1] = oc0 + min(k, w.len - 1);
+          for (int r = 0; r + 1 < NRING; ++r) last[r] = last[r + 1];
+          last[NRING - 1] = oc0 + min(k, w.len - 1);
           if (++k == w.len + 2) {
             k = 0;
             oc0 += w.len;
@@ -314,12 +337,12 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(NTHREADS, 1) ppconv_
         uint4 h[4], l[4];
 #pragma unroll
         for (int j = 0; j < 4; ++j) split_f16x8_max(v[j], p.xscale, h[j], l[j], hmax);
-        const int s = sq % RING;
+        const int s = sq % NRING;
         const bool one = un == units - 1, in = !one || lane < 4 * p.nch;
         const int off = one ? (lane >> 2) * ROW_CHUNK + ((lane >> 1) & 1) * ROW_HALF + (128 + (lane & 1)) * 16
                             : (un >> 1) * ROW_CHUNK + (un & 1) * ROW_HALF + lane * 16;
-        uint4* dst = reinterpret_cast<uint4*>(smem + X_OFF + s * ROW_BYTES + (in ? off : 0));
-        if (!__all_sync(0xffffffffu, sq < RING || wait(&acc_full[last[0] & 1], (uint32_t)((last[0] >> 1) & 1)))) break;
+        uint4* dst = reinterpret_cast<uint4*>(smem + X_OFF + s * ENTRY + (in ? off : 0));
+        if (!__all_sync(0xffffffffu, sq < NRING || wait(&acc_full[last[0] & 1], (uint32_t)((last[0] >> 1) & 1)))) break;
         store(dst, 2 * ROW_HALF / 16, h, l, in, one, &full[s]);
         un += nload;
         settle();
@@ -329,15 +352,15 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(NTHREADS, 1) ppconv_
     } else {
       // (NLOADW < 2 UNITS: no warp skips two stages' entries, see above)
       static_assert(NLOADW <= 2 * UNITS, "a parity wait needs the phase before");
-      // tile it, chunk c, unit un of the chunk in stage s: un < 8 is row un >> 1, K half un & 1 and pixels 32 j + lane;
-      // unit 8 holds pixels 128 and 129 (lane l < 16: row l >> 2, K half (l >> 1) & 1, pixel l & 1)
-      int it = 0, c = 0, un = warp - LOAD_WARP0, s = 0, use = 0, n = 0, r0 = 0, c0 = 0;
-      bool ok = tile_of(0, n, r0, c0);
+      // tile it, chunk c, unit un of the chunk in stage s: un < 2 BROWS is row un >> 1, K half un & 1 and pixels 32 j +
+      // lane; the last holds pixels 128 and 129 (lane l: row l >> 2, K half (l >> 1) & 1, pixel l & 1)
+      int it = 0, c = 0, un = warp - LOAD_WARP0, s = 0, use = 0, n = 0, r0 = 0, c0 = 0, fb = 0;
+      bool ok = tile_of(0, n, r0, c0, fb);
       auto settle = [&]() {
         bool moved = false;
         while (un >= UNITS) {
           un -= UNITS;
-          if (++s == NST) {
+          if (++s == NRING) {
             s = 0;
             ++use;
           }
@@ -347,14 +370,14 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(NTHREADS, 1) ppconv_
             moved = true;
           }
         }
-        if (moved) ok = tile_of(it, n, r0, c0);
+        if (moved) ok = tile_of(it, n, r0, c0, fb);
       };
       settle();
       float v[4][4];
       auto load = [&]() {
         const bool one = un == UNITS - 1;
         fetch(v, n, c * KCH32 + (one ? (lane >> 1) & 1 : un & 1) * 4, r0 - 1 + (one ? lane >> 2 : un >> 1),
-              c0 - 1 + (one ? 128 + (lane & 1) : lane), ok && (!one || lane < 16), one);
+              c0 - 1 + (one ? 128 + (lane & 1) : lane), ok && (!one || lane < 4 * G::BROWS), one);
       };
       if (it < nmine) load();
       while (it < nmine) {
@@ -370,23 +393,33 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(NTHREADS, 1) ppconv_
                             __float_as_uint(v[j][3] - __uint_as_float(h[j].w)));
         }
         const int su = s, uu = use;
-        const bool one = un == UNITS - 1, in = !one || lane < 16;
-        uint4* dst = reinterpret_cast<uint4*>(smem + X_OFF + s * STAGE) +
+        const bool one = un == UNITS - 1, in = !one || lane < 4 * G::BROWS, head = un == 0;
+        const unsigned char* wsrc = p.wt + ((size_t)(fb * p.nch + c) * 2 + rank) * W_CHUNK;
+        uint4* dst = reinterpret_cast<uint4*>(smem + X_OFF + s * ENTRY) +
                      (one ? (in ? ((lane >> 1) & 1) * NPIX + (lane >> 2) * BCOLS + 128 + (lane & 1) : 0)
                           : (un & 1) * NPIX + (un >> 1) * BCOLS + lane);
         un += NLOADW;
         settle();
         if (it < nmine) load();
         if (!__all_sync(0xffffffffu, uu == 0 || wait(&empty[su], (uint32_t)((uu - 1) & 1)))) break;
+        if (STREAM && head && lane == 0) {  // the warp with a stage's first unit copies its weights
+          uint64_t* bar = rank == 0 ? &full[su] : &wfull[su];
+          mbar_arrive_expect_tx(su32(bar), W_CHUNK);
+          asm volatile(
+              "cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(
+                  su32(smem + su * ENTRY)),
+              "l"(wsrc), "r"(W_CHUNK), "r"(su32(bar))
+              : "memory");
+        }
         store(dst, IN_BYTES / 16, h, l, in, one, &full[su]);
       }
     }
     __syncwarp();
   } else if (warp >= MMA_WARP) {
     // ------------------------------------------------------------ MMA issuers (even CTA, for the pair)
-    if (lane == 0 && rank == 0) {
-      constexpr uint32_t ID1 = F16 ? idesc_f16(256, 128) : idesc_tf32(256, 128);
-      constexpr uint32_t ID2 = F16 ? idesc_f16(256, 64) : idesc_tf32(256, 64);
+    if (lane == 0 && rank == 0 && warp - MMA_WARP < NISS) {
+      constexpr uint32_t ID1 = F16 ? idesc_f16(256, 2 * FB) : idesc_tf32(256, 2 * FB);
+      constexpr uint32_t ID2 = F16 ? idesc_f16(256, FB) : idesc_tf32(256, FB);
       const int rr = warp - MMA_WARP;  // which issuer
       const uint32_t x_base = su32(smem) + X_OFF;
       if constexpr (F16) {
@@ -405,8 +438,8 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(NTHREADS, 1) ppconv_
 #pragma unroll
             for (int r = 0; r < 3; ++r) {  // the input rows' ring entries; the run's previous row waited for the first two
               const int q = sq + y + r;
-              if (ok && (r == 2 || y == 0)) ok = wait(&full[q % RING], (uint32_t)((q / RING) & 1));
-              xd[r] = smem_desc(x_base + (uint32_t)((q % RING) * ROW_BYTES + rr * 2 * ROW_HALF), ROW_HALF);
+              if (ok && (r == 2 || y == 0)) ok = wait(&full[q % NRING], (uint32_t)((q / NRING) & 1));
+              xd[r] = smem_desc(x_base + (uint32_t)((q % NRING) * ENTRY + rr * 2 * ROW_HALF), ROW_HALF);
             }
             if (!ok) break;
             tm_fence_after();
@@ -431,21 +464,22 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(NTHREADS, 1) ppconv_
           if (i >= NSLOT / R) ok = wait(&acc_empty[slot], (uint32_t)(sph ^ 1));
           const uint32_t d = tmem + (uint32_t)(slot * SLOTC);
           uint64_t w0 = smem_desc(su32(smem), FB * 16);
-          for (int c = 0; c < p.nch && ok; ++c, w0 += W_CHUNK / 16) {
+          for (int c = 0; c < p.nch && ok; ++c, w0 += STREAM ? 0 : W_CHUNK / 16) {
             ok = wait(&full[s], (uint32_t)ph);
             if (!ok) break;
             tm_fence_after();
-            const uint64_t xh0 = smem_desc(x_base + (uint32_t)(s * STAGE), IN_HALF) + (uint64_t)(rr * BCOLS);
+            const uint64_t xh0 = smem_desc(x_base + (uint32_t)(s * ENTRY), IN_HALF) + (uint64_t)(rr * BCOLS);
+            const uint64_t ws = w0 + (uint64_t)(STREAM ? s * (ENTRY / 16) : 0);
             const uint32_t acc0 = c == 0 ? 0u : 1u;
 #pragma unroll
             for (int t = 0; t < NTAP; ++t) {
               const uint64_t xh = xh0 + (uint64_t)((t / 3) * BCOLS + t % 3);  // pixels of 16 bytes
-              const uint64_t w = w0 + (uint64_t)(t * W_TAP / 16);
+              const uint64_t w = ws + (uint64_t)(t * W_TAP / 16);
               mma_tf32_pair(d, xh, w, ID1, t == 0 ? acc0 : 1u);
               mma_tf32_pair(d, xh + IN_BYTES / 16, w, ID2, 1u);
             }
             mma_commit_pair(su32(&empty[s]), (uint16_t)3);
-            if (++s == NST) {
+            if (++s == NRING) {
               s = 0;
               ph ^= 1;
             }
@@ -464,7 +498,18 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(NTHREADS, 1) ppconv_
       asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
       mma_commit_pair(su32(&done_bar), (uint16_t)1);
       wait(&done_bar, 0u);
-    } else if (lane == 0) {
+    } else if (lane == 0 && rank == 1 && warp == MMA_WARP) {
+      if (STREAM) {  // reports the odd CTA's weights of each chunk to the even one
+        int s = 0, ph = 0;
+        for (int g = 0; g < nmine * p.nch; ++g) {
+          if (!wait(&wfull[s], (uint32_t)ph)) break;
+          mbar_arrive_remote(map_rank(su32(&full[s]), 0));
+          if (++s == NRING) {
+            s = 0;
+            ph ^= 1;
+          }
+        }
+      }
       asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
     }
     __syncwarp();
@@ -474,15 +519,28 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(NTHREADS, 1) ppconv_
     const int q = warp & 3, half = warp >> 2;
     const bool relu = p.flags & PP_RELU;
     constexpr int EB = POOL ? 8 : 16;  // filters handled together (pooling holds two rows of them)
-    const int f0 = 32 * half, nf = p.Co - f0;  // first filter, and how many from there on exist
+    constexpr int Q = FB / 2;     // filters of a half, columns of a quarter
+    const int f0 = Q * half;      // first filter of this half
+    int fbase = 0, nf = p.Co - f0;  // the block's first filter; how many filters from f0 on exist
     const int HW = p.H * p.W, Wo = p.W / 2, HWo = (p.H / 2) * Wo;
     const uint32_t lanebase = tmem + ((uint32_t)(32 * q) << 16);
+    // bias and output channel x plane of filters f0 + j .. + 3 (past the last filter: anything)
+    auto bias4 = [&](int j) -> float4 {
+      if (FB == 64) return *reinterpret_cast<const float4*>(&bias_s[f0 + j]);
+      return p.bias && j < nf ? __ldg(reinterpret_cast<const float4*>(p.bias + fbase + f0 + j)) : make_float4(0.f, 0.f, 0.f, 0.f);
+    };
+    auto plane4 = [&](int j, bool y) -> int4 {
+      if (FB == 64) return *reinterpret_cast<const int4*>(y ? &yoff[f0 + j] : &soff[f0 + j]);
+      const int4 o = j < nf ? __ldg(reinterpret_cast<const int4*>(p.perm + fbase + f0 + j)) : make_int4(0, 0, 0, 0);
+      // a vector's entries past the last filter are padding, not channels
+      return make_int4(o.x * HW, j + 1 < nf ? o.y * HW : 0, j + 2 < nf ? o.z * HW : 0, j + 3 < nf ? o.w * HW : 0);
+    };
     // filters f0 + jj .. + EB - 1, with their bias, from a slot's accumulators (warp-collective)
     auto get = [&](int slot, int jj, float(&a)[EB]) {
       const uint32_t b = lanebase + (uint32_t)(slot * SLOTC + jj);
       float a2[EB];
-      tm_ld(b + (half ? 64 : 0), a);
-      tm_ld(b + (half ? 32 : 96), a2);
+      tm_ld(b + (half ? 2 * Q : 0), a);
+      tm_ld(b + (half ? Q : 3 * Q), a2);
       if constexpr (F16) {
         const uint64_t e = pack2(0x1p-11f, 0x1p-11f);
         float a3[EB];
@@ -502,7 +560,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(NTHREADS, 1) ppconv_
         tm_wait_ld();
 #pragma unroll
         for (int k = 0; k < EB; k += 4) {
-          const float4 bv = *reinterpret_cast<const float4*>(&bias_s[f0 + jj + k]);
+          const float4 bv = bias4(jj + k);
           unpack2(add2(add2(pack2(a[k], a[k + 1]), pack2(a2[k], a2[k + 1])), pack2(bv.x, bv.y)), a[k], a[k + 1]);
           unpack2(add2(add2(pack2(a[k + 2], a[k + 3]), pack2(a2[k + 2], a2[k + 3])), pack2(bv.z, bv.w)), a[k + 2],
                   a[k + 3]);
@@ -538,10 +596,11 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(NTHREADS, 1) ppconv_
         if (sbase) {
 #pragma unroll
           for (int k0 = 0; k0 < EB; k0 += 8) {
+            const int4 so[2] = {plane4(jj + k0, false), plane4(jj + k0 + 4, false)};
             float sv[8], tv[POOL ? 8 : 1];
 #pragma unroll
             for (int k = 0; k < 8; ++k) {
-              const int o = soff[f0 + jj + k0 + k];
+              const int o = (k & 3) == 0 ? so[k >> 2].x : (k & 3) == 1 ? so[k >> 2].y : (k & 3) == 2 ? so[k >> 2].z : so[k >> 2].w;
               sv[k] = __ldg(sbase + (in0 ? o + roff : 0));
               if constexpr (POOL) tv[k] = __ldg(sbase + (in0 ? o + roff + p.W : 0));
             }
@@ -561,7 +620,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(NTHREADS, 1) ppconv_
         }
 #pragma unroll
         for (int k = 0; k < EB; k += 4) {
-          const int4 o4 = *reinterpret_cast<const int4*>(&yoff[f0 + jj + k]);
+          const int4 o4 = plane4(jj + k, true);
           const int o[4] = {o4.x, o4.y, o4.z, o4.w};
 #pragma unroll
           for (int e = 0; e < 4; ++e) {
@@ -576,11 +635,11 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(NTHREADS, 1) ppconv_
         }
       };
 #pragma unroll(POOL ? 1 : 2)
-      for (int jj = 0; jj < 32; jj += EB) {
+      for (int jj = 0; jj < Q; jj += EB) {
         float a[EB], bb[POOL ? EB : 1];
         get(s0, jj, a);
         if constexpr (POOL) get(s1, jj, bb);
-        if (jj == 32 - EB) release();
+        if (jj == Q - EB) release();
         finish(jj, a, bb);
       }
       return true;
@@ -595,13 +654,20 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(NTHREADS, 1) ppconv_
         for (int y = 0; y < w.len && ok; y += STEP, r += STEP) ok = emit(r, w.n, w.row0 + w.y + y, w.c0, w.ok);
     } else {
       for (int i = 0; i < nmine && ok; ++i) {
-        int n = 0, r0 = 0, c0 = 0;
-        const bool valid = tile_of(i, n, r0, c0);
+        int n = 0, r0 = 0, c0 = 0, fb = 0;
+        const bool valid = tile_of(i, n, r0, c0, fb);
+        if (FB == 128) {
+          fbase = fb * FB;
+          nf = p.Co - fbase - f0;
+        }
         for (int rr = 0; rr < R && ok; rr += STEP) ok = emit(i * R + rr, n, r0 + rr, c0, valid);
       }
     }
   }
 
+  // after a wait that gave up, weight copies may still be in flight: a millisecond outlasts them
+  if (STREAM && abort_s)
+    for (int k = 0; k < 1000; ++k) __nanosleep(1000);
   // neither CTA leaves (or frees its TMEM) while the pair's MMAs or arrivals may still reach it
   tm_fence_before();
   __syncwarp();
@@ -612,13 +678,15 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(NTHREADS, 1) ppconv_
 }
 
 // Pairs that fit on the current device at once, per instantiation (0: pairs cannot be launched).
-int g_pairs[ppc::DeviceOnce::kMaxDevices][2][2];
+enum { K_TF32, K_TF32_POOL, K_F16, K_F16_POOL, K_STREAM64, K_STREAM64_POOL, K_STREAM128, K_COUNT };
+int g_pairs[ppc::DeviceOnce::kMaxDevices][K_COUNT];
 ppc::DeviceOnce g_once;
 
-template <bool F16, bool POOL>
-cudaError_t setup(int dev) {
-  const cudaError_t e =
-      cudaFuncSetAttribute(ppconv_tcr_kernel<F16, POOL>, cudaFuncAttributeMaxDynamicSharedMemorySize, (F16 ? SMEM16 : SMEM32));
+template <bool F16, bool POOL, int FB, bool STREAM>
+cudaError_t setup(int dev, int k) {
+  constexpr int SMEM = Geo<F16, FB, STREAM>::SMEM;
+  const auto kernel = ppconv_tcr_kernel<F16, POOL, FB, STREAM>;
+  const cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM);
   if (e != cudaSuccess) return e;
   cudaLaunchConfig_t cfg = {};
   cudaLaunchAttribute at[1];
@@ -628,43 +696,61 @@ cudaError_t setup(int dev) {
   at[0].val.clusterDim.z = 1;
   cfg.gridDim = dim3(2);
   cfg.blockDim = dim3(NTHREADS);
-  cfg.dynamicSmemBytes = (F16 ? SMEM16 : SMEM32);
+  cfg.dynamicSmemBytes = SMEM;
   cfg.attrs = at;
   cfg.numAttrs = 1;
   int n = 0;
-  if (cudaOccupancyMaxActiveClusters(&n, ppconv_tcr_kernel<F16, POOL>, &cfg) != cudaSuccess) {
+  if (cudaOccupancyMaxActiveClusters(&n, kernel, &cfg) != cudaSuccess) {
     cudaGetLastError();
     n = 0;
   }
-  g_pairs[dev][F16][POOL] = n;
+  g_pairs[dev][k] = n;
   return cudaSuccess;
 }
 
 cudaError_t prepare() {
   return g_once.run([](int dev) {
     cudaError_t e;
-    if ((e = setup<false, false>(dev)) != cudaSuccess) return e;
-    if ((e = setup<false, true>(dev)) != cudaSuccess) return e;
-    if ((e = setup<true, false>(dev)) != cudaSuccess) return e;
-    return setup<true, true>(dev);
+    if ((e = setup<false, false, 64, false>(dev, K_TF32)) != cudaSuccess) return e;
+    if ((e = setup<false, true, 64, false>(dev, K_TF32_POOL)) != cudaSuccess) return e;
+    if ((e = setup<true, false, 64, false>(dev, K_F16)) != cudaSuccess) return e;
+    if ((e = setup<true, true, 64, false>(dev, K_F16_POOL)) != cudaSuccess) return e;
+    if ((e = setup<false, false, 64, true>(dev, K_STREAM64)) != cudaSuccess) return e;
+    if ((e = setup<false, true, 64, true>(dev, K_STREAM64_POOL)) != cudaSuccess) return e;
+    return setup<false, false, 128, true>(dev, K_STREAM128);
   });
 }
 
-template <bool F16, bool POOL>
+template <bool F16, bool POOL, int FB, bool STREAM>
 cudaError_t launch(const TcrParams& p, int pairs, cudaStream_t stream) {
   cudaLaunchConfig_t cfg = {};
-  // tf32: pairs of tiles; f16: pairs of strip pieces, row by row (pooled: row pair by row pair)
-  const int64_t work = F16 ? (int64_t)((p.nstrips * p.split + 1) / 2) * (p.srows / (POOL ? 2 : 1)) : (p.ntiles + 1) / 2;
+  // tf32: pairs of tiles and filter blocks; f16: pairs of strip pieces, row by row (pooled: row pair by row pair)
+  const int64_t work = F16 ? (int64_t)((p.nstrips * p.split + 1) / 2) * (p.srows / (POOL ? 2 : 1))
+                           : (int64_t)((p.ntiles + 1) / 2) * p.nfb;
   cfg.gridDim = dim3((unsigned)(2 * std::min<int64_t>(work, pairs)));
   cfg.blockDim = dim3(NTHREADS);
-  cfg.dynamicSmemBytes = (F16 ? SMEM16 : SMEM32);
+  cfg.dynamicSmemBytes = Geo<F16, FB, STREAM>::SMEM;
   cfg.stream = stream;
   cudaLaunchAttribute at[1];
   at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
   at[0].val.programmaticStreamSerializationAllowed = 1;
   cfg.attrs = at;
   cfg.numAttrs = 1;
-  return cudaLaunchKernelEx(&cfg, ppconv_tcr_kernel<F16, POOL>, p);
+  return cudaLaunchKernelEx(&cfg, ppconv_tcr_kernel<F16, POOL, FB, STREAM>, p);
+}
+
+// The tf32 weight tiles in the order that the pairs stream them: block (filter block, chunk, rank) of [9][K half][FB
+// rows][16 bytes], rank 0 the rows [w_hi F0 ; w_lo F1], rank 1 [w_hi F1 ; w_lo F0] (F0 / F1: first / last FB / 2 filters).
+__global__ void pair_layout_kernel(const uint4* a, uint4* ap, int64_t n, int FB) {
+  for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
+    const int r = (int)(i % FB);
+    int64_t t = i / FB;
+    const int th = (int)(t % (2 * NTAP));  // tap and K half
+    t /= 2 * NTAP;
+    const int rank = (int)(t & 1);
+    const int src = rank == 0 ? (r < FB / 2 ? r : FB + r) : (r < FB / 2 ? FB / 2 + r : FB / 2 + r);
+    ap[i] = a[((t >> 1) * (2 * NTAP) + th) * (2 * FB) + src];
+  }
 }
 
 }  // namespace
@@ -676,25 +762,60 @@ namespace ppc {
 // one tile (64 -> 64, tf32 / f16: 8 x 28 x 28, 112 tiles, 18.1 -> 15.2 / 14.3 -> 13.0 us; 8 x 40 x 40, 160 tiles,
 // 17.5 -> 21.6 / 14.2 -> 15.7 us).
 bool tcr_applicable(const TcLayout& T, int Ci, int N, int H, bool narrow) {
-  return T.FB == FB && Ci <= MAX_CI && (!narrow || (int64_t)N * ((H + R - 1) / R) <= device_sms());
+  if (T.FB == 128) return !T.f16 && T.ap && !narrow;
+  if (Ci > MAX_CI && (T.f16 || !T.ap)) return false;
+  return !narrow || (int64_t)N * ((H + 1) / 2) <= device_sms();
+}
+
+bool tcr_streams(const TcLayout& T, int Ci) { return T.FB == 128 || Ci > MAX_CI; }
+
+pp_status tcr_pair_layout(TcLayout* T, cudaStream_t stream) {
+  if (T->ap) return PP_OK;
+  const int64_t bytes = (int64_t)T->nfb * T->nch * 2 * NTAP * 2 * T->FB * 16;
+  void* d = nullptr;
+  if (cudaMalloc(&d, (size_t)bytes) != cudaSuccess) {
+    cudaGetLastError();
+    return PP_ERR_OOM;
+  }
+  const int64_t n = bytes / 16;
+  pair_layout_kernel<<<(unsigned)std::min<int64_t>((n + 255) / 256, 4096), 256, 0, stream>>>(
+      reinterpret_cast<const uint4*>(T->a), static_cast<uint4*>(d), n, T->FB);
+  if (cudaGetLastError() != cudaSuccess || cudaStreamSynchronize(stream) != cudaSuccess) {
+    cudaFree(d);
+    return PP_ERR_CUDA;
+  }
+  T->ap = static_cast<unsigned char*>(d);
+  T->dbytesp = (size_t)bytes;
+  return PP_OK;
+}
+
+void tcr_pair_free(TcLayout* T) {
+  if (T->ap) cudaFree(T->ap);
+  T->ap = nullptr;
+  T->dbytesp = 0;
 }
 
 pp_status tcr_launch(const TcLayout& T, const LayerMeta& M, const float* x, float* y, const float* skip, int N, int H,
                      int W, int flags, cudaStream_t stream) {
-  if (T.FB != FB || M.Ci > MAX_CI) return PP_ERR_UNSUPPORTED;
   if (prepare() != cudaSuccess) return PP_ERR_CUDA;
   int dev = 0;
   if (cudaGetDevice(&dev) != cudaSuccess) return PP_ERR_CUDA;
   const bool f16 = T.f16;
   const bool pool = flags & PP_POOL2;
-  const int pairs = g_pairs[dev][f16][pool];
+  const bool streams = tcr_streams(T, M.Ci);
+  if (streams && (f16 || !T.ap || (pool && T.FB == 128))) return PP_ERR_UNSUPPORTED;
+  const int k = f16 ? (pool ? K_F16_POOL : K_F16)
+                    : T.FB == 128 ? K_STREAM128
+                                  : streams ? (pool ? K_STREAM64_POOL : K_STREAM64) : (pool ? K_TF32_POOL : K_TF32);
+  const int pairs = g_pairs[dev][k];
+  const int R = T.FB == 128 ? 1 : 2;
   TcrParams p;
   p.rscale = T.rscale;
   p.xscale = T.xscale;
   p.x = x;
   p.y = y;
   p.skip = (flags & PP_ADD_SKIP) ? skip : nullptr;
-  p.wt = f16 ? T.a16 : T.a;
+  p.wt = streams ? T.ap : f16 ? T.a16 : T.a;
   p.perm = M.perm;
   p.bias = M.bias;
   p.status = T.status;
@@ -708,14 +829,23 @@ pp_status tcr_launch(const TcLayout& T, const LayerMeta& M, const float* x, floa
   p.tiles_x = (W + TW - 1) / TW;
   p.tiles_y = (H + R - 1) / R;
   const int64_t ns = (int64_t)p.tiles_x * N, nt = ns * p.tiles_y;
-  if (pairs <= 0 || ns * (H + 2) > INT32_MAX / 2) return PP_ERR_UNSUPPORTED;
+  if (pairs <= 0 || ns * (H + 2) * T.nfb > INT32_MAX / 2) return PP_ERR_UNSUPPORTED;
+  p.nfb = T.nfb;
   p.ntiles = (int)nt;
   p.nstrips = (int)ns;
   // an odd number of strips is cut at half height, so that every pair of CTAs has two pieces
   p.split = ns & 1 ? 2 : 1;
   p.srows = p.split == 2 ? (pool ? (H / 2 + 1) / 2 * 2 : (H + 1) / 2) : H;
-  const cudaError_t e = f16 ? (pool ? launch<true, true>(p, pairs, stream) : launch<true, false>(p, pairs, stream))
-                            : (pool ? launch<false, true>(p, pairs, stream) : launch<false, false>(p, pairs, stream));
+  cudaError_t e;
+  switch (k) {
+    case K_TF32: e = launch<false, false, 64, false>(p, pairs, stream); break;
+    case K_TF32_POOL: e = launch<false, true, 64, false>(p, pairs, stream); break;
+    case K_F16: e = launch<true, false, 64, false>(p, pairs, stream); break;
+    case K_F16_POOL: e = launch<true, true, 64, false>(p, pairs, stream); break;
+    case K_STREAM64: e = launch<false, false, 64, true>(p, pairs, stream); break;
+    case K_STREAM64_POOL: e = launch<false, true, 64, true>(p, pairs, stream); break;
+    default: e = launch<false, false, 128, true>(p, pairs, stream); break;
+  }
   if (e != cudaSuccess) {
     cudaGetLastError();
     return PP_ERR_CUDA;

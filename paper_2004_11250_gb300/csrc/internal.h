@@ -91,6 +91,8 @@ struct TcLayout {
   void* dmem = nullptr;
   size_t dbytes = 0;
   const unsigned char* a = nullptr;
+  unsigned char* ap = nullptr;  // the tf32 tiles again, as CTA pairs stream them (conv_tcr.cu); null unless built
+  size_t dbytesp = 0;
   int* status = nullptr;        // device word: bit 0 a timed-out wait, bit 1 an input out of the f16 range
   TcState* state = nullptr;  // owned; see tc_free
   // fp16 split: [nfb][nch16][9][2 FB x 16 f16] tiles (hi rows, then lo rows scaled by 2^11) and, per
@@ -115,9 +117,12 @@ pp_status tc_status(const TcLayout& T, int* device_error);
 // Build the f16 tiles and scales (precision PP_PRECISION_F16X3) for inputs bounded by input_bound.
 pp_status tc_build16(TcLayout* T, const pp_packed* pk, float input_bound, cudaStream_t stream);
 void tc_free(TcLayout* T);
-// Layers with at most 64 filters and 64 input channels: weights resident in shared memory, CTA pairs (conv_tcr.cu);
-// returns PP_ERR_UNSUPPORTED for others and where pairs cannot be launched.  narrow: the row-tiled kernel would
-// flatten the map's rows.
+// CTA pairs (conv_tcr.cu): layers of at most 64 filters (weights resident up to 64 input channels, else streamed, tf32)
+// and of 128-filter blocks on wide maps (tf32); the streaming ones need the pair layout.  Returns PP_ERR_UNSUPPORTED for
+// others and where pairs cannot be launched.  narrow: the row-tiled kernel would flatten the map's rows.
+bool tcr_streams(const TcLayout& T, int Ci);
+pp_status tcr_pair_layout(TcLayout* T, cudaStream_t stream);  // builds ap from a; synchronous on stream
+void tcr_pair_free(TcLayout* T);
 bool tcr_applicable(const TcLayout& T, int Ci, int N, int H, bool narrow);
 pp_status tcr_prepare();
 pp_status tcr_launch(const TcLayout& T, const LayerMeta& M, const float* x, float* y, const float* skip, int N, int H,

@@ -1160,3 +1160,44 @@ def test_direct_kernels_dense(pp, runner, oracle_mod, shape, flags):
     g = run_layer(pp, runner, D, x, skip, "relu" in flags, pool)
     y, s = oracle_layer_full(oracle_mod, D, x, skip, "relu" in flags, pool)
     check_within(g, y, s, f"dense {shape} {flags}")
+
+
+# The same kernel streaming weights to CTA pairs (tf32): 64-filter layers with more than 64 input channels, and 128-filter
+# blocks on maps at least 96 wide once a layer has been tuned; ragged chunks, filters past the last block's end, one and
+# several blocks, odd numbers of tiles, more work than CTAs.
+STREAM_CASES = [
+    # N, Ci, Co, H, W
+    (1, 65, 64, 3, 130), (2, 72, 9, 5, 63), (1, 200, 40, 10, 28), (3, 100, 33, 40, 129), (1, 80, 64, 330, 257),
+    (1, 8, 65, 2, 96), (1, 9, 128, 3, 129), (2, 24, 131, 7, 128), (1, 40, 260, 33, 200), (3, 16, 130, 130, 140),
+]
+
+
+@pytest.mark.parametrize("case", STREAM_CASES)
+@pytest.mark.parametrize("flags", ["none", "skip_relu", "skip_pool_relu"])
+def test_streamed_weight_pairs(pp, runner, oracle_mod, case, flags):
+    N, Ci, Co, H, W = case
+    pool = "pool" in flags
+    if pool:
+        H, W = H + H % 2, W + W % 2
+    rng = np.random.default_rng(sum(case) + len(flags))
+    L = synth.small_random_layer(rng, Co, Ci, P=8, keep=0.5)
+    x = rng.uniform(-1, 1, (N, Ci, H, W)).astype(np.float32)
+    skip = rng.uniform(-1, 1, (N, Co, H, W)).astype(np.float32) if "skip" in flags else None
+    fl = (pp.PP_ADD_SKIP if skip is not None else 0) | (pp.PP_RELU if "relu" in flags else 0) | (pp.PP_POOL2 if pool else 0)
+    y, s = oracle_layer_full(oracle_mod, L, x, skip, "relu" in flags, pool)
+    d = runner.DeviceLayer(L)
+    try:
+        st = torch.cuda.current_stream()
+        pp.pp_layer_autotune(d.handle, N, H, W, fl, st)
+        pp.pp_layer_set_kernel(d.handle, pp.PP_KERNEL_TC)
+        outs = []
+        for _ in range(2):
+            g = torch.full(y.shape, float("nan"), device="cuda")
+            d.forward(dev(x), g, None if skip is None else dev(skip), N, H, W, fl, st)
+            torch.cuda.synchronize()
+            assert pp.pp_layer_device_status(d.handle) == 0
+            outs.append(g.cpu().numpy())
+    finally:
+        d.close()
+    check_within(outs[0], y, s, f"streamed weights {case} {flags}")
+    assert np.array_equal(outs[0], outs[1])
