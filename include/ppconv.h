@@ -267,7 +267,9 @@ pp_status pp_layer_precision(const pp_layer* layer, int* precision, float* input
  * PP_KERNEL_AUTO picks by an estimate of each kernel's time for the layer's
  * density (the direct kernel for Ci <= 4, and in place of an FMA kernel that it
  * beats, then also with more channels).  Setting a kernel the layer cannot
- * run returns PP_ERR_UNSUPPORTED. */
+ * run returns PP_ERR_UNSUPPORTED.  The kernels that run all 9 taps (TC, TC_FLAT,
+ * DIRECT) multiply pruned taps as zeros: an input that is not finite then also
+ * reaches outputs whose kept taps do not touch it. */
 #define PP_KERNEL_AUTO 0
 #define PP_KERNEL_TMEM 1
 #define PP_KERNEL_REGISTER 2
@@ -285,7 +287,9 @@ pp_status pp_layer_kernel(const pp_layer* layer, int* kernel);
  * keeps the winning one for launches of this shape.  The kernels differ in speed by layer shape:
  * the tensor-core kernel needs many output tiles to fill the GPU, the FMA
  * kernels split small layers across thread-block clusters.  Allocates and
- * frees scratch device memory; must not be called during stream capture.
+ * frees scratch device memory, and for a tf32 layer of more than 64 filters on
+ * a map at least 96 wide keeps a second copy of its weight tiles with the layer
+ * (pp_layer_info counts it); must not be called during stream capture.
  * Errors: PP_ERR_INVALID_ARG, PP_ERR_UNSUPPORTED, PP_ERR_CUDA, PP_ERR_OOM. */
 pp_status pp_layer_autotune(pp_layer* layer, int N, int H, int W, int flags, void* stream);
 

@@ -877,17 +877,19 @@ extern "C" pp_status pp_layer_autotune(pp_layer* L, int N, int H, int W, int fla
     if (c.kernel == PP_KERNEL_TC_FLAT) ppc::tcf_pin(L->tc, N, H, W, flags, c.R, c.S);
     for (int w = 0; w < 2 && st == PP_OK; ++w) st = launch(L, x, y, sk, N, H, W, flags, stream);
     if (st != PP_OK) break;
-    if (cudaEventRecord(e0, stream) != cudaSuccess) {
-      st = PP_ERR_CUDA;
-      break;
+    // the faster of two groups of 4 launches: one group of 5 let a stray delay pick a slower kernel now and then
+    // (VGG-16 op 2 row-tiled, 264 instead of 250 us a frame)
+    float ms = 1e30f;
+    for (int group = 0; group < 2 && st == PP_OK; ++group) {
+      float t = 0.f;
+      if (cudaEventRecord(e0, stream) != cudaSuccess) st = PP_ERR_CUDA;
+      for (int r = 0; r < 4 && st == PP_OK; ++r) st = launch(L, x, y, sk, N, H, W, flags, stream);
+      if (st == PP_OK && (cudaEventRecord(e1, stream) != cudaSuccess || cudaEventSynchronize(e1) != cudaSuccess ||
+                          cudaEventElapsedTime(&t, e0, e1) != cudaSuccess))
+        st = PP_ERR_CUDA;
+      ms = std::min(ms, t);
     }
-    for (int r = 0; r < 5 && st == PP_OK; ++r) st = launch(L, x, y, sk, N, H, W, flags, stream);
-    float ms = 0.f;
-    if (st != PP_OK || cudaEventRecord(e1, stream) != cudaSuccess || cudaEventSynchronize(e1) != cudaSuccess ||
-        cudaEventElapsedTime(&ms, e0, e1) != cudaSuccess) {
-      st = st != PP_OK ? st : PP_ERR_CUDA;
-      break;
-    }
+    if (st != PP_OK) break;
     if (c.kernel == PP_KERNEL_TC) tc_ms = ms;
     if (ms < best_ms) {
       best_ms = ms;

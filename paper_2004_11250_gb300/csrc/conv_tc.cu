@@ -975,8 +975,10 @@ pp_status tc_build(TcLayout* T, const pp_packed* pk, cudaStream_t stream) {
   T->dbytes = total + 256;
   T->a = static_cast<const unsigned char*>(d);
   T->status = reinterpret_cast<int*>(static_cast<unsigned char*>(d) + total);
-  // 64-filter layers whose weights do not stay resident stream them in the pairs' order
-  return FB == 64 && tcr_streams(*T, Ci) ? tcr_pair_layout(T, stream) : PP_OK;
+  // 64-filter layers whose weights do not stay resident stream them in the pairs' order (without memory for the copy
+  // they run the row-tiled kernel)
+  if (FB == 64 && tcr_streams(*T, Ci) && tcr_pair_layout(T, stream) == PP_ERR_CUDA) return PP_ERR_CUDA;
+  return PP_OK;
 }
 
 // The same layer for the fp16 split (PP_PRECISION_F16X3): per (filter block,
