@@ -46,6 +46,7 @@ if ROOT not in sys.path:
 
 HBM_PEAK_GBS_FALLBACK = 6800.0
 CONFIG_CPU_SECONDS = 4.0  # oracle sample per workload of the all-configs table
+# by kernel choice; the row-tiled choice (3) launches ppconv_tcr_kernel where CTA pairs take the layer
 KERNEL_NAMES = {1: "ppconv_tm_kernel", 2: "ppconv_kernel", 3: "ppconv_tc_kernel", 4: "ppconv_tcf_kernel",
                 5: "ppconv_direct_kernel"}
 FP32_LANES_PER_SM = 128

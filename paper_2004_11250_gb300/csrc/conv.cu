@@ -878,9 +878,10 @@ extern "C" pp_status pp_layer_autotune(pp_layer* L, int N, int H, int W, int fla
     for (int w = 0; w < 2 && st == PP_OK; ++w) st = launch(L, x, y, sk, N, H, W, flags, stream);
     if (st != PP_OK) break;
     // the faster of two groups of 4 launches: one group of 5 let a stray delay pick a slower kernel now and then
-    // (VGG-16 op 2 row-tiled, 264 instead of 250 us a frame)
+    // (VGG-16 op 2 row-tiled, 264 instead of 250 us a frame).  A candidate that took over twice the best one's time
+    // needs no second group.
     float ms = 1e30f;
-    for (int group = 0; group < 2 && st == PP_OK; ++group) {
+    for (int group = 0; group < 2 && st == PP_OK && (group == 0 || ms < 2.f * best_ms); ++group) {
       float t = 0.f;
       if (cudaEventRecord(e0, stream) != cudaSuccess) st = PP_ERR_CUDA;
       for (int r = 0; r < 4 && st == PP_OK; ++r) st = launch(L, x, y, sk, N, H, W, flags, stream);
