@@ -320,7 +320,7 @@ pp_status pp_layer_flat_geometry(const pp_layer* layer, int N, int H, int W, int
 pp_status pp_layer_pin_flat_geometry(pp_layer* layer, int N, int H, int W, int flags, int R, int S);
 
 /* Synchronous: *device_error = 0 unless a launch of this layer's tensor-core
- * kernels met an error since the last read, and its output is then invalid:
+ * kernels, or of its direct kernels' box copies, met an error since the last read, and its output is then invalid:
  * bit 0 (value 1) a bounded wait gave up; bit 1 (value 2) under
  * PP_PRECISION_F16X3 an input was not finite or overflowed fp16 (|x s_x| >=
  * 65520) after the layer's input scale.  The word is cleared by the read. */

@@ -935,10 +935,14 @@ extern "C" pp_status pp_layer_pin_flat_geometry(pp_layer* L, int N, int H, int W
 extern "C" pp_status pp_layer_device_status(const pp_layer* L, int* device_error) {
   if (!L || !device_error) return PP_ERR_INVALID_ARG;
   *device_error = 0;
-  if (!L->tc_ok) return PP_OK;
-  pp_status st = ppc::tc_status(L->tc, device_error);
-  if (st == PP_OK && *device_error && cudaMemset(L->tc.status, 0, sizeof(int)) != cudaSuccess) return PP_ERR_CUDA;
-  return st;
+  for (int* word : {L->tc_ok ? L->tc.status : nullptr, L->direct.status}) {
+    int v = 0;
+    if (!word) continue;
+    if (cudaMemcpy(&v, word, sizeof(int), cudaMemcpyDeviceToHost) != cudaSuccess) return PP_ERR_CUDA;
+    *device_error |= v;
+    if (v && cudaMemset(word, 0, sizeof(int)) != cudaSuccess) return PP_ERR_CUDA;
+  }
+  return PP_OK;
 }
 
 extern "C" pp_status pp_layer_info(const pp_layer* L, int* Co, int* Ci, int64_t* device_bytes) {

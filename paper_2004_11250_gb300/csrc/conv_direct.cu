@@ -10,13 +10,18 @@
 // The weights are expanded to the dense 9 taps (pruned taps and kernels are
 // exact zeros, so the sum is the one of Section 2 with zero terms added).  Input
 // channels are staged a few at a time (tile plus one-pixel zero halo) together
-// with their weights, in a ring of stages filled by cp.async.  Epilogue: + bias, + skip,
+// with their weights, in a ring of stages.  Where a tensor map can describe x (W a
+// multiple of 4, x 16-byte aligned) a stage's input is one box copy, issued by one
+// thread; else every thread copies by cp.async, whose issue slots and load-store
+// work then bound the kernels (64 -> 1 at 720 x 1280 52 us against 36 with boxes).
+// Waits on the boxes' mbarriers are bounded; one that gives up is recorded in the
+// layer's device status word.  Epilogue: + bias, + skip,
 // ReLU, optional 2 x 2 max pool, stored in the original channel order.
 //
 // ppconv_direct_kernel: a CTA of 256 threads owns FBD filters of a tile; a
 // thread owns a 2 x 2 pixel block and FBD x 4 accumulators.  What bounds it is
 // instruction issue and, on large maps, the FMA pipe (64 -> 64 at 224 x 224,
-// batch 4: 45 of 73 TFLOP/s), so two filters share each packed FMA
+// batch 4: 51 of 73 TFLOP/s, 45 with cp.async copies), so two filters share each packed FMA
 // (fma.rn.f32x2): the weights lie as pairs of filters, 9 pairs per channel padded
 // to 80 bytes, read as broadcasts; the thread's 4 x 4 window is duplicated once
 // per channel.  Maps with few tiles split the staged channels over KS groups of
@@ -32,7 +37,8 @@
 // for 36 FMAs) took longer than the copies.  A thread owns 4 x 4 pixels, a warp 4
 // rows of 128, so a window row is one 16-byte read and two shuffles for 12 FMAs a
 // row and filter, and three stages of two channels keep 40 KB per CTA in flight.
-// 64 -> 1 at 720 x 1280 with the residual: 97 -> 61 us (4.0 TB/s of the input).
+// 64 -> 1 at 720 x 1280 with the residual, alone: 97 us (2 x 2 blocks), 61 (cp.async), 43 (boxes; 36 among
+// other launches, 6.7 TB/s of input, residual and output: HBM bounds it).
 //
 // ppconv_direct_first_kernel: at most 4 input channels (a network's first
 // layer) on maps wider than a tile's half.  These write far more than they read:
@@ -64,6 +70,7 @@ struct DirectParams {
   int N, Ci, Co, H, W, flags;
   int npair;
   int tiles_x, tiles_y;
+  int* status;  // device status word
   int vec;  // x 16-byte aligned and W a multiple of 4: rows staged in 16-byte copies
 };
 
@@ -125,6 +132,59 @@ struct XStage {
   }
 };
 
+// Where x can be box-copied (a tensor map: W a multiple of 4, x 16-byte aligned) a stage's input is one copy by one thread
+// that completes on the stage's mbarrier, with its zeros outside the image; XStage's copies are the other maps' path.
+// One per CTA; every thread calls wait for every chunk, in order.
+template <int NS>
+struct BoxRing {
+  uint64_t* full;   // [NS] in shared memory
+  int issued = 0;   // thread 0: chunks whose copy was issued
+  bool dead = false;
+  __device__ __forceinline__ void init(int tid) {
+    if (tid == 0) {
+      for (int s = 0; s < NS; ++s) mbar_init(su32(full + s), 1);
+      asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+    }
+    __syncthreads();
+  }
+  // Thread 0: channels ch0 .. of image n from row r0 - 1, column c0 - 4 into dst, as chunk ch; `more` further bytes of the
+  // stage are copied by the caller.
+  __device__ __forceinline__ void copy(const CUtensorMap* m, float* dst, int bytes, int more, int ch, int ch0, int r0,
+                                       int c0, int n) {
+    mbar_arrive_expect_tx(su32(full + ch % NS), bytes + more);
+    asm volatile(
+        "cp.async.bulk.tensor.4d.shared::cluster.global.tile.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3, %4, "
+        "%5}], [%6];" ::"r"(su32(dst)),
+        "l"(reinterpret_cast<uint64_t>(m)), "r"(c0 - 4), "r"(r0 - 1), "r"(ch0), "r"(n), "r"(su32(full + ch % NS))
+        : "memory");
+    issued = ch + 1;
+  }
+  __device__ __forceinline__ bool poll(int ch) const {
+    bool ok = false;
+    for (long q = 0; q < PP_WAIT_POLLS && !ok; ++q) ok = mbar_try(su32(full + ch % NS), (uint32_t)((ch / NS) & 1));
+    return ok;
+  }
+  // A wait that gives up is recorded, and the thread waits (and thread 0 copies) no more.
+  __device__ __forceinline__ void wait(int ch, int* status) {
+    if (dead || poll(ch)) return;
+    dead = true;
+    atomicOr(status, ppc::kStatusTimeout);
+  }
+  // Thread 0, after the last chunk: no copy may be in flight when the CTA's shared memory is reused or given back.
+  __device__ __forceinline__ void drain() const {
+    if (!dead) return;
+    for (int ch = issued > NS ? issued - NS : 0; ch < issued; ++ch) poll(ch);
+  }
+};
+
+// The tensor map as a kernel argument, nothing where there is none.
+template <bool BOX>
+struct BoxMap {
+  CUtensorMap m;
+};
+template <>
+struct BoxMap<false> {};
+
 template <int CC, int FBD, int KS>
 struct DirectGeo {
   static constexpr int TH = KS == 1 ? 32 : 16, TW = KS == 4 ? 16 : 32;  // tile of 1024 / KS pixels
@@ -134,15 +194,19 @@ struct DirectGeo {
   // stages: one chunk's arithmetic does not cover the copies' latency (small tiles have less of it)
   static constexpr int NS = KS == 1 ? 3 : 4;
   static constexpr int FLOATS = NS * (XS + WS) > RED ? NS * (XS + WS) : RED;
+  static_assert(CC != 4 || XS * 4 % 128 == 0, "box copies start at 128 bytes");
   static_assert(CC % KS == 0 && FBD % 2 == 0, "channels over the groups, filters in pairs");
 };
 
-template <int CC, int FBD, int KS>
-__global__ void __launch_bounds__(DTHREADS, 2) ppconv_direct_kernel(const DirectParams p) {
+template <int CC, int FBD, int KS, bool BOX>
+__global__ void __launch_bounds__(DTHREADS, 2) ppconv_direct_kernel(const DirectParams p, const __grid_constant__ BoxMap<BOX> xmap) {
   using G = DirectGeo<CC, FBD, KS>;
   constexpr int NP = FBD / 2, GT = DTHREADS / KS, TX = G::TW / 2;
+  // boxes start at 128 bytes, so the weights lie after them all; else in their stage
+  constexpr int XSTEP = BOX ? G::XS : G::XS + G::WS, WSTEP = BOX ? G::WS : XSTEP, W0 = BOX ? G::NS * G::XS : G::XS;
   // NS stages of [CC][ROWS][COLS] input and [CC][NP][WPAIR] weights; at the end the groups' sums
-  extern __shared__ __align__(16) float dsm[];
+  extern __shared__ __align__(128) float dsm[];
+  __shared__ uint64_t full[G::NS];
   const int tid = threadIdx.x, grp = tid / GT, gt = tid % GT, tx = gt % TX, ty = gt / TX;
   int t = (int)blockIdx.x;
   const int bx = t % p.tiles_x;
@@ -156,15 +220,31 @@ __global__ void __launch_bounds__(DTHREADS, 2) ppconv_direct_kernel(const Direct
   const int nchunks = (p.Ci + CC - 1) / CC;
 
   XStage<G::ROWS, G::COLS, DTHREADS> xst;
-  xst.init(p, r0, c0, tid);
+  BoxRing<G::NS> ring{full};
+  if constexpr (BOX) ring.init(tid);
+  else xst.init(p, r0, c0, tid);
   auto stage = [&](int ch) {
-    float* xs = dsm + (ch % G::NS) * (G::XS + G::WS);
+    float* xs = dsm + (ch % G::NS) * XSTEP;
+    float* ws = dsm + W0 + (ch % G::NS) * WSTEP;
+    if constexpr (BOX) {
+      if (tid == 0 && ch < nchunks && !ring.dead) {
+        const int have = min(CC, p.Ci - ch * CC);  // the weights of these channels, a bulk copy each
+        ring.copy(&xmap.m, xs, G::XS * 4, have * NP * WPAIR * 4, ch, ch * CC, r0, c0, n);
+        for (int k = 0; k < have; ++k)
+          asm volatile(
+              "cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(
+                  su32(ws + k * NP * WPAIR)),
+              "l"(p.w + ((size_t)(ch * CC + k) * p.npair + q0) * WPAIR), "r"(NP * WPAIR * 4), "r"(su32(full + ch % G::NS))
+              : "memory");
+      }
+      return;
+    }
     if (ch < nchunks) {
       xst.template copy<CC>(xs, p, xb, ch * CC, r0, c0, tid);
       for (int e = tid; e < CC * NP * (WPAIR / 4); e += DTHREADS) {  // the layout is padded to FBMAX filters
         const int k = e / (NP * (WPAIR / 4)), rem = e - k * (NP * (WPAIR / 4));
         const bool in = ch * CC + k < p.Ci;
-        cp_async16(xs + G::XS + 4 * e, in ? p.w + ((size_t)(ch * CC + k) * p.npair + q0) * WPAIR + 4 * rem : p.w, in);
+        cp_async16(ws + 4 * e, in ? p.w + ((size_t)(ch * CC + k) * p.npair + q0) * WPAIR + 4 * rem : p.w, in);
       }
     }
     asm volatile("cp.async.commit_group;" ::: "memory");  // one group per step, empty past the last chunk
@@ -182,11 +262,13 @@ __global__ void __launch_bounds__(DTHREADS, 2) ppconv_direct_kernel(const Direct
 #pragma unroll
   for (int st = 0; st < G::NS - 1; ++st) stage(st);
   for (int ch = 0; ch < nchunks; ++ch) {
-    asm volatile("cp.async.wait_group %0;" ::"n"(G::NS - 2) : "memory");
-    __syncthreads();  // chunk ch has landed; every thread is done with the stage that is filled next
+    if constexpr (BOX) asm volatile("fence.proxy.async.shared::cta;" ::: "memory");  // reads, before the next copy
+    else asm volatile("cp.async.wait_group %0;" ::"n"(G::NS - 2) : "memory");
+    __syncthreads();  // chunk ch has landed (cp.async); every thread is done with the stage that is filled next
     stage(ch + G::NS - 1);
-    const float* xs = dsm + (ch % G::NS) * (G::XS + G::WS);
-    const float* ws = xs + G::XS;
+    if constexpr (BOX) ring.wait(ch, p.status);
+    const float* xs = dsm + (ch % G::NS) * XSTEP;
+    const float* ws = dsm + W0 + (ch % G::NS) * WSTEP;
     uint64_t part[NP][4];  // the chunk's sum: added to acc as one term, which keeps the rounding error of long sums low
 #pragma unroll
     for (int o = 0; o < NP; ++o)
@@ -235,6 +317,8 @@ __global__ void __launch_bounds__(DTHREADS, 2) ppconv_direct_kernel(const Direct
       for (int q = 0; q < 4; ++q) acc[o][q] = add2(acc[o][q], part[o][q]);
   }
 
+  if constexpr (BOX)
+    if (tid == 0) ring.drain();
   // the next kernel may start its prologue (it waits for this grid to finish)
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
   if (KS > 1) {
@@ -301,12 +385,14 @@ constexpr int VH = 16, VW = 128;             // tile: 4 rows of 128 pixels per w
 constexpr int VROWS = VH + 2, VCOLS = VW + 8;
 constexpr int VCC = 2, VST = 3;              // channels per stage, stages
 constexpr int VX = VCC * VROWS * VCOLS;
+static_assert(VX * 4 % 128 == 0, "box copies start at 128 bytes");
 
-template <int CO>
-__global__ void __launch_bounds__(VTHREADS, 3) ppconv_direct_wide_kernel(const DirectParams p) {
-  // VST stages of [VCC][VROWS][VCOLS] input and [VCC][CO][9][2] weights (each twice, for packed FMAs)
+template <int CO, bool BOX>
+__global__ void __launch_bounds__(VTHREADS, 3) ppconv_direct_wide_kernel(const DirectParams p, const __grid_constant__ BoxMap<BOX> xmap) {
+  // VST stages of [VCC][VROWS][VCOLS] input, then of [VCC][CO][9][2] weights (each twice, for packed FMAs)
   constexpr int VWS = VCC * CO * 20;
-  extern __shared__ __align__(16) float dsm[];
+  extern __shared__ __align__(128) float dsm[];
+  __shared__ uint64_t full[VST];
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   int t = (int)blockIdx.x;
   const int bx = t % p.tiles_x;
@@ -318,15 +404,22 @@ __global__ void __launch_bounds__(VTHREADS, 3) ppconv_direct_wide_kernel(const D
   const int nchunks = (p.Ci + VCC - 1) / VCC;
 
   XStage<VROWS, VCOLS, VTHREADS> xst;
-  xst.init(p, r0, c0, tid);
+  BoxRing<VST> ring{full};
+  if constexpr (BOX) ring.init(tid);
+  else xst.init(p, r0, c0, tid);
+  float* const wsm = dsm + VST * VX;
   auto stage = [&](int ch) {
-    float* xs = dsm + (ch % VST) * (VX + VWS);
+    const int st = ch % VST;
     if (ch < nchunks) {
-      xst.template copy<VCC>(xs, p, xb, ch * VCC, r0, c0, tid);
+      if constexpr (BOX) {
+        if (tid == 0 && !ring.dead) ring.copy(&xmap.m, dsm + st * VX, VX * 4, 0, ch, ch * VCC, r0, c0, n);
+      } else {
+        xst.template copy<VCC>(dsm + st * VX, p, xb, ch * VCC, r0, c0, tid);
+      }
       for (int e = tid; e < VCC * CO * 18; e += VTHREADS) {
         const int k = e / (CO * 18), rem = e - k * (CO * 18), o = rem / 18, tap = (rem - o * 18) >> 1;
         const bool in = ch * VCC + k < p.Ci;
-        cp_async4(xs + VX + (k * CO + o) * 20 + (rem - o * 18),
+        cp_async4(wsm + st * VWS + (k * CO + o) * 20 + (rem - o * 18),
                   in ? p.w + ((size_t)(ch * VCC + k) * p.npair + (o >> 1)) * WPAIR + 2 * tap + (o & 1) : p.w, in);
       }
     }
@@ -344,9 +437,12 @@ __global__ void __launch_bounds__(VTHREADS, 3) ppconv_direct_wide_kernel(const D
   for (int s = 0; s < VST - 1; ++s) stage(s);
   for (int ch = 0; ch < nchunks; ++ch) {
     asm volatile("cp.async.wait_group %0;" ::"n"(VST - 2) : "memory");
-    __syncthreads();  // chunk ch has landed; every thread is done with the stage that is filled next
+    if constexpr (BOX) asm volatile("fence.proxy.async.shared::cta;" ::: "memory");  // reads, before the next copy
+    __syncthreads();  // chunk ch has landed (cp.async); every thread is done with the stage that is filled next
     stage(ch + VST - 1);
-    const float* xs = dsm + (ch % VST) * (VX + VWS);
+    if constexpr (BOX) ring.wait(ch, p.status);
+    const float* xs = dsm + (ch % VST) * VX;
+    const float* ws = wsm + (ch % VST) * VWS;
 #pragma unroll
     for (int k = 0; k < VCC; ++k) {
       if (ch * VCC + k >= p.Ci) break;
@@ -368,7 +464,7 @@ __global__ void __launch_bounds__(VTHREADS, 3) ppconv_direct_wide_kernel(const D
       }
 #pragma unroll
       for (int o = 0; o < CO; ++o) {
-        const float* wp = xs + VX + (k * CO + o) * 20;
+        const float* wp = ws + (k * CO + o) * 20;
         uint64_t wt[9];
 #pragma unroll
         for (int e = 0; e < 4; ++e) {
@@ -390,6 +486,8 @@ __global__ void __launch_bounds__(VTHREADS, 3) ppconv_direct_wide_kernel(const D
     }
   }
 
+  if constexpr (BOX)
+    if (tid == 0) ring.drain();
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
   asm volatile("cp.async.wait_group 0;" ::: "memory");
   const bool relu = p.flags & PP_RELU, pool = p.flags & PP_POOL2;
@@ -588,8 +686,18 @@ cudaError_t launch_one(DirectParams p, cudaStream_t stream) {
   const int64_t nt = (int64_t)p.N * p.tiles_x * p.tiles_y, nfb = (p.Co + FBD - 1) / FBD;
   if (nt > INT32_MAX) return cudaErrorInvalidConfiguration;
   const unsigned gy = (unsigned)std::min<int64_t>(nfb, 65535);  // the grid's y extent; the rest in z
-  return launch_kernel(ppconv_direct_kernel<CC, FBD, KS>, once, dim3((unsigned)nt, gy, (unsigned)((nfb + gy - 1) / gy)),
-                       DTHREADS, G::FLOATS * 4, stream, p);
+  const dim3 grid((unsigned)nt, gy, (unsigned)((nfb + gy - 1) / gy));
+  // Boxes where the grid is large (64 -> 64 at 224 x 224 94 -> 83 us, 96 -> 96 at 112 x 112 73.5 -> 70.5); with four
+  // groups on small tiles a box's latency costs more than the copies it saves (64 -> 64 at 56 x 56 14.6 against 14.0).
+  if constexpr (CC == 4 && KS <= 2) {
+    BoxMap<true> xmap;
+    if (p.Ci > CC && ppc::image_map(&xmap.m, p.x, p.N, p.Ci, p.H, p.W, G::COLS, G::ROWS, CC)) {
+      static ppc::DeviceOnce box;
+      return launch_kernel(ppconv_direct_kernel<CC, FBD, KS, true>, box, grid, DTHREADS, G::FLOATS * 4, stream, p, xmap);
+    }
+  }
+  return launch_kernel(ppconv_direct_kernel<CC, FBD, KS, false>, once, grid, DTHREADS, G::FLOATS * 4, stream, p,
+                       BoxMap<false>());
 }
 
 template <int CO>
@@ -599,8 +707,14 @@ cudaError_t launch_wide(DirectParams p, cudaStream_t stream) {
   p.tiles_y = (p.H + VH - 1) / VH;
   const int64_t nt = (int64_t)p.N * p.tiles_x * p.tiles_y;
   if (nt > INT32_MAX) return cudaErrorInvalidConfiguration;
-  return launch_kernel(ppconv_direct_wide_kernel<CO>, once, dim3((unsigned)nt), VTHREADS,
-                       VST * (VX + VCC * CO * 20) * 4, stream, p);
+  constexpr int bytes = VST * (VX + VCC * CO * 20) * 4;
+  BoxMap<true> xmap;
+  if (ppc::image_map(&xmap.m, p.x, p.N, p.Ci, p.H, p.W, VCOLS, VROWS, VCC)) {
+    static ppc::DeviceOnce box;
+    return launch_kernel(ppconv_direct_wide_kernel<CO, true>, box, dim3((unsigned)nt), VTHREADS, bytes, stream, p, xmap);
+  }
+  return launch_kernel(ppconv_direct_wide_kernel<CO, false>, once, dim3((unsigned)nt), VTHREADS, bytes, stream, p,
+                       BoxMap<false>());
 }
 
 template <int CI>
@@ -645,11 +759,13 @@ pp_status direct_build(DirectLayout* D, const float* w_dense, const float* bias,
       for (int t = 0; t < 9; ++t) dst[2 * t] = src[t];
     }
   void* d = nullptr;
-  if (cudaMalloc(&d, (nw + nb) * 4) != cudaSuccess) {
+  if (cudaMalloc(&d, (nw + nb + 1) * 4) != cudaSuccess) {
     cudaGetLastError();
     return PP_ERR_OOM;
   }
-  if (cudaMemcpyAsync(d, host.data(), nw * 4, cudaMemcpyHostToDevice, stream) != cudaSuccess ||
+  int* status = reinterpret_cast<int*>(static_cast<float*>(d) + nw + nb);
+  if (cudaMemsetAsync(status, 0, sizeof(int), stream) != cudaSuccess ||
+      cudaMemcpyAsync(d, host.data(), nw * 4, cudaMemcpyHostToDevice, stream) != cudaSuccess ||
       (nb && cudaMemcpyAsync(static_cast<float*>(d) + nw, bias, nb * 4, cudaMemcpyHostToDevice, stream) !=
                  cudaSuccess) ||
       cudaStreamSynchronize(stream) != cudaSuccess) {
@@ -657,7 +773,8 @@ pp_status direct_build(DirectLayout* D, const float* w_dense, const float* bias,
     return PP_ERR_CUDA;
   }
   D->dmem = d;
-  D->dbytes = (nw + nb) * 4;
+  D->dbytes = (nw + nb + 1) * 4;
+  D->status = status;
   D->w = static_cast<const float*>(d);
   D->bias = nb ? static_cast<const float*>(d) + nw : nullptr;
   D->npair = npair;
@@ -677,6 +794,7 @@ pp_status direct_launch(const DirectLayout& D, const float* x, float* y, const f
   p.skip = (flags & PP_ADD_SKIP) ? skip : nullptr;
   p.w = D.w;
   p.bias = D.bias;
+  p.status = D.status;
   p.N = N;
   p.Ci = D.Ci;
   p.Co = D.Co;
@@ -691,7 +809,7 @@ pp_status direct_launch(const DirectLayout& D, const float* x, float* y, const f
   };
   cudaError_t e;
   if (D.Co <= 4 && D.Ci >= 8 && ctas(VH, VW, 4) >= sms) {
-    // (64 -> 1 at 720 x 1280 61 us, 64 -> 3 109 us; 2 x 2 pixel blocks 97 and 147.  Fewer tiles than SMs: the split
+    // (64 -> 1 at 720 x 1280 43 us, 64 -> 3 88; 2 x 2 pixel blocks 97 and 147.  Fewer tiles than SMs: the split
     // channels below, 64 -> 1 at 224 x 224 10.5 us)
     switch (D.Co) {
       case 1: e = launch_wide<1>(p, stream); break;

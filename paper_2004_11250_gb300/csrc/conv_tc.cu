@@ -849,21 +849,6 @@ typedef CUresult (*EncodeTiledFn)(CUtensorMap*, CUtensorMapDataType, cuuint32_t,
 std::atomic<EncodeTiledFn> g_encode{nullptr};
 ppc::DeviceOnce g_encode_once;
 
-// 4-D map over x viewed as [N][Ci][H][W] (W innermost), box [1][KCH][R+2][TW+8].
-template <int ORI, int TW, int FB, bool F16>
-bool make_xmap(CUtensorMap* m, const TcParams& p) {
-  using G = Geo<ORI, TW, FB, F16>;
-  const EncodeTiledFn encode = g_encode.load(std::memory_order_acquire);
-  if (!encode) return false;
-  const cuuint64_t dims[4] = {(cuuint64_t)p.W, (cuuint64_t)p.H, (cuuint64_t)p.Ci, (cuuint64_t)p.N};
-  const cuuint64_t strides[3] = {(cuuint64_t)p.W * 4, (cuuint64_t)p.W * p.H * 4, (cuuint64_t)p.W * p.H * p.Ci * 4};
-  const cuuint32_t box[4] = {(cuuint32_t)G::RAW_W, (cuuint32_t)G::BROWS, (cuuint32_t)G::KCH, 1};
-  const cuuint32_t estr[4] = {1, 1, 1, 1};
-  return encode(m, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 4, const_cast<float*>(p.x), dims, strides, box, estr,
-                  CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE, CU_TENSOR_MAP_L2_PROMOTION_L2_128B,
-                  CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
-}
-
 template <int ORI, int TW, int FB, bool F16>
 cudaError_t launch_one(const TcParams& p0, cudaStream_t stream, int sms) {
   using G = Geo<ORI, TW, FB, F16>;
@@ -873,8 +858,7 @@ cudaError_t launch_one(const TcParams& p0, cudaStream_t stream, int sms) {
   p.tiles_y = (p.H + G::R - 1) / G::R;
   CUtensorMap xmap;
   std::memset(&xmap, 0, sizeof(xmap));
-  p.use_tma =
-      ((p.W & 3) == 0 && (reinterpret_cast<uintptr_t>(p.x) & 15) == 0 && make_xmap<ORI, TW, FB, F16>(&xmap, p)) ? 1 : 0;
+  p.use_tma = ppc::image_map(&xmap, p.x, p.N, p.Ci, p.H, p.W, G::RAW_W, G::BROWS, G::KCH) ? 1 : 0;
   const int64_t nt = (int64_t)p.tiles_x * p.tiles_y * p.nfb * p.N;
   if (nt > INT32_MAX) return cudaErrorInvalidValue;
   p.ntiles = (int)nt;
@@ -903,8 +887,13 @@ cudaError_t launch(const TcParams& p, cudaStream_t stream, int sms, bool f16) {
 namespace ppc {
 
 pp_status tc_prepare() {
-  if (prepare() != cudaSuccess || device_sms() <= 0 || tcr_prepare() != PP_OK) return PP_ERR_CUDA;
-  // the entry point is process-wide; looked up at the first set-up of each device
+  return prepare() == cudaSuccess && device_sms() > 0 && tcr_prepare() == PP_OK ? PP_OK : PP_ERR_CUDA;
+}
+
+// 4-D map over x viewed as [N][Ci][H][W] (W innermost), box [1][bc][bh][bw].
+bool image_map(CUtensorMap* m, const float* x, int N, int Ci, int H, int W, int bw, int bh, int bc) {
+  if ((W & 3) != 0 || (reinterpret_cast<uintptr_t>(x) & 15) != 0) return false;
+  // the entry point is process-wide; looked up at the first use on each device
   const cudaError_t e = g_encode_once.run([](int) {
     void* fn = nullptr;
     cudaDriverEntryPointQueryResult q;
@@ -915,7 +904,15 @@ pp_status tc_prepare() {
       cudaGetLastError();  // without the entry point every launch uses per-thread loads
     return cudaSuccess;
   });
-  return e == cudaSuccess ? PP_OK : PP_ERR_CUDA;
+  const EncodeTiledFn encode = g_encode.load(std::memory_order_acquire);
+  if (e != cudaSuccess || !encode) return false;
+  const cuuint64_t dims[4] = {(cuuint64_t)W, (cuuint64_t)H, (cuuint64_t)Ci, (cuuint64_t)N};
+  const cuuint64_t strides[3] = {(cuuint64_t)W * 4, (cuuint64_t)W * H * 4, (cuuint64_t)W * H * Ci * 4};
+  const cuuint32_t box[4] = {(cuuint32_t)bw, (cuuint32_t)bh, (cuuint32_t)bc, 1};
+  const cuuint32_t estr[4] = {1, 1, 1, 1};
+  return encode(m, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 4, const_cast<float*>(x), dims, strides, box, estr,
+                CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE, CU_TENSOR_MAP_L2_PROMOTION_L2_128B,
+                CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 
 // Dense per-tap weights of every (FB-filter block, 8-channel chunk), split into
@@ -1134,13 +1131,6 @@ void tc_free(TcLayout* T) {
   T->f16 = false;
   delete T->state;
   T->state = nullptr;
-}
-
-pp_status tc_status(const TcLayout& T, int* device_error) {
-  int v = 0;
-  if (cudaMemcpy(&v, T.status, sizeof(int), cudaMemcpyDeviceToHost) != cudaSuccess) return PP_ERR_CUDA;
-  *device_error = v;
-  return PP_OK;
 }
 
 }  // namespace ppc

@@ -1,6 +1,7 @@
 // Internal declarations shared by the library's translation units.
 #pragma once
 
+#include <cuda.h>
 #include <cuda_runtime.h>
 
 #include <atomic>
@@ -110,10 +111,12 @@ constexpr int kStatusTimeout = 1;
 constexpr int kStatusF16Range = 2;
 
 pp_status tc_prepare();
+// Tensor map for box copies out of x viewed as [N][Ci][H][W], box [1][bc][bh][bw]; zeros outside the image.  False where
+// such copies are not possible (x not 16-byte aligned, W not a multiple of 4, no driver entry point).
+bool image_map(CUtensorMap* m, const float* x, int N, int Ci, int H, int W, int bw, int bh, int bc);
 pp_status tc_build(TcLayout* T, const pp_packed* pk, cudaStream_t stream);
 pp_status tc_launch(const TcLayout& T, const LayerMeta& M, const float* x, float* y, const float* skip, int N,
                     int H, int W, int flags, cudaStream_t stream);
-pp_status tc_status(const TcLayout& T, int* device_error);
 // Build the f16 tiles and scales (precision PP_PRECISION_F16X3) for inputs bounded by input_bound.
 pp_status tc_build16(TcLayout* T, const pp_packed* pk, float input_bound, cudaStream_t stream);
 void tc_free(TcLayout* T);
@@ -151,6 +154,7 @@ struct DirectLayout {
   int npair = 0;
   const float* w = nullptr;
   const float* bias = nullptr;
+  int* status = nullptr;  // device status word
   int Co = 0, Ci = 0;
 };
 bool direct_applicable(int Co, int Ci);
