@@ -31,14 +31,18 @@
 // which halves the rounding error of one long sum (1.1e-7 against 2.2e-7 of the
 // result at 64 channels).
 //
-// ppconv_direct_wide_kernel: at most 4 filters on wide maps (a network's last
+// ppconv_direct_wide_kernel: at most 3 filters on wide maps (a network's last
 // layer).  These read far more than they compute (64 -> 1 at 720 x 1280: 236 MB
 // of input), and with 2 x 2 blocks the shared-memory reads of the windows (16
 // for 36 FMAs) took longer than the copies.  A thread owns 4 x 4 pixels, a warp 4
 // rows of 128, so a window row is one 16-byte read and two shuffles for 12 FMAs a
-// row and filter, and three stages of two channels keep 40 KB per CTA in flight.
-// 64 -> 1 at 720 x 1280 with the residual, alone: 97 us (2 x 2 blocks), 61 (cp.async), 43 (boxes; 36 among
-// other launches, 6.7 TB/s of input, residual and output: HBM bounds it).
+// row and filter.  A warp of its own copies, and the others free a stage each for
+// itself: with a barrier over the CTA per chunk their reads and their FMAs came in
+// turns.  Three stages of two channels keep 40 KB per CTA in flight; where the
+// tiles leave SMs without three CTAs, groups of warps share a tile's channels.
+// 64 -> 1 at 720 x 1280 with the residual, alone: 97 us (2 x 2 blocks), 61
+// (cp.async), 43 (boxes), 42 (copying warp), 36 among other launches, 6.7 TB/s of
+// input, residual and output, where HBM bounds it; at 360 x 640 27.2 -> 16.3.
 //
 // ppconv_direct_first_kernel: at most 4 input channels (a network's first
 // layer) on maps wider than a tile's half.  These write far more than they read:
@@ -70,7 +74,8 @@ struct DirectParams {
   int N, Ci, Co, H, W, flags;
   int npair;
   int tiles_x, tiles_y;
-  int* status;  // device status word
+  const float* wdup;  // at most 3 filters: [Ci][Co][20], tap t twice at 2 t, 2 t + 1
+  int* status;        // device status word
   int vec;  // x 16-byte aligned and W a multiple of 4: rows staged in 16-byte copies
 };
 
@@ -134,11 +139,34 @@ struct XStage {
 
 // Where x can be box-copied (a tensor map: W a multiple of 4, x 16-byte aligned) a stage's input is one copy by one thread
 // that completes on the stage's mbarrier, with its zeros outside the image; XStage's copies are the other maps' path.
-// One per CTA; every thread calls wait for every chunk, in order.
+// Channels ch0 .. of image n from row r0 - 1, column c0 - 4 into dst; `more` further bytes come by bulk_copy.
+__device__ __forceinline__ void box_copy(const CUtensorMap* m, float* dst, int bytes, int more, int ch0, int r0, int c0,
+                                         int n, uint64_t* full) {
+  mbar_arrive_expect_tx(su32(full), bytes + more);
+  asm volatile(
+      "cp.async.bulk.tensor.4d.shared::cluster.global.tile.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3, %4, "
+      "%5}], [%6];" ::"r"(su32(dst)),
+      "l"(reinterpret_cast<uint64_t>(m)), "r"(c0 - 4), "r"(r0 - 1), "r"(ch0), "r"(n), "r"(su32(full))
+      : "memory");
+}
+__device__ __forceinline__ void bulk_copy(float* dst, const float* src, int bytes, uint64_t* full) {
+  asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(su32(dst)),
+               "l"(src), "r"(bytes), "r"(su32(full))
+               : "memory");
+}
+// A bounded wait: false when it gave up.
+__device__ __forceinline__ bool mbar_poll(uint32_t bar, uint32_t parity) {
+  for (long q = 0; q < PP_WAIT_POLLS; ++q)
+    if (mbar_try(bar, parity)) return true;
+  return false;
+}
+
+// The full barriers of a ring whose stages are freed by a barrier over the CTA: every thread calls wait for every chunk,
+// in order; thread 0 copies.
 template <int NS>
 struct BoxRing {
-  uint64_t* full;   // [NS] in shared memory
-  int issued = 0;   // thread 0: chunks whose copy was issued
+  uint64_t* full;  // [NS] in shared memory
+  int issued = 0;  // thread 0: chunks whose copy was issued
   bool dead = false;
   __device__ __forceinline__ void init(int tid) {
     if (tid == 0) {
@@ -147,22 +175,8 @@ struct BoxRing {
     }
     __syncthreads();
   }
-  // Thread 0: channels ch0 .. of image n from row r0 - 1, column c0 - 4 into dst, as chunk ch; `more` further bytes of the
-  // stage are copied by the caller.
-  __device__ __forceinline__ void copy(const CUtensorMap* m, float* dst, int bytes, int more, int ch, int ch0, int r0,
-                                       int c0, int n) {
-    mbar_arrive_expect_tx(su32(full + ch % NS), bytes + more);
-    asm volatile(
-        "cp.async.bulk.tensor.4d.shared::cluster.global.tile.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3, %4, "
-        "%5}], [%6];" ::"r"(su32(dst)),
-        "l"(reinterpret_cast<uint64_t>(m)), "r"(c0 - 4), "r"(r0 - 1), "r"(ch0), "r"(n), "r"(su32(full + ch % NS))
-        : "memory");
-    issued = ch + 1;
-  }
   __device__ __forceinline__ bool poll(int ch) const {
-    bool ok = false;
-    for (long q = 0; q < PP_WAIT_POLLS && !ok; ++q) ok = mbar_try(su32(full + ch % NS), (uint32_t)((ch / NS) & 1));
-    return ok;
+    return mbar_poll(su32(full + ch % NS), (uint32_t)((ch / NS) & 1));
   }
   // A wait that gives up is recorded, and the thread waits (and thread 0 copies) no more.
   __device__ __forceinline__ void wait(int ch, int* status) {
@@ -229,13 +243,11 @@ __global__ void __launch_bounds__(DTHREADS, 2) ppconv_direct_kernel(const Direct
     if constexpr (BOX) {
       if (tid == 0 && ch < nchunks && !ring.dead) {
         const int have = min(CC, p.Ci - ch * CC);  // the weights of these channels, a bulk copy each
-        ring.copy(&xmap.m, xs, G::XS * 4, have * NP * WPAIR * 4, ch, ch * CC, r0, c0, n);
+        uint64_t* bar = full + ch % G::NS;
+        box_copy(&xmap.m, xs, G::XS * 4, have * NP * WPAIR * 4, ch * CC, r0, c0, n, bar);
         for (int k = 0; k < have; ++k)
-          asm volatile(
-              "cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(
-                  su32(ws + k * NP * WPAIR)),
-              "l"(p.w + ((size_t)(ch * CC + k) * p.npair + q0) * WPAIR), "r"(NP * WPAIR * 4), "r"(su32(full + ch % G::NS))
-              : "memory");
+          bulk_copy(ws + k * NP * WPAIR, p.w + ((size_t)(ch * CC + k) * p.npair + q0) * WPAIR, NP * WPAIR * 4, bar);
+        ring.issued = ch + 1;
       }
       return;
     }
@@ -380,51 +392,72 @@ __global__ void __launch_bounds__(DTHREADS, 2) ppconv_direct_kernel(const Direct
   }
 }
 
-constexpr int VTHREADS = 128;                // 4 warps
-constexpr int VH = 16, VW = 128;             // tile: 4 rows of 128 pixels per warp
+constexpr int VH = 16, VW = 128;             // tile: 4 rows of 128 pixels per warp of a group
 constexpr int VROWS = VH + 2, VCOLS = VW + 8;
-constexpr int VCC = 2, VST = 3;              // channels per stage, stages
-constexpr int VX = VCC * VROWS * VCOLS;
-static_assert(VX * 4 % 128 == 0, "box copies start at 128 bytes");
 
-template <int CO, bool BOX>
-__global__ void __launch_bounds__(VTHREADS, 3) ppconv_direct_wide_kernel(const DirectParams p, const __grid_constant__ BoxMap<BOX> xmap) {
+// KS groups of 4 warps take the channels of a stage in turn; group 0 adds their sums.
+template <int CO, int KS, bool BOX>
+struct WideGeo {
+  static constexpr int NT = 128 * KS, VCC = KS == 4 ? 4 : 2;          // computing threads, channels per stage
+  static constexpr int VST = KS == 1 ? 3 : 5;                         // stages
+  static constexpr int THREADS = NT + (BOX ? 32 : 0);                 // and the warp that issues the copies
+  static constexpr int XS = VCC * VROWS * VCOLS, WS = VCC * CO * 20;  // floats of a stage
+  static constexpr int BYTES = VST * (XS + WS) * 4;
+  static_assert(XS * 4 % 128 == 0, "box copies start at 128 bytes");
+  static_assert((KS - 1) * CO * 8 * 128 * 8 <= BYTES, "the groups' sums lie over the stages");
+};
+
+template <int CO, int KS, bool BOX>
+__global__ void __launch_bounds__(WideGeo<CO, KS, BOX>::THREADS, KS == 1 ? 3 : 1)
+    ppconv_direct_wide_kernel(const DirectParams p, const __grid_constant__ BoxMap<BOX> xmap) {
+  using G = WideGeo<CO, KS, BOX>;
+  constexpr int VCC = G::VCC, VST = G::VST;
   // VST stages of [VCC][VROWS][VCOLS] input, then of [VCC][CO][9][2] weights (each twice, for packed FMAs)
-  constexpr int VWS = VCC * CO * 20;
   extern __shared__ __align__(128) float dsm[];
-  __shared__ uint64_t full[VST];
-  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  __shared__ uint64_t full[VST], empty[VST];
+  float* const wsm = dsm + VST * G::XS;
+  const int tid = threadIdx.x, grp = tid >> 7, gt = tid & 127, warp = gt >> 5, lane = tid & 31;
   int t = (int)blockIdx.x;
   const int bx = t % p.tiles_x;
   t /= p.tiles_x;
   const int by = t % p.tiles_y;
   const int n = t / p.tiles_y;
   const int r0 = by * VH, c0 = bx * VW;
-  const float* xb = p.x + (size_t)n * p.Ci * p.H * p.W;
   const int nchunks = (p.Ci + VCC - 1) / VCC;
 
-  XStage<VROWS, VCOLS, VTHREADS> xst;
-  BoxRing<VST> ring{full};
-  if constexpr (BOX) ring.init(tid);
-  else xst.init(p, r0, c0, tid);
-  float* const wsm = dsm + VST * VX;
-  auto stage = [&](int ch) {
-    const int st = ch % VST;
-    if (ch < nchunks) {
-      if constexpr (BOX) {
-        if (tid == 0 && !ring.dead) ring.copy(&xmap.m, dsm + st * VX, VX * 4, 0, ch, ch * VCC, r0, c0, n);
-      } else {
-        xst.template copy<VCC>(dsm + st * VX, p, xb, ch * VCC, r0, c0, tid);
+  if constexpr (BOX) {
+    if (tid == 0) {
+      for (int s = 0; s < VST; ++s) {
+        mbar_init(su32(full + s), 1);
+        mbar_init(su32(empty + s), 4 * KS);  // one arrival per computing warp
       }
-      for (int e = tid; e < VCC * CO * 18; e += VTHREADS) {
-        const int k = e / (CO * 18), rem = e - k * (CO * 18), o = rem / 18, tap = (rem - o * 18) >> 1;
-        const bool in = ch * VCC + k < p.Ci;
-        cp_async4(wsm + st * VWS + (k * CO + o) * 20 + (rem - o * 18),
-                  in ? p.w + ((size_t)(ch * VCC + k) * p.npair + (o >> 1)) * WPAIR + 2 * tap + (o & 1) : p.w, in);
-      }
+      asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
-    asm volatile("cp.async.commit_group;" ::: "memory");  // one group per step, empty past the last chunk
-  };
+    __syncthreads();
+  }
+  asm volatile("griddepcontrol.wait;" ::: "memory");
+  if constexpr (BOX) {
+    if (tid >= G::NT) {
+      // One thread copies a chunk's input box and weights into its stage once every warp is done with the chunk before.
+      if (lane == 0) {
+        int ch = 0;
+        for (; ch < nchunks; ++ch) {
+          const int st = ch % VST;
+          if (ch >= VST && !mbar_poll(su32(empty + st), (uint32_t)((ch / VST - 1) & 1))) {
+            atomicOr(p.status, ppc::kStatusTimeout);
+            break;
+          }
+          const int wbytes = min(VCC, p.Ci - ch * VCC) * CO * 80;
+          box_copy(&xmap.m, dsm + st * G::XS, G::XS * 4, wbytes, ch * VCC, r0, c0, n, full + st);
+          bulk_copy(wsm + st * G::WS, p.wdup + (size_t)ch * VCC * CO * 20, wbytes, full + st);
+        }
+        // no copy may be in flight when the CTA exits (the computing warps waited for them unless a wait gave up)
+        for (int c = ch > VST ? ch - VST : 0; c < ch; ++c) mbar_poll(su32(full + c % VST), (uint32_t)((c / VST) & 1));
+      }
+      asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+      return;
+    }
+  }
 
   uint64_t acc[CO][4][2];  // 4 rows x 4 columns as pairs of columns
 #pragma unroll
@@ -432,19 +465,12 @@ __global__ void __launch_bounds__(VTHREADS, 3) ppconv_direct_wide_kernel(const D
 #pragma unroll
     for (int r = 0; r < 4; ++r) acc[o][r][0] = acc[o][r][1] = 0;
 
-  asm volatile("griddepcontrol.wait;" ::: "memory");
+  auto compute = [&](int ch) {
+    const float* xs = dsm + (ch % VST) * G::XS;
+    const float* ws = wsm + (ch % VST) * G::WS;
 #pragma unroll
-  for (int s = 0; s < VST - 1; ++s) stage(s);
-  for (int ch = 0; ch < nchunks; ++ch) {
-    asm volatile("cp.async.wait_group %0;" ::"n"(VST - 2) : "memory");
-    if constexpr (BOX) asm volatile("fence.proxy.async.shared::cta;" ::: "memory");  // reads, before the next copy
-    __syncthreads();  // chunk ch has landed (cp.async); every thread is done with the stage that is filled next
-    stage(ch + VST - 1);
-    if constexpr (BOX) ring.wait(ch, p.status);
-    const float* xs = dsm + (ch % VST) * VX;
-    const float* ws = wsm + (ch % VST) * VWS;
-#pragma unroll
-    for (int k = 0; k < VCC; ++k) {
+    for (int kk = 0; kk < VCC / KS; ++kk) {
+      const int k = kk * KS + grp;
       if (ch * VCC + k >= p.Ci) break;
       // window rows 0 .. 5, columns -1 .. 4 of the thread's block: pairs starting at each of the columns -1 .. 3
       uint64_t xp[6][5];
@@ -484,12 +510,66 @@ __global__ void __launch_bounds__(VTHREADS, 3) ppconv_direct_wide_kernel(const D
                 acc[o][r][h] = fma2(wt[dy * 3 + dx], xp[r + dy][2 * h + dx], acc[o][r][h]);
       }
     }
+  };
+
+  if constexpr (BOX) {
+    bool dead = false;  // after a wait that gave up the thread waits no more; the output is invalid
+    for (int ch = 0; ch < nchunks; ++ch) {
+      const int st = ch % VST;
+      if (!dead && !mbar_poll(su32(full + st), (uint32_t)((ch / VST) & 1))) {
+        dead = true;
+        atomicOr(p.status, ppc::kStatusTimeout);
+      }
+      compute(ch);
+      asm volatile("fence.proxy.async.shared::cta;" ::: "memory");  // these reads, before the next copy into the stage
+      __syncwarp();
+      if (lane == 0) mbar_arrive(su32(empty + st));
+    }
+  } else {
+    const float* xb = p.x + (size_t)n * p.Ci * p.H * p.W;
+    XStage<VROWS, VCOLS, G::NT> xst;
+    xst.init(p, r0, c0, tid);
+    auto stage = [&](int ch) {
+      const int st = ch % VST;
+      if (ch < nchunks) {
+        xst.template copy<VCC>(dsm + st * G::XS, p, xb, ch * VCC, r0, c0, tid);
+        const int have = min(VCC, p.Ci - ch * VCC) * CO * 5;
+        for (int e = tid; e < have; e += G::NT)
+          cp_async16(wsm + st * G::WS + 4 * e, p.wdup + (size_t)ch * VCC * CO * 20 + 4 * e, true);
+      }
+      asm volatile("cp.async.commit_group;" ::: "memory");  // one group per step, empty past the last chunk
+    };
+#pragma unroll
+    for (int s = 0; s < VST - 1; ++s) stage(s);
+    for (int ch = 0; ch < nchunks; ++ch) {
+      asm volatile("cp.async.wait_group %0;" ::"n"(VST - 2) : "memory");
+      __syncthreads();  // chunk ch has landed; every thread is done with the stage that is filled next
+      stage(ch + VST - 1);
+      compute(ch);
+    }
+    asm volatile("cp.async.wait_group 0;" ::: "memory");
   }
 
-  if constexpr (BOX)
-    if (tid == 0) ring.drain();
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
-  asm volatile("cp.async.wait_group 0;" ::: "memory");
+  if constexpr (KS > 1) {
+    uint64_t* red = reinterpret_cast<uint64_t*>(dsm);
+    group_sync<G::NT>();  // every thread is done with the stages
+    if (grp > 0) {
+#pragma unroll
+      for (int o = 0; o < CO; ++o)
+#pragma unroll
+        for (int e = 0; e < 8; ++e) red[(((grp - 1) * CO + o) * 8 + e) * 128 + gt] = acc[o][e >> 1][e & 1];
+    }
+    group_sync<G::NT>();
+    if (grp > 0) return;
+#pragma unroll
+    for (int g = 0; g < KS - 1; ++g)
+#pragma unroll
+      for (int o = 0; o < CO; ++o)
+#pragma unroll
+        for (int e = 0; e < 8; ++e)
+          acc[o][e >> 1][e & 1] = add2(acc[o][e >> 1][e & 1], red[((g * CO + o) * 8 + e) * 128 + gt]);
+  }
   const bool relu = p.flags & PP_RELU, pool = p.flags & PP_POOL2;
   const float* skip = (p.flags & PP_ADD_SKIP) ? p.skip : nullptr;
   const int row0 = r0 + 4 * warp, c = c0 + 4 * lane;
@@ -700,21 +780,24 @@ cudaError_t launch_one(DirectParams p, cudaStream_t stream) {
                        BoxMap<false>());
 }
 
-template <int CO>
+template <int CO, int KS, bool BOX>
+cudaError_t launch_wide_one(const DirectParams& p, int64_t nt, const BoxMap<BOX>& xmap, cudaStream_t stream) {
+  using G = WideGeo<CO, KS, BOX>;
+  static ppc::DeviceOnce once;  // one per instantiation
+  return launch_kernel(ppconv_direct_wide_kernel<CO, KS, BOX>, once, dim3((unsigned)nt), G::THREADS, G::BYTES, stream, p,
+                       xmap);
+}
+
+template <int CO, int KS>
 cudaError_t launch_wide(DirectParams p, cudaStream_t stream) {
-  static ppc::DeviceOnce once;
   p.tiles_x = (p.W + VW - 1) / VW;
   p.tiles_y = (p.H + VH - 1) / VH;
   const int64_t nt = (int64_t)p.N * p.tiles_x * p.tiles_y;
   if (nt > INT32_MAX) return cudaErrorInvalidConfiguration;
-  constexpr int bytes = VST * (VX + VCC * CO * 20) * 4;
   BoxMap<true> xmap;
-  if (ppc::image_map(&xmap.m, p.x, p.N, p.Ci, p.H, p.W, VCOLS, VROWS, VCC)) {
-    static ppc::DeviceOnce box;
-    return launch_kernel(ppconv_direct_wide_kernel<CO, true>, box, dim3((unsigned)nt), VTHREADS, bytes, stream, p, xmap);
-  }
-  return launch_kernel(ppconv_direct_wide_kernel<CO, false>, once, dim3((unsigned)nt), VTHREADS, bytes, stream, p,
-                       BoxMap<false>());
+  if (ppc::image_map(&xmap.m, p.x, p.N, p.Ci, p.H, p.W, VCOLS, VROWS, WideGeo<CO, KS, true>::VCC))
+    return launch_wide_one<CO, KS, true>(p, nt, xmap, stream);
+  return launch_wide_one<CO, KS, false>(p, nt, BoxMap<false>(), stream);
 }
 
 template <int CI>
@@ -750,13 +833,16 @@ pp_status direct_build(DirectLayout* D, const float* w_dense, const float* bias,
                        cudaStream_t stream) {
   // pairs of filters, padded to whole CTAs of FBMAX filters (zero weights)
   const int npair = (Co + FBMAX - 1) / FBMAX * (FBMAX / 2);
-  const size_t nw = (size_t)Ci * npair * WPAIR, nb = bias ? (size_t)Co : 0;
+  const size_t ndup = Co <= 3 ? (size_t)Ci * Co * WPAIR : 0;  // the wide kernel's weights, each twice
+  const size_t np = (size_t)Ci * npair * WPAIR, nw = np + ndup, nb = bias ? (size_t)Co : 0;
   std::vector<float> host(nw, 0.f);
   for (int o = 0; o < Co; ++o)
     for (int i = 0; i < Ci; ++i) {
       float* dst = &host[((size_t)i * npair + (o >> 1)) * WPAIR + (o & 1)];
       const float* src = w_dense + ((size_t)o * Ci + i) * 9;
       for (int t = 0; t < 9; ++t) dst[2 * t] = src[t];
+      if (ndup)
+        for (int t = 0; t < 18; ++t) host[np + ((size_t)i * Co + o) * WPAIR + t] = src[t >> 1];
     }
   void* d = nullptr;
   if (cudaMalloc(&d, (nw + nb + 1) * 4) != cudaSuccess) {
@@ -777,6 +863,7 @@ pp_status direct_build(DirectLayout* D, const float* w_dense, const float* bias,
   D->status = status;
   D->w = static_cast<const float*>(d);
   D->bias = nb ? static_cast<const float*>(d) + nw : nullptr;
+  D->wdup = ndup ? static_cast<const float*>(d) + np : nullptr;
   D->npair = npair;
   D->Co = Co;
   D->Ci = Ci;
@@ -794,6 +881,7 @@ pp_status direct_launch(const DirectLayout& D, const float* x, float* y, const f
   p.skip = (flags & PP_ADD_SKIP) ? skip : nullptr;
   p.w = D.w;
   p.bias = D.bias;
+  p.wdup = D.wdup;
   p.status = D.status;
   p.N = N;
   p.Ci = D.Ci;
@@ -808,15 +896,22 @@ pp_status direct_launch(const DirectLayout& D, const float* x, float* y, const f
     return (int64_t)N * ((H + th - 1) / th) * ((W + tw - 1) / tw) * ((D.Co + fbd - 1) / fbd);
   };
   cudaError_t e;
-  if (D.Co <= 4 && D.Ci >= 8 && ctas(VH, VW, 4) >= sms) {
-    // (64 -> 1 at 720 x 1280 43 us, 64 -> 3 88; 2 x 2 pixel blocks 97 and 147.  Fewer tiles than SMs: the split
-    // channels below, 64 -> 1 at 224 x 224 10.5 us)
-    switch (D.Co) {
-      case 1: e = launch_wide<1>(p, stream); break;
-      case 2: e = launch_wide<2>(p, stream); break;
-      case 3: e = launch_wide<3>(p, stream); break;
-      default: e = launch_wide<4>(p, stream); break;
-    }
+  // The wide kernel by its tiles: one filter from half a tile per SM (fewer: the split channels of the 2 x 2 kernel, 64 ->
+  // 1 at 240 x 240, 30 tiles, 10.7 us against 15.8), with more groups of warps the fewer there are (64 -> 1 at 360 x 640,
+  // 115 tiles: 1 / 2 / 4 groups 21.0 / 18.8 / 16.3, 2 x 2 kernel 27.2; 540 x 960, 272 tiles: 38.9 / 30.4 / 34.3, 42.9;
+  // 720 x 1280, 450 tiles: 40.6 / 46.3 / 51.2, 70.5).  Two filters share the 2 x 2 kernel's packed FMAs and need two
+  // tiles per SM to lose (43 against 51 - 61 at 540 x 960, 71 against 61 at 720 x 1280), three leave a fourth of them
+  // idle (40.5 against 35.3 at 360 x 640, 111 against 84), four never lose by it (111 against 115).  Without boxes (W not
+  // a multiple of 4) the copies bound it and two groups of warps gain nothing (64 -> 1 at 540 x 959 57.6 against 61.8,
+  // 64 -> 3 at 361 x 643 54.8, 2 x 2 kernel 48.4).
+  const int64_t vt = D.Ci >= 8 && D.Co <= 3 ? ctas(VH, VW, 4) : 0;
+  if (D.Co == 1 && vt * 2 >= sms) {
+    e = vt >= (p.vec ? 2 : 1) * sms ? launch_wide<1, 1>(p, stream)
+                                    : vt > sms ? launch_wide<1, 2>(p, stream) : launch_wide<1, 4>(p, stream);
+  } else if (D.Co == 2 && vt >= 2 * sms) {
+    e = launch_wide<2, 1>(p, stream);
+  } else if (D.Co == 3 && (vt >= sms || (p.vec && vt * 3 >= sms * 2))) {
+    e = vt >= 2 * sms ? launch_wide<3, 1>(p, stream) : launch_wide<3, 2>(p, stream);
   } else if (D.Ci <= 4 && W > UW / 2 && D.Co > 4 && D.Co <= 65535 && ctas(UH, UW, FBMAX) >= sms / 2) {
     // (1 -> 64 at 720 x 1280 48 us against 86 with the 32 x 32 tiles, 3 -> 64 at 224 x 224 7.2 against 9.1; below half
     // a CTA per SM the smaller tiles win: 1 -> 64 at 64 x 96, 64 CTAs, 3.0 against 2.7)

@@ -154,7 +154,8 @@ struct DirectLayout {
   int npair = 0;
   const float* w = nullptr;
   const float* bias = nullptr;
-  int* status = nullptr;  // device status word
+  const float* wdup = nullptr;  // at most 3 filters
+  int* status = nullptr;        // device status word
   int Co = 0, Ci = 0;
 };
 bool direct_applicable(int Co, int Ci);

@@ -1136,12 +1136,14 @@ def test_resident_weight_kernel_unaligned_input(pp, runner, oracle_mod, precisio
 
 
 # The direct kernels: dense layers between wide layers, channel groups (1, 2 or 4) on small and large grids, ragged
-# channel counts and filter pairs; the wide kernel of last layers (1 - 4 filters) and the first-layer kernel (1 - 4
+# channel counts and filter pairs; the wide kernel of last layers (1 - 3 filters; 1, 2 or 4 groups of warps, with boxes and
+# without) and the first-layer kernel (1 - 4
 # channels) at tile edges, with and without rows of whole 16-byte groups, with more than one filter block per CTA.
 DIRECT_SHAPES = [
     # N, Ci, Co, H, W
     (1, 33, 47, 14, 14), (2, 20, 24, 40, 37), (1, 18, 17, 1, 1), (1, 64, 64, 33, 65), (5, 24, 40, 96, 96), (3, 17, 21, 130, 128),
     (2, 8, 1, 720, 260), (1, 9, 2, 1250, 255), (3, 10, 3, 416, 256), (1, 16, 4, 2500, 130), (1, 8, 3, 16, 128),
+    (1, 9, 1, 130, 1028), (1, 13, 1, 131, 1030), (1, 64, 1, 300, 1280), (1, 8, 1, 313, 1281), (1, 11, 3, 300, 700), (2, 9, 3, 160, 1284), (1, 10, 2, 520, 1284),
     (1, 1, 64, 18, 129), (2, 2, 70, 64, 130), (1, 3, 130, 41, 200), (1, 4, 9, 300, 257), (1, 3, 33, 6, 66), (2, 1, 5, 2000, 68),
 ]
 
