@@ -727,7 +727,11 @@ cudaError_t launch(const TcrParams& p, int pairs, cudaStream_t stream) {
   // tf32: pairs of tiles and filter blocks; f16: pairs of strip pieces, row by row (pooled: row pair by row pair)
   const int64_t work = F16 ? (int64_t)((p.nstrips * p.split + 1) / 2) * (p.srows / (POOL ? 2 : 1))
                            : (int64_t)((p.ntiles + 1) / 2) * p.nfb;
-  cfg.gridDim = dim3((unsigned)(2 * std::min<int64_t>(work, pairs)));
+  // No more pairs than the busiest one's share calls for, and in f16 at least two rows each (a row alone fetches three):
+  // the SMs left over run what else is in flight (f16, three networks on streams of their own, a frame: 8 layers of 64
+  // channels at 205 x 59 95 -> 75 us, 7 at 54 x 220 56 -> 39; alone a layer takes 12.8 -> 12.0 and 10.0 -> 11.0).
+  const int64_t share = std::max<int64_t>((work + pairs - 1) / pairs, F16 && !POOL ? 2 : 1);
+  cfg.gridDim = dim3((unsigned)(2 * ((work + share - 1) / share)));
   cfg.blockDim = dim3(NTHREADS);
   cfg.dynamicSmemBytes = Geo<F16, FB, STREAM>::SMEM;
   cfg.stream = stream;
