@@ -896,8 +896,8 @@ pp_status direct_launch(const DirectLayout& D, const float* x, float* y, const f
     return (int64_t)N * ((H + th - 1) / th) * ((W + tw - 1) / tw) * ((D.Co + fbd - 1) / fbd);
   };
   cudaError_t e;
-  // The wide kernel by its tiles: one filter from half a tile per SM (fewer: the split channels of the 2 x 2 kernel, 64 ->
-  // 1 at 240 x 240, 30 tiles, 10.7 us against 15.8), with more groups of warps the fewer there are (64 -> 1 at 360 x 640,
+  // The wide kernel by its tiles: one filter from two tiles for five SMs (64 -> 1 at 128 x 128, batch 8, 64 tiles: 16.0 us
+  // against the 2 x 2 kernel's 19.6; fewer: its split channels, 240 x 240, 30 tiles, 10.7 against 15.8), with more groups of warps the fewer there are (64 -> 1 at 360 x 640,
   // 115 tiles: 1 / 2 / 4 groups 21.0 / 18.8 / 16.3, 2 x 2 kernel 27.2; 540 x 960, 272 tiles: 38.9 / 30.4 / 34.3, 42.9;
   // 720 x 1280, 450 tiles: 40.6 / 46.3 / 51.2, 70.5).  Two filters share the 2 x 2 kernel's packed FMAs and need two
   // tiles per SM to lose (43 against 51 - 61 at 540 x 960, 71 against 61 at 720 x 1280), three leave a fourth of them
@@ -905,7 +905,7 @@ pp_status direct_launch(const DirectLayout& D, const float* x, float* y, const f
   // a multiple of 4) the copies bound it and two groups of warps gain nothing (64 -> 1 at 540 x 959 57.6 against 61.8,
   // 64 -> 3 at 361 x 643 54.8, 2 x 2 kernel 48.4).
   const int64_t vt = D.Ci >= 8 && D.Co <= 3 ? ctas(VH, VW, 4) : 0;
-  if (D.Co == 1 && vt * 2 >= sms) {
+  if (D.Co == 1 && vt * (p.vec ? 5 : 4) >= 2 * sms) {
     e = vt >= (p.vec ? 2 : 1) * sms ? launch_wide<1, 1>(p, stream)
                                     : vt > sms ? launch_wide<1, 2>(p, stream) : launch_wide<1, 4>(p, stream);
   } else if (D.Co == 2 && vt >= 2 * sms) {
