@@ -1034,7 +1034,9 @@ struct FlatGeo {
 // 16-byte aligned and each thread loads its own; start-up, pipeline fill and
 // teardown of ~9000 cycles; the last tile's copy out of tensor memory at ~16
 // cycles a column and the remote part of a split's partials at ~24 more;
-// clusters of 16 start late (~12000); and clusters beyond those co-resident on
+// clusters of 16 start the later the more of them there are (up to ~12000; a few
+// are worth it: 387 -> 78 at 10 x 15 split in 16 10.4 us, in 8 13.4; 512
+// -> 512 at 7 x 7 12.4 against 16.2); and clusters beyond those co-resident on
 // the GPU run in later waves.  CTA pairs measured slower than their halves apart
 // (39.6 against 31.4 us at 512 -> 512, 28 x 28): 1.15 of the chunk time.  Against
 // every accepted geometry of 21 shapes the model's choice measured within 1 % of
@@ -1116,8 +1118,9 @@ int flat_candidates(int N, int H, int W, int nch, int nfb, bool pool, bool allow
           cost = waves * nch * per_chunk + 9000.0 + (wide ? waves : 1.0) * 16.0 * G.ncols;
         } else {
           // clusters beyond those that fit on the GPU at once run in a later wave
+          const double full = std::min(1.0, (double)G.ntiles / D.max_clusters[cs]);
           const double waves = std::ceil((double)G.ntiles / D.max_clusters[cs]);
-          cost = waves * (std::ceil((double)nch / s) * per_chunk + 9000.0 + (cs == 16 ? 12000.0 : 0.0) +
+          cost = waves * (std::ceil((double)nch / s) * per_chunk + 9000.0 + (cs == 16 ? 12000.0 * full * full : 0.0) +
                           (16.0 + 24.0 * (s - 1) / s) * G.ncols);
         }
         G.split = s;
