@@ -267,9 +267,11 @@ pp_status pp_layer_precision(const pp_layer* layer, int* precision, float* input
  * PP_KERNEL_AUTO picks by an estimate of each kernel's time for the layer's
  * density (the direct kernel for Ci <= 4, and in place of an FMA kernel that it
  * beats, then also with more channels).  Setting a kernel the layer cannot
- * run returns PP_ERR_UNSUPPORTED.  The kernels that run all 9 taps (TC, TC_FLAT,
- * DIRECT) multiply pruned taps as zeros: an input that is not finite then also
- * reaches outputs whose kept taps do not touch it. */
+ * run returns PP_ERR_UNSUPPORTED.  The tensor-core kernels, and
+ * the direct kernel on layers that would else run a tensor-core kernel or that
+ * have at most 4 input channels, multiply pruned taps as zeros: an input that
+ * is not finite then also reaches outputs whose kept taps do not touch it.  The
+ * other kernels, and the direct kernel in their place, sum the kept taps alone. */
 #define PP_KERNEL_AUTO 0
 #define PP_KERNEL_TMEM 1
 #define PP_KERNEL_REGISTER 2

@@ -412,6 +412,7 @@ struct pp_layer {
   float* bias = nullptr;
   std::vector<int32_t> pk_perm;     // the packer's filter permutation (host copy)
   std::vector<float> direct_w;      // direct layout's dense weights [Co][Ci][9], original filter order
+  std::vector<uint16_t> direct_kept;  // and a bit per kept tap, [Co][Ci] (empty where pruned taps may count as zeros)
   std::vector<float> direct_bias;   // and its bias (empty: none)
   pp_packed packed;                 // host copy of the packed layer (tensor-core layers: f16 layout built on demand)
   int precision = PP_PRECISION_TF32X3;
@@ -708,18 +709,23 @@ extern "C" pp_status pp_layer_create(const pp_packed* pk, const float* bias, voi
   // layers with a handful of input channels (a network's first layer) run the
   // direct kernel: the others cannot fill their tiles
   L->direct_ok = ppc::direct_applicable(pk->Co, pk->Ci);
+  const bool redo = direct_auto && pk->Ci > 4;
   if (direct_auto || (L->direct_ok && pk->Ci <= 4)) L->auto_kernel = PP_KERNEL_DIRECT;
   if (st == PP_OK && (L->direct_ok || direct_auto)) {
     // dense [Co][Ci][9] in the original filter order, zeros where pruned
     std::vector<float> wd((size_t)pk->Co * pk->Ci * 9, 0.f);
+    // where a kernel over the kept taps alone would be the default, their sums stay free of the pruned taps' inputs
+    std::vector<uint16_t> kept(redo ? (size_t)pk->Co * pk->Ci : 0, 0);
     for (int j = 0; j < pk->Co; ++j)
       for (int32_t e = pk->kptr[j]; e < pk->kptr[j + 1]; ++e) {
         const uint8_t* t = &pk->taps[4 * pk->kpat[e]];
-        for (int s = 0; s < 4; ++s)
-          wd[((size_t)pk->perm[j] * pk->Ci + pk->kidx[e]) * 9 + t[s]] = pk->kw[(size_t)e * 4 + s];
+        const size_t k = (size_t)pk->perm[j] * pk->Ci + pk->kidx[e];
+        if (redo) kept[k] = ppc::tap_mask(t);
+        for (int s = 0; s < 4; ++s) wd[k * 9 + t[s]] = pk->kw[(size_t)e * 4 + s];
       }
-    st = ppc::direct_build(&L->direct, wd.data(), bias, pk->Co, pk->Ci, (cudaStream_t)stream);
+    st = ppc::direct_build(&L->direct, wd.data(), redo ? kept.data() : nullptr, bias, pk->Co, pk->Ci, (cudaStream_t)stream);
     L->direct_w.swap(wd);
+    L->direct_kept.swap(kept);
     if (bias) L->direct_bias.assign(bias, bias + pk->Co);
   }
   if (st != PP_OK) {
@@ -748,11 +754,14 @@ extern "C" pp_status pp_layer_set_output_order(pp_layer* L, const int32_t* order
   ppc::DirectLayout D;
   if (L->direct.w) {
     std::vector<float> w((size_t)Co * Ci * 9), b(L->direct_bias.empty() ? 0 : Co);
+    std::vector<uint16_t> kept(L->direct_kept.size());
     for (int o = 0; o < Co; ++o) {
+      if (!kept.empty()) std::copy_n(&L->direct_kept[(size_t)o * Ci], Ci, &kept[(size_t)ord[o] * Ci]);
       std::memcpy(&w[(size_t)ord[o] * Ci * 9], &L->direct_w[(size_t)o * Ci * 9], (size_t)Ci * 9 * sizeof(float));
       if (!b.empty()) b[ord[o]] = L->direct_bias[o];
     }
-    const pp_status st = ppc::direct_build(&D, w.data(), b.empty() ? nullptr : b.data(), Co, Ci, stream);
+    const pp_status st = ppc::direct_build(&D, w.data(), kept.empty() ? nullptr : kept.data(),
+                                           b.empty() ? nullptr : b.data(), Co, Ci, stream);
     if (st != PP_OK) return st;
   }
   // every other kernel stores reordered filter j at channel perm[j]
@@ -996,7 +1005,7 @@ extern "C" pp_status pp_dense_create(const float* w, const float* bias, int Co, 
   if (!D) return PP_ERR_OOM;
   D->base.Co = Co;
   D->base.Ci = Ci;
-  const pp_status st = ppc::direct_build(&D->base.direct, w, bias, Co, Ci, (cudaStream_t)stream);
+  const pp_status st = ppc::direct_build(&D->base.direct, w, nullptr, bias, Co, Ci, (cudaStream_t)stream);
   D->base.kernel = D->base.auto_kernel = PP_KERNEL_DIRECT;
   if (st != PP_OK) {
     pp_dense_destroy(D);

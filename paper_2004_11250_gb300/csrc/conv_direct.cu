@@ -8,7 +8,8 @@
 // 2 % of the FP32 rate.
 //
 // The weights are expanded to the dense 9 taps (pruned taps and kernels are
-// exact zeros, so the sum is the one of Section 2 with zero terms added).  Input
+// exact zeros, so the sum is the one of Section 2 with zero terms added; where
+// an input is not finite, layers that need it sum the kept taps alone again: redo).  Input
 // channels are staged a few at a time (tile plus one-pixel zero halo) together
 // with their weights, in a ring of stages.  Where a tensor map can describe x (W a
 // multiple of 4, x 16-byte aligned) a stage's input is one box copy, issued by one
@@ -63,21 +64,73 @@ using namespace ppc_ptx;
 
 constexpr int DTHREADS = 256;
 constexpr int FBMAX = 8;      // filters per CTA at most
-constexpr int WPAIR = 20;     // floats of one channel of a filter pair: 9 taps x 2 filters, padded to 80 bytes
+constexpr int WPAIR = 20;     // floats of one channel of a filter pair: 9 taps x 2 filters, the 2 filters' kept taps (bits)
 
 struct DirectParams {
   const float* x;
   float* y;
   const float* skip;
-  const float* w;     // [Ci][npair][WPAIR]: tap t of filters 2 q, 2 q + 1 at 2 t, 2 t + 1; original filter order
+  // [Ci][npair][WPAIR]: tap t of filters 2 q, 2 q + 1 at 2 t, 2 t + 1, a bit per kept tap of each at 18, 19; original
+  // filter order
+  const float* w;
   const float* bias;  // [Co] or null
   int N, Ci, Co, H, W, flags;
   int npair;
   int tiles_x, tiles_y;
   const float* wdup;  // at most 3 filters: [Ci][Co][20], tap t twice at 2 t, 2 t + 1
   int* status;        // device status word
+  int redo;           // sums that are not finite are computed again: see redo
   int vec;  // x 16-byte aligned and W a multiple of 4: rows staged in 16-byte copies
 };
+
+__device__ __forceinline__ bool nan2(uint64_t v) {
+  float a, b;
+  unpack2(v, a, b);
+  return a != a || b != b;
+}
+
+// A pruned tap is no part of the sum, but the kernels multiply it as a zero weight, and zero times an infinity or a NaN is
+// not zero.  Every such product makes its output NaN.  In the instantiations with REDO a thread that meets a sum which is
+// not finite computes its block of outputs (filters o0 .., rows r0 .., columns c0 ..) again over the kept taps alone,
+// straight from x, after its stores.  Layers that run these kernels by default where a kernel over kept taps alone would
+// else run them take those: within 2 % of the others' time in the wide kernel (256 -> 1 at 720 x 1280 150.7 -> 153.4 us),
+// at it in the 2 x 2 kernel (64 -> 16 at 224 x 224 31.1 -> 30.8).
+__device__ __forceinline__ void redo(const DirectParams& p, int n, int o0, int no, int r0, int nr, int c0, int nc) {
+  const size_t plane = (size_t)p.H * p.W;
+  const auto output = [&](int o, int r, int c) -> float {
+    const float* w = p.w + (size_t)(o >> 1) * WPAIR + (o & 1);
+    const float* x = p.x + (size_t)n * p.Ci * plane;
+    float sum = 0.f;
+    for (int i = 0; i < p.Ci; ++i, w += (size_t)p.npair * WPAIR, x += plane) {
+      const uint32_t kept = __float_as_uint(__ldg(w + 18));
+      for (int t = 0; t < 9; ++t) {
+        if (!(kept >> t & 1)) continue;
+        const int row = r - 1 + t / 3, col = c - 1 + t % 3;
+        const bool in = (unsigned)row < (unsigned)p.H && (unsigned)col < (unsigned)p.W;
+        sum = fmaf(__ldg(w + 2 * t), in ? __ldg(x + (size_t)row * p.W + col) : 0.f, sum);
+      }
+    }
+    if (p.bias) sum += __ldg(p.bias + o);
+    if (p.flags & PP_ADD_SKIP) sum += __ldg(p.skip + ((size_t)n * p.Co + o) * plane + (size_t)r * p.W + c);
+    return p.flags & PP_RELU ? fmaxf(sum, 0.f) : sum;
+  };
+  for (int o = o0; o < min(o0 + no, p.Co); ++o)
+    for (int r = r0; r < min(r0 + nr, p.H); r += p.flags & PP_POOL2 ? 2 : 1)
+      for (int c = c0; c < min(c0 + nc, p.W); c += p.flags & PP_POOL2 ? 2 : 1) {
+        const size_t q = (size_t)n * p.Co + o;
+        if (p.flags & PP_POOL2)
+          p.y[(q * (p.H / 2) + r / 2) * (p.W / 2) + c / 2] =
+              fmaxf(fmaxf(output(o, r, c), output(o, r, c + 1)), fmaxf(output(o, r + 1, c), output(o, r + 1, c + 1)));
+        else
+          p.y[(q * p.H + r) * p.W + c] = output(o, r, c);
+      }
+}
+
+// The same as a call: inlined it costs the 2 x 2 kernel registers (70 -> 90 for two filters, a CTA less per SM), while
+// a call costs the wide kernel 8 %.
+__device__ __noinline__ void redo_call(const DirectParams p, int n, int o0, int no, int r0, int nr, int c0, int nc) {
+  redo(p, n, o0, no, r0, nr, c0, nc);
+}
 
 __device__ __forceinline__ void cp_async4(float* dst, const float* src, bool valid) {
   const uint32_t d = (uint32_t)__cvta_generic_to_shared(dst);
@@ -212,7 +265,7 @@ struct DirectGeo {
   static_assert(CC % KS == 0 && FBD % 2 == 0, "channels over the groups, filters in pairs");
 };
 
-template <int CC, int FBD, int KS, bool BOX>
+template <int CC, int FBD, int KS, bool BOX, bool REDO>
 __global__ void __launch_bounds__(DTHREADS, 2) ppconv_direct_kernel(const DirectParams p, const __grid_constant__ BoxMap<BOX> xmap) {
   using G = DirectGeo<CC, FBD, KS>;
   constexpr int NP = FBD / 2, GT = DTHREADS / KS, TX = G::TW / 2;
@@ -355,6 +408,13 @@ __global__ void __launch_bounds__(DTHREADS, 2) ppconv_direct_kernel(const Direct
   const bool relu = p.flags & PP_RELU, pool = p.flags & PP_POOL2;
   const float* skip = (p.flags & PP_ADD_SKIP) ? p.skip : nullptr;
   const int r = r0 + 2 * ty, c = c0 + 2 * tx;
+  uint64_t bad = 0;  // zero times every sum: NaN once one is not finite
+  if constexpr (REDO) {
+#pragma unroll
+    for (int o = 0; o < NP; ++o)
+#pragma unroll
+      for (int q = 0; q < 4; ++q) bad = fma2(acc[o][q], 0, bad);
+  }
 #pragma unroll
   for (int o = 0; o < FBD; ++o) {
     const int oo = 2 * q0 + o;
@@ -390,6 +450,7 @@ __global__ void __launch_bounds__(DTHREADS, 2) ppconv_direct_kernel(const Direct
       }
     }
   }
+  if (REDO && nan2(bad)) redo_call(p, n, 2 * q0, FBD, r, 2, c, 2);
 }
 
 constexpr int VH = 16, VW = 128;             // tile: 4 rows of 128 pixels per warp of a group
@@ -407,7 +468,7 @@ struct WideGeo {
   static_assert((KS - 1) * CO * 8 * 128 * 8 <= BYTES, "the groups' sums lie over the stages");
 };
 
-template <int CO, int KS, bool BOX>
+template <int CO, int KS, bool BOX, bool REDO>
 __global__ void __launch_bounds__(WideGeo<CO, KS, BOX>::THREADS, KS == 1 ? 3 : 1)
     ppconv_direct_wide_kernel(const DirectParams p, const __grid_constant__ BoxMap<BOX> xmap) {
   using G = WideGeo<CO, KS, BOX>;
@@ -574,6 +635,13 @@ __global__ void __launch_bounds__(WideGeo<CO, KS, BOX>::THREADS, KS == 1 ? 3 : 1
   const float* skip = (p.flags & PP_ADD_SKIP) ? p.skip : nullptr;
   const int row0 = r0 + 4 * warp, c = c0 + 4 * lane;
   const bool wide = (p.W & 3) == 0;
+  uint64_t bad = 0;  // zero times every sum: NaN once one is not finite
+  if constexpr (REDO) {
+#pragma unroll
+    for (int o = 0; o < CO; ++o)
+#pragma unroll
+      for (int e = 0; e < 8; ++e) bad = fma2(acc[o][e >> 1][e & 1], 0, bad);
+  }
 #pragma unroll
   for (int o = 0; o < CO; ++o) {
     const size_t plane = (size_t)n * p.Co + o;
@@ -613,6 +681,7 @@ __global__ void __launch_bounds__(WideGeo<CO, KS, BOX>::THREADS, KS == 1 ? 3 : 1
       }
     }
   }
+  if (REDO && nan2(bad)) redo(p, n, 0, CO, row0, 4, c, 4);
 }
 
 constexpr int UTHREADS = 128;                // 4 warps
@@ -772,20 +841,31 @@ cudaError_t launch_one(DirectParams p, cudaStream_t stream) {
   if constexpr (CC == 4 && KS <= 2) {
     BoxMap<true> xmap;
     if (p.Ci > CC && ppc::image_map(&xmap.m, p.x, p.N, p.Ci, p.H, p.W, G::COLS, G::ROWS, CC)) {
-      static ppc::DeviceOnce box;
-      return launch_kernel(ppconv_direct_kernel<CC, FBD, KS, true>, box, grid, DTHREADS, G::FLOATS * 4, stream, p, xmap);
+      static ppc::DeviceOnce box, box_redo;
+      return p.redo ? launch_kernel(ppconv_direct_kernel<CC, FBD, KS, true, true>, box_redo, grid, DTHREADS, G::FLOATS * 4,
+                                    stream, p, xmap)
+                    : launch_kernel(ppconv_direct_kernel<CC, FBD, KS, true, false>, box, grid, DTHREADS, G::FLOATS * 4,
+                                    stream, p, xmap);
     }
   }
-  return launch_kernel(ppconv_direct_kernel<CC, FBD, KS, false>, once, grid, DTHREADS, G::FLOATS * 4, stream, p,
+  if constexpr (CC == 4) {  // with fewer channels no other kernel runs a layer by default
+    static ppc::DeviceOnce once_redo;
+    if (p.redo)
+      return launch_kernel(ppconv_direct_kernel<CC, FBD, KS, false, true>, once_redo, grid, DTHREADS, G::FLOATS * 4, stream,
+                           p, BoxMap<false>());
+  }
+  return launch_kernel(ppconv_direct_kernel<CC, FBD, KS, false, false>, once, grid, DTHREADS, G::FLOATS * 4, stream, p,
                        BoxMap<false>());
 }
 
 template <int CO, int KS, bool BOX>
 cudaError_t launch_wide_one(const DirectParams& p, int64_t nt, const BoxMap<BOX>& xmap, cudaStream_t stream) {
   using G = WideGeo<CO, KS, BOX>;
-  static ppc::DeviceOnce once;  // one per instantiation
-  return launch_kernel(ppconv_direct_wide_kernel<CO, KS, BOX>, once, dim3((unsigned)nt), G::THREADS, G::BYTES, stream, p,
-                       xmap);
+  static ppc::DeviceOnce once, once_redo;  // one per instantiation
+  return p.redo ? launch_kernel(ppconv_direct_wide_kernel<CO, KS, BOX, true>, once_redo, dim3((unsigned)nt), G::THREADS,
+                                G::BYTES, stream, p, xmap)
+                : launch_kernel(ppconv_direct_wide_kernel<CO, KS, BOX, false>, once, dim3((unsigned)nt), G::THREADS,
+                                G::BYTES, stream, p, xmap);
 }
 
 template <int CO, int KS>
@@ -829,7 +909,7 @@ bool direct_applicable(int Co, int Ci) {
   return (Ci <= kDirectMaxSmall || Co <= kDirectMaxSmall) && (int64_t)Co * Ci <= (int64_t(1) << 20);
 }
 
-pp_status direct_build(DirectLayout* D, const float* w_dense, const float* bias, int Co, int Ci,
+pp_status direct_build(DirectLayout* D, const float* w_dense, const uint16_t* kept, const float* bias, int Co, int Ci,
                        cudaStream_t stream) {
   // pairs of filters, padded to whole CTAs of FBMAX filters (zero weights)
   const int npair = (Co + FBMAX - 1) / FBMAX * (FBMAX / 2);
@@ -841,6 +921,8 @@ pp_status direct_build(DirectLayout* D, const float* w_dense, const float* bias,
       float* dst = &host[((size_t)i * npair + (o >> 1)) * WPAIR + (o & 1)];
       const float* src = w_dense + ((size_t)o * Ci + i) * 9;
       for (int t = 0; t < 9; ++t) dst[2 * t] = src[t];
+      const uint32_t bits = kept ? kept[(size_t)o * Ci + i] : 0x1ffu;
+      std::memcpy(dst + 18, &bits, 4);
       if (ndup)
         for (int t = 0; t < 18; ++t) host[np + ((size_t)i * Co + o) * WPAIR + t] = src[t >> 1];
     }
@@ -865,6 +947,7 @@ pp_status direct_build(DirectLayout* D, const float* w_dense, const float* bias,
   D->bias = nb ? static_cast<const float*>(d) + nw : nullptr;
   D->wdup = ndup ? static_cast<const float*>(d) + np : nullptr;
   D->npair = npair;
+  D->redo = kept != nullptr;
   D->Co = Co;
   D->Ci = Ci;
   return PP_OK;
@@ -883,6 +966,7 @@ pp_status direct_launch(const DirectLayout& D, const float* x, float* y, const f
   p.bias = D.bias;
   p.wdup = D.wdup;
   p.status = D.status;
+  p.redo = D.redo;
   p.N = N;
   p.Ci = D.Ci;
   p.Co = D.Co;

@@ -156,10 +156,13 @@ struct DirectLayout {
   const float* bias = nullptr;
   const float* wdup = nullptr;  // at most 3 filters
   int* status = nullptr;        // device status word
+  bool redo = false;            // sums that are not finite: again, over the kept taps alone
   int Co = 0, Ci = 0;
 };
 bool direct_applicable(int Co, int Ci);
-pp_status direct_build(DirectLayout* D, const float* w_dense, const float* bias, int Co, int Ci, cudaStream_t stream);
+// kept: [Co][Ci], a bit per kept tap, for layers whose pruned taps must not meet inputs that are not finite; else null
+pp_status direct_build(DirectLayout* D, const float* w_dense, const uint16_t* kept, const float* bias, int Co, int Ci,
+                       cudaStream_t stream);
 pp_status direct_launch(const DirectLayout& D, const float* x, float* y, const float* skip, int N, int H, int W,
                         int flags, cudaStream_t stream);
 void direct_free(DirectLayout* D);

@@ -1203,3 +1203,69 @@ def test_streamed_weight_pairs(pp, runner, oracle_mod, case, flags):
         d.close()
     check_within(outs[0], y, s, f"streamed weights {case} {flags}")
     assert np.array_equal(outs[0], outs[1])
+
+
+# Inputs that are not finite, in layers that run the direct kernels by default (channel groups of 1, 2 and 4, with boxes
+# and without; wide, with 1, 2 and 4 groups of warps): a pruned tap is no part of the sum, whatever value it would meet.
+NONFINITE_SHAPES = [
+    # N, Ci, Co, H, W
+    (1, 17, 16, 260, 1032), (1, 20, 13, 260, 1030), (1, 24, 12, 160, 500), (2, 29, 9, 20, 21), (1, 64, 24, 30, 34),
+    (1, 100, 3, 17, 16), (1, 256, 1, 720, 1284), (1, 256, 1, 300, 1280), (1, 257, 1, 131, 1030), (1, 130, 2, 520, 1284),
+    (1, 91, 3, 300, 700),
+]
+
+
+@pytest.mark.parametrize("shape", NONFINITE_SHAPES)
+@pytest.mark.parametrize("flags", ["none", "skip_relu", "skip_pool_relu"])
+def test_direct_kernel_nonfinite_inputs(pp, runner, oracle_mod, shape, flags):
+    N, Ci, Co, H, W = shape
+    pool = "pool" in flags
+    if pool:
+        H, W = H + H % 2, W + W % 2
+    rng = np.random.default_rng(sum(shape) + len(flags))
+    L = synth.small_random_layer(rng, Co, Ci, P=8, keep=0.4, ring=False)
+    x = rng.uniform(-1, 1, (N, Ci, H, W)).astype(np.float32)
+    at = [(0, 0), (H - 1, W - 1), (H // 2, W // 2), (H // 3, W - 1), (H - 1, W // 3)]
+    for k, (r, c) in enumerate(at):  # the third where filter 0 has a kernel, the others anywhere
+        ch = np.flatnonzero(L.mask[0])[0] if k == 2 else rng.integers(Ci)
+        x[k % N, ch, r, c] = (np.inf, -np.inf, np.nan)[k % 3]
+    skip = rng.uniform(-1, 1, (N, Co, H, W)).astype(np.float32) if "skip" in flags else None
+    d = runner.DeviceLayer(L)
+    assert pp.pp_layer_kernel(d.handle) == pp.PP_KERNEL_DIRECT
+    d.close()
+    g = run_layer(pp, runner, L, x, skip, "relu" in flags, pool)
+    with np.errstate(invalid="ignore"):
+        y, s = oracle_layer_full(oracle_mod, L, x, skip, "relu" in flags, pool)
+        # no value that is not finite under a kept tap (in none of a pooled output's four)
+        finite = np.isfinite(oracle_layer_full(oracle_mod, L, x, skip)[1])
+    if pool:
+        finite = finite.reshape(N, Co, H // 2, 2, W // 2, 2).all(axis=(3, 5))
+    assert finite.any() and not finite.all()
+    check_within(g[finite], y[finite], s[finite], f"direct {shape} {flags}")
+    if flags == "none":
+        assert np.array_equal(np.isnan(g), np.isnan(y)) and np.array_equal(np.isposinf(g), np.isposinf(y))
+        assert np.array_equal(np.isneginf(g), np.isneginf(y))
+
+
+def test_direct_kernel_nonfinite_input_output_order(pp, runner, oracle_mod):
+    """The kept taps move with their filters when the output order changes."""
+    rng = np.random.default_rng(61)
+    L = synth.small_random_layer(rng, 24, 64, P=8, keep=0.4, ring=False)
+    x = rng.uniform(-1, 1, (1, 64, 9, 13)).astype(np.float32)
+    x[0, 7, 4, 5], x[0, 40, 8, 12] = np.inf, np.nan
+    order = rng.permutation(24).astype(np.int32)
+    d = runner.DeviceLayer(L)
+    try:
+        assert pp.pp_layer_kernel(d.handle) == pp.PP_KERNEL_DIRECT
+        pp.pp_layer_set_output_order(d.handle, order, None)
+        out = torch.empty((1, 24, 9, 13), device="cuda")
+        d.forward(dev(x), out, None, 1, 9, 13, 0, torch.cuda.current_stream())
+        torch.cuda.synchronize()
+        g = out.cpu().numpy()[:, order]
+    finally:
+        d.close()
+    with np.errstate(invalid="ignore"):
+        y, s = oracle_layer_full(oracle_mod, L, x)
+    finite = np.isfinite(s)
+    check_within(g[finite], y[finite], s[finite], "direct kernel, inputs not finite, output order")
+    assert np.array_equal(np.isfinite(g), np.isfinite(y))
