@@ -80,7 +80,8 @@ struct DirectParams {
   const float* wdup;  // at most 3 filters: [Ci][Co][20], tap t twice at 2 t, 2 t + 1
   int* status;        // device status word
   int redo;           // sums that are not finite are computed again: see redo
-  int vec;  // x 16-byte aligned and W a multiple of 4: rows staged in 16-byte copies
+  // x 16-byte aligned, W a multiple of 4 and offsets within a channel in 32 bits: rows staged in 16-byte copies
+  int vec;
 };
 
 __device__ __forceinline__ bool nan2(uint64_t v) {
@@ -975,7 +976,7 @@ pp_status direct_launch(const DirectLayout& D, const float* x, float* y, const f
   p.flags = flags;
   p.npair = D.npair;
   p.tiles_x = p.tiles_y = 0;
-  p.vec = (W & 3) == 0 && ((uintptr_t)x & 15) == 0;
+  p.vec = (W & 3) == 0 && ((uintptr_t)x & 15) == 0 && (int64_t)H * W <= INT32_MAX;
   const auto ctas = [&](int th, int tw, int fbd) {
     return (int64_t)N * ((H + th - 1) / th) * ((W + tw - 1) / tw) * ((D.Co + fbd - 1) / fbd);
   };

@@ -1269,3 +1269,27 @@ def test_direct_kernel_nonfinite_input_output_order(pp, runner, oracle_mod):
     finite = np.isfinite(s)
     check_within(g[finite], y[finite], s[finite], "direct kernel, inputs not finite, output order")
     assert np.array_equal(np.isfinite(g), np.isfinite(y))
+
+
+@pytest.mark.parametrize("Co", [1, 8])
+def test_direct_kernel_channel_beyond_32_bit_offsets(pp, Co):
+    """One channel of more than 2^31 pixels, in rows of whole 16-byte groups: its last rows are read where they lie."""
+    H, W, ROWS = 46344, 46344, 20
+    assert H * W > 2 ** 31 and (H - ROWS // 2) * W < 2 ** 31
+    rng = np.random.default_rng(71)
+    w = rng.standard_normal((Co, 1, 9)).astype(np.float32)
+    d = pp.pp_dense_create(w)
+    try:
+        x = torch.zeros((1, 1, H, W), device="cuda")
+        x[:, :, -ROWS:] = torch.rand((ROWS, W), device="cuda") - 0.5
+        y = torch.empty((1, Co, H // 2, W // 2), device="cuda")
+        pp.pp_dense_forward(d, x, y, None, 1, H, W, pp.PP_POOL2, torch.cuda.current_stream())
+        torch.cuda.synchronize()
+        e = torch.nn.functional.conv2d(x[:, :, -ROWS:].double(), torch.from_numpy(w).cuda().double().reshape(Co, 1, 3, 3), padding=1)
+        e = torch.nn.functional.max_pool2d(e, 2)
+        # nine products of |x| <= 0.5, each with a rounding or two: well below 1e-5 of the largest sum
+        bound = 1e-5 * 0.5 * np.abs(w).sum(axis=2).max()
+        assert (y[:, :, -ROWS // 2:].double() - e).abs().max().item() <= bound
+    finally:
+        pp.pp_dense_destroy(d)
+        torch.cuda.empty_cache()
