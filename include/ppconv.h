@@ -263,15 +263,17 @@ pp_status pp_layer_precision(const pp_layer* layer, int* precision, float* input
  *   PP_KERNEL_DIRECT    FP32 FMA over all 9 taps of dense weights (zeros where
  *                       pruned), a block of pixels and up to 8 filters per
  *                       thread; layers with at most 16 input or at most 16
- *                       output channels (first and last layers).
+ *                       output channels (first and last layers), and layers
+ *                       for which PP_KERNEL_AUTO picks it.
  * PP_KERNEL_AUTO picks by an estimate of each kernel's time for the layer's
  * density (the direct kernel for Ci <= 4, and in place of an FMA kernel that it
  * beats, then also with more channels).  Setting a kernel the layer cannot
- * run returns PP_ERR_UNSUPPORTED.  The tensor-core kernels, and
- * the direct kernel on layers that would else run a tensor-core kernel or that
- * have at most 4 input channels, multiply pruned taps as zeros: an input that
- * is not finite then also reaches outputs whose kept taps do not touch it.  The
- * other kernels, and the direct kernel in their place, sum the kept taps alone. */
+ * run returns PP_ERR_UNSUPPORTED; what pp_layer_kernel reports can be set.  The
+ * tensor-core kernels, and the direct kernel on layers that would else run a
+ * tensor-core kernel or that have at most 4 input channels, multiply pruned taps
+ * as zeros: an input that is not finite then also reaches outputs whose kept
+ * taps do not touch it.  The other kernels, and the direct kernel in their
+ * place, sum the kept taps alone. */
 #define PP_KERNEL_AUTO 0
 #define PP_KERNEL_TMEM 1
 #define PP_KERNEL_REGISTER 2

@@ -399,7 +399,6 @@ struct pp_layer {
   ppc::TmLayout tm;
   ppc::TcLayout tc;
   ppc::DirectLayout direct;  // built for layers with few input or output channels and where the default choice is it
-  bool direct_ok = false;    // few input or output channels: pp_layer_set_kernel accepts PP_KERNEL_DIRECT
   int G = 0, nch = 0;
   int64_t nE = 0;
   bool has_bias = false;
@@ -708,10 +707,10 @@ extern "C" pp_status pp_layer_create(const pp_packed* pk, const float* bias, voi
   const bool direct_auto = fma && pairs >= 256 && pairs <= (int64_t(1) << 20);
   // layers with a handful of input channels (a network's first layer) run the
   // direct kernel: the others cannot fill their tiles
-  L->direct_ok = ppc::direct_applicable(pk->Co, pk->Ci);
+  const bool direct_ok = ppc::direct_applicable(pk->Co, pk->Ci);
   const bool redo = direct_auto && pk->Ci > 4;
-  if (direct_auto || (L->direct_ok && pk->Ci <= 4)) L->auto_kernel = PP_KERNEL_DIRECT;
-  if (st == PP_OK && (L->direct_ok || direct_auto)) {
+  if (direct_auto || (direct_ok && pk->Ci <= 4)) L->auto_kernel = PP_KERNEL_DIRECT;
+  if (st == PP_OK && (direct_ok || direct_auto)) {
     // dense [Co][Ci][9] in the original filter order, zeros where pruned
     std::vector<float> wd((size_t)pk->Co * pk->Ci * 9, 0.f);
     // where a kernel over the kept taps alone would be the default, their sums stay free of the pruned taps' inputs
@@ -821,7 +820,7 @@ extern "C" pp_status pp_layer_set_kernel(pp_layer* L, int kernel) {
       return PP_OK;
     case PP_KERNEL_REGISTER: L->kernel = kernel; return PP_OK;
     case PP_KERNEL_DIRECT:
-      if (!L->direct_ok) return PP_ERR_UNSUPPORTED;
+      if (!L->direct.w) return PP_ERR_UNSUPPORTED;
       L->kernel = kernel;
       return PP_OK;
     default: return PP_ERR_INVALID_ARG;

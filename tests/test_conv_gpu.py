@@ -1293,3 +1293,22 @@ def test_direct_kernel_channel_beyond_32_bit_offsets(pp, Co):
     finally:
         pp.pp_dense_destroy(d)
         torch.cuda.empty_cache()
+
+
+@pytest.mark.parametrize("Ci,Co,keep,ring", [(64, 24, 0.3, False), (20, 20, 0.4, False), (64, 24, 0.3, True), (128, 128, 0.4, True)])
+@pytest.mark.parametrize("tune", [False, True])
+def test_reported_kernel_can_be_set(pp, runner, Ci, Co, keep, ring, tune):
+    """A kernel read with pp_layer_kernel, by default or after tuning, is accepted by the same layer built again."""
+    rng = np.random.default_rng(81)
+    L = synth.small_random_layer(rng, Co, Ci, P=8, keep=keep, ring=ring)
+    a, b = runner.DeviceLayer(L), runner.DeviceLayer(L)
+    try:
+        if tune:
+            pp.pp_layer_autotune(a.handle, 1, 20, 24, 0, None)
+        k = pp.pp_layer_kernel(a.handle)
+        pp.pp_layer_set_kernel(b.handle, pp.PP_KERNEL_REGISTER)
+        pp.pp_layer_set_kernel(b.handle, k)
+        assert pp.pp_layer_kernel(b.handle) == k
+    finally:
+        a.close()
+        b.close()
