@@ -264,16 +264,18 @@ pp_status pp_layer_precision(const pp_layer* layer, int* precision, float* input
  *                       pruned), a block of pixels and up to 8 filters per
  *                       thread; layers with at most 16 input or at most 16
  *                       output channels (first and last layers), and layers
- *                       for which PP_KERNEL_AUTO picks it.
+ *                       of 256 to 2^20 (filter, channel) pairs whose density
+ *                       calls for an FMA kernel (up to 32 filters, or not
+ *                       ring patterns).
  * PP_KERNEL_AUTO picks by an estimate of each kernel's time for the layer's
  * density (the direct kernel for Ci <= 4, and in place of an FMA kernel that it
- * beats, then also with more channels).  Setting a kernel the layer cannot
- * run returns PP_ERR_UNSUPPORTED; what pp_layer_kernel reports can be set.  The
- * tensor-core kernels, and the direct kernel on layers that would else run a
- * tensor-core kernel or that have at most 4 input channels, multiply pruned taps
- * as zeros: an input that is not finite then also reaches outputs whose kept
- * taps do not touch it.  The other kernels, and the direct kernel in their
- * place, sum the kept taps alone. */
+ * beats on maps of any size).  Setting a kernel the layer cannot run returns
+ * PP_ERR_UNSUPPORTED; what pp_layer_kernel reports can be set.  The tensor-core
+ * kernels, and the direct kernel on layers of the former kind only (at most 16
+ * channels on a side), multiply pruned taps as zeros: an input that is not
+ * finite then also reaches outputs whose kept taps do not touch it.  The other
+ * kernels, and the direct kernel on layers of the latter kind with more than 4
+ * input channels, sum the kept taps alone. */
 #define PP_KERNEL_AUTO 0
 #define PP_KERNEL_TMEM 1
 #define PP_KERNEL_REGISTER 2

@@ -398,7 +398,7 @@ struct pp_layer {
   int auto_kernel = 2;
   ppc::TmLayout tm;
   ppc::TcLayout tc;
-  ppc::DirectLayout direct;  // built for layers with few input or output channels and where the default choice is it
+  ppc::DirectLayout direct;  // built for layers with few input or output channels and where an FMA kernel is the choice
   int G = 0, nch = 0;
   int64_t nE = 0;
   bool has_bias = false;
@@ -698,19 +698,33 @@ extern "C" pp_status pp_layer_create(const pp_packed* pk, const float* bias, voi
   const double fma_cycles = 4.0 * nk / 32.0;
   L->auto_kernel = (L->tc_ok && tc_cycles < fma_cycles) ? (L->tc.FB == 128 ? PP_KERNEL_TC_FLAT : PP_KERNEL_TC)
                                                          : (L->tm_ok ? PP_KERNEL_TMEM : PP_KERNEL_REGISTER);
-  // Where the estimate wants FP32, the direct kernel's 9 taps on packed FMAs beat the register kernel's dispatch at
-  // any density (64 -> 24 at 128 x 128, keep 0.2 / 0.5 / 0.9: 21 us against 54 / 110 / 181) and the TMEM kernel on
-  // layers that leave its 64-filter CTAs half empty (21 against 21 / 25 / 30; 64 -> 48 keep 0.2: 31 against 25).  Layers
-  // of a few dozen kernels are bound by the launch and keep their choice.
-  const bool fma = L->auto_kernel == PP_KERNEL_REGISTER || (L->auto_kernel == PP_KERNEL_TMEM && pk->Co <= 32);
+  // Where the estimate wants FP32, the direct kernel's 9 taps on packed FMAs are a candidate (its layout is built), and take
+  // the place of
+  //  * the register kernel's dispatch where they are no slower on any map from 7 x 7 to 1080 x 1920.  Their time does not
+  //    depend on the density, the register kernel's does: 64 -> 24 at 128 x 128 21 us against 18 / 26 / 33 / 52 / 105 at
+  //    keep 0.02 / 0.05 / 0.1 / 0.2 / 0.5; more filters need more (64 -> 64 on its worst map, keep 0.1 / 0.12: 1.03 / 0.91
+  //    of the register kernel's time), few entries a channel leave it ahead on small maps (300 -> 1 at 7 x 7, keep 0.3,
+  //    33 us against 25), and from 128 filters on or many channels the middling maps do (97 x 131, keep 0.12: 256 -> 64
+  //    1.06, 96 -> 200 1.07, 512 -> 128 1.48);
+  //  * the TMEM kernel on layers that leave most of its 64-filter CTAs empty: of its time at 720 x 1280, keep 0.1 / 0.15 /
+  //    0.4, 16 -> 16 0.98 / 0.92 / 0.71, 64 -> 16 1.05 / 0.95 / 0.69, 64 -> 24 1.40 / 1.26 / 0.98, 16 -> 32 1.50 / 1.40 /
+  //    1.05; on maps up to 56 x 56 0.1 to 0.8, but 256 -> 16 at 97 x 131 1.7 / 1.6 / 1.2.
+  // Layers of a few dozen kernels are bound by the launch and keep their choice.
   const int64_t pairs = (int64_t)pk->Co * pk->Ci;
-  const bool direct_auto = fma && pairs >= 256 && pairs <= (int64_t(1) << 20);
+  const double keep = nk / (double)pairs;
+  const bool reg = L->auto_kernel == PP_KERNEL_REGISTER;
+  const bool direct_more =
+      (reg || (L->auto_kernel == PP_KERNEL_TMEM && pk->Co <= 32)) && pairs >= 256 && pairs <= (int64_t(1) << 20);
+  const bool direct_auto =
+      direct_more && (reg ? nk >= 1.2 * pk->Ci && (pk->Co <= 32 ? keep >= 0.07 && pk->Ci <= 1024
+                                                                : keep >= 0.12 && pk->Co <= 128 && pk->Ci <= 192)
+                          : pk->Ci <= 96 && (pk->Co <= 16 ? keep >= 0.18 : pk->Co <= 24 && keep >= 0.4));
   // layers with a handful of input channels (a network's first layer) run the
   // direct kernel: the others cannot fill their tiles
   const bool direct_ok = ppc::direct_applicable(pk->Co, pk->Ci);
-  const bool redo = direct_auto && pk->Ci > 4;
+  const bool redo = direct_more && pk->Ci > 4;
   if (direct_auto || (direct_ok && pk->Ci <= 4)) L->auto_kernel = PP_KERNEL_DIRECT;
-  if (st == PP_OK && (direct_ok || direct_auto)) {
+  if (st == PP_OK && (direct_ok || direct_more)) {
     // dense [Co][Ci][9] in the original filter order, zeros where pruned
     std::vector<float> wd((size_t)pk->Co * pk->Ci * 9, 0.f);
     // where a kernel over the kept taps alone would be the default, their sums stay free of the pruned taps' inputs

@@ -93,8 +93,8 @@ __device__ __forceinline__ bool nan2(uint64_t v) {
 // A pruned tap is no part of the sum, but the kernels multiply it as a zero weight, and zero times an infinity or a NaN is
 // not zero.  Every such product makes its output NaN.  In the instantiations with REDO a thread that meets a sum which is
 // not finite computes its block of outputs (filters o0 .., rows r0 .., columns c0 ..) again over the kept taps alone,
-// straight from x, after its stores.  Layers that run these kernels by default where a kernel over kept taps alone would
-// else run them take those: within 2 % of the others' time in the wide kernel (256 -> 1 at 720 x 1280 150.7 -> 153.4 us),
+// straight from x, after its stores.  Layers whose choice without these kernels would be one over the kept taps alone take
+// those: within 2 % of the others' time in the wide kernel (256 -> 1 at 720 x 1280 150.7 -> 153.4 us),
 // at it in the 2 x 2 kernel (64 -> 16 at 224 x 224 31.1 -> 30.8).
 __device__ __forceinline__ void redo(const DirectParams& p, int n, int o0, int no, int r0, int nr, int c0, int nc) {
   const size_t plane = (size_t)p.H * p.W;

@@ -1205,13 +1205,13 @@ def test_streamed_weight_pairs(pp, runner, oracle_mod, case, flags):
     assert np.array_equal(outs[0], outs[1])
 
 
-# Inputs that are not finite, in layers that run the direct kernels by default (channel groups of 1, 2 and 4, with boxes
+# Inputs that are not finite, in layers whose FMA kernel may be the direct one (channel groups of 1, 2 and 4, with boxes
 # and without; wide, with 1, 2 and 4 groups of warps): a pruned tap is no part of the sum, whatever value it would meet.
 NONFINITE_SHAPES = [
     # N, Ci, Co, H, W
     (1, 17, 16, 260, 1032), (1, 20, 13, 260, 1030), (1, 24, 12, 160, 500), (2, 29, 9, 20, 21), (1, 64, 24, 30, 34),
     (1, 100, 3, 17, 16), (1, 256, 1, 720, 1284), (1, 256, 1, 300, 1280), (1, 257, 1, 131, 1030), (1, 130, 2, 520, 1284),
-    (1, 91, 3, 300, 700),
+    (1, 91, 3, 300, 700), (1, 89, 3, 420, 1283),
 ]
 
 
@@ -1230,10 +1230,7 @@ def test_direct_kernel_nonfinite_inputs(pp, runner, oracle_mod, shape, flags):
         ch = np.flatnonzero(L.mask[0])[0] if k == 2 else rng.integers(Ci)
         x[k % N, ch, r, c] = (np.inf, -np.inf, np.nan)[k % 3]
     skip = rng.uniform(-1, 1, (N, Co, H, W)).astype(np.float32) if "skip" in flags else None
-    d = runner.DeviceLayer(L)
-    assert pp.pp_layer_kernel(d.handle) == pp.PP_KERNEL_DIRECT
-    d.close()
-    g = run_layer(pp, runner, L, x, skip, "relu" in flags, pool)
+    g = run_layer(pp, runner, L, x, skip, "relu" in flags, pool, kernel=pp.PP_KERNEL_DIRECT)
     with np.errstate(invalid="ignore"):
         y, s = oracle_layer_full(oracle_mod, L, x, skip, "relu" in flags, pool)
         # no value that is not finite under a kept tap (in none of a pooled output's four)
@@ -1312,3 +1309,21 @@ def test_reported_kernel_can_be_set(pp, runner, Ci, Co, keep, ring, tune):
     finally:
         a.close()
         b.close()
+
+
+@pytest.mark.parametrize("Ci,Co,keep,ring,direct", [
+    (64, 24, 0.08, False, True), (64, 24, 0.06, False, False), (64, 64, 0.13, False, True), (64, 64, 0.11, False, False),
+    (300, 2, 0.5, False, False), (300, 2, 0.7, False, True), (256, 64, 0.15, False, False), (100, 130, 0.15, False, False),
+    (32, 16, 0.2, True, True), (32, 16, 0.15, True, False), (64, 20, 0.45, True, True), (64, 20, 0.3, True, False),
+    (32, 32, 0.3, True, False), (256, 16, 0.5, True, False),
+])
+def test_default_direct_kernel_by_density(pp, runner, Ci, Co, keep, ring, direct):
+    """The direct kernel is a layer's default in place of an FMA kernel over the kept taps only from the density on where
+    it is no slower."""
+    rng = np.random.default_rng(91)
+    d = runner.DeviceLayer(synth.small_random_layer(rng, Co, Ci, P=8, keep=keep, ring=ring))
+    try:
+        other = pp.PP_KERNEL_TMEM if ring else pp.PP_KERNEL_REGISTER
+        assert pp.pp_layer_kernel(d.handle) == (pp.PP_KERNEL_DIRECT if direct else other)
+    finally:
+        d.close()
