@@ -293,9 +293,13 @@ pp_status pp_layer_kernel(const pp_layer* layer, int* kernel);
  * keeps the winning one for launches of this shape.  The kernels differ in speed by layer shape:
  * the tensor-core kernel needs many output tiles to fill the GPU, the FMA
  * kernels split small layers across thread-block clusters.  Allocates and
- * frees scratch device memory, and for a tf32 layer of more than 64 filters on
- * a map at least 96 wide keeps a second copy of its weight tiles with the layer
- * (pp_layer_info counts it); must not be called during stream capture.
+ * frees scratch device memory.  A tf32 layer of more than 64 filters tuned
+ * without pooling on a map at least 96 wide, and for which PP_KERNEL_TC wins,
+ * keeps a second copy of its weight tiles (pp_layer_info counts it), with which
+ * PP_KERNEL_TC streams weights to CTA pairs on every map at least 96 wide that
+ * is not pooled; without it (a layer as loaded, or a stored choice set with
+ * pp_layer_set_kernel) the same layer runs the slower row-tiled form.  Must not
+ * be called during stream capture.
  * Errors: PP_ERR_INVALID_ARG, PP_ERR_UNSUPPORTED, PP_ERR_CUDA, PP_ERR_OOM. */
 pp_status pp_layer_autotune(pp_layer* layer, int N, int H, int W, int flags, void* stream);
 

@@ -867,9 +867,19 @@ extern "C" pp_status pp_layer_autotune(pp_layer* L, int N, int H, int W, int fla
   if (L->tm_ok) cand.push_back({PP_KERNEL_TMEM, 0, 0});
   if (L->direct.w) cand.push_back({PP_KERNEL_DIRECT, 0, 0});
   if (cand.empty()) cand.push_back({PP_KERNEL_REGISTER, 0, 0});
+  // Wide maps of 128-filter tf32 blocks: the row-tiled kernel's place is taken by the one that streams weights to CTA
+  // pairs, which needs its own copy of the weight tiles (without memory for it the row-tiled kernel runs).  A copy made
+  // here is kept if the choice uses it: a captured graph may then, too.
+  const bool had_pairs = L->tc_ok && L->tc.ap;
+  const auto make_pairs = [&]() -> pp_status {
+    if (!L->tc_ok || L->tc.FB != 128 || L->tc.f16 || (flags & PP_POOL2) || W < 96) return PP_OK;
+    const pp_status e = ppc::tcr_pair_layout(&L->tc, stream);
+    return e == PP_ERR_OOM ? PP_OK : e;
+  };
   if (cand.size() == 1) {
-    L->kernel = cand[0].kernel;
-    return PP_OK;
+    const pp_status e = cand[0].kernel == PP_KERNEL_TC ? make_pairs() : PP_OK;
+    if (e == PP_OK) L->kernel = cand[0].kernel;
+    return e;
   }
   const size_t in_elems = (size_t)N * L->Ci * H * W, out_elems = (size_t)N * L->Co * H * W;
   float *x = nullptr, *y = nullptr, *sk = nullptr;
@@ -880,13 +890,9 @@ extern "C" pp_status pp_layer_autotune(pp_layer* L, int N, int H, int W, int fla
     cudaFree(y);
     return PP_ERR_OOM;
   }
-  // Wide maps of 128-filter tf32 blocks: the row-tiled kernel's place is taken by the one that streams weights to CTA
-  // pairs, which needs its own copy of the weight tiles (built once, kept: a captured graph may use it from now on;
-  // without memory for it the row-tiled kernel runs).
-  if (L->tc_ok && L->tc.FB == 128 && !L->tc.f16 && !(flags & PP_POOL2) && W >= 96) ppc::tcr_pair_layout(&L->tc, stream);
-  pp_status st = PP_OK;
-  if (cudaMemsetAsync(x, 0, in_elems * 4, stream) != cudaSuccess ||
-      (sk && cudaMemsetAsync(sk, 0, out_elems * 4, stream) != cudaSuccess))
+  pp_status st = make_pairs();
+  if (st == PP_OK && (cudaMemsetAsync(x, 0, in_elems * 4, stream) != cudaSuccess ||
+                      (sk && cudaMemsetAsync(sk, 0, out_elems * 4, stream) != cudaSuccess)))
     st = PP_ERR_CUDA;
   cudaEvent_t e0 = nullptr, e1 = nullptr;
   if (st == PP_OK && (cudaEventCreate(&e0) != cudaSuccess || cudaEventCreate(&e1) != cudaSuccess)) st = PP_ERR_CUDA;
@@ -931,6 +937,7 @@ extern "C" pp_status pp_layer_autotune(pp_layer* L, int N, int H, int W, int fla
   if (e0) cudaEventDestroy(e0);
   if (e1) cudaEventDestroy(e1);
   cudaStreamSynchronize(stream);
+  if (!had_pairs && (st != PP_OK || best.kernel != PP_KERNEL_TC)) ppc::tcr_pair_free(&L->tc);
   cudaFree(x);
   cudaFree(y);
   cudaFree(sk);

@@ -6,6 +6,9 @@ including all 48 sweep points and the multi-tile repeatability shapes.  Bound:
 |gpu - oracle| <= 1e-5 * S per output (see tests/parity.py); integer-valued
 cases must be bit-exact.
 """
+import re
+import warnings
+
 import numpy as np
 import pytest
 import torch
@@ -51,6 +54,19 @@ def run_layer(pp, runner, layer, x, skip=None, relu=False, pool=False, kernel=No
         return y.cpu().numpy()
     finally:
         L.close()
+
+
+def launched(call, tmp_path):
+    """The mangled names of the kernels that call() launches on the current stream, from a captured graph's dump."""
+    g = torch.cuda.CUDAGraph(keep_graph=True)
+    g.enable_debug_mode()
+    with torch.cuda.graph(g):
+        call()
+    dot = tmp_path / "graph.dot"
+    with warnings.catch_warnings():
+        warnings.simplefilter("ignore")
+        g.debug_dump(str(dot))
+    return re.findall(r"ppconv_\w+", dot.read_text())
 
 
 SMALL = [
@@ -1170,19 +1186,19 @@ def test_direct_kernels_dense(pp, runner, oracle_mod, shape, flags):
 STREAM_CASES = [
     # N, Ci, Co, H, W
     (1, 65, 64, 3, 130), (2, 72, 9, 5, 63), (1, 200, 40, 10, 28), (3, 100, 33, 40, 129), (1, 80, 64, 330, 257),
-    (1, 8, 65, 2, 96), (1, 9, 128, 3, 129), (2, 24, 131, 7, 128), (1, 40, 260, 33, 200), (3, 16, 130, 130, 140),
+    (1, 17, 65, 2, 96), (1, 18, 128, 3, 129), (2, 24, 131, 7, 128), (1, 40, 260, 33, 200), (3, 20, 130, 130, 140),
 ]
 
 
 @pytest.mark.parametrize("case", STREAM_CASES)
 @pytest.mark.parametrize("flags", ["none", "skip_relu", "skip_pool_relu"])
-def test_streamed_weight_pairs(pp, runner, oracle_mod, case, flags):
+def test_streamed_weight_pairs(pp, runner, oracle_mod, tmp_path, case, flags):
     N, Ci, Co, H, W = case
     pool = "pool" in flags
     if pool:
         H, W = H + H % 2, W + W % 2
     rng = np.random.default_rng(sum(case) + len(flags))
-    L = synth.small_random_layer(rng, Co, Ci, P=8, keep=0.5)
+    L = synth.small_random_layer(rng, Co, Ci, P=8, keep=0.5, ring=False)
     x = rng.uniform(-1, 1, (N, Ci, H, W)).astype(np.float32)
     skip = rng.uniform(-1, 1, (N, Co, H, W)).astype(np.float32) if "skip" in flags else None
     fl = (pp.PP_ADD_SKIP if skip is not None else 0) | (pp.PP_RELU if "relu" in flags else 0) | (pp.PP_POOL2 if pool else 0)
@@ -1190,8 +1206,12 @@ def test_streamed_weight_pairs(pp, runner, oracle_mod, case, flags):
     d = runner.DeviceLayer(L)
     try:
         st = torch.cuda.current_stream()
-        pp.pp_layer_autotune(d.handle, N, H, W, fl, st)
+        pp.pp_layer_autotune(d.handle, 1, 4, 160, 0, st)  # the flat kernel cannot run it: the weight copy is made
         pp.pp_layer_set_kernel(d.handle, pp.PP_KERNEL_TC)
+        xd, sd, g = dev(x), None if skip is None else dev(skip), torch.empty(y.shape, device="cuda")
+        names = launched(lambda: d.forward(xd, g, sd, N, H, W, fl, torch.cuda.current_stream()), tmp_path)
+        # pooled 128-filter layers are the row-tiled kernel's
+        assert len(names) == 1 and ("ppconv_tcr_kernel" in names[0]) == (Co <= 64 or not pool)
         outs = []
         for _ in range(2):
             g = torch.full(y.shape, float("nan"), device="cuda")
@@ -1325,5 +1345,51 @@ def test_default_direct_kernel_by_density(pp, runner, Ci, Co, keep, ring, direct
     try:
         other = pp.PP_KERNEL_TMEM if ring else pp.PP_KERNEL_REGISTER
         assert pp.pp_layer_kernel(d.handle) == (pp.PP_KERNEL_DIRECT if direct else other)
+    finally:
+        d.close()
+
+
+def pair_copy_bytes(Co, Ci):
+    """The second copy of a 128-filter tf32 layer's weight tiles: 9 taps, hi and lo, 8 channels a chunk."""
+    return (Co + 127) // 128 * ((Ci + 7) // 8) * 9 * 2 * 128 * 8 * 4
+
+
+@pytest.mark.parametrize("N,Ci,Co,H,W", [(1, 24, 130, 6, 140), (2, 72, 256, 120, 160)])
+def test_autotune_single_candidate_gets_pair_copy(pp, runner, oracle_mod, tmp_path, N, Ci, Co, H, W):
+    """A tf32 layer of more than 64 filters whose only candidate is PP_KERNEL_TC (no ring patterns, a map wider than the
+    flat kernel's) runs the kernel on CTA pairs once it is tuned."""
+    rng = np.random.default_rng(101)
+    L = synth.small_random_layer(rng, Co, Ci, P=8, keep=0.5, ring=False)
+    x = rng.uniform(-1, 1, (N, Ci, H, W)).astype(np.float32)
+    d = runner.DeviceLayer(L)
+    try:
+        before = pp.pp_layer_info(d.handle)[2]
+        pp.pp_layer_autotune(d.handle, N, H, W, 0, None)
+        assert pp.pp_layer_kernel(d.handle) == pp.PP_KERNEL_TC
+        assert pp.pp_layer_info(d.handle)[2] - before == pair_copy_bytes(Co, Ci)
+        xd, out = dev(x), torch.empty((N, Co, H, W), device="cuda")
+        names = launched(lambda: d.forward(xd, out, None, N, H, W, 0, torch.cuda.current_stream()), tmp_path)
+        assert len(names) == 1 and "ppconv_tcr_kernel" in names[0]
+        d.forward(xd, out, None, N, H, W, 0, torch.cuda.current_stream())
+        torch.cuda.synchronize()
+        assert pp.pp_layer_device_status(d.handle) == 0
+    finally:
+        d.close()
+    y, s = oracle_layer_full(oracle_mod, L, x)
+    check_within(out.cpu().numpy(), y, s, "tuned layer with a single candidate")
+
+
+@pytest.mark.parametrize("N,Ci,Co,H,W", [(1, 128, 128, 8, 100), (1, 512, 256, 4, 96), (1, 128, 128, 128, 128), (4, 64, 200, 60, 120)])
+def test_autotune_keeps_pair_copy_only_if_used(pp, runner, N, Ci, Co, H, W):
+    rng = np.random.default_rng(103)
+    d = runner.DeviceLayer(synth.small_random_layer(rng, Co, Ci, P=8, keep=0.5))
+    try:
+        before = pp.pp_layer_info(d.handle)[2]
+        pp.pp_layer_autotune(d.handle, N, H, W, 0, None)
+        kept = pp.pp_layer_info(d.handle)[2] - before
+        assert kept == (pair_copy_bytes(Co, Ci) if pp.pp_layer_kernel(d.handle) == pp.PP_KERNEL_TC else 0)
+        if kept:  # another shape's tuning leaves it, whatever wins there
+            pp.pp_layer_autotune(d.handle, 1, 4, 96, 0, None)
+            assert pp.pp_layer_info(d.handle)[2] - before == kept
     finally:
         d.close()
