@@ -201,10 +201,11 @@ pp_status pp_conv_forward_noalloc(const pp_layer* layer, const float* x, float* 
  * j, so the epilogue writes the filters in the order they are computed), and
  * pack layer k + 1 from weights whose input channels were permuted the same
  * way (pp_permute_input_channels with layout = perm_k).
- * Synchronous on stream (uploads Co indices; layers with a direct-kernel
- * layout also rebuild it).  A CUDA graph captured earlier keeps the direct
- * kernel's old weights: re-capture after calling this (pp_net_use_graph).
- * Errors: PP_ERR_INVALID_ARG (not a permutation), PP_ERR_CUDA, PP_ERR_OOM. */
+ * Synchronous on stream (uploads Co indices, and for layers with a
+ * direct-kernel layout its weights, into the memory that they have): no launch
+ * of the layer may be in flight on another stream.  A CUDA graph captured
+ * earlier stores in the new order from then on.
+ * Errors: PP_ERR_INVALID_ARG (not a permutation), PP_ERR_CUDA. */
 pp_status pp_layer_set_output_order(pp_layer* layer, const int32_t* order, void* stream);
 
 /*

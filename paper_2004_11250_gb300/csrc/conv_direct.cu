@@ -910,13 +910,12 @@ bool direct_applicable(int Co, int Ci) {
   return (Ci <= kDirectMaxSmall || Co <= kDirectMaxSmall) && (int64_t)Co * Ci <= (int64_t(1) << 20);
 }
 
-pp_status direct_build(DirectLayout* D, const float* w_dense, const uint16_t* kept, const float* bias, int Co, int Ci,
-                       cudaStream_t stream) {
-  // pairs of filters, padded to whole CTAs of FBMAX filters (zero weights)
-  const int npair = (Co + FBMAX - 1) / FBMAX * (FBMAX / 2);
-  const size_t ndup = Co <= 3 ? (size_t)Ci * Co * WPAIR : 0;  // the wide kernel's weights, each twice
-  const size_t np = (size_t)Ci * npair * WPAIR, nw = np + ndup, nb = bias ? (size_t)Co : 0;
-  std::vector<float> host(nw, 0.f);
+// Weights (npair pairs of filters, padded to whole CTAs of FBMAX filters with zeros), the wide kernel's (each twice), bias.
+static std::vector<float> direct_host(const float* w_dense, const uint16_t* kept, const float* bias, int Co, int Ci,
+                                      int npair) {
+  const size_t ndup = Co <= 3 ? (size_t)Ci * Co * WPAIR : 0;
+  const size_t np = (size_t)Ci * npair * WPAIR, nw = np + ndup;
+  std::vector<float> host(nw + (bias ? Co : 0), 0.f);
   for (int o = 0; o < Co; ++o)
     for (int i = 0; i < Ci; ++i) {
       float* dst = &host[((size_t)i * npair + (o >> 1)) * WPAIR + (o & 1)];
@@ -927,30 +926,47 @@ pp_status direct_build(DirectLayout* D, const float* w_dense, const uint16_t* ke
       if (ndup)
         for (int t = 0; t < 18; ++t) host[np + ((size_t)i * Co + o) * WPAIR + t] = src[t >> 1];
     }
+  if (bias) std::copy_n(bias, Co, &host[nw]);
+  return host;
+}
+
+pp_status direct_build(DirectLayout* D, const float* w_dense, const uint16_t* kept, const float* bias, int Co, int Ci,
+                       cudaStream_t stream) {
+  const int npair = (Co + FBMAX - 1) / FBMAX * (FBMAX / 2);
+  const std::vector<float> host = direct_host(w_dense, kept, bias, Co, Ci, npair);
   void* d = nullptr;
-  if (cudaMalloc(&d, (nw + nb + 1) * 4) != cudaSuccess) {
+  if (cudaMalloc(&d, (host.size() + 1) * 4) != cudaSuccess) {
     cudaGetLastError();
     return PP_ERR_OOM;
   }
-  int* status = reinterpret_cast<int*>(static_cast<float*>(d) + nw + nb);
+  int* status = reinterpret_cast<int*>(static_cast<float*>(d) + host.size());
   if (cudaMemsetAsync(status, 0, sizeof(int), stream) != cudaSuccess ||
-      cudaMemcpyAsync(d, host.data(), nw * 4, cudaMemcpyHostToDevice, stream) != cudaSuccess ||
-      (nb && cudaMemcpyAsync(static_cast<float*>(d) + nw, bias, nb * 4, cudaMemcpyHostToDevice, stream) !=
-                 cudaSuccess) ||
+      cudaMemcpyAsync(d, host.data(), host.size() * 4, cudaMemcpyHostToDevice, stream) != cudaSuccess ||
       cudaStreamSynchronize(stream) != cudaSuccess) {
     cudaFree(d);
     return PP_ERR_CUDA;
   }
   D->dmem = d;
-  D->dbytes = (nw + nb + 1) * 4;
+  D->dbytes = (host.size() + 1) * 4;
   D->status = status;
   D->w = static_cast<const float*>(d);
-  D->bias = nb ? static_cast<const float*>(d) + nw : nullptr;
-  D->wdup = ndup ? static_cast<const float*>(d) + np : nullptr;
+  D->bias = bias ? static_cast<const float*>(d) + host.size() - Co : nullptr;
+  D->wdup = Co <= 3 ? static_cast<const float*>(d) + (size_t)Ci * npair * WPAIR : nullptr;
   D->npair = npair;
   D->redo = kept != nullptr;
   D->Co = Co;
   D->Ci = Ci;
+  return PP_OK;
+}
+
+pp_status direct_update(const DirectLayout& D, const float* w_dense, const uint16_t* kept, const float* bias,
+                        cudaStream_t stream) {
+  const std::vector<float> host = direct_host(w_dense, kept, bias, D.Co, D.Ci, D.npair);
+  if (cudaMemcpyAsync(D.dmem, host.data(), host.size() * 4, cudaMemcpyHostToDevice, stream) != cudaSuccess ||
+      cudaStreamSynchronize(stream) != cudaSuccess) {
+    cudaGetLastError();
+    return PP_ERR_CUDA;
+  }
   return PP_OK;
 }
 

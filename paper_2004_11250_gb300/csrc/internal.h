@@ -163,6 +163,9 @@ bool direct_applicable(int Co, int Ci);
 // kept: [Co][Ci], a bit per kept tap, for layers whose pruned taps must not meet inputs that are not finite; else null
 pp_status direct_build(DirectLayout* D, const float* w_dense, const uint16_t* kept, const float* bias, int Co, int Ci,
                        cudaStream_t stream);
+// Other weights and bias for the same layout (kept and bias null as when it was built), in the same device memory.
+pp_status direct_update(const DirectLayout& D, const float* w_dense, const uint16_t* kept, const float* bias,
+                        cudaStream_t stream);
 pp_status direct_launch(const DirectLayout& D, const float* x, float* y, const float* skip, int N, int H, int W,
                         int flags, cudaStream_t stream);
 void direct_free(DirectLayout* D);

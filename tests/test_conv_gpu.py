@@ -1393,3 +1393,30 @@ def test_autotune_keeps_pair_copy_only_if_used(pp, runner, N, Ci, Co, H, W):
             assert pp.pp_layer_info(d.handle)[2] - before == kept
     finally:
         d.close()
+
+
+@pytest.mark.parametrize("Ci,Co", [(64, 24), (8, 3), (3, 64), (64, 100)])
+def test_captured_graph_follows_output_order(pp, runner, oracle_mod, Ci, Co):
+    """The output order is changed where the layer's kernels read it, so a graph captured before stores in the new order
+    (and never reads memory that was given back)."""
+    rng = np.random.default_rng(111)
+    L = synth.small_random_layer(rng, Co, Ci, P=8, keep=0.5, ring=False)
+    x = rng.uniform(-1, 1, (1, Ci, 20, 70)).astype(np.float32)
+    y, s = oracle_layer_full(oracle_mod, L, x)
+    d = runner.DeviceLayer(L)
+    try:
+        xd, out = dev(x), torch.empty((1, Co, 20, 70), device="cuda")
+        g = torch.cuda.CUDAGraph()
+        with torch.cuda.graph(g):
+            d.forward(xd, out, None, 1, 20, 70, 0, torch.cuda.current_stream())
+        bytes_before = pp.pp_layer_info(d.handle)[2]
+        for order in (rng.permutation(Co).astype(np.int32), None):
+            pp.pp_layer_set_output_order(d.handle, order, None)
+            out.fill_(float("nan"))
+            g.replay()
+            torch.cuda.synchronize()
+            o = out.cpu().numpy()
+            check_within(o if order is None else o[:, order], y, s, "graph captured before the order changed")
+        assert pp.pp_layer_info(d.handle)[2] == bytes_before
+    finally:
+        d.close()
