@@ -723,6 +723,7 @@ extern "C" pp_status pp_layer_create(const pp_packed* pk, const float* bias, voi
   // direct kernel: the others cannot fill their tiles
   const bool direct_ok = ppc::direct_applicable(pk->Co, pk->Ci);
   const bool redo = direct_more && pk->Ci > 4;
+  const int fma_kernel = L->auto_kernel;
   if (direct_auto || (direct_ok && pk->Ci <= 4)) L->auto_kernel = PP_KERNEL_DIRECT;
   if (st == PP_OK && (direct_ok || direct_more)) {
     // dense [Co][Ci][9] in the original filter order, zeros where pruned
@@ -737,9 +738,14 @@ extern "C" pp_status pp_layer_create(const pp_packed* pk, const float* bias, voi
         for (int s = 0; s < 4; ++s) wd[k * 9 + t[s]] = pk->kw[(size_t)e * 4 + s];
       }
     st = ppc::direct_build(&L->direct, wd.data(), redo ? kept.data() : nullptr, bias, pk->Co, pk->Ci, (cudaStream_t)stream);
-    L->direct_w.swap(wd);
-    L->direct_kept.swap(kept);
-    if (bias) L->direct_bias.assign(bias, bias + pk->Co);
+    if (st == PP_OK) {
+      L->direct_w.swap(wd);
+      L->direct_kept.swap(kept);
+      if (bias) L->direct_bias.assign(bias, bias + pk->Co);
+    } else if (st == PP_ERR_OOM && !direct_ok) {  // without memory for it the other FMA kernel runs
+      L->auto_kernel = fma_kernel;
+      st = PP_OK;
+    }
   }
   if (st != PP_OK) {
     pp_layer_destroy(L);

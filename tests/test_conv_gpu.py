@@ -6,7 +6,11 @@ including all 48 sweep points and the multi-tile repeatability shapes.  Bound:
 |gpu - oracle| <= 1e-5 * S per output (see tests/parity.py); integer-valued
 cases must be bit-exact.
 """
+import json
+import os
 import re
+import subprocess
+import sys
 import warnings
 
 import numpy as np
@@ -1420,3 +1424,71 @@ def test_captured_graph_follows_output_order(pp, runner, oracle_mod, Ci, Co):
         assert pp.pp_layer_info(d.handle)[2] == bytes_before
     finally:
         d.close()
+
+
+# A layer where one device allocation fails: a preloaded cudaMalloc answers cudaErrorMemoryAllocation for one size, and a
+# child process prints the kernel that the layer picks, the one that a call launches, and the call's output.
+OOM_MALLOC = r"""
+#include <dlfcn.h>
+#include <stdlib.h>
+int cudaMalloc(void** p, size_t n) {
+  const char* s = getenv("PP_TEST_NO_MEMORY_FOR");
+  if (s && (size_t)atoll(s) == n) return 2;
+  return ((int (*)(void**, size_t))dlsym(dlopen("libcudart.so.13", RTLD_LAZY), "cudaMalloc"))(p, n);
+}
+"""
+
+OOM_CHILD = r"""
+import json, os, pathlib, sys
+sys.path[:0] = sys.argv[1:3]
+import numpy as np, torch
+import test_conv_gpu as t
+from paper_2004_11250_gb300 import ppconv as pp, runner, synth
+N, Ci, Co, H, W, kernel, nbytes, where = json.loads(sys.argv[3])
+L = synth.small_random_layer(np.random.default_rng(7), Co, Ci, P=8, keep=0.4, ring=False)
+x = np.random.default_rng(8).uniform(-1, 1, (N, Ci, H, W)).astype(np.float32)
+os.environ["PP_TEST_NO_MEMORY_FOR"] = str(nbytes)
+d = runner.DeviceLayer(L)
+picked = pp.pp_layer_kernel(d.handle)
+if kernel:
+    pp.pp_layer_set_kernel(d.handle, kernel)
+xd, y = t.dev(x), torch.full((N, Co, H, W), float("nan"), device="cuda")
+call = lambda: d.forward(xd, y, None, N, H, W, 0, torch.cuda.current_stream())
+names = t.launched(call, pathlib.Path(where))
+call()
+torch.cuda.synchronize()
+assert pp.pp_layer_device_status(d.handle) == 0
+np.save(os.path.join(where, "y.npy"), y.cpu().numpy())
+d.close()
+print(json.dumps([picked, names]))
+"""
+
+
+def pair_copy_bytes_64(Ci):
+    return (Ci + 7) // 8 * 9 * 2 * 64 * 8 * 4
+
+
+@pytest.mark.parametrize("case,kernel,nbytes,picked,launches", [
+    # no memory for the direct kernel's weights: the register kernel runs, as it would without a direct kernel
+    ((1, 64, 24, 20, 30), 0, (64 * 12 * 20 + 24 + 1) * 4, 2, "ppconv_kernel"),
+    # no memory for the pairs' weight copy of 64 filters: the row-tiled kernel, in tiles of 128 columns
+    ((1, 72, 64, 5, 130), 3, pair_copy_bytes_64(72), 3, "ppconv_tc_kernelILi1ELi128ELi64ELb0E"),
+    ((2, 100, 40, 7, 257), 3, pair_copy_bytes_64(100), 3, "ppconv_tc_kernelILi1ELi128ELi64ELb0E"),
+])
+def test_no_memory_for_optional_layouts(pp, oracle_mod, tmp_path, case, kernel, nbytes, picked, launches):
+    N, Ci, Co, H, W = case
+    src, so = tmp_path / "m.c", tmp_path / "m.so"
+    src.write_text(OOM_MALLOC)
+    subprocess.run(["gcc", "-shared", "-fPIC", "-o", str(so), str(src), "-ldl"], check=True)
+    here = os.path.dirname(os.path.abspath(__file__))
+    r = subprocess.run([sys.executable, "-c", OOM_CHILD, os.path.dirname(here), here,
+                        json.dumps([N, Ci, Co, H, W, kernel, nbytes, str(tmp_path)])],
+                       env=dict(os.environ, LD_PRELOAD=str(so)), capture_output=True, text=True, timeout=300)
+    assert r.returncode == 0, r.stderr[-2000:]
+    got, names = json.loads(r.stdout.splitlines()[-1])
+    assert got == picked or kernel
+    assert len(names) == 1 and launches in names[0]
+    L = synth.small_random_layer(np.random.default_rng(7), Co, Ci, P=8, keep=0.4, ring=False)
+    x = np.random.default_rng(8).uniform(-1, 1, (N, Ci, H, W)).astype(np.float32)
+    y, s = oracle_layer_full(oracle_mod, L, x)
+    check_within(np.load(tmp_path / "y.npy"), y, s, f"no memory for {nbytes} bytes")
