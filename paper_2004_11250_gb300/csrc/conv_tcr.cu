@@ -175,6 +175,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(NTHREADS, 1) ppconv_
   // loaders wait for too); acc_empty (even CTA): both CTAs' epilogues have read it
   __shared__ __align__(8) uint64_t full[NRING], empty[NRING], acc_full[NSLOT], acc_empty[NSLOT], done_bar;
   __shared__ __align__(8) uint64_t wfull[NRING];  // STREAM, odd CTA: its weights of a stage have landed
+  __shared__ volatile int wuse[NRING];            // STREAM: last use of a stage for which this CTA's copy was issued, or -1
   __shared__ uint32_t tmem_s;
   // per filter: output channel x plane size of y and of skip (0 past the last filter), bias, inverse scale
   // (64 filters; 128-filter layers may have several blocks and read them from memory)
@@ -204,6 +205,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(NTHREADS, 1) ppconv_
       mbar_init(su32(&full[s]), 2 * units + (STREAM ? 2 : 0));
       mbar_init(su32(&empty[s]), NISS);
       mbar_init(su32(&wfull[s]), 1);
+      wuse[s] = -1;
     }
     for (int s = 0; s < NSLOT; ++s) {
       mbar_init(su32(&acc_full[s]), F16 ? 2 : 1);
@@ -404,6 +406,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(NTHREADS, 1) ppconv_
         if (!__all_sync(0xffffffffu, uu == 0 || wait(&empty[su], (uint32_t)((uu - 1) & 1)))) break;
         if (STREAM && head && lane == 0) {  // the warp with a stage's first unit copies its weights
           uint64_t* bar = rank == 0 ? &full[su] : &wfull[su];
+          wuse[su] = uu;
           mbar_arrive_expect_tx(su32(bar), W_CHUNK);
           asm volatile(
               "cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(
@@ -665,9 +668,6 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(NTHREADS, 1) ppconv_
     }
   }
 
-  // after a wait that gave up, weight copies may still be in flight: a millisecond outlasts them
-  if (STREAM && abort_s)
-    for (int k = 0; k < 1000; ++k) __nanosleep(1000);
   // neither CTA leaves (or frees its TMEM) while the pair's MMAs or arrivals may still reach it
   tm_fence_before();
   __syncwarp();
@@ -675,6 +675,16 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(NTHREADS, 1) ppconv_
   tm_fence_after();
   if (warp == MMA_WARP)
     asm volatile("tcgen05.dealloc.cta_group::2.sync.aligned.b32 %0, %1;" ::"r"(tmem), "n"(512));
+  // After a wait that gave up, this CTA's weight copies may still be in flight: none may write shared memory once the
+  // CTA has exited.  No more are issued (every loader has passed the barrier above); wait, bounded, for the last into
+  // each stage.  (The even CTA's stage barriers may lack loader arrivals and never complete; the bounded wait then
+  // outlasts any copy.)
+  if (STREAM && abort_s && tid == 0) {
+    long polls = 0;
+    for (int s = 0; s < NRING; ++s)
+      while (wuse[s] >= 0 && polls < WAIT_LIMIT && !mbar_try(su32(rank == 0 ? &full[s] : &wfull[s]), (uint32_t)(wuse[s] & 1)))
+        ++polls;
+  }
 }
 
 // Pairs that fit on the current device at once, per instantiation (0: pairs cannot be launched).

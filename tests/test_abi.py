@@ -238,3 +238,11 @@ def test_fold_groups_of_the_workloads():
     g = runner.fold_groups(net)
     # dense end layers and the global skip keep the original order, the 18 pruned layers' outputs are free
     assert g[0] and g[1] and g[-1] and g[-2] is False and not any(g[2:-2])
+
+
+def test_kernels_wait_for_copies_and_do_not_sleep():
+    """A sleep has no guaranteed length, so no kernel may count on one to outlast a copy in flight: each waits, bounded,
+    on the copies' barriers."""
+    csrc = os.path.join(ROOT, "paper_2004_11250_gb300", "csrc")
+    for name in sorted(os.listdir(csrc)):
+        assert "nanosleep" not in open(os.path.join(csrc, name)).read(), name
