@@ -331,13 +331,15 @@ pp_status pp_layer_flat_geometry(const pp_layer* layer, int N, int H, int W, int
 pp_status pp_layer_pin_flat_geometry(pp_layer* layer, int N, int H, int W, int flags, int R, int S);
 
 /* Synchronous: *device_error = 0 unless a launch of this layer's tensor-core
- * kernels, or of its direct kernels' box copies, met an error since the last read, and its output is then invalid:
+ * kernels or direct kernels, alone or in a network, met an error since the last
+ * read, and its output is then invalid:
  * bit 0 (value 1) a bounded wait gave up; bit 1 (value 2) under
  * PP_PRECISION_F16X3 an input was not finite or overflowed fp16 (|x s_x| >=
  * 65520) after the layer's input scale.  The word is cleared by the read. */
 pp_status pp_layer_device_status(const pp_layer* layer, int* device_error);
 
-/* Polls of an mbarrier after which a wait in the tensor-core kernels gives up:
+/* Polls of an mbarrier after which a wait in the tensor-core kernels, or for a
+ * box copy in the direct kernels, gives up:
  * the kernel then sets the layer's device status word, skips the rest of its
  * work, waits (with the same bound) for its own copies in flight and exits.
  * A poll that finds the phase incomplete suspends the thread for a few
@@ -399,6 +401,9 @@ pp_status pp_dense_forward(const pp_dense* layer, const float* x, float* y, cons
 
 /* Co and Ci of a dense layer (either may be NULL). */
 pp_status pp_dense_info(const pp_dense* layer, int* Co, int* Ci);
+/* As pp_layer_device_status, for the layer's launches, in a network too: 0, or
+ * 1 when a bounded wait for a box copy gave up and the output is invalid. */
+pp_status pp_dense_device_status(const pp_dense* layer, int* device_error);
 
 void pp_dense_destroy(pp_dense* layer);
 

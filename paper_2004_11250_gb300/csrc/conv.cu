@@ -958,8 +958,8 @@ extern "C" pp_status pp_layer_pin_flat_geometry(pp_layer* L, int N, int H, int W
   return PP_OK;
 }
 
-extern "C" pp_status pp_layer_device_status(const pp_layer* L, int* device_error) {
-  if (!L || !device_error) return PP_ERR_INVALID_ARG;
+// Reads and clears a layer's status words: the tensor-core kernels' and the direct kernels'.
+static pp_status read_status(const pp_layer* L, int* device_error) {
   *device_error = 0;
   for (int* word : {L->tc_ok ? L->tc.status : nullptr, L->direct.status}) {
     int v = 0;
@@ -969,6 +969,10 @@ extern "C" pp_status pp_layer_device_status(const pp_layer* L, int* device_error
     if (v && cudaMemset(word, 0, sizeof(int)) != cudaSuccess) return PP_ERR_CUDA;
   }
   return PP_OK;
+}
+
+extern "C" pp_status pp_layer_device_status(const pp_layer* L, int* device_error) {
+  return L && device_error ? read_status(L, device_error) : PP_ERR_INVALID_ARG;
 }
 
 extern "C" pp_status pp_layer_info(const pp_layer* L, int* Co, int* Ci, int64_t* device_bytes) {
@@ -1043,6 +1047,10 @@ extern "C" pp_status pp_dense_info(const pp_dense* D, int* Co, int* Ci) {
   if (Co) *Co = D->base.Co;
   if (Ci) *Ci = D->base.Ci;
   return PP_OK;
+}
+
+extern "C" pp_status pp_dense_device_status(const pp_dense* D, int* device_error) {
+  return D && device_error ? read_status(&D->base, device_error) : PP_ERR_INVALID_ARG;
 }
 
 extern "C" void pp_dense_destroy(pp_dense* D) {

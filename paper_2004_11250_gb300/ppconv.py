@@ -91,6 +91,7 @@ _SIGS = {
     "pp_dense_create": ([_P, _P, _I, _I, _P, _PP], _I),
     "pp_dense_forward": ([_P, _P, _P, _P, _I, _I, _I, _I, _P], _I),
     "pp_dense_info": ([_P, _P, _P], _I),
+    "pp_dense_device_status": ([_P, _P], _I),
     "pp_dense_destroy": ([_P], None),
     "pp_net_create": ([_I, _I, _I, _I, _PP], _I),
     "pp_net_add_conv": ([_P, _P, _I, _I], _I),
@@ -359,6 +360,12 @@ def pp_dense_info(layer):
     co, ci = _I(), _I()
     _check(lib.pp_dense_info(layer, ctypes.byref(co), ctypes.byref(ci)), "pp_dense_info")
     return co.value, ci.value
+
+
+def pp_dense_device_status(layer) -> int:
+    v = _I()
+    _check(lib.pp_dense_device_status(layer, ctypes.byref(v)), "pp_dense_device_status")
+    return v.value
 
 
 def pp_dense_destroy(layer):

@@ -40,6 +40,12 @@ def test_status_strings(pp):
     assert pp.pp_version() >= 100
 
 
+def test_device_status_of_both_kinds_of_layers(pp):
+    """Every kind of layer whose kernels have bounded waits has a status to read."""
+    for name in ("pp_layer_device_status", "pp_dense_device_status"):
+        assert getattr(pp.lib, name)(None, None) == pp.PP_ERR_INVALID_ARG
+
+
 def layers_for_pack():
     rng = np.random.default_rng(0)
     out = [synth.small_random_layer(rng, 16, 16, P=8, keep=0.5),

@@ -53,8 +53,7 @@ def run_layer(pp, runner, layer, x, skip=None, relu=False, pool=False, kernel=No
         flags = (pp.PP_ADD_SKIP if skip is not None else 0) | (pp.PP_RELU if relu else 0) | (pp.PP_POOL2 if pool else 0)
         L.forward(dev(x), y, None if skip is None else dev(skip), N, H, W, flags, torch.cuda.current_stream())
         torch.cuda.synchronize()
-        if not L.dense:
-            assert pp.pp_layer_device_status(L.handle) == 0
+        assert (pp.pp_dense_device_status if L.dense else pp.pp_layer_device_status)(L.handle) == 0
         return y.cpu().numpy()
     finally:
         L.close()
@@ -656,8 +655,7 @@ def layerwise_check(pp, runner, oracle_mod, net, check_net=True, fold_perm=False
             dn.run_host(xh, yh)
             assert torch.equal(yh, final.cpu())
         for L in dn.layers:
-            if not L.dense:
-                assert pp.pp_layer_device_status(L.handle) == 0
+            assert (pp.pp_dense_device_status if L.dense else pp.pp_layer_device_status)(L.handle) == 0
         return worst
     finally:
         dn.close()
