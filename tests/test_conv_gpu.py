@@ -176,8 +176,8 @@ def test_tensor_core_split_and_tiles(pp, runner, oracle_mod):
 @pytest.mark.parametrize("shape", [(1, 40, 130, 7, 100), (2, 16, 200, 4, 144), (1, 24, 64, 6, 160)])
 @pytest.mark.parametrize("flags", ["none", "skip_relu", "pool_relu"])
 def test_tensor_core_pixel_major(pp, runner, oracle_mod, shape, flags):
-    """Maps at least 96 wide: the row-tiled kernel's pixel-major tiles (merged hi/lo weight operand), 64- and
-    128-filter blocks, ragged filter blocks and row ends; pooled 128-filter layers take filter-major tiles."""
+    """Maps at least 96 wide: the row-tiled kernel's pixel-major tiles (merged hi/lo weight operand) of 128-filter blocks,
+    ragged filter blocks and row ends; pooled 128-filter layers take filter-major tiles, 64-filter ones CTA pairs."""
     N, Ci, Co, H, W = shape
     if flags == "pool_relu" and (H % 2 or W % 2):
         pytest.skip("pool needs even sizes")
@@ -208,8 +208,8 @@ FLAT_CASES = [
 
 
 PFR_CASES = [
-    # N, Ci, Co, H, W: 64-filter layers on maps at most 62 wide run the row-tiled
-    # kernel with whole rows flattened into the 128-pixel M side (16/32/64-pixel pitch)
+    # N, Ci, Co, H, W: 64-filter layers on a few maps at most 62 wide (CTA pairs; batches
+    # of them: test_row_tiled_kernel_where_pairs_do_not_run)
     (1, 64, 64, 56, 56),
     (2, 24, 40, 20, 14),
     (1, 16, 64, 33, 30),
@@ -221,7 +221,7 @@ PFR_CASES = [
 @pytest.mark.parametrize("case", PFR_CASES)
 @pytest.mark.parametrize("flags", ["none", "skip_relu"])
 def test_tensor_core_flattened_rows(pp, runner, oracle_mod, case, flags):
-    """Row-tiled tensor-core kernel, pixel-major with flattened rows, against the oracle."""
+    """64-filter layers on narrow maps by PP_KERNEL_TC, against the oracle."""
     N, Ci, Co, H, W = case
     rng = np.random.default_rng(13 * sum(case) + len(flags))
     L = synth.small_random_layer(rng, Co, Ci, P=8, keep=0.4)
@@ -229,7 +229,57 @@ def test_tensor_core_flattened_rows(pp, runner, oracle_mod, case, flags):
     skip = rng.uniform(-1, 1, (N, Co, H, W)).astype(np.float32) if flags == "skip_relu" else None
     g = run_layer(pp, runner, L, x, skip, flags != "none", False, kernel=pp.PP_KERNEL_TC)
     y, s = oracle_layer_full(oracle_mod, L, x, skip, flags != "none", False)
-    check_within(g, y, s, f"flattened-row tensor-core kernel {case} {flags}")
+    check_within(g, y, s, f"64 filters, narrow map {case} {flags}")
+
+
+# Where PP_KERNEL_TC still runs the row-tiled kernel: narrow maps of more than one tile per SM (whole rows flattened into
+# the 128-pixel M side at a pitch of 16, 32 or 64 pixels), in fp16 64-filter layers of more than 64 channels, 128-filter
+# blocks without the pairs' weight copy and pooled ones.  Orientation (0 filter-major, 1 pixel-major, 2 flattened rows),
+# tile width and filters per block as in the kernel's template arguments.
+ROW_TILED_CASES = [
+    # N, Ci, Co, H, W, pool, precisions, (orientation, width, filters)
+    (40, 24, 40, 9, 5, False, (0, 1), (2, 16, 64)),
+    (32, 64, 64, 14, 14, False, (0, 1), (2, 16, 64)),
+    (40, 72, 20, 8, 13, False, (0, 1), (2, 16, 64)),
+    (16, 20, 33, 20, 30, False, (0, 1), (2, 32, 64)),
+    (17, 9, 64, 19, 15, False, (0, 1), (2, 32, 64)),
+    (8, 16, 64, 40, 56, False, (0, 1), (2, 64, 64)),
+    (6, 72, 64, 55, 62, False, (0, 1), (2, 64, 64)),
+    (1, 72, 64, 23, 62, False, (1,), (2, 64, 64)),
+    (1, 72, 64, 6, 160, False, (1,), (1, 128, 64)),
+    (2, 100, 40, 7, 257, False, (1,), (1, 128, 64)),
+    (1, 80, 33, 5, 63, False, (1,), (1, 128, 64)),
+    (1, 130, 64, 20, 22, True, (1,), (1, 128, 64)),
+    (1, 40, 130, 7, 100, False, (0, 1), (1, 128, 128)),
+    (1, 24, 130, 6, 100, True, (0,), (0, 128, 128)),
+    (1, 24, 130, 6, 100, True, (1,), (0, 64, 128)),
+    (1, 24, 130, 12, 14, False, (0, 1), (0, 16, 128)),
+]
+
+
+@pytest.mark.parametrize("case,precision", [(c, p) for c in ROW_TILED_CASES for p in c[6]])
+@pytest.mark.parametrize("epilogue", ["none", "skip_relu"])
+def test_row_tiled_kernel_where_pairs_do_not_run(pp, runner, oracle_mod, tmp_path, case, precision, epilogue):
+    N, Ci, Co, H, W, pool, _, (ori, tw, fb) = case
+    rng = np.random.default_rng(sum(case[:5]) + precision + len(epilogue))
+    L = synth.small_random_layer(rng, Co, Ci, P=8, keep=0.4)
+    x = rng.uniform(-1, 1, (N, Ci, H, W)).astype(np.float32)
+    skip = rng.uniform(-1, 1, (N, Co, H, W)).astype(np.float32) if epilogue == "skip_relu" else None
+    fl = (pp.PP_ADD_SKIP | pp.PP_RELU if skip is not None else 0) | (pp.PP_POOL2 if pool else 0)
+    y, s = oracle_layer_full(oracle_mod, L, x, skip, skip is not None, pool)
+    d = runner.DeviceLayer(L, precision=precision)
+    try:
+        pp.pp_layer_set_kernel(d.handle, pp.PP_KERNEL_TC)
+        xd, sd, out = dev(x), None if skip is None else dev(skip), torch.full(y.shape, float("nan"), device="cuda")
+        call = lambda: d.forward(xd, out, sd, N, H, W, fl, torch.cuda.current_stream())
+        names = launched(call, tmp_path)
+        assert len(names) == 1 and f"ppconv_tc_kernelILi{ori}ELi{tw}ELi{fb}ELb{precision}E" in names[0], names
+        call()
+        torch.cuda.synchronize()
+        assert pp.pp_layer_device_status(d.handle) == 0
+    finally:
+        d.close()
+    check_within(out.cpu().numpy(), y, s, f"row-tiled kernel {case} precision {precision} {epilogue}")
 
 
 @pytest.mark.parametrize("case", FLAT_CASES)
@@ -970,7 +1020,8 @@ def test_f16_flat_wide_tiles(pp, runner, oracle_mod, case):
 @pytest.mark.parametrize("shape", [(1, 40, 130, 7, 100), (2, 16, 200, 4, 144), (1, 24, 64, 6, 160)] + PFR_CASES)
 @pytest.mark.parametrize("flags", ["none", "skip_relu", "pool_relu"])
 def test_f16_row_tiled(pp, runner, oracle_mod, shape, flags):
-    """Row-tiled kernel under f16: pixel-major (128- and 64-filter blocks), flattened rows, filter-major."""
+    """PP_KERNEL_TC under f16: the row-tiled kernel's pixel-major 128-filter and filter-major tiles, CTA pairs for at most
+    64 filters and 64 channels, flattened rows for more channels."""
     N, Ci, Co, H, W = shape
     pool = flags == "pool_relu"
     if pool and (H % 2 or W % 2):
@@ -1111,7 +1162,7 @@ RESIDENT_CASES = [
 @pytest.mark.parametrize("case", RESIDENT_CASES)
 @pytest.mark.parametrize("flags", ["none", "skip_relu", "skip_pool_relu"])
 @pytest.mark.parametrize("precision", [0, 1])
-def test_resident_weight_kernel(pp, runner, oracle_mod, case, flags, precision):
+def test_resident_weight_kernel(pp, runner, oracle_mod, tmp_path, case, flags, precision):
     N, Ci, Co, H, W = case
     pool = "pool" in flags
     if pool:
@@ -1126,6 +1177,15 @@ def test_resident_weight_kernel(pp, runner, oracle_mod, case, flags, precision):
     # a second launch gives the same bits (a fixed order of sums)
     g2 = run_layer(pp, runner, L, x, skip, "relu" in flags, pool, kernel=pp.PP_KERNEL_TC, precision=precision)
     assert np.array_equal(g, g2)
+    d = runner.DeviceLayer(L, precision=precision)
+    try:
+        pp.pp_layer_set_kernel(d.handle, pp.PP_KERNEL_TC)
+        xd, sd, out = dev(x), None if skip is None else dev(skip), torch.empty(y.shape, device="cuda")
+        fl = (pp.PP_ADD_SKIP if skip is not None else 0) | (pp.PP_RELU if "relu" in flags else 0) | (pp.PP_POOL2 if pool else 0)
+        names = launched(lambda: d.forward(xd, out, sd, N, H, W, fl, torch.cuda.current_stream()), tmp_path)
+        assert len(names) == 1 and f"ppconv_tcr_kernelILb{precision}ELb{int(pool)}ELi64ELb0E" in names[0]
+    finally:
+        d.close()
 
 
 @pytest.mark.parametrize("precision", [0, 1])
