@@ -1222,6 +1222,7 @@ DIRECT_SHAPES = [
     (1, 33, 47, 14, 14), (2, 20, 24, 40, 37), (1, 18, 17, 1, 1), (1, 64, 64, 33, 65), (5, 24, 40, 96, 96), (3, 17, 21, 130, 128),
     (2, 8, 1, 720, 260), (1, 9, 2, 1250, 255), (3, 10, 3, 416, 256), (1, 16, 4, 2500, 130), (1, 8, 3, 16, 128),
     (1, 9, 1, 130, 1028), (1, 13, 1, 131, 1030), (1, 64, 1, 300, 1280), (1, 8, 1, 313, 1281), (1, 11, 3, 300, 700), (2, 9, 3, 160, 1284), (1, 10, 2, 520, 1284),
+    (1, 9, 1, 719, 1284), (1, 12, 3, 701, 1100), (1, 11, 3, 700, 1101), (1, 10, 2, 521, 1285), (1, 17, 22, 290, 1100), (1, 18, 17, 291, 1101),
     (1, 1, 64, 18, 129), (2, 2, 70, 64, 130), (1, 3, 130, 41, 200), (1, 4, 9, 300, 257), (1, 3, 33, 6, 66), (2, 1, 5, 2000, 68),
 ]
 
