@@ -253,6 +253,20 @@ __device__ __forceinline__ void split_reduce(const FlatParams& p, const Tile& T,
   }
 }
 
+// A load that stays where it is written: the compiler moved plain ones behind the wait that follows them, where their
+// latency was in series with every chunk.  Zero unless in.
+__device__ __forceinline__ float ld_here(const float* a, bool in) {
+  float v;
+  asm volatile("{ .reg .pred p; setp.ne.b32 p, %2, 0; mov.b32 %0, 0; @p ld.global.nc.f32 %0, [%1]; }"
+               : "=f"(v)
+               : "l"(a), "r"((int)in));
+  return v;
+}
+
+// EARLY (f16): the input comes through a box ring; without it per-thread loads or a box in the stage itself.  An
+// instantiation of its own each: in one, the loaders without boxes were 15 % slower for the code of those with them (128 ->
+// 128 at 113 x 66, R = 2, split in 2: 15.7 us before that code, 18.1 beside it, 14.7 apart and with ld_here), and those
+// with boxes 5 % (512 -> 512 at 28 x 28 18.9 -> 17.9).
 // PAIR: the CTAs of a cluster form pairs (cluster ranks 2k, 2k + 1) that run
 // two filter blocks of the same tile and channel range with cta_group::2 MMAs
 // (M = 256): each CTA holds its own block's weights (A) and stages half of
@@ -260,7 +274,7 @@ __device__ __forceinline__ void split_reduce(const FlatParams& p, const Tile& T,
 // odd one); the even CTA's MMA thread issues for both, once the odd CTA has
 // reported its stage full, and its commits arrive in both CTAs.  Pairs run in
 // cluster-split mode (one tile per CTA).
-template <bool SPLIT, bool F16, bool PAIR>
+template <bool SPLIT, bool F16, bool PAIR, bool EARLY>
 __global__ void __launch_bounds__(flat_threads<SPLIT, F16>(), 1) ppconv_tcf_kernel(const FlatParams p, const __grid_constant__ CUtensorMap xmap) {
   static_assert(SPLIT || !PAIR, "CTA pairs run in cluster-split mode");
   constexpr bool WR = weight_ring<SPLIT, F16>();
@@ -299,7 +313,7 @@ __global__ void __launch_bounds__(flat_threads<SPLIT, F16>(), 1) ppconv_tcf_kern
       // chunk's weight copies (one more arrival each,
       // with its bytes: the three group copies, or without the ring the whole
       // chunk) have landed: the MMA thread waits on one barrier per chunk
-      mbar_init(su32(&full[s]), (F16 && p.use_tma && p.sep ? MMA_WARP : NLOAD) + (WR ? NGRP : 1));
+      mbar_init(su32(&full[s]), (EARLY ? MMA_WARP : NLOAD) + (WR ? NGRP : 1));
       mbar_init(su32(&raw_full[s]), 1);
       mbar_init(su32(&raw_empty[s]), MMA_WARP);
       mbar_init(su32(&empty[s]), 1);
@@ -439,7 +453,7 @@ __global__ void __launch_bounds__(flat_threads<SPLIT, F16>(), 1) ppconv_tcf_kern
         issue_raw(raw_issued, smem + p.raw_off + raw_issued * p.raw_slot);
     bool stop = false;  // identical in every loader thread (decided by group_any), f16 with a box ring in every lane of a warp
     __half2 hmax = __floats2half2_rn(0.f, 0.f);  // f16: largest |x| after scaling: infinite or NaN out of fp16's range
-    const bool early = p.use_tma && p.sep;
+    const bool early = F16 ? EARLY : p.use_tma && p.sep;
     const int nit = (2 * p.npix + NLOAD - 1) / NLOAD;  // items per thread
     for (int i = 0; i < nmine && !stop; ++i) {
       const Tile T = my_tile(tile_index(i));
@@ -458,7 +472,8 @@ __global__ void __launch_bounds__(flat_threads<SPLIT, F16>(), 1) ppconv_tcf_kern
         if (early) {
           // f16: no barrier over the loader warps; each waits for the box itself, and thread 0 alone waits until all
           // have read it before it issues the next copy into the slot (256 -> 256 at 56 x 56, batch 8: 70.8 -> 67.9 us
-          // with the cheaper split; the tf32 loaders, whose warps have little to do per chunk, ran 5 % slower so).
+          // with the cheaper split, 65.4 with an instantiation of its own; the tf32 loaders, whose warps have little to do
+          // per chunk, ran 5 % slower so).
           const bool landed = wait(&raw_full[s], (uint32_t)(use & 1));
           if (F16 ? !__all_sync(0xffffffffu, landed) : group_any<NLOAD>(!landed)) {
             stop = true;
@@ -507,16 +522,20 @@ __global__ void __launch_bounds__(flat_threads<SPLIT, F16>(), 1) ppconv_tcf_kern
             }
           }
         }
-        if (!p.use_tma) {
+        if (!EARLY && !p.use_tma) {
 #pragma unroll
           for (int b = 0; b < ITEMS_MAX; ++b) {
+            if (F16 && b >= nit) break;
             const int kh = rowcol[b] >> 30, br = (rowcol[b] >> 15) & 0x7FFF, bc = rowcol[b] & 0x7FFF;
             const int r = T.r0 - 1 + br, cc = bc - 1;
             const bool inside = doff[b] >= 0 && (unsigned)r < (unsigned)p.H && (unsigned)cc < (unsigned)p.W;
 #pragma unroll
             for (int k = 0; k < CPH; ++k) {
               const int ch = c * KCH + kh * CPH + k;
-              v[b][k] = (inside && ch < p.Ci) ? __ldg(xb + ((size_t)ch * p.H + r) * p.W + cc) : 0.f;
+              if constexpr (F16)
+                v[b][k] = ld_here(xb + ((size_t)ch * p.H + r) * p.W + cc, inside && ch < p.Ci);
+              else
+                v[b][k] = (inside && ch < p.Ci) ? __ldg(xb + ((size_t)ch * p.H + r) * p.W + cc) : 0.f;
             }
           }
         }
@@ -533,7 +552,7 @@ __global__ void __launch_bounds__(flat_threads<SPLIT, F16>(), 1) ppconv_tcf_kern
             issue_w(g, s);
             ++w_issued;
           }
-          if (p.use_tma && !p.sep) {
+          if (!EARLY && p.use_tma && !p.sep) {
             issue_raw(g, reinterpret_cast<unsigned char*>(lo));  // lands in the lo operand, split in place below
             ++raw_issued;
           }
@@ -947,36 +966,30 @@ struct DeviceState {
 DeviceState g_dev[ppc::DeviceOnce::kMaxDevices];
 ppc::DeviceOnce g_dev_once;  // fills g_dev[dev] once per device (its ready flag publishes it)
 
+template <bool SPLIT, bool F16, bool PAIR, bool EARLY>
+cudaError_t set_attributes() {
+  const auto kernel = ppconv_tcf_kernel<SPLIT, F16, PAIR, EARLY>;
+  const cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM_ALLOC);
+  // without larger clusters only portable sizes (up to 8) can be used
+  if (e == cudaSuccess && SPLIT &&
+      cudaFuncSetAttribute(kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) != cudaSuccess)
+    cudaGetLastError();
+  return e;
+}
+
 cudaError_t init_device(int dev) {
   DeviceState& D = g_dev[dev];
   cudaError_t e = cudaDeviceGetAttribute(&D.sms, cudaDevAttrMultiProcessorCount, dev);
-  if (e != cudaSuccess) return e;
-  if ((e = cudaFuncSetAttribute(ppconv_tcf_kernel<false, false, false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                SMEM_ALLOC)) != cudaSuccess ||
-      (e = cudaFuncSetAttribute(ppconv_tcf_kernel<true, false, false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                SMEM_ALLOC)) != cudaSuccess ||
-      (e = cudaFuncSetAttribute(ppconv_tcf_kernel<false, true, false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                SMEM_ALLOC)) != cudaSuccess ||
-      (e = cudaFuncSetAttribute(ppconv_tcf_kernel<true, true, false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                SMEM_ALLOC)) != cudaSuccess ||
-      (e = cudaFuncSetAttribute(ppconv_tcf_kernel<true, false, true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                SMEM_ALLOC)) != cudaSuccess ||
-      (e = cudaFuncSetAttribute(ppconv_tcf_kernel<true, true, true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                SMEM_ALLOC)) != cudaSuccess)
+  if (e != cudaSuccess || (e = set_attributes<false, false, false, false>()) != cudaSuccess ||
+      (e = set_attributes<true, false, false, false>()) != cudaSuccess ||
+      (e = set_attributes<true, false, true, false>()) != cudaSuccess ||
+      (e = set_attributes<false, true, false, false>()) != cudaSuccess ||
+      (e = set_attributes<true, true, false, false>()) != cudaSuccess ||
+      (e = set_attributes<true, true, true, false>()) != cudaSuccess ||
+      (e = set_attributes<false, true, false, true>()) != cudaSuccess ||
+      (e = set_attributes<true, true, false, true>()) != cudaSuccess ||
+      (e = set_attributes<true, true, true, true>()) != cudaSuccess)
     return e;
-  // then only portable sizes (up to 8) can be used
-  if (cudaFuncSetAttribute(ppconv_tcf_kernel<true, false, false>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) !=
-      cudaSuccess)
-    cudaGetLastError();
-  if (cudaFuncSetAttribute(ppconv_tcf_kernel<true, true, false>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) !=
-      cudaSuccess)
-    cudaGetLastError();
-  if (cudaFuncSetAttribute(ppconv_tcf_kernel<true, false, true>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) !=
-      cudaSuccess)
-    cudaGetLastError();
-  if (cudaFuncSetAttribute(ppconv_tcf_kernel<true, true, true>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) !=
-      cudaSuccess)
-    cudaGetLastError();
   for (int s = 2; s <= MAX_SPLIT; s *= 2) {
     cudaLaunchConfig_t cfg = {};
     cudaLaunchAttribute at[1];
@@ -991,7 +1004,7 @@ cudaError_t init_device(int dev) {
     cfg.numAttrs = 1;
     int n = 0;
     // split launches run 576 threads in both precisions, one CTA per SM, with the same shared memory
-    if (cudaOccupancyMaxActiveClusters(&n, ppconv_tcf_kernel<true, false, false>, &cfg) != cudaSuccess) {
+    if (cudaOccupancyMaxActiveClusters(&n, ppconv_tcf_kernel<true, false, false, false>, &cfg) != cudaSuccess) {
       cudaGetLastError();
       n = 0;
     }
@@ -1029,9 +1042,11 @@ struct FlatGeo {
 // ~1850 per cycle and its operand reads (4 KB of weights + 32 N bytes of
 // input) at 128 shared-memory bytes per cycle; a chunk also needs its 73.7 KB
 // of weights from L2 (~48 bytes per cycle) and the loaders' round of its input,
-// which measured 2250 cycles in tf32 at any width up to 128 columns and 2550 +
-// 7 N in f16 (16 channels to split), 900 more where rows and planes are not
-// 16-byte aligned and each thread loads its own; start-up, pipeline fill and
+// which measured 2250 cycles in tf32 at any width up to 128 columns, 900 more
+// where rows and planes are not 16-byte aligned and each thread loads its own; in
+// f16 (16 channels to split) it is taken as 2550 + 7 N, and 900, which was measured
+// before boxes and per-thread loads had loaders of their own (now 2400 at N = 64,
+// 2550 at 120, 3550 at 176 with boxes) and still ranks the geometries; start-up, pipeline fill and
 // teardown of ~9000 cycles; the last tile's copy out of tensor memory at ~16
 // cycles a column and the remote part of a split's partials at ~24 more;
 // clusters of 16 start the later the more of them there are (up to ~12000; a few
@@ -1039,8 +1054,9 @@ struct FlatGeo {
 // -> 512 at 7 x 7 12.4 against 16.2); and clusters beyond those co-resident on
 // the GPU run in later waves.  CTA pairs measured slower than their halves apart
 // (39.6 against 31.4 us at 512 -> 512, 28 x 28): 1.15 of the chunk time.  Against
-// every accepted geometry of 21 shapes the model's choice measured within 1 % of
-// the fastest; the model before it (1500 cycles a chunk, pairs at 0.8, start-up
+// every accepted geometry the model's choice measured within 1 % of the fastest in
+// tf32 (21 shapes), in f16 1.3 % on average over 90 and 18 % at worst (36 -> 338 at
+// 138 x 80, R = 2 22.9 us, R = 1 19.4); the model before it (1500 cycles a chunk, pairs at 0.8, start-up
 // 5000) was up to 1.8 times off it (100 -> 200 at 45 x 61: R = 2 unsplit, 42 us,
 // against R = 4 split in 2, 23).
 // Every geometry the kernel can run for this shape, best first by the model;
@@ -1280,6 +1296,7 @@ pp_status launch_geo(const FlatGeo& G, const DeviceState& Dref, const ppc::TcLay
       }
     }
   }
+  const bool early = f16 && p.use_tma && p.sep;
   cudaLaunchConfig_t cfg = {};
   cudaLaunchAttribute at[2];
   // programmatic dependent launch: the kernel waits (griddepcontrol.wait) for
@@ -1299,8 +1316,9 @@ pp_status launch_geo(const FlatGeo& G, const DeviceState& Dref, const ppc::TcLay
     at[1].val.clusterDim.z = 1;
     cfg.numAttrs = 2;
     cfg.gridDim = dim3((unsigned)(G.ntiles * 2 * G.split));
-    e = f16 ? cudaLaunchKernelEx(&cfg, ppconv_tcf_kernel<true, true, true>, p, xmap)
-            : cudaLaunchKernelEx(&cfg, ppconv_tcf_kernel<true, false, true>, p, xmap);
+    e = early ? cudaLaunchKernelEx(&cfg, ppconv_tcf_kernel<true, true, true, true>, p, xmap)
+        : f16 ? cudaLaunchKernelEx(&cfg, ppconv_tcf_kernel<true, true, true, false>, p, xmap)
+              : cudaLaunchKernelEx(&cfg, ppconv_tcf_kernel<true, false, true, false>, p, xmap);
   } else if (G.split > 1 || one) {
     at[1].id = cudaLaunchAttributeClusterDimension;
     at[1].val.clusterDim.x = (unsigned)G.split;
@@ -1308,12 +1326,14 @@ pp_status launch_geo(const FlatGeo& G, const DeviceState& Dref, const ppc::TcLay
     at[1].val.clusterDim.z = 1;
     cfg.numAttrs = 2;
     cfg.gridDim = dim3((unsigned)(G.ntiles * G.split));
-    e = f16 ? cudaLaunchKernelEx(&cfg, ppconv_tcf_kernel<true, true, false>, p, xmap)
-            : cudaLaunchKernelEx(&cfg, ppconv_tcf_kernel<true, false, false>, p, xmap);
+    e = early ? cudaLaunchKernelEx(&cfg, ppconv_tcf_kernel<true, true, false, true>, p, xmap)
+        : f16 ? cudaLaunchKernelEx(&cfg, ppconv_tcf_kernel<true, true, false, false>, p, xmap)
+              : cudaLaunchKernelEx(&cfg, ppconv_tcf_kernel<true, false, false, false>, p, xmap);
   } else {
     cfg.gridDim = dim3((unsigned)std::min(G.ntiles, D->sms));
-    e = f16 ? cudaLaunchKernelEx(&cfg, ppconv_tcf_kernel<false, true, false>, p, xmap)
-            : cudaLaunchKernelEx(&cfg, ppconv_tcf_kernel<false, false, false>, p, xmap);
+    e = early ? cudaLaunchKernelEx(&cfg, ppconv_tcf_kernel<false, true, false, true>, p, xmap)
+        : f16 ? cudaLaunchKernelEx(&cfg, ppconv_tcf_kernel<false, true, false, false>, p, xmap)
+              : cudaLaunchKernelEx(&cfg, ppconv_tcf_kernel<false, false, false, false>, p, xmap);
   }
   if (e != cudaSuccess) {
     cudaGetLastError();

@@ -959,6 +959,50 @@ def test_f16_flat_kernel(pp, runner, oracle_mod, case, flags):
     check_within(g, y, s, f"f16 flat {case} {flags}")
 
 
+# The flat kernel's f16 loaders by their input: boxes through a ring, and per-thread loads (rows and planes not 16-byte
+# aligned, or x itself not); one item a thread up to the most, split and unsplit, several tiles a CTA.
+F16_LOADER_CASES = [
+    # N, Ci, Co, H, W, offset of x in floats, boxes
+    (1, 136, 256, 28, 28, 0, True), (1, 40, 129, 30, 22, 0, True), (4, 33, 128, 64, 60, 0, True), (9, 16, 130, 112, 112, 0, True),
+    (1, 136, 256, 28, 28, 1, False), (1, 100, 200, 45, 61, 0, False), (1, 33, 128, 113, 66, 0, False), (5, 24, 130, 211, 50, 0, False),
+    (3, 40, 128, 585, 19, 0, False), (1, 200, 66, 7, 5, 0, False), (2, 17, 129, 33, 125, 0, False),
+]
+
+
+@pytest.mark.parametrize("case", F16_LOADER_CASES)
+@pytest.mark.parametrize("skip", [False, True])
+def test_f16_flat_loaders(pp, runner, oracle_mod, tmp_path, case, skip):
+    N, Ci, Co, H, W, off, boxes = case
+    rng = np.random.default_rng(sum(case[:6]))
+    L = synth.small_random_layer(rng, Co, Ci, P=8, keep=0.4)
+    x = rng.uniform(-1, 1, (N, Ci, H, W)).astype(np.float32)
+    sk = rng.uniform(-1, 1, (N, Co, H, W)).astype(np.float32) if skip else None
+    d = runner.DeviceLayer(L, precision=F16)
+    try:
+        pp.pp_layer_set_kernel(d.handle, pp.PP_KERNEL_TC_FLAT)
+        buf = torch.empty(x.size + off, device="cuda")
+        buf[off:] = torch.from_numpy(x.ravel()).cuda()
+        sd, out = None if sk is None else dev(sk), torch.full((N, Co, H, W), float("nan"), device="cuda")
+        call = lambda: d.forward(buf[off:], out, sd, N, H, W, pp.PP_ADD_SKIP if skip else 0, torch.cuda.current_stream())
+        names = launched(call, tmp_path)
+        assert len(names) == 1 and re.search(r"ppconv_tcf_kernelILb[01]ELb1ELb[01]ELb%dE" % boxes, names[0]), names
+        call()
+        torch.cuda.synchronize()
+        assert pp.pp_layer_device_status(d.handle) == 0
+        buf[off + x.size // 2] = float("inf")
+        call()
+        torch.cuda.synchronize()
+        assert pp.pp_layer_device_status(d.handle) == pp.PP_STATUS_F16_RANGE
+        buf[off + x.size // 2] = float(x.ravel()[x.size // 2])
+        call()
+        torch.cuda.synchronize()
+        assert pp.pp_layer_device_status(d.handle) == 0
+    finally:
+        d.close()
+    y, s = oracle_layer_full(oracle_mod, L, x, sk)
+    check_within(out.cpu().numpy(), y, s, f"f16 loaders {case}")
+
+
 WIDE_F16_CASES = [
     # N, Ci, Co, H, W, flags, whether split geometries exist; flat-kernel f16 tiles of more than 128 columns
     # (the second accumulator in the other TMEM buffer, single-buffered)
