@@ -1238,12 +1238,15 @@ pp_status launch_geo(const FlatGeo& G, const DeviceState& Dref, const ppc::TcLay
   p.raw_w = G.raw_w;
   p.raw_bytes = G.raw_bytes;
   // without the weight ring (unsplit tf32): two whole-chunk weight slots, 6 group slots
-  // One tile per CTA, and rows that do not allow 16-byte stores or a residual: the split instantiation with a split of
-  // 1 (a cluster of one CTA).  Its second phase finishes a tile with whole rows per warp, where the other epilogue has a
-  // filter per lane and touches 32 planes with every 4-byte access (100 -> 200 at 45 x 61, batch 3, with residual, R = 2:
-  // 42.3 -> 26.9 us).  Aligned rows without residual leave in 16-byte stores as fast (128 -> 128 at 128 x 128, tf32 27.8
-  // against 27.4, f16 21.1 against 22.4).
-  const bool one = G.split == 1 && !G.pair && G.ntiles <= D->sms && ((W & 3) || (flags & PP_ADD_SKIP));
+  // One tile per CTA, and a residual or, unless pooled, rows that do not allow 16-byte stores: the split instantiation with
+  // a split of 1 (a cluster of one CTA).  Its second phase finishes a tile with whole rows per warp, where the other
+  // epilogue has a filter per lane and touches 32 planes with every 4-byte access (100 -> 200 at 45 x 61, batch 3, with
+  // residual, R = 2: 42.3 -> 26.9 us).  Aligned rows without residual leave in 16-byte stores as fast (128 -> 128 at 128 x
+  // 128, tf32 27.8 against 27.4, f16 21.1 against 22.4), and pooled ones write a quarter: without residual the second phase
+  // cost them up to 16 % (128 -> 128 at 30 x 30, tf32, R = 6 28.9 -> 31.0 us; 40 -> 80 at 34 x 46, batch 2, R = 4 12.9 ->
+  // 14.9; with a residual 37.9 -> 25.4 and 22.0 -> 15.7).
+  const bool one = G.split == 1 && !G.pair && G.ntiles <= D->sms &&
+                   ((flags & PP_ADD_SKIP) || ((W & 3) && !(flags & PP_POOL2)));
   const bool ring = G.split > 1 || G.pair || f16 || one;
   p.wsl = ring ? G.wsl : 6;
   p.xoff = p.wsl * GRP_BYTES;

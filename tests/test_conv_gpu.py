@@ -1595,3 +1595,31 @@ def test_no_memory_for_optional_layouts(pp, oracle_mod, tmp_path, case, kernel, 
     x = np.random.default_rng(8).uniform(-1, 1, (N, Ci, H, W)).astype(np.float32)
     y, s = oracle_layer_full(oracle_mod, L, x)
     check_within(np.load(tmp_path / "y.npy"), y, s, f"no memory for {nbytes} bytes")
+
+
+@pytest.mark.parametrize("flags,split_form", [("pool", False), ("skip_pool", True), ("none", True)])
+@pytest.mark.parametrize("precision", [0, 1])
+def test_flat_unsplit_ragged_rows_form(pp, runner, oracle_mod, tmp_path, flags, split_form, precision):
+    """Unsplit one-tile launches with rows of no whole 16-byte groups finish in the split instantiation's second phase,
+    pooled ones only with a residual."""
+    rng = np.random.default_rng(121)
+    L = synth.small_random_layer(rng, 80, 40, P=8, keep=0.5)
+    N, H, W, pool = 2, 34, 46, "pool" in flags
+    x = rng.uniform(-1, 1, (N, 40, H, W)).astype(np.float32)
+    skip = rng.uniform(-1, 1, (N, 80, H, W)).astype(np.float32) if "skip" in flags else None
+    fl = (pp.PP_POOL2 if pool else 0) | (pp.PP_ADD_SKIP if skip is not None else 0)
+    y, s = oracle_layer_full(oracle_mod, L, x, skip, False, pool)
+    d = runner.DeviceLayer(L, precision=precision)
+    try:
+        pp.pp_layer_set_kernel(d.handle, pp.PP_KERNEL_TC_FLAT)
+        pp.pp_layer_pin_flat_geometry(d.handle, N, H, W, fl, 4, 1)
+        xd, sd, out = dev(x), None if skip is None else dev(skip), torch.full(y.shape, float("nan"), device="cuda")
+        call = lambda: d.forward(xd, out, sd, N, H, W, fl, torch.cuda.current_stream())
+        names = launched(call, tmp_path)
+        assert len(names) == 1 and f"ppconv_tcf_kernelILb{int(split_form)}E" in names[0], names
+        call()
+        torch.cuda.synchronize()
+        assert pp.pp_layer_device_status(d.handle) == 0
+    finally:
+        d.close()
+    check_within(out.cpu().numpy(), y, s, f"unsplit tile, ragged rows, {flags}")
