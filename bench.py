@@ -387,12 +387,16 @@ def code_lines(text: str) -> str:
     return "\n".join(out)
 
 
+KERNEL_SOURCES = ("conv.cu", "conv_tm.cu", "conv_tc.cu", "conv_tcf.cu", "conv_tcr.cu", "conv_direct.cu", "tc_ptx.cuh",
+                  "internal.h")
+
+
 def kernel_source_hash():
     """sha256 over the conv kernel sources' code, comments left out (a profile taken on other code is
     stale; an edit of a comment does not change the kernels)."""
     import hashlib
     h = hashlib.sha256()
-    for name in ("conv.cu", "conv_tm.cu", "conv_tc.cu", "conv_tcf.cu", "conv_direct.cu", "tc_ptx.cuh", "internal.h"):
+    for name in KERNEL_SOURCES:
         with open(os.path.join(ROOT, "paper_2004_11250_gb300", "csrc", name), encoding="utf-8") as f:
             h.update(code_lines(f.read()).encode())
     return h.hexdigest()

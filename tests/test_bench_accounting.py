@@ -7,6 +7,7 @@ that do not depend on the generated weights.  The totals below are written out f
 definitions, not from the code under test.
 """
 import os
+import re
 import sys
 
 import pytest
@@ -79,6 +80,15 @@ def test_source_hash_ignores_comments_only():
     assert bench.code_lines(src) == "int a = 1;\nint b = a + 2;"
     assert bench.code_lines(src.replace("// one", "// another note")) == bench.code_lines(src)
     assert bench.code_lines(src.replace("a + 2", "a + 3")) != bench.code_lines(src)
+
+
+def test_source_hash_covers_every_convolution_kernel():
+    """A traffic figure is stale once any source that defines a convolution kernel has changed."""
+    csrc = os.path.join(ROOT, "paper_2004_11250_gb300", "csrc")
+    with_kernels = {n for n in os.listdir(csrc) if n.endswith(".cu") and re.search(
+        r"__global__[^;{]*ppconv_\w*kernel", open(os.path.join(csrc, n), encoding="utf-8").read())}
+    assert len(with_kernels) >= 6
+    assert with_kernels <= set(bench.KERNEL_SOURCES)
 
 
 def test_traffic_read_only_for_matching_code(tmp_path, monkeypatch):
