@@ -32,11 +32,13 @@ import argparse
 import json
 import math
 import os
+import re
 import statistics
 import subprocess
 import sys
 import tempfile
 import time
+import warnings
 
 import numpy as np
 
@@ -46,9 +48,7 @@ if ROOT not in sys.path:
 
 HBM_PEAK_GBS_FALLBACK = 6800.0
 CONFIG_CPU_SECONDS = 4.0  # oracle sample per workload of the all-configs table
-# by kernel choice; the row-tiled choice (3) launches ppconv_tcr_kernel where CTA pairs take the layer
-KERNEL_NAMES = {1: "ppconv_tm_kernel", 2: "ppconv_kernel", 3: "ppconv_tc_kernel", 4: "ppconv_tcf_kernel",
-                5: "ppconv_direct_kernel"}
+TENSOR_KERNELS = ("ppconv_tc_kernel", "ppconv_tcf_kernel", "ppconv_tcr_kernel")
 FP32_LANES_PER_SM = 128
 SM_MAX_MHZ = 2070.0
 L2_FLUSH_BYTES = 512 << 20
@@ -329,6 +329,33 @@ def time_ops_in_frame(dn, acts, steps, flush, stream):
     return [statistics.median(v) for v in per]
 
 
+def op_kernels(dn, acts):
+    """The kernel that each op launches, by name, from the dump of a graph captured of its call."""
+    import torch
+    from paper_2004_11250_gb300 import runner
+    names = []
+    with tempfile.TemporaryDirectory() as tmp, warnings.catch_warnings():
+        warnings.simplefilter("ignore")  # the dump announces itself as one
+        dot = os.path.join(tmp, "graph.dot")
+        for k, (op, L) in enumerate(zip(dn.spec.ops, dn.layers)):
+            N, _, H, W = acts[k].shape
+            g = torch.cuda.CUDAGraph(keep_graph=True)
+            g.enable_debug_mode()
+            with torch.cuda.graph(g):
+                L.forward(acts[k], acts[k + 1], acts[op.skip_from] if op.skip_from >= 0 else None, N, H, W,
+                          runner.op_flags(op), torch.cuda.current_stream())
+            g.debug_dump(dot)
+            with open(dot) as f:
+                names.append(kernel_name(f.read()))
+    return names
+
+
+def kernel_name(dump: str) -> str:
+    """The kernel's name without template arguments, from the dump of a graph that holds one launch."""
+    found = re.findall(r"ppconv_(?:[a-z]+_)*kernel", dump)
+    return found[0] if len(found) == 1 else "?"
+
+
 def time_graph_of_launches(dn, acts, reps, steps, stream):
     """Per-launch time (ms) of op 0 replayed back to back: one CUDA graph of `reps` launches of the op on the
     same buffers (no L2 flush between them: weights and input stay warm), replayed `steps` times.  With a
@@ -409,7 +436,7 @@ def tensor_view(shapes, kern, op_ms, pruned, f16=False):
     """Tensor-pipe view of the pruned ops that run on a tensor-core kernel: their dense 9-tap contraction
     in 3 passes (hi*hi, lo*hi, hi*lo) per second against the measured kind::tf32 (or kind::f16) MMA
     peak; None without such ops."""
-    tc_ops = [k for k in pruned if kern[k] in ("ppconv_tc_kernel", "ppconv_tcf_kernel")]
+    tc_ops = [k for k in pruned if kern[k] in TENSOR_KERNELS]
     kind = "f16" if f16 else "tf32"
     if not tc_ops or kind not in TENSOR_PEAKS:
         return None
@@ -441,10 +468,9 @@ def bench_config(name, steps, warmup, flush, stream, hbm, fold_too=False, precis
         ms = statistics.median(ts)
         fr = [roof_time_s(s["flops"], s["bytes"], hbm) / (t * 1e-3) for s, t in zip(shapes, op_ms)]
         pr = [f for s, f in zip(shapes, fr) if s["pruned"]]
+        per_op = op_kernels(dn, acts)
         del acts
-        from paper_2004_11250_gb300 import ppconv as pp
-        per_op = [KERNEL_NAMES.get(pp.pp_layer_kernel(L.handle), "?") if not L.dense else "dense" for L in dn.layers]
-        kern = sorted(set(k for k in per_op if k != "dense"))
+        kern = sorted(set(k for k, s in zip(per_op, shapes) if s["pruned"]))
         tv = tensor_view(shapes, per_op, op_ms, [k for k, s in enumerate(shapes) if s["pruned"]], f16=precision == 1)
         graph_us = None
         if name == "single":
@@ -681,6 +707,7 @@ def main():
     torch.cuda.synchronize()
     op_ms = time_ops_in_frame(dn, acts, max(5, args.steps // 2), flush, stream)
     op_ms_alone = time_ops(dn, acts, max(5, args.steps // 2), flush, stream)
+    kern = op_kernels(dn, acts)
     del acts
     pruned = [k for k, s in enumerate(shapes) if s["pruned"]]
     kf = sum(shapes[k]["flops"] for k in pruned)
@@ -688,8 +715,6 @@ def main():
     achieved_all = kf / kt / 1e12
     # which kernel each op runs (autotuned by pp_net_finalize) and the tensor-pipe view
     from paper_2004_11250_gb300 import ppconv as pp
-    kern = [KERNEL_NAMES.get(pp.pp_layer_kernel(L.handle), "?") if not L.dense else "ppconv_kernel (dense)"
-            for L in dn.layers]
     # the flat kernel's tile geometry per op ("R:S", as --kernels flat:R:S takes it)
     geo = []
     for L, op, sh in zip(dn.layers, spec.ops, shapes):

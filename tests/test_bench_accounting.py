@@ -91,6 +91,13 @@ def test_source_hash_covers_every_convolution_kernel():
     assert with_kernels <= set(bench.KERNEL_SOURCES)
 
 
+def test_kernel_name_from_a_graph_dump():
+    dump = 'label="{KERNEL\n| {ID | 0 | _ZN44_GLOBAL__N__60_11_conv_%s_cu_89517%sILb0ELi64EEEvNS_9TcrParamsE\\<\\<\\<16,768\\>}"'
+    for name in ("ppconv_tcr_kernel", "ppconv_direct_first_kernel", "ppconv_kernel", "ppconv_tcf_kernel"):
+        assert bench.kernel_name(dump % (name[:3], name)) == name
+    assert bench.kernel_name("no launch") == "?"
+
+
 def test_traffic_read_only_for_matching_code(tmp_path, monkeypatch):
     """roofline.traffic comes from a committed summary only while that summary's recorded source hash is
     the current one; otherwise the bench reports null."""
