@@ -52,7 +52,9 @@
 // Epilogue: bias, +skip, ReLU, 2x2 max pool from tcgen05.ld, stores to each
 // filter's original channel.  tc_launch hands the pixel-major tiles that CTA
 // pairs run faster to conv_tcr.cu: 64-filter blocks (in fp16 up to 64 channels)
-// and 128-filter tf32 blocks with a pair weight layout.  This kernel has no channel split: layers with
+// and 128-filter tf32 blocks with a pair weight layout (so the tf32 64-filter
+// instantiation runs only without memory for that layout, or where pairs cannot
+// be launched).  This kernel has no channel split: layers with
 // more than 64 filters on maps at most 128 wide can also run the flat kernel
 // (conv_tcf.cu), which splits the chunks of small grids over a cluster.
 //

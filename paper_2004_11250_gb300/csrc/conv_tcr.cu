@@ -47,7 +47,7 @@
 // pipe.  Arrivals on the even CTA's barriers have the default scope: what they hand over (operands behind a proxy
 // fence, tensor memory) does not need the cluster-scope release, which waits for the thread's global stores.
 //
-// Measured, 64 -> 64 channels at 720 x 1280 (back to back): tf32 250 -> 219 us, f16 198 -> 149 us against the row-tiled
+// Measured, 64 -> 64 channels at 720 x 1280 (back to back): tf32 250 -> 219 us, f16 198 -> 143 us against the row-tiled
 // kernel; 321 x 481 (rows not 16-byte aligned), tf32, 89 -> 44 us.  tf32 is bound by the tensor pipe (197 us with every
 // load, store and epilogue left out: 110 clocks per tap and row, N = 64 MMAs taking 46 where 32 would be their rate);
 // f16 by the epilogue and loader instructions beside the MMAs (117-126 us with them left out).  Tried and slower in f16:
@@ -739,7 +739,8 @@ cudaError_t launch(const TcrParams& p, int pairs, cudaStream_t stream) {
                            : (int64_t)((p.ntiles + 1) / 2) * p.nfb;
   // No more pairs than the busiest one's share calls for, and in f16 at least two rows each (a row alone fetches three):
   // the SMs left over run what else is in flight (f16, three networks on streams of their own, a frame: 8 layers of 64
-  // channels at 205 x 59 95 -> 75 us, 7 at 54 x 220 56 -> 39; alone a layer takes 12.8 -> 12.0 and 10.0 -> 11.0).
+  // channels at 205 x 59 95 -> 75 us, 7 at 54 x 220 56 -> 39; alone a layer takes 12.8 -> 12.0 and 10.0 -> 11.0, the
+  // row-tiled kernel 18.1 and 14.4).
   const int64_t share = std::max<int64_t>((work + pairs - 1) / pairs, F16 && !POOL ? 2 : 1);
   cfg.gridDim = dim3((unsigned)(2 * ((work + share - 1) / share)));
   cfg.blockDim = dim3(NTHREADS);
