@@ -32,8 +32,8 @@
 // which halves the rounding error of one long sum (1.1e-7 against 2.2e-7 of the
 // result at 64 channels).
 //
-// ppconv_direct_wide_kernel: at most 3 filters on wide maps (a network's last
-// layer).  These read far more than they compute (64 -> 1 at 720 x 1280: 236 MB
+// ppconv_direct_wide_kernel: at most 3 filters on maps that its rows of 128 pixels
+// do not mostly miss (a network's last layer).  These read far more than they compute (64 -> 1 at 720 x 1280: 236 MB
 // of input), and with 2 x 2 blocks the shared-memory reads of the windows (16
 // for 36 FMAs) took longer than the copies.  A thread owns 4 x 4 pixels, a warp 4
 // rows of 128, so a window row is one 16-byte read and two shuffles for 12 FMAs a
@@ -996,22 +996,48 @@ pp_status direct_launch(const DirectLayout& D, const float* x, float* y, const f
   const auto ctas = [&](int th, int tw, int fbd) {
     return (int64_t)N * ((H + th - 1) / th) * ((W + tw - 1) / tw) * ((D.Co + fbd - 1) / fbd);
   };
-  cudaError_t e;
-  // The wide kernel by its tiles: one filter from two tiles for five SMs (64 -> 1 at 128 x 128, batch 8, 64 tiles: 16.0 us
-  // against the 2 x 2 kernel's 19.6; fewer: its split channels, 240 x 240, 30 tiles, 10.7 against 15.8), with more groups of warps the fewer there are (64 -> 1 at 360 x 640,
-  // 115 tiles: 1 / 2 / 4 groups 21.0 / 18.8 / 16.3, 2 x 2 kernel 27.2; 540 x 960, 272 tiles: 38.9 / 30.4 / 34.3, 42.9;
-  // 720 x 1280, 450 tiles: 40.6 / 46.3 / 51.2, 70.5).  Two filters share the 2 x 2 kernel's packed FMAs and need two
-  // tiles per SM to lose (43 against 51 - 61 at 540 x 960, 71 against 61 at 720 x 1280), three leave a fourth of them
-  // idle (40.5 against 35.3 at 360 x 640, 111 against 84), four never lose by it (111 against 115).  Without boxes (W not
-  // a multiple of 4) the copies bound it and two groups of warps gain nothing (64 -> 1 at 540 x 959 57.6 against 61.8,
-  // 64 -> 3 at 361 x 643 54.8, 2 x 2 kernel 48.4).
+  // 2 x 2 kernel, filters per CTA: as many as there are, up to 8; channel groups while the grid would leave SMs without two
+  // CTAs, and fewer filters (the input tile is then staged more often) only when even four groups leave a quarter of the
+  // SMs idle (64 -> 64 at 56 x 56, 128 CTAs of 8 filters: 13.5 us, of 4 filters 19.7).
+  int fbd = D.Co > 4 ? 8 : D.Co > 2 ? 4 : 2, ks = 1;
+  const auto grid = [&]() { return ctas(ks == 1 ? 32 : 16, ks == 4 ? 16 : 32, fbd); };
+  if (D.Ci > 4) {
+    if (grid() < 2 * sms) ks = 2;
+    if (grid() < 2 * sms) ks = 4;
+  }
+  while (fbd > 2 && grid() < (ks == 4 ? sms * 3 / 4 : 2 * sms)) fbd /= 2;
+
+  // The wide kernel where it has tiles for two SMs in five (64 -> 1 at 128 x 128, batch 8, 64 tiles: 16.0 us against the 2 x
+  // 2 kernel's 19.6), with more groups of warps the fewer there are (64 -> 1 at 360 x 640, 115 tiles: 1 / 2 / 4 groups 21.0
+  // / 18.8 / 16.3, 2 x 2 kernel 27.2; 540 x 960, 272 tiles: 38.9 / 30.4 / 34.3, 42.9; 720 x 1280, 450 tiles: 40.6 / 46.3 /
+  // 51.2, 70.5), and where its 128 columns are not spent on the map's edge: both kernels' time goes by the CTAs of the
+  // busiest SM, and the wide kernel's take about as long as the 2 x 2 kernel's with half as many pixels.  The figures
+  // below are us at 64 channels (they scale with the channels) on 252 maps of 8 .. 640 columns, where this choice is within
+  // 9 % of the better kernel; by tiles alone narrow maps took up to 4.9 times as long (64 -> 3 at 781 x 16, batch 4, 68.9
+  // against 13.9; 64 x 3125 157 against 96; 64 -> 1 at 6250 x 32 127 against 61).
   const int64_t vt = D.Ci >= 8 && D.Co <= 3 ? ctas(VH, VW, 4) : 0;
-  if (D.Co == 1 && vt * (p.vec ? 5 : 4) >= 2 * sms) {
+  const auto rounds = [&](int64_t n) { return (double)((n + sms - 1) / sms); };
+  bool wide = vt && (D.Co == 1   ? vt * (p.vec ? 5 : 4) >= 2 * sms
+                     : D.Co == 2 ? vt >= 2 * sms
+                                 : vt >= sms || (p.vec && vt * 3 >= sms * 2));
+  if (wide) {
+    const double c = rounds(vt);
+    const double tw = D.Co == 1 ? (p.vec ? (vt <= sms ? 16.2 : vt < 2 * sms ? 29.2 : 10.8 * c + 8.6)
+                                         : (vt < sms ? 28.3 : 22.2 * c + 11.0))
+                      : D.Co == 2 ? (p.vec ? 17.4 * c + 8.0 : 30.5 * c + 14.0)
+                                  : (p.vec ? (vt < 2 * sms ? 34.7 * c : 24.6 * c + 9.8)
+                                           : (vt < 2 * sms ? 53.4 * c : 39.2 * c + 13.0));
+    // us of one CTA for each SM, by channel groups (1, 2, 4): rows of whole 16-byte groups or not, 2 or 4 filters
+    static const double round_us[2][2][3] = {{{16.3, 9.6, 6.0}, {21.2, 12.5, 8.0}}, {{10.1, 6.6, 5.05}, {16.0, 10.4, 7.0}}};
+    wide = tw < round_us[p.vec][fbd > 2][ks == 4 ? 2 : ks - 1] * rounds(grid());
+  }
+  cudaError_t e;
+  if (wide && D.Co == 1) {
     e = vt >= (p.vec ? 2 : 1) * sms ? launch_wide<1, 1>(p, stream)
                                     : vt > sms ? launch_wide<1, 2>(p, stream) : launch_wide<1, 4>(p, stream);
-  } else if (D.Co == 2 && vt >= 2 * sms) {
+  } else if (wide && D.Co == 2) {
     e = launch_wide<2, 1>(p, stream);
-  } else if (D.Co == 3 && (vt >= sms || (p.vec && vt * 3 >= sms * 2))) {
+  } else if (wide) {
     e = vt >= 2 * sms ? launch_wide<3, 1>(p, stream) : launch_wide<3, 2>(p, stream);
   } else if (D.Ci <= 4 && W > UW / 2 && D.Co > 4 && D.Co <= 65535 && ctas(UH, UW, FBMAX) >= sms / 2) {
     // (1 -> 64 at 720 x 1280 48 us against 86 with the 32 x 32 tiles, 3 -> 64 at 224 x 224 7.2 against 9.1; below half
@@ -1025,16 +1051,6 @@ pp_status direct_launch(const DirectLayout& D, const float* x, float* y, const f
       default: e = launch_first<4>(p, fpc, stream); break;
     }
   } else {
-    // Filters per CTA: as many as there are, up to 8; channel groups while the grid would leave SMs without two CTAs,
-    // and fewer filters (the input tile is then staged more often) only when even four groups leave a quarter of the
-    // SMs idle (64 -> 64 at 56 x 56, 128 CTAs of 8 filters: 13.5 us, of 4 filters 19.7).
-    int fbd = D.Co > 4 ? 8 : D.Co > 2 ? 4 : 2, ks = 1;
-    const auto grid = [&]() { return ctas(ks == 1 ? 32 : 16, ks == 4 ? 16 : 32, fbd); };
-    if (D.Ci > 4) {
-      if (grid() < 2 * sms) ks = 2;
-      if (grid() < 2 * sms) ks = 4;
-    }
-    while (fbd > 2 && grid() < (ks == 4 ? sms * 3 / 4 : 2 * sms)) fbd /= 2;
     if (D.Ci <= 4) {
       switch (D.Ci) {
         case 1: e = launch_fbd<1, 1>(p, fbd, stream); break;

@@ -1267,6 +1267,7 @@ DIRECT_SHAPES = [
     (2, 8, 1, 720, 260), (1, 9, 2, 1250, 255), (3, 10, 3, 416, 256), (1, 16, 4, 2500, 130), (1, 8, 3, 16, 128),
     (1, 9, 1, 130, 1028), (1, 13, 1, 131, 1030), (1, 64, 1, 300, 1280), (1, 8, 1, 313, 1281), (1, 11, 3, 300, 700), (2, 9, 3, 160, 1284), (1, 10, 2, 520, 1284),
     (1, 9, 1, 719, 1284), (1, 12, 3, 701, 1100), (1, 11, 3, 700, 1101), (1, 10, 2, 521, 1285), (1, 17, 22, 290, 1100), (1, 18, 17, 291, 1101),
+    (1, 9, 1, 719, 1279), (4, 9, 1, 128, 390), (1, 10, 2, 720, 1280), (1, 10, 2, 719, 1279), (1, 11, 3, 719, 1279), (1, 9, 3, 640, 384),
     (1, 1, 64, 18, 129), (2, 2, 70, 64, 130), (1, 3, 130, 41, 200), (1, 4, 9, 300, 257), (1, 3, 33, 6, 66), (2, 1, 5, 2000, 68),
 ]
 
@@ -1337,8 +1338,8 @@ def test_streamed_weight_pairs(pp, runner, oracle_mod, tmp_path, case, flags):
 NONFINITE_SHAPES = [
     # N, Ci, Co, H, W
     (1, 17, 16, 260, 1032), (1, 20, 13, 260, 1030), (1, 24, 12, 160, 500), (2, 29, 9, 20, 21), (1, 64, 24, 30, 34),
-    (1, 100, 3, 17, 16), (1, 256, 1, 720, 1284), (1, 256, 1, 300, 1280), (1, 257, 1, 131, 1030), (1, 130, 2, 520, 1284),
-    (1, 91, 3, 300, 700), (1, 89, 3, 420, 1283),
+    (1, 100, 3, 17, 16), (1, 256, 1, 720, 1284), (1, 256, 1, 300, 1280), (1, 257, 1, 130, 1028), (1, 130, 2, 720, 1280),
+    (1, 91, 3, 640, 384), (1, 89, 3, 719, 1279),
 ]
 
 
@@ -1623,3 +1624,21 @@ def test_flat_unsplit_ragged_rows_form(pp, runner, oracle_mod, tmp_path, flags, 
     finally:
         d.close()
     check_within(out.cpu().numpy(), y, s, f"unsplit tile, ragged rows, {flags}")
+
+
+@pytest.mark.parametrize("shape,wide", [
+    ((1, 64, 1, 720, 1280), True), ((1, 64, 1, 360, 640), True), ((1, 64, 2, 720, 1280), True), ((1, 64, 3, 720, 1280), True),
+    ((1, 64, 1, 719, 1279), True), ((4, 64, 1, 1785, 112), True), ((4, 64, 1, 3125, 64), False), ((4, 64, 1, 6250, 32), False),
+    ((4, 64, 3, 3125, 64), False), ((4, 64, 2, 12500, 16), False), ((8, 64, 3, 96, 40), False), ((4, 64, 3, 384, 130), False),
+    ((4, 64, 1, 312, 160), False), ((4, 64, 1, 769, 65), False),
+])
+def test_wide_direct_kernel_by_map(pp, runner, tmp_path, shape, wide):
+    """Layers of at most 3 filters run the direct kernel with 128-pixel rows only on maps that its rows do not mostly miss."""
+    N, Ci, Co, H, W = shape
+    d = runner.DeviceLayer(synth.make_dense_layer(np.random.default_rng(131), Co, Ci, synth.he_std(Ci), 0.01))
+    try:
+        x, y = torch.zeros((N, Ci, H, W), device="cuda"), torch.empty((N, Co, H, W), device="cuda")
+        names = launched(lambda: d.forward(x, y, None, N, H, W, 0, torch.cuda.current_stream()), tmp_path)
+    finally:
+        d.close()
+    assert len(names) == 1 and ("ppconv_direct_wide_kernel" in names[0]) == wide, names
