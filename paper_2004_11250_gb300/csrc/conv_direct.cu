@@ -46,7 +46,7 @@
 // input, residual and output, where HBM bounds it; at 360 x 640 27.2 -> 16.3.
 //
 // ppconv_direct_first_kernel: at most 4 input channels (a network's first
-// layer) on maps wider than a tile's half.  These write far more than they read:
+// layer) on maps wider than a tile's half whose columns its tiles do not miss too much of.  These write far more than they read:
 // a CTA stages its tile's input once for up to 64 filters, 8 at a time, and a
 // thread's 2 x 4 pixels leave in 16-byte stores.
 #include <cuda_runtime.h>
@@ -266,8 +266,10 @@ struct DirectGeo {
   static_assert(CC % KS == 0 && FBD % 2 == 0, "channels over the groups, filters in pairs");
 };
 
+// Fewer than 4 channels are one chunk: latency decides, and a third CTA per SM hides it (1 -> 64 at 446 x 56, batch 2, 8.4 us
+// against 6.1, although 8 filters of 2 or 3 channels then spill some 100 bytes).
 template <int CC, int FBD, int KS, bool BOX, bool REDO>
-__global__ void __launch_bounds__(DTHREADS, 2) ppconv_direct_kernel(const DirectParams p, const __grid_constant__ BoxMap<BOX> xmap) {
+__global__ void __launch_bounds__(DTHREADS, CC < 4 ? 3 : 2) ppconv_direct_kernel(const DirectParams p, const __grid_constant__ BoxMap<BOX> xmap) {
   using G = DirectGeo<CC, FBD, KS>;
   constexpr int NP = FBD / 2, GT = DTHREADS / KS, TX = G::TW / 2;
   // boxes start at 128 bytes, so the weights lie after them all; else in their stage
@@ -1039,9 +1041,12 @@ pp_status direct_launch(const DirectLayout& D, const float* x, float* y, const f
     e = launch_wide<2, 1>(p, stream);
   } else if (wide) {
     e = vt >= 2 * sms ? launch_wide<3, 1>(p, stream) : launch_wide<3, 2>(p, stream);
-  } else if (D.Ci <= 4 && W > UW / 2 && D.Co > 4 && D.Co <= 65535 && ctas(UH, UW, FBMAX) >= sms / 2) {
+  } else if (D.Ci <= 4 && W > UW / 2 && D.Co > 4 && D.Co <= 65535 && ctas(UH, UW, FBMAX) >= sms / 2 &&
+             10 * ((W + UW - 1) / UW * UW) < 13 * ((W + 31) / 32 * 32)) {
     // (1 -> 64 at 720 x 1280 48 us against 86 with the 32 x 32 tiles, 3 -> 64 at 224 x 224 7.2 against 9.1; below half
-    // a CTA per SM the smaller tiles win: 1 -> 64 at 64 x 96, 64 CTAs, 3.0 against 2.7)
+    // a CTA per SM the smaller tiles win: 1 -> 64 at 64 x 96, 64 CTAs, 3.0 against 2.7; where its rows of 128 pixels are
+    // 1.3 times the columns that the others pad to, or more, these: 4 -> 64 at 625 x 160, batch 2, 52 against 33, 1 -> 16
+    // at 666 x 150 8.7 against 6.7)
     int fpc = UFMAX;
     while (fpc > FBMAX && ctas(UH, UW, fpc) < 2 * sms) fpc /= 2;
     switch (D.Ci) {

@@ -1269,6 +1269,7 @@ DIRECT_SHAPES = [
     (1, 9, 1, 719, 1284), (1, 12, 3, 701, 1100), (1, 11, 3, 700, 1101), (1, 10, 2, 521, 1285), (1, 17, 22, 290, 1100), (1, 18, 17, 291, 1101),
     (1, 9, 1, 719, 1279), (4, 9, 1, 128, 390), (1, 10, 2, 720, 1280), (1, 10, 2, 719, 1279), (1, 11, 3, 719, 1279), (1, 9, 3, 640, 384),
     (1, 1, 64, 18, 129), (2, 2, 70, 64, 130), (1, 3, 130, 41, 200), (1, 4, 9, 300, 257), (1, 3, 33, 6, 66), (2, 1, 5, 2000, 68),
+    (2, 2, 70, 64, 128), (1, 4, 9, 600, 255), (2, 1, 5, 2000, 100), (1, 2, 40, 800, 150), (1, 3, 33, 900, 160), (1, 4, 12, 900, 160),
 ]
 
 
@@ -1642,3 +1643,20 @@ def test_wide_direct_kernel_by_map(pp, runner, tmp_path, shape, wide):
     finally:
         d.close()
     assert len(names) == 1 and ("ppconv_direct_wide_kernel" in names[0]) == wide, names
+
+
+@pytest.mark.parametrize("shape,first", [
+    ((1, 1, 64, 720, 1280), True), ((1, 3, 64, 224, 224), True), ((2, 3, 64, 200, 100), True), ((1, 4, 32, 300, 300), True),
+    ((2, 4, 64, 625, 160), False), ((2, 1, 16, 666, 150), False), ((2, 3, 64, 156, 160), False), ((2, 1, 64, 96, 258), False),
+    ((2, 3, 64, 200, 64), False),
+])
+def test_first_layer_direct_kernel_by_map(pp, runner, tmp_path, shape, first):
+    """Layers of at most 4 channels run the kernel with 128-pixel rows only on maps that its rows do not miss too much of."""
+    N, Ci, Co, H, W = shape
+    d = runner.DeviceLayer(synth.make_dense_layer(np.random.default_rng(137), Co, Ci, synth.he_std(Ci), 0.01))
+    try:
+        x, y = torch.zeros((N, Ci, H, W), device="cuda"), torch.empty((N, Co, H, W), device="cuda")
+        names = launched(lambda: d.forward(x, y, None, N, H, W, 0, torch.cuda.current_stream()), tmp_path)
+    finally:
+        d.close()
+    assert len(names) == 1 and ("ppconv_direct_first_kernel" in names[0]) == first, names
