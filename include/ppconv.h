@@ -270,8 +270,10 @@ pp_status pp_layer_precision(const pp_layer* layer, int* precision, float* input
  *                       ring patterns).
  * PP_KERNEL_AUTO picks by an estimate of each kernel's time for the layer's
  * density (the direct kernel for Ci <= 4, and in place of an FMA kernel that it
- * beats on maps of any size).  Setting a kernel the layer cannot run returns
- * PP_ERR_UNSUPPORTED; what pp_layer_kernel reports can be set.  The tensor-core
+ * beats: on maps of any size, or, where pp_layer_kernel reports TMEM or REGISTER,
+ * on the maps where it is estimated to).  Setting a kernel the layer cannot run returns
+ * PP_ERR_UNSUPPORTED; what pp_layer_kernel reports can be set, and then runs on
+ * every map.  The tensor-core
  * kernels, and the direct kernel on layers of the former kind only (at most 16
  * channels on a side), multiply pruned taps as zeros: an input that is not
  * finite then also reaches outputs whose kept taps do not touch it.  The other
@@ -284,7 +286,8 @@ pp_status pp_layer_precision(const pp_layer* layer, int* precision, float* input
 #define PP_KERNEL_TC_FLAT 4
 #define PP_KERNEL_DIRECT 5
 pp_status pp_layer_set_kernel(pp_layer* layer, int kernel);
-/* The kernel that pp_conv_forward will run (one of the PP_KERNEL_ values above, not _AUTO). */
+/* The kernel that pp_conv_forward will run (one of the PP_KERNEL_ values above, not _AUTO); by default on
+ * some maps the direct kernel in place of TMEM or REGISTER, see PP_KERNEL_AUTO. */
 pp_status pp_layer_kernel(const pp_layer* layer, int* kernel);
 /* Time the kernels that can run this layer (tensor-core, TMEM and direct
  * kernels where their layouts exist; the register kernel only when none of

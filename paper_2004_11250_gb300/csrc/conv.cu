@@ -396,6 +396,9 @@ struct pp_layer {
   bool tc_ok = false;    // the tensor-core kernel can run it
   int kernel = 2;        // PP_KERNEL_TMEM / _REGISTER / _TC
   int auto_kernel = 2;
+  // The default choice is an FMA kernel over the kept taps with the direct kernel as a candidate: each launch takes the one
+  // that the estimates find faster on its map.  Off once a kernel is set or tuned.
+  bool by_map = false, by_map_default = false;
   ppc::TmLayout tm;
   ppc::TcLayout tc;
   ppc::DirectLayout direct;  // built for layers with few input or output channels and where an FMA kernel is the choice
@@ -546,26 +549,32 @@ int choose_split(int64_t base_ctas, int nch) {
   return ks;
 }
 
-pp_status launch(const pp_layer* L, const float* x, float* y, const float* skip, int N, int H, int W, int flags,
-                 cudaStream_t stream) {
-  if (!L || !x || !y || N < 1 || H < 1 || W < 1) return PP_ERR_INVALID_ARG;
-  if (flags & ~(PP_ADD_SKIP | PP_RELU | PP_POOL2)) return PP_ERR_INVALID_ARG;
-  if ((flags & PP_ADD_SKIP) && !skip) return PP_ERR_INVALID_ARG;
-  if ((flags & PP_POOL2) && ((H & 1) || (W & 1))) return PP_ERR_UNSUPPORTED;
-  if (((uintptr_t)y & 15) || ((uintptr_t)x & 3)) return PP_ERR_INVALID_ARG;
-  if (L->kernel == PP_KERNEL_DIRECT) return ppc::direct_launch(L->direct, x, y, skip, N, H, W, flags, stream);
-  if (L->kernel == PP_KERNEL_TMEM || L->kernel == PP_KERNEL_TC || L->kernel == PP_KERNEL_TC_FLAT) {
+// us of a launch of the register kernel: within 32 % for nine in ten of 184 random layers and maps that it was not fitted to
+// (5 .. 512 channels, 4 .. 253 filters, 5 x 5 to 800 x 1300).
+double register_estimate_us(const pp_layer* L, int N, int H, int W) {
+  const int64_t base = (int64_t)((H + TH - 1) / TH) * ((W + TW - 1) / TW) * ((L->G + NWF - 1) / NWF) * N;
+  const int ks = choose_split(base, L->nch);
+  const double waves = (double)((base * ks + 2 * 152 - 1) / (2 * 152)), chunks = (double)((L->nch + ks - 1) / ks);
+  const double entries = (double)L->nE / L->G / L->nch;  // of a warp in a chunk
+  return 1.0 + waves * (8.0 + chunks * (3.2 + 0.73 * entries + ((W & 3) ? 0.42 : 0.0))) *
+                   (1.0 + 0.15 * (std::min(NWF, L->G) - 1));
+}
+
+pp_status run_kernel(const pp_layer* L, int kernel, const float* x, float* y, const float* skip, int N, int H, int W,
+                     int flags, cudaStream_t stream) {
+  if (kernel == PP_KERNEL_DIRECT) return ppc::direct_launch(L->direct, x, y, skip, N, H, W, flags, stream);
+  if (kernel == PP_KERNEL_TMEM || kernel == PP_KERNEL_TC || kernel == PP_KERNEL_TC_FLAT) {
     ppc::LayerMeta M;
     M.Co = L->Co;
     M.Ci = L->Ci;
     M.perm = L->perm;
     M.bias = L->has_bias ? L->bias : nullptr;
-    if (L->kernel == PP_KERNEL_TC_FLAT) {
+    if (kernel == PP_KERNEL_TC_FLAT) {
       const pp_status st = ppc::tcf_launch(L->tc, M, x, y, skip, N, H, W, flags, stream);
       if (st != PP_ERR_UNSUPPORTED) return st;
       // maps wider than the flat kernel's tiles run the row-tiled tensor-core kernel
     }
-    if (L->kernel == PP_KERNEL_TC || L->kernel == PP_KERNEL_TC_FLAT) {
+    if (kernel == PP_KERNEL_TC || kernel == PP_KERNEL_TC_FLAT) {
       const pp_status st = ppc::tc_launch(L->tc, M, x, y, skip, N, H, W, flags, stream);
       if (st != PP_ERR_UNSUPPORTED) return st;
       // shapes beyond the tensor-core kernel's 32-bit offsets run on an FMA kernel
@@ -626,6 +635,30 @@ pp_status launch(const pp_layer* L, const float* x, float* y, const float* skip,
     return PP_ERR_CUDA;
   }
   return PP_OK;
+}
+
+// Where neither kernel wins on every map (by_map): the direct kernel unless its estimate is the larger.  Over the better
+// kernel's time, geometric mean and worst of 542 random layers and maps beside the TMEM kernel: the choice 1.009 and 1.32,
+// the direct kernel alone 1.05 and 2.5, the TMEM kernel alone 1.60 and 7.2; of 184 beside the register kernel: 1.008 and
+// 1.34, 1.08 and 2.5, 1.86 and 10.7.
+bool direct_on_map(const pp_layer* L, int N, int H, int W) {
+  const double other = L->kernel == PP_KERNEL_TMEM ? ppc::tm_estimate_us(L->tm, L->nE, N, H, W)
+                                                   : register_estimate_us(L, N, H, W);
+  return ppc::direct_estimate_us(L->direct, N, H, W) <= other;
+}
+
+pp_status launch(const pp_layer* L, const float* x, float* y, const float* skip, int N, int H, int W, int flags,
+                 cudaStream_t stream) {
+  if (!L || !x || !y || N < 1 || H < 1 || W < 1) return PP_ERR_INVALID_ARG;
+  if (flags & ~(PP_ADD_SKIP | PP_RELU | PP_POOL2)) return PP_ERR_INVALID_ARG;
+  if ((flags & PP_ADD_SKIP) && !skip) return PP_ERR_INVALID_ARG;
+  if ((flags & PP_POOL2) && ((H & 1) || (W & 1))) return PP_ERR_UNSUPPORTED;
+  if (((uintptr_t)y & 15) || ((uintptr_t)x & 3)) return PP_ERR_INVALID_ARG;
+  const int kernel = L->by_map && direct_on_map(L, N, H, W) ? PP_KERNEL_DIRECT : L->kernel;
+  const pp_status st = run_kernel(L, kernel, x, y, skip, N, H, W, flags, stream);
+  if (st != PP_ERR_UNSUPPORTED || !L->by_map) return st;
+  // batches and maps beyond one kernel's grid run the other
+  return run_kernel(L, kernel == L->kernel ? PP_KERNEL_DIRECT : L->kernel, x, y, skip, N, H, W, flags, stream);
 }
 
 }  // namespace
@@ -699,7 +732,7 @@ extern "C" pp_status pp_layer_create(const pp_packed* pk, const float* bias, voi
   L->auto_kernel = (L->tc_ok && tc_cycles < fma_cycles) ? (L->tc.FB == 128 ? PP_KERNEL_TC_FLAT : PP_KERNEL_TC)
                                                          : (L->tm_ok ? PP_KERNEL_TMEM : PP_KERNEL_REGISTER);
   // Where the estimate wants FP32, the direct kernel's 9 taps on packed FMAs are a candidate (its layout is built), and take
-  // the place of
+  // the place of the others on maps where an estimate finds it faster (by_map), and on every map of
   //  * the register kernel's dispatch where they are no slower on any map from 7 x 7 to 1080 x 1920.  Their time does not
   //    depend on the density, the register kernel's does: 64 -> 24 at 128 x 128 21 us against 18 / 26 / 33 / 52 / 105 at
   //    keep 0.02 / 0.05 / 0.1 / 0.2 / 0.5; more filters need more (64 -> 64 on its worst map, keep 0.1 / 0.12: 1.03 / 0.91
@@ -753,6 +786,7 @@ extern "C" pp_status pp_layer_create(const pp_packed* pk, const float* bias, voi
   }
   L->pk_perm = pk->perm;
   L->kernel = L->auto_kernel;
+  L->by_map = L->by_map_default = redo && L->direct.w && L->auto_kernel != PP_KERNEL_DIRECT;
   *out = L;
   return PP_OK;
 }
@@ -815,27 +849,20 @@ extern "C" pp_status pp_layer_precision(const pp_layer* L, int* precision, float
 
 extern "C" pp_status pp_layer_set_kernel(pp_layer* L, int kernel) {
   if (!L) return PP_ERR_INVALID_ARG;
+  bool can = true;
   switch (kernel) {
-    case PP_KERNEL_AUTO: L->kernel = L->auto_kernel; return PP_OK;
-    case PP_KERNEL_TMEM:
-      if (!L->tm_ok) return PP_ERR_UNSUPPORTED;
-      L->kernel = kernel;
-      return PP_OK;
-    case PP_KERNEL_TC:
-      if (!L->tc_ok) return PP_ERR_UNSUPPORTED;
-      L->kernel = kernel;
-      return PP_OK;
-    case PP_KERNEL_TC_FLAT:
-      if (!L->tc_ok || L->tc.FB != 128) return PP_ERR_UNSUPPORTED;
-      L->kernel = kernel;
-      return PP_OK;
-    case PP_KERNEL_REGISTER: L->kernel = kernel; return PP_OK;
-    case PP_KERNEL_DIRECT:
-      if (!L->direct.w) return PP_ERR_UNSUPPORTED;
-      L->kernel = kernel;
-      return PP_OK;
+    case PP_KERNEL_AUTO:
+    case PP_KERNEL_REGISTER: break;
+    case PP_KERNEL_TMEM: can = L->tm_ok; break;
+    case PP_KERNEL_TC: can = L->tc_ok; break;
+    case PP_KERNEL_TC_FLAT: can = L->tc_ok && L->tc.FB == 128; break;
+    case PP_KERNEL_DIRECT: can = L->direct.w != nullptr; break;
     default: return PP_ERR_INVALID_ARG;
   }
+  if (!can) return PP_ERR_UNSUPPORTED;
+  L->kernel = kernel == PP_KERNEL_AUTO ? L->auto_kernel : kernel;
+  L->by_map = kernel == PP_KERNEL_AUTO && L->by_map_default;
+  return PP_OK;
 }
 
 extern "C" pp_status pp_layer_kernel(const pp_layer* L, int* kernel) {
@@ -875,7 +902,10 @@ extern "C" pp_status pp_layer_autotune(pp_layer* L, int N, int H, int W, int fla
   };
   if (cand.size() == 1) {
     const pp_status e = cand[0].kernel == PP_KERNEL_TC ? make_pairs() : PP_OK;
-    if (e == PP_OK) L->kernel = cand[0].kernel;
+    if (e == PP_OK) {
+      L->kernel = cand[0].kernel;
+      L->by_map = false;
+    }
     return e;
   }
   const size_t in_elems = (size_t)N * L->Ci * H * W, out_elems = (size_t)N * L->Co * H * W;
@@ -894,6 +924,8 @@ extern "C" pp_status pp_layer_autotune(pp_layer* L, int N, int H, int W, int fla
   cudaEvent_t e0 = nullptr, e1 = nullptr;
   if (st == PP_OK && (cudaEventCreate(&e0) != cudaSuccess || cudaEventCreate(&e1) != cudaSuccess)) st = PP_ERR_CUDA;
   const int saved = L->kernel;
+  const bool saved_by_map = L->by_map;
+  L->by_map = false;
   Cand best = {saved, 0, 0};
   float best_ms = 1e30f, tc_ms = 1e30f;
   for (const Cand& c : cand) {
@@ -928,6 +960,7 @@ extern "C" pp_status pp_layer_autotune(pp_layer* L, int N, int H, int W, int fla
   // replaces the row-tiled one only when it is more than 10 % faster alone.
   if (best.kernel == PP_KERNEL_TC_FLAT && tc_ms <= 1.1f * best_ms) best = {PP_KERNEL_TC, 0, 0};
   L->kernel = st == PP_OK ? best.kernel : saved;
+  if (st != PP_OK) L->by_map = saved_by_map;
   // the flat kernel keeps the geometry that won for this shape (none if it lost)
   if (L->tc_ok && L->tc.FB == 128)
     ppc::tcf_pin(L->tc, N, H, W, flags, st == PP_OK && best.kernel == PP_KERNEL_TC_FLAT ? best.R : 0, best.S);

@@ -972,6 +972,84 @@ pp_status direct_update(const DirectLayout& D, const float* w_dense, const uint1
   return PP_OK;
 }
 
+// CTAs of tiles of th x tw pixels and f filters.
+static int64_t tiles(const DirectLayout& D, int N, int H, int W, int th, int tw, int f) {
+  return (int64_t)N * ((H + th - 1) / th) * ((W + tw - 1) / tw) * ((D.Co + f - 1) / f);
+}
+
+// Which of the 2 x 2 and wide kernels a layer runs on a map, and in which form.
+struct Plan {
+  int fbd = 0, ks = 1;   // 2 x 2 kernel: filters per CTA, channel groups
+  int64_t grid = 0;      // and its CTAs
+  int64_t vt = 0;        // tiles of the wide kernel, 0 for layers that it does not run
+  bool wide = false;
+  double wide_us = 0;    // its time at 64 channels where it was considered
+};
+static Plan make_plan(const DirectLayout& D, int N, int H, int W, bool vec, int64_t sms) {
+  Plan pl;
+  const auto ctas = [&](int th, int tw, int f) { return tiles(D, N, H, W, th, tw, f); };
+  // 2 x 2 kernel, filters per CTA: as many as there are, up to 8; channel groups while the grid would leave SMs without two
+  // CTAs, and fewer filters (the input tile is then staged more often) only when even four groups leave a quarter of the
+  // SMs idle (64 -> 64 at 56 x 56, 128 CTAs of 8 filters: 13.5 us, of 4 filters 19.7).
+  int fbd = D.Co > 4 ? 8 : D.Co > 2 ? 4 : 2, ks = 1;
+  const auto grid = [&]() { return ctas(ks == 1 ? 32 : 16, ks == 4 ? 16 : 32, fbd); };
+  if (D.Ci > 4) {
+    if (grid() < 2 * sms) ks = 2;
+    if (grid() < 2 * sms) ks = 4;
+  }
+  while (fbd > 2 && grid() < (ks == 4 ? sms * 3 / 4 : 2 * sms)) fbd /= 2;
+
+  // The wide kernel where it has tiles for two SMs in five (64 -> 1 at 128 x 128, batch 8, 64 tiles: 16.0 us against the 2 x
+  // 2 kernel's 19.6), with more groups of warps the fewer there are (64 -> 1 at 360 x 640, 115 tiles: 1 / 2 / 4 groups 21.0
+  // / 18.8 / 16.3, 2 x 2 kernel 27.2; 540 x 960, 272 tiles: 38.9 / 30.4 / 34.3, 42.9; 720 x 1280, 450 tiles: 40.6 / 46.3 /
+  // 51.2, 70.5), and where its 128 columns are not spent on the map's edge: both kernels' time goes by the CTAs of the
+  // busiest SM, and the wide kernel's take about as long as the 2 x 2 kernel's with half as many pixels.  The figures
+  // below are us at 64 channels (they scale with the channels) on 252 maps of 8 .. 640 columns, where this choice is within
+  // 9 % of the better kernel; by tiles alone narrow maps took up to 4.9 times as long (64 -> 3 at 781 x 16, batch 4, 68.9
+  // against 13.9; 64 x 3125 157 against 96; 64 -> 1 at 6250 x 32 127 against 61).
+  const int64_t vt = D.Ci >= 8 && D.Co <= 3 ? ctas(VH, VW, 4) : 0;
+  const auto rounds = [&](int64_t n) { return (double)((n + sms - 1) / sms); };
+  bool wide = vt && (D.Co == 1   ? vt * (vec ? 5 : 4) >= 2 * sms
+                     : D.Co == 2 ? vt >= 2 * sms
+                                 : vt >= sms || (vec && vt * 3 >= sms * 2));
+  if (wide) {
+    const double c = rounds(vt);
+    const double tw = D.Co == 1 ? (vec ? (vt <= sms ? 16.2 : vt < 2 * sms ? 29.2 : 10.8 * c + 8.6)
+                                         : (vt < sms ? 28.3 : 22.2 * c + 11.0))
+                      : D.Co == 2 ? (vec ? 17.4 * c + 8.0 : 30.5 * c + 14.0)
+                                  : (vec ? (vt < 2 * sms ? 34.7 * c : 24.6 * c + 9.8)
+                                           : (vt < 2 * sms ? 53.4 * c : 39.2 * c + 13.0));
+    // us of one CTA for each SM, by channel groups (1, 2, 4): rows of whole 16-byte groups or not, 2 or 4 filters
+    static const double round_us[2][2][3] = {{{16.3, 9.6, 6.0}, {21.2, 12.5, 8.0}}, {{10.1, 6.6, 5.05}, {16.0, 10.4, 7.0}}};
+    pl.wide_us = tw;
+    wide = tw < round_us[vec ? 1 : 0][fbd > 2][ks == 4 ? 2 : ks - 1] * rounds(grid());
+  }
+  pl.fbd = fbd;
+  pl.ks = ks;
+  pl.grid = grid();
+  pl.vt = vt;
+  pl.wide = wide;
+  return pl;
+}
+
+// us of a launch with more than 4 channels: within 12 % for nine in ten of 726 random pruned layers and maps that it was not
+// fitted to (5 .. 512 channels, 1 .. 253 filters, 5 x 5 to 800 x 1300): a pass over the channels and a round of CTAs over
+// the SMs, both in proportion to the channels.
+double direct_estimate_us(const DirectLayout& D, int N, int H, int W) {
+  const int64_t sms = device_sms();
+  if (sms <= 0) return 0.0;
+  const Plan pl = make_plan(D, N, H, W, (W & 3) == 0, sms);
+  if (pl.wide) return 2.2 + D.Ci / 64.0 * pl.wide_us;
+  static const double pass_us[3] = {0.7, 4.0, 3.0};  // 64 channels, by groups (1, 2, 4)
+  // by filters (2, 4, 8), groups, rows of whole 16-byte groups or not
+  static const double round_us[3][3][2] = {{{10.1, 16.3}, {4.6, 6.6}, {2.5, 3.6}},
+                                           {{15.3, 20.6}, {8.3, 10.4}, {4.5, 5.7}},
+                                           {{27.3, 32.0}, {14.2, 16.6}, {8.2, 9.6}}};
+  const int f = pl.fbd == 2 ? 0 : pl.fbd == 4 ? 1 : 2, k = pl.ks == 4 ? 2 : pl.ks - 1;
+  return 2.2 + ((D.Ci + 3) / 4) / 16.0 *
+                   (pass_us[k] + (double)((pl.grid + sms - 1) / sms) * round_us[f][k][(W & 3) ? 1 : 0]);
+}
+
 pp_status direct_launch(const DirectLayout& D, const float* x, float* y, const float* skip, int N, int H, int W,
                         int flags, cudaStream_t stream) {
   if (!D.w) return PP_ERR_UNSUPPORTED;
@@ -995,44 +1073,11 @@ pp_status direct_launch(const DirectLayout& D, const float* x, float* y, const f
   p.npair = D.npair;
   p.tiles_x = p.tiles_y = 0;
   p.vec = (W & 3) == 0 && ((uintptr_t)x & 15) == 0 && (int64_t)H * W <= INT32_MAX;
-  const auto ctas = [&](int th, int tw, int fbd) {
-    return (int64_t)N * ((H + th - 1) / th) * ((W + tw - 1) / tw) * ((D.Co + fbd - 1) / fbd);
-  };
-  // 2 x 2 kernel, filters per CTA: as many as there are, up to 8; channel groups while the grid would leave SMs without two
-  // CTAs, and fewer filters (the input tile is then staged more often) only when even four groups leave a quarter of the
-  // SMs idle (64 -> 64 at 56 x 56, 128 CTAs of 8 filters: 13.5 us, of 4 filters 19.7).
-  int fbd = D.Co > 4 ? 8 : D.Co > 2 ? 4 : 2, ks = 1;
-  const auto grid = [&]() { return ctas(ks == 1 ? 32 : 16, ks == 4 ? 16 : 32, fbd); };
-  if (D.Ci > 4) {
-    if (grid() < 2 * sms) ks = 2;
-    if (grid() < 2 * sms) ks = 4;
-  }
-  while (fbd > 2 && grid() < (ks == 4 ? sms * 3 / 4 : 2 * sms)) fbd /= 2;
-
-  // The wide kernel where it has tiles for two SMs in five (64 -> 1 at 128 x 128, batch 8, 64 tiles: 16.0 us against the 2 x
-  // 2 kernel's 19.6), with more groups of warps the fewer there are (64 -> 1 at 360 x 640, 115 tiles: 1 / 2 / 4 groups 21.0
-  // / 18.8 / 16.3, 2 x 2 kernel 27.2; 540 x 960, 272 tiles: 38.9 / 30.4 / 34.3, 42.9; 720 x 1280, 450 tiles: 40.6 / 46.3 /
-  // 51.2, 70.5), and where its 128 columns are not spent on the map's edge: both kernels' time goes by the CTAs of the
-  // busiest SM, and the wide kernel's take about as long as the 2 x 2 kernel's with half as many pixels.  The figures
-  // below are us at 64 channels (they scale with the channels) on 252 maps of 8 .. 640 columns, where this choice is within
-  // 9 % of the better kernel; by tiles alone narrow maps took up to 4.9 times as long (64 -> 3 at 781 x 16, batch 4, 68.9
-  // against 13.9; 64 x 3125 157 against 96; 64 -> 1 at 6250 x 32 127 against 61).
-  const int64_t vt = D.Ci >= 8 && D.Co <= 3 ? ctas(VH, VW, 4) : 0;
-  const auto rounds = [&](int64_t n) { return (double)((n + sms - 1) / sms); };
-  bool wide = vt && (D.Co == 1   ? vt * (p.vec ? 5 : 4) >= 2 * sms
-                     : D.Co == 2 ? vt >= 2 * sms
-                                 : vt >= sms || (p.vec && vt * 3 >= sms * 2));
-  if (wide) {
-    const double c = rounds(vt);
-    const double tw = D.Co == 1 ? (p.vec ? (vt <= sms ? 16.2 : vt < 2 * sms ? 29.2 : 10.8 * c + 8.6)
-                                         : (vt < sms ? 28.3 : 22.2 * c + 11.0))
-                      : D.Co == 2 ? (p.vec ? 17.4 * c + 8.0 : 30.5 * c + 14.0)
-                                  : (p.vec ? (vt < 2 * sms ? 34.7 * c : 24.6 * c + 9.8)
-                                           : (vt < 2 * sms ? 53.4 * c : 39.2 * c + 13.0));
-    // us of one CTA for each SM, by channel groups (1, 2, 4): rows of whole 16-byte groups or not, 2 or 4 filters
-    static const double round_us[2][2][3] = {{{16.3, 9.6, 6.0}, {21.2, 12.5, 8.0}}, {{10.1, 6.6, 5.05}, {16.0, 10.4, 7.0}}};
-    wide = tw < round_us[p.vec][fbd > 2][ks == 4 ? 2 : ks - 1] * rounds(grid());
-  }
+  const Plan pl = make_plan(D, N, H, W, p.vec, sms);
+  const int64_t vt = pl.vt;
+  const bool wide = pl.wide;
+  const int fbd = pl.fbd, ks = pl.ks;
+  const auto ctas = [&](int th, int tw, int f) { return tiles(D, N, H, W, th, tw, f); };
   cudaError_t e;
   if (wide && D.Co == 1) {
     e = vt >= (p.vec ? 2 : 1) * sms ? launch_wide<1, 1>(p, stream)

@@ -168,6 +168,7 @@ pp_status direct_update(const DirectLayout& D, const float* w_dense, const uint1
                         cudaStream_t stream);
 pp_status direct_launch(const DirectLayout& D, const float* x, float* y, const float* skip, int N, int H, int W,
                         int flags, cudaStream_t stream);
+double direct_estimate_us(const DirectLayout& D, int N, int H, int W);
 void direct_free(DirectLayout* D);
 
 // True when every pattern of the set is one of the ring patterns (centre plus
@@ -175,6 +176,7 @@ void direct_free(DirectLayout* D);
 bool tm_supports(const uint8_t* taps, int P, std::vector<int>& ring_of);
 pp_status tm_prepare();
 pp_status tm_build(TmLayout* T, const pp_packed* pk, const std::vector<int>& ring_of, cudaStream_t stream);
+double tm_estimate_us(const TmLayout& T, int64_t kernels, int N, int H, int W);  // at most 32 filters
 pp_status tm_launch(const TmLayout& T, const LayerMeta& M, const float* x, float* y, const float* skip, int N,
                     int H, int W, int flags, cudaStream_t stream);
 

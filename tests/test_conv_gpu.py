@@ -125,6 +125,24 @@ def test_register_kernel_on_ring_layers(pp, runner, oracle_mod, case, flags):
 
 @pytest.mark.parametrize("case", SMALL)
 @pytest.mark.parametrize("flags", ["none", "skip_relu", "pool_relu"])
+def test_kept_tap_kernels(pp, runner, oracle_mod, case, flags):
+    """The tensor-memory kernel on every small ring case, the register kernel on the others: by default many of these maps
+    run the direct kernel."""
+    N, Ci, Co, H, W, P, ring, keep = case
+    if flags == "pool_relu" and (H % 2 or W % 2):
+        pytest.skip("pool needs even sizes")
+    rng = np.random.default_rng(5 * sum(case[:5]) + len(flags))
+    L = synth.small_random_layer(rng, Co, Ci, P=P, keep=keep, ring=ring)
+    x = rng.uniform(-1, 1, (N, Ci, H, W)).astype(np.float32)
+    skip = rng.uniform(-1, 1, (N, Co, H, W)).astype(np.float32) if flags == "skip_relu" else None
+    g = run_layer(pp, runner, L, x, skip, flags != "none", flags == "pool_relu",
+                  kernel=pp.PP_KERNEL_TMEM if ring else pp.PP_KERNEL_REGISTER)
+    y, s = oracle_layer_full(oracle_mod, L, x, skip, flags != "none", flags == "pool_relu")
+    check_within(g, y, s, f"kept-tap kernel {case} {flags}")
+
+
+@pytest.mark.parametrize("case", SMALL)
+@pytest.mark.parametrize("flags", ["none", "skip_relu", "pool_relu"])
 def test_tensor_core_kernel(pp, runner, oracle_mod, case, flags):
     """The 3xTF32 implicit-GEMM kernel on every small case (fewer than 8 input channels: one ragged chunk)."""
     N, Ci, Co, H, W, P, ring, keep = case
@@ -1456,6 +1474,57 @@ def test_default_direct_kernel_by_density(pp, runner, Ci, Co, keep, ring, direct
         assert pp.pp_layer_kernel(d.handle) == (pp.PP_KERNEL_DIRECT if direct else other)
     finally:
         d.close()
+
+
+@pytest.mark.parametrize("Ci,Co,keep,ring,maps", [
+    (64, 32, 0.3, True, [((1, 14, 14), True), ((1, 56, 56), True), ((1, 720, 1280), False)]),
+    (16, 32, 0.2, True, [((1, 56, 56), True), ((2, 97, 131), True), ((1, 720, 1280), False)]),
+    (128, 128, 0.05, False, [((1, 14, 14), True), ((1, 56, 56), False), ((2, 97, 131), False)]),
+])
+def test_direct_kernel_by_map(pp, runner, tmp_path, Ci, Co, keep, ring, maps):
+    """Where neither wins on every map, a layer's launches take the direct kernel or its default by the map; the default
+    runs on every map once it is set."""
+    d = runner.DeviceLayer(synth.small_random_layer(np.random.default_rng(93), Co, Ci, P=8, keep=keep, ring=ring))
+    try:
+        other = pp.pp_layer_kernel(d.handle)
+        assert other == (pp.PP_KERNEL_TMEM if ring else pp.PP_KERNEL_REGISTER)
+        for (N, H, W), direct in maps:
+            x, y = torch.zeros((N, Ci, H, W), device="cuda"), torch.empty((N, Co, H, W), device="cuda")
+            for kernel, want in ((other, False), (pp.PP_KERNEL_AUTO, direct)):
+                pp.pp_layer_set_kernel(d.handle, kernel)
+                assert pp.pp_layer_kernel(d.handle) == other
+                names = launched(lambda: d.forward(x, y, None, N, H, W, 0, torch.cuda.current_stream()), tmp_path)
+                assert ("ppconv_direct" in names[0]) == want, (N, H, W, kernel, names)
+        pp.pp_layer_autotune(d.handle, 1, 14, 14, 0, None)
+        if pp.pp_layer_kernel(d.handle) == pp.PP_KERNEL_DIRECT:  # a tuned layer keeps its kernel
+            x, y = torch.zeros((1, Ci, 720, 1280), device="cuda"), torch.empty((1, Co, 720, 1280), device="cuda")
+            names = launched(lambda: d.forward(x, y, None, 1, 720, 1280, 0, torch.cuda.current_stream()), tmp_path)
+            assert "ppconv_direct" in names[0], names
+    finally:
+        d.close()
+
+
+def test_direct_kernel_by_map_batch_beyond_the_others_grid(pp, runner, oracle_mod):
+    """A batch that the FMA kernel of a layer's default cannot launch runs the direct kernel, whatever the estimates."""
+    N, Ci, Co, H, W = 65536, 16, 32, 4, 4
+    rng = np.random.default_rng(95)
+    L = synth.small_random_layer(rng, Co, Ci, P=8, keep=0.2, ring=True)
+    xs = rng.uniform(-1, 1, (3, Ci, H, W)).astype(np.float32)
+    at = [0, 40000, N - 1]
+    d = runner.DeviceLayer(L)
+    try:
+        assert pp.pp_layer_kernel(d.handle) == pp.PP_KERNEL_TMEM
+        x, y = torch.zeros((N, Ci, H, W), device="cuda"), torch.empty((N, Co, H, W), device="cuda")
+        x[at] = torch.from_numpy(xs).cuda()
+        d.forward(x, y, None, N, H, W, 0, torch.cuda.current_stream())
+        got = y[at].cpu().numpy()
+        pp.pp_layer_set_kernel(d.handle, pp.PP_KERNEL_TMEM)
+        with pytest.raises(pp.PPError):
+            d.forward(x, y, None, N, H, W, 0, torch.cuda.current_stream())
+    finally:
+        d.close()
+    y_ref, s = oracle_layer_full(oracle_mod, L, xs)
+    check_within(got, y_ref, s, "batch beyond the TMEM kernel's grid")
 
 
 def pair_copy_bytes(Co, Ci):
